@@ -118,8 +118,8 @@ typedef struct {
                            orthorhombic fully separable case): rho(n) as a sliced bf16 tcgen05 matrix
                            product over (pair record, i, j), split form and orthorhombic cells only
                            (EUNSUPPORTED otherwise), whole sphere (pair_gcut_eps = 0); the
-                           back-contraction (Alg. S1) takes the same form where the sphere's
-                           (n_a, n_b) rows fit one exact accumulation, else the split walk
+                           back-contraction (Alg. S1) takes the same form where its columns fit the
+                           MMA width and its factor tables shared memory, else the split walk
                            (ftcj_info.j_contraction says which) */
     int tc_wait_log2;   /* tensor-core kernels: each wait between their roles gives up after
                            2^tc_wait_log2 clock cycles (0: 2^32, about 2 s), raises the plan's device
@@ -182,7 +182,7 @@ typedef struct {
                                  product and padding column included) of one structure-factor pass over
                                  max_dens densities; 0 for the walks */
     int j_contraction;        /* the back-contraction's form: FTCJ_CONTRACT_TC where a tensor-core plan's
-                                 rows fit one exact accumulation (<= 672 rows of (n_a, n_b)), else
+                                 columns fit the MMA width and its tables shared memory, else
                                  FTCJ_CONTRACT_WALK */
     int64_t tc_j_mma_flops;   /* the same count for one tensor-core back-contraction; 0 for the walk */
     int tc_column_axis;       /* tensor-core form: the lattice axis of the columns (n_c), 0..2 */

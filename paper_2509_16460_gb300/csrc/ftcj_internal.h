@@ -146,6 +146,12 @@ struct CellConst {
 
 struct Gpw;
 
+// One pass of the tensor-core structure-factor product: windows [w0, w0 + nwin)
+// over ngroups CTA groups, its partial rows from out_row0, its deal at sched.
+struct TcPass {
+    int w0, nwin, ngroups, out_row0, sched;
+};
+
 }  // namespace ftcj
 
 struct ftcj_plan {
@@ -230,33 +236,45 @@ struct ftcj_plan {
     int tc_axis[3] = {0, 1, 2};  // row axes a, b and the column axis c
     int tc_ncols = 0, tc_nd = 0, tc_npad = 0;  // n_c = 0..ncols-1; densities per launch; MMA N
     int tc_colw = 0, tc_G = 0;                 // real columns per (i, j) block; blocks per window
-    int tc_rows = 0, tc_mtiles = 0, tc_nna = 0, tc_nnb = 0, tc_tabw = 0;
-    int64_t tc_nkappa = 0;
-    int tc_nwin = 0, tc_wpg = 0, tc_ngroups = 0;  // K windows, windows per group, groups (partial rows)
-    int tc_tslots = 0;                            // stage-table slots in shared memory
-    int64_t tc_mma_flops = 0;                     // bf16 MMA flops of one pass over max_dens densities
-    void* d_tc_rows = nullptr;   // int2 [rows]
-    int* d_tc_map = nullptr;     // [rows][ncols]
-    int* d_tc_kappa = nullptr;   // [nwin * 512] record ids of each window
+    int tc_rows = 0, tc_nslots = 0;            // signed (n_a, n_b); real row slots (|n_a|, |n_b|, types)
+    int tc_mtiles = 0, tc_nna = 0, tc_nnb = 0, tc_tws = 0;  // tws: X and Y entries per record, rounded up to odd
+    int tc_nwin = 0, tc_wlen = 0;              // K windows, records per window
+    std::vector<ftcj::TcPass> tc_passes;       // window ranges sharing the B workspace
+    int tc_out_rows = 0;                       // partial rows over all passes
+    int tc_nbuf = 0, tc_tslots = 0;            // stage buffers and stage-table slots in shared memory
+    int64_t tc_mma_flops = 0;                  // bf16 MMA flops of one pass over max_dens densities
+    int* d_tc_slots = nullptr;   // [mtiles * 128]
+    int* d_tc_quads = nullptr;   // [nslots / 4]
+    int* d_tc_map = nullptr;     // [2 nna - 1][2 nnb - 1][ncols]
     int* d_tc_wpairs = nullptr;  // (i | j << 3) of the windows' blocks
-    void* d_tc_winfo = nullptr;  // int4 [nwin]: class, blocks, first block
-    void* d_tc_tab = nullptr;    // float4 [npairs][tabw]
-    float* d_tc_cl = nullptr;    // [npairs]
+    void* d_tc_winfo = nullptr;  // int4 [nwin]: class, blocks, first block, first position
+    int* d_tc_wcnt = nullptr;    // [nwin]: records
+    long long* d_tc_boff = nullptr;  // [nwin]: start of the window's B tiles
+    int* d_tc_sched = nullptr;   // per pass: group offsets, then window ids
+    void* d_tc_b = nullptr;      // sliced B stage tiles of one pass
+    void* d_tc_tab = nullptr;    // float4 [npairs][tws], record order
+    void* d_tc_tabk = nullptr;   // the same in the K order of all classes
+    void* d_tc_tabz = nullptr;   // float4 [npairs][ncols], K order
+    float* d_tc_cl = nullptr;    // [npairs] widths, K order
+    int* d_tc_kpos = nullptr;    // [npairs] position of each record in that order
     int* d_tc_err = nullptr;     // device error word of the bounded waits
     int* d_tc_pos = nullptr;     // [npairs]: position of each record in its class's K order
-    int* d_tc_ebw = nullptr;     // [nwin][128]: the windows' column scales, per build
     float* d_tc_clw = nullptr;   // [nwin]: the windows' smallest widths
     long long tc_dp_base[ftcj::kNclass] = {}, tc_dp_stride[ftcj::kNclass] = {}, tc_dp_total = 0;
     // tensor-core form of the back-contraction (tc.cu); false: the split walk runs it
     bool tc_j = false;
-    int tc_jnd = 0, tc_jgw = 0, tc_jG = 0, tc_jnpad = 0;  // densities per launch, columns per density, blocks per item, MMA N
-    int tc_jnstage = 0, tc_jnitems = 0;                     // 8-row stages, work items
-    int tc_jparts = 0, tc_jspp = 0;                         // row parts (one exact accumulation each), stages per part
+    int tc_jnd = 0, tc_jgw = 0, tc_jG = 0, tc_jnpad = 0;  // densities per launch, columns per density, blocks per group, MMA N
+    int tc_jnstage = 0, tc_jgrid = 0, tc_jnbuf = 0;         // 16-slot stages, CTAs, stage buffers
+    int tc_jparts = 0, tc_jspp = 0;                         // slot parts (one exact accumulation each), stages per part
     int64_t tc_j_mma_flops = 0;                             // bf16 MMA flops of one pass over max_dens densities
-    void* d_tc_jitems = nullptr;  // int4 [items]: class, blocks, first block, first record
-    int* d_tc_jpairs = nullptr;   // (i | j << 3) of the items' blocks
-    void* d_tc_vs = nullptr;      // bf16 sliced V_ij stage tiles
-    int* d_tc_ev = nullptr;       // their column scales
+    void* d_tc_jitems = nullptr;   // int4 [units]: class | part << 8, first block group, block groups, first record
+    void* d_tc_jgroups = nullptr;  // int2 [groups]: first block, blocks
+    int* d_tc_jpairs = nullptr;    // (i | j << 3) of the groups' blocks
+    int* d_tc_jsched = nullptr;    // CTA offsets, then unit ids
+    void* d_tc_vs = nullptr;       // bf16 sliced V_ij stage tiles by block group
+    long long* d_tc_voff = nullptr;  // start of each block group's tiles
+    int* d_tc_vplace = nullptr;    // block groups that hold each (i, j)
+    int* d_tc_ev = nullptr;        // their column bounds
     int rho_rows = 0;            // partial rows the rho reduction sums (walk blocks or tensor-core groups)
     // density classification (Sec. 2.6): the records a plan keeps (0 all, 1 compact, 2 DD)
     int rec_filter = 0;

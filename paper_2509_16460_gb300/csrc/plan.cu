@@ -301,10 +301,11 @@ void free_device(ftcj_plan* P) {
                     P->d_gvec, P->d_vg, P->d_tw, P->d_Tmat, P->d_D0n, P->d_J0n, P->d_cbuf0, P->d_cbuf1,
                     P->d_Dp, P->d_Jp, P->d_rho_part, P->d_rho, P->d_W, P->d_Epart, P->d_Dk_stage,
                     P->d_Jk_stage, P->d_EJ_stage, P->d_check, P->d_split_init, P->d_split_const, P->d_Jg,
-                    P->d_maps, P->d_map_off, P->d_sched, P->d_rec_gcut, P->d_tc_rows, P->d_tc_map,
-                    P->d_tc_kappa, P->d_tc_tab, P->d_tc_cl, P->d_tc_err, P->d_tc_wpairs, P->d_tc_winfo,
-                    P->d_tc_pos, P->d_tc_jitems, P->d_tc_jpairs, P->d_tc_vs, P->d_tc_ev,
-                    P->d_tc_ebw, P->d_tc_clw};
+                    P->d_maps, P->d_map_off, P->d_sched, P->d_rec_gcut, P->d_tc_slots, P->d_tc_quads,
+                    P->d_tc_map, P->d_tc_tab, P->d_tc_tabk, P->d_tc_tabz, P->d_tc_kpos, P->d_tc_cl, P->d_tc_err, P->d_tc_wpairs,
+                    P->d_tc_winfo, P->d_tc_wcnt, P->d_tc_boff, P->d_tc_sched, P->d_tc_b, P->d_tc_pos,
+                    P->d_tc_jitems, P->d_tc_jgroups, P->d_tc_jpairs, P->d_tc_jsched, P->d_tc_vs, P->d_tc_ev,
+                    P->d_tc_clw, P->d_tc_voff, P->d_tc_vplace};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     free_gpw(P);
@@ -547,7 +548,7 @@ int create(const ftcj_cell* cell, const ftcj_basis* basis, const int kmesh[3], c
     if ((rc = build_rho_schedule(P))) return rc;
     if (P->tc && !P->ortho) return fail(FTCJ_EUNSUPPORTED, "the tensor-core contraction needs an orthorhombic cell");
     if (P->tc && (rc = setup_tc(P))) return rc;
-    P->rho_rows = P->tc ? P->tc_ngroups : P->npb;
+    P->rho_rows = P->tc ? P->tc_out_rows : P->npb;
 
     size_t nn = (size_t)P->nao * P->nao;
     size_t md = (size_t)P->max_dens;

@@ -1,5 +1,5 @@
-// Tensor-core form of the structure-factor pass (Alg. 1) for orthorhombic
-// cells.
+// Tensor-core form of the structure-factor pass (Alg. 1) and of the
+// back-contraction (Alg. S1) for orthorhombic cells.
 //
 // In an orthorhombic cell the pair prefactor factorises over the three axes
 // (Sec. 2.4, the orthorhombic fully separable case; App. D):
@@ -8,56 +8,79 @@
 // f_a the fractional coordinate of the pair centre.  With a pair record's
 // Hermite densities D'_{ijk} (the walks' convention: the record adds
 // X Y Z sum_ijk D'_ijk (-i n_a)^i (-i n_b)^j (-i n_c)^k to rho(n)),
-//   rho(n_a, n_b, n_c) = sum_{(i,j)} P_ij(n_a, n_b) sum_r A[(n_a, n_b), r] B_ij[r, n_c]
-//   A = X_r(n_a) Y_r(n_b)                              (geometry only)
-//   B_ij = Z_r(n_c) sum_k D'_{r,ijk} (-i n_c)^k         (per density)
-//   P_ij = (-i n_a)^i (-i n_b)^j                        (exact small integers)
-// For the records of one class L, all (i, j) with i + j <= L share A, so the
-// column blocks B_ij (up to G of them side by side) form one complex matrix
-// product over K = records: rows are the (n_a, n_b) of the sphere's
-// projection, columns (i, j) x n_c >= 0 x densities (the stored half sphere
-// maps to n_c >= 0, through -n and a conjugate where n_c < 0).  The powers
-// P_ij are applied to each block's sums when tensor memory is drained, so
-// that A carries only the Gaussian and the phase: a row's entries over a
-// window of records sorted by their width differ little in size, which is
-// what keeps the slicing below at full relative precision.
+//   rho(n_a, n_b, n_c) = sum_{(i,j)} (-i n_a)^i (-i n_b)^j sum_r X_r(n_a) Y_r(n_b) B_ij[r, n_c]
+//   B_ij = Z_r(n_c) sum_k D'_{r,ijk} (-i n_c)^k         (per density).
+//
+// Real form.  X(-n) = conj X(n), so with X(s n) = X_0(n) + i s X_1(n) (real
+// and imaginary part, s = +-1) the four sign combinations of (n_a, n_b) are
+// sums of the four REAL products X_ta(|n_a|) Y_tb(|n_b|), ta, tb in {0, 1}:
+//   X(s_a |n_a|) Y(s_b |n_b|) = sum_{ta,tb} i^{ta+tb} s_a^ta s_b^tb X_ta Y_tb.
+// The matrix product over the records is therefore formed with real A
+// (rows = "slots" (|n_a|, |n_b|, ta, tb), K = records) and complex B
+// (columns = (Re, Im) of (i, j) x n_c >= 0 x densities); the signs are put
+// back when the sums leave the kernel.  Against the complex form (rows
+// (n_a, n_b), two K entries and two columns per complex product) this is half
+// the multiply-adds, half the operand bytes, and one real product per A entry
+// instead of a complex one.  For the records of one class L, all (i, j) with
+// i + j <= L share A, so up to G column blocks B_ij go side by side.  A block
+// contributes with (-i)^{i+j} n_a^i n_b^j, whose sign s_a^i s_b^j moves a
+// product of type (ta, tb) to the sign character (ta + i, tb + j) mod 2: the
+// four slots of a point sit in four adjacent lanes, and the drain exchanges
+// their sums with one xor shuffle per block.  A carries only the Gaussian and
+// the phase, so a row's entries over a window of records sorted by their width
+// differ little in size, which is what keeps the slicing below at full
+// relative precision.
 //
 // Precision.  bf16 products summed in FP32 carry 8 bits; the target is FP64-
 // class.  The operands are therefore split after Ozaki, Ogita, Oishi and Rump
 // ("Error-free transformations of matrix multiplication by using fast
 // routines of matrix multiplication", Numer. Algorithms 59, 2012): every row
-// of A and every column of B, over a window of 512 records, gets a
-// power-of-two scale 2^e bounding its entries, and each entry is cut into six
-// slices m_s 2^{e-6-7s} with integers |m_s| <= 64.  Slice s of A times slice t
-// of B is a tcgen05.mma of kind::f16 (bf16 operands, FP32 accumulator in
-// tensor memory); products with s + t <= 5 are formed (21 per k-step), the
-// others fall below 2^-40 of the window's scale.  Products of the same level
-// s + t land in one accumulator: levels 0, 1, 2 are exact integer sums
-// (|m| <= 64, at most 3 products per level and 1024 real K terms per window
-// keep every partial sum below 2^24), levels 3..5 share a fourth, rounded
-// accumulator.  At each window's end the accumulators are scaled by
-// 2^{eA+eB}, multiplied by P_ij and added in double-float (FP32 pairs,
-// df.cuh) to sums kept in tensor memory, which are written as FP64 partial
-// rows and summed across window groups in fixed order by the row reduction.
+// of A and every column of B, over a window of at most 1024 records, gets a
+// power-of-two bound 2^e of its entries, and each entry is cut into six slices
+// m_s 2^{e-6-7s} with integers |m_s| <= 64 (kept at their own magnitude: bf16
+// has FP32's exponent range, so no scaling is undone later).  Slice s of A
+// times slice t of B is a tcgen05.mma of kind::f16 (bf16 operands, FP32
+// accumulator in tensor memory); products with s + t <= 5 are formed (21 per
+// k-step), the others fall below 2^-40 of the window's scale.  Products of the
+// same level s + t land in one accumulator: levels 0 to 3 are exact integer
+// sums (|m| <= 64, at most 4 products per level and 1024 K terms keep every
+// partial sum at or below 2^24), levels 4 and 5 share a fifth, rounded
+// accumulator, 2^-28 of the first.  At each window's end the level sums are
+// added in double-float (FP32 pairs, df.cuh) to sums kept in registers, which
+// are written as FP64 partial rows and summed across window groups in fixed
+// order by the row reduction.
 //
-// Kernel shape (one CTA per SM: 512 tensor-memory columns and ~200 KB of
-// shared memory), thirteen warps: warps 0-10 form the operand slices of a
-// 16-record stage into one of two shared-memory buffers (plain 16-byte stores
-// in the no-swizzle K-major core-matrix layout the MMA descriptors name);
-// lane 0 of warp 11 issues the MMAs; warp 12 stages each stage's record
-// factor tables with bulk copies (cp.async.bulk, completion counted in bytes
-// on an mbarrier) and their Hermite terms into a ring of shared-memory slots
-// ahead of use.  Warps 0-11 also compute the window scales and drain tensor
-// memory.  Stages are handed over with mbarriers (arrivals; tcgen05.commit
-// for the MMA side).  Every wait is bounded: past ~2 s of clock a waiting
-// thread raises the CTA's abort flag and the plan's device error word, every
-// thread leaves its loops, the copies and MMAs in flight are waited for
-// (again bounded) and tensor memory is freed before the CTA exits.
+// Kernel shape.  B does not depend on the row, and a sphere has several row
+// tiles, so B is sliced once per build (k_tc_rho_b) into stage tiles in global
+// memory, already in the core-matrix layout of the MMA descriptors, and comes
+// in with one bulk copy per stage.  k_tc_rho runs one CTA per SM (512
+// tensor-memory columns, ~200 KB of shared memory), 19 warps: warps 0-15, two
+// groups in turn, form the A slices of a 16-record stage (one thread per row
+// and eight records: one 16-byte core-matrix row per slice) into a ring of up
+// to four buffers; one elected lane of warp 16 issues the MMAs; warp 17 brings
+// the records' factor tables and warp 18 the B tiles in (cp.async.bulk,
+// completion counted in bytes on mbarriers).  Warps 0-15 also drain tensor
+// memory.  Stages are handed over with mbarriers (arrivals; tcgen05.commit for
+// the MMA side).  Every wait is bounded: past ~2 s of clock a waiting thread
+// raises the CTA's abort flag and the plan's device error word, every thread
+// leaves its loops, the copies and MMAs in flight are waited for (again
+// bounded) and tensor memory is freed before the CTA exits.
+//
+// What bounds it (molecular crystal, 1056 AOs, 2 densities, GB300): the product
+// takes 1.07 ms, of which the MMAs alone (operands left unformed) need 0.89 ms:
+// their operand reads from shared memory (15 MMAs of N = 96 or 192 per k-step,
+// 123 KB) beside the operand and table writes.  B tiles in global memory cost
+// 0.28 ms more (0.49 GB written).  What took the pass from 4.76 ms there: the
+// real form (half of everything), B formed once instead of once per row tile,
+// one bulk copy per stage instead of one per record and block (each copy takes
+// ~100 cycles of the copy engine whatever its size: 1.32 ms for the loads
+// alone), and MMAs issued from warp-uniform code (1.57 -> 1.35 ms).
 #include <cuda_bf16.h>
 
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <queue>
 #include <set>
 #include <vector>
 
@@ -68,50 +91,60 @@ namespace ftcj {
 namespace {
 
 constexpr int kTcM = 128;                      // rows per tile (MMA M)
-constexpr int kTcStageK = 16;                  // records per stage: two MMA k-steps of 16 real (re, im)
-constexpr int kTcWin = 512;                    // records per exact-accumulation window (1024 real K)
-constexpr int kTcStagesPerWin = kTcWin / kTcStageK;
-constexpr int kTcNmma = 256;                   // MMA N at most
+constexpr int kTcStageK = 16;                  // records per stage: one MMA k-step
+constexpr int kTcWinMax = 1024;                // records per exact-accumulation window at most
+constexpr int kTcNmax = 96;                    // MMA N at most: five level accumulators in the 512 columns
 constexpr int kTcS = 6;                        // slices per operand
-constexpr int kTcAcc = 4;                      // accumulators: levels 0, 1, 2 exact, levels 3..5 rounded
+constexpr int kTcAcc = 5;                      // accumulators: levels 0-3 exact, levels 4, 5 rounded
 constexpr int kTcTmemCols = 512;
 constexpr int kTcGmax = 15;                    // (i, j) blocks per window at most (class 4 has 15)
-constexpr int kTcEbMax = 128;                  // column scales per window at most
-constexpr int kTcNbuf = 2;                     // stage buffers
-constexpr int kTcTabSlotsMax = 4;              // stage tables in flight
-constexpr int kTcAsliceBytes = kTcM * 2 * kTcStageK * 2;  // 128 rows x 32 real K x bf16
+constexpr int kTcNbufMax = 4;                  // stage buffers at most
+constexpr int kTcTabSlotsMax = 6;              // stage tables in flight at most
+constexpr int kTcAsliceBytes = kTcM * kTcStageK * 2;      // 128 rows x 16 K x bf16
+constexpr long long kTcBWorkMax = 8LL << 30;              // bytes of B tiles per pass
 constexpr long long kTcSpinCycles = 1LL << 32;            // ~2 s of SM clock per wait
 
+// a slot: bits 0-7 |n_a|, 8-15 |n_b|, 16 ta, 17 tb, 18 / 19: the lane's bit 0
+// (1) is the sign of n_a (n_b), 20: valid
+__host__ __device__ constexpr int slot_pack(int na, int nb, int ta, int tb, int da, int db, int valid) {
+    return na | (nb << 8) | (ta << 16) | (tb << 17) | (da << 18) | (db << 19) | (valid << 20);
+}
+
 struct TcArgs {
-    const int2* rows;    // (n_a, n_b) per row
-    const int* map;      // [rows][ncols]: half-sphere index, ~index where the stored point is -n, INT_MIN none
-    const int* wrec;     // [nwin][kTcWin]: record ids of each window, -1 for padding
+    const int* slots;    // row slots, a multiple of kTcM
+    const int* map;      // [2 nam + 1][2 nbm + 1][ncols]: half-sphere index of (n_a, n_b, n_c), ~index where the
+                         // stored point is -n, INT_MIN none
     const int4* winfo;   // [nwin]: class L, number of (i,j) blocks, first block index into wpairs,
                          // position of the window's first record in its class's K order
+    const int* wcnt;     // [nwin]: records of the window
+    const long long* boff;  // [nwin]: start of the window's B tiles in bs (16-byte units)
+    const int* sched;    // [ngroups + 1] offsets, then window ids grouped by CTA group
     const int* wpairs;   // (i | j << 3) of each block
-    const float4* tab;   // per record [tabw]: X(0..), Y(0..), Z(0..) as complex double-float
-    const float* cl;     // per record c log2(e)
+    const float4* tabk;  // X(0..), Y(0..) as complex double-float, [tws] per record in the K order of all classes
+    const float4* tabz;  // Z(0..), [ncols] per record in the same order
+    const float* clk;    // c log2(e) in the same order
+    long long kbase[kNclass];  // first record of each class in that order
     const float2* Dp;    // Hermite densities (double-float) in the K order: [dens][class][term][position]
     long long dp_total;
     long long dp_base[kNclass];
     long long dp_stride[kNclass];
-    double2* out;        // partial rows [dens][ngroups][ng_half]
+    uint4* bs;           // sliced B stage tiles of this pass
+    float* clw;          // [nwin]: smallest c log2(e) of each window's records
+    double2* out;        // partial rows [dens][out_rows][ng_half], this pass's from out_row0
     long long ng_half;
+    int out_rows, out_row0;
     int* err;            // device error word (bit 0: a bounded wait gave up)
     float Maa, Mbb, Mcc;
     int ax, bx, cx;      // lattice axes of the row indices (a, b) and of the column index (c)
-    int tabw, offY, offZ;
+    int nam, nbm;
+    int tws, offY;       // table entries per record (X and Y, rounded up to odd), start of Y
     int ncols;           // complex columns per density and block: n_c = 0 .. ncols-1
     int nd, d0;          // densities of this launch, first density
-    int colw;            // real columns per block: 2 nd ncols
-    int G;               // blocks per window at most
-    int npad;            // MMA N: G colw rounded up to 16
-    int accw;            // real columns of the double-float sums: colw rounded up to 8
-    int nwin, win_per_group, ngroups;
-    int nrows;
+    int colw;            // real columns per block: 2 nd ncols rounded up to 8
+    int npad;            // MMA N of a full window: G colw rounded up to 16
+    int w0;              // first window of this pass
+    int nslots;
     long long spin;      // clock cycles a wait between roles may take before it gives up
-    int* ebw;            // [nwin][kTcEbMax]: column scales of each window (k_tc_rho_bounds)
-    float* clw;          // [nwin]: smallest c log2(e) of each window's records
 };
 
 // ---- PTX wrappers -----------------------------------------------------------
@@ -150,15 +183,15 @@ __device__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag
     return true;
 }
 
-// A bounded barrier of the eight operand warps (an mbarrier counting one
-// arrival per warp): unlike bar.sync it cannot hang when a thread has left
-// after a failed wait.  The outcome is the same for every lane of a warp.
-__device__ bool prod_sync(uint64_t* b, uint32_t& ph, volatile int* abort_flag, int lane, long long spin) {
-    __syncwarp();
-    if (lane == 0) mbar_arrive(b);
-    const bool ok = mbar_wait(b, ph, abort_flag, spin);
-    ph ^= 1u;
-    return __all_sync(0xffffffffu, ok);
+// One lane of a converged warp, always the same one.  The MMA warp runs its
+// loops with all lanes on warp-uniform values and only the MMAs and commits
+// under this predicate, so that descriptors stay in uniform registers: with
+// the loops inside a one-lane branch every MMA cost ~90 cycles of register
+// moves, whatever its width.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+    return p != 0;
 }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -166,9 +199,9 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 
 // shared-memory matrix descriptor: K-major, no swizzle, core matrices of 8
 // rows x 16 B; K-adjacent core matrices 128 B apart (leading byte offset),
-// 8-row groups 512 B apart (stride byte offset: 32 real K per stage row)
+// 8-row groups 256 B apart (stride byte offset: 16 K per stage row)
 __device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
-    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(128u >> 4) << 16) | ((uint64_t)(512u >> 4) << 32) |
+    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(128u >> 4) << 16) | ((uint64_t)(256u >> 4) << 32) |
            (1ull << 46);
 }
 
@@ -185,25 +218,74 @@ __device__ __forceinline__ void tc_commit(uint64_t* b) {
                  : "memory");
 }
 
-__device__ __forceinline__ void tc_ld8(uint32_t taddr, float (&v)[8]) {
-    uint32_t r[8];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+// The slice products of one k-step, A_s B_t with s + t < S, into the level
+// accumulators min(s + t, ACC - 1) (nw columns each, side by side).  The slices
+// of B follow each other in shared memory in the same core-matrix layout, so up
+// to W of them whose levels have accumulators of their own go into one MMA of
+// N = W nw columns (<= 256): A_s is then read from shared memory once for all
+// of them, and fewer MMAs are issued.  acc false: the window's first k-step,
+// whose s = 0 products start each level's accumulator.
+template <int S, int ACC, int W>
+__device__ __forceinline__ void issue_kstep(uint32_t tmem, uint64_t ad, uint32_t astep, uint64_t bd, uint32_t bstep,
+                                            uint32_t nw, uint32_t idesc, bool acc) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+    for (int s = 0; s < S; ++s) {
+        const int nt = S - s;  // t = 0 .. nt - 1
+#pragma unroll
+        for (int t = 0; t < nt; ++t) {
+            const int own = ACC - s;  // t below this has a level accumulator that no other t of this s shares
+            const int lead = t < own ? t % W : 0;
+            if (lead != 0) continue;  // part of the previous MMA
+            const int lim = own < nt ? own : nt;
+            const int n = t < own ? (lim - t < W ? lim - t : W) : 1;
+            const int lv = s + t < ACC - 1 ? s + t : ACC - 1;
+            const uint32_t on = s == 0 && t < ACC ? (acc ? 1u : 0u) : 1u;
+            tc_mma(tmem + (uint32_t)lv * nw, ad + (uint64_t)(s * astep), bd + (uint64_t)(t * bstep),
+                   idesc + ((((uint32_t)n * nw) >> 3) << 17), on);
+        }
+    }
 }
 
-__device__ __forceinline__ void tc_st8(uint32_t taddr, const float (&v)[8]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr),
-                 "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
-                 "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
-                 "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7]))
-                 : "memory");
+// W slices side by side for nw columns each
+template <int S, int ACC>
+__device__ __forceinline__ void issue_kstep(uint32_t tmem, uint64_t ad, uint32_t astep, uint64_t bd, uint32_t bstep,
+                                            uint32_t nw, uint32_t idesc, bool acc) {
+    if (nw > 80) issue_kstep<S, ACC, 2>(tmem, ad, astep, bd, bstep, nw, idesc, acc);
+    else if (nw > 64) issue_kstep<S, ACC, 3>(tmem, ad, astep, bd, bstep, nw, idesc, acc);
+    else if (nw > 48) issue_kstep<S, ACC, 4>(tmem, ad, astep, bd, bstep, nw, idesc, acc);
+    else issue_kstep<S, ACC, 5>(tmem, ad, astep, bd, bstep, nw, idesc, acc);
 }
 
-__device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// Tensor-memory reads of 4 (8) columns of the five level accumulators, npad
+// columns apart, with the wait for them in the same statement, so that no use
+// of the values can be scheduled before it.
+__device__ __forceinline__ void tc_ld_levels4(uint32_t taddr, uint32_t npad, float (&v)[5][4]) {
+    uint32_t r[20];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%20];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%21];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%8,%9,%10,%11}, [%22];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%12,%13,%14,%15}, [%23];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%16,%17,%18,%19}, [%24];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19])
+        : "r"(taddr), "r"(taddr + npad), "r"(taddr + 2 * npad), "r"(taddr + 3 * npad), "r"(taddr + 4 * npad)
+        : "memory");
+#pragma unroll
+    for (int l = 0; l < 5; ++l)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[l][i] = __uint_as_float(r[4 * l + i]);
+}
+
+// the sum of the five level sums of one real output, double-float (|lo| may
+// exceed ulp(hi)/2 by a few units)
+__device__ __forceinline__ df level_sum(float t0, float t1, float t2, float t3, float t4) {
+    const df a = two_sum(t0, t1), b = two_sum(t2, t3);
+    const df s = two_sum(a.hi, b.hi);
+    return df{s.hi, __fadd_rn(__fadd_rn(s.lo, a.lo), __fadd_rn(b.lo, t4))};
+}
 
 // ---- operand slices ---------------------------------------------------------
 
@@ -213,38 +295,59 @@ __device__ __forceinline__ float pow2f(int k) {
     return __int_as_float((k + 127) << 23);
 }
 
-// Slices of x = hi + lo (|x| < 2^e, sc = 2^(6-e)): o[s] = m_s 2^(-7s) with
-// integers |m_s| <= 64 (<= 72 for s = 3, which takes the low part's
-// rounding), so that x = 2^(e-6) sum_s o[s] up to 2^(e-41).  Each slice rounds
-// the remainder to a multiple of 2^(-7s) by adding and subtracting 1.5 x
-// 2^(23-7s) (round to nearest even, no fast-math reassociation); slices 0-2
-// peel the high part exactly, the low part joins at slice 3 with one rounding
-// below 2^(e-45).
-__device__ __forceinline__ void slice6(float hi, float lo, float sc, float (&o)[kTcS]) {
-    float h = hi * sc;
-    const float l = lo * sc;
-    o[0] = (h + 0x1.8p23f) - 0x1.8p23f;
-    h -= o[0];
-    o[1] = (h + 0x1.8p16f) - 0x1.8p16f;
-    h -= o[1];
-    o[2] = (h + 0x1.8p9f) - 0x1.8p9f;
-    h = (h - o[2]) + l;
-    o[3] = (h + 0x1.8p2f) - 0x1.8p2f;
-    h -= o[3];
-    o[4] = (h + 0x1.8p-5f) - 0x1.8p-5f;
-    h -= o[4];
-    o[5] = (h + 0x1.8p-12f) - 0x1.8p-12f;
-}
+// Slices of x = h + l (|x| < 2^e): o[s] = m_s u 2^(-7s) with u = 2^(e-6) and
+// integers |m_s| <= 64 (<= 72 for s = 3, which takes the low part's rounding),
+// so that x = sum_s o[s] up to 2^(e-41).  Each slice rounds the remainder to a
+// multiple of u 2^(-7s) by adding and subtracting 1.5 x 2^(23-7s) u (round to
+// nearest even, no fast-math reassociation); slices 0-2 peel the high part
+// exactly, the low part joins at slice 3 with one rounding below 2^(e-45).
+struct Slicer6 {
+    float c[kTcS];
+    __device__ __forceinline__ explicit Slicer6(float u) {
+        c[0] = 0x1.8p23f * u;
+        c[1] = 0x1.8p16f * u;
+        c[2] = 0x1.8p9f * u;
+        c[3] = 0x1.8p2f * u;
+        c[4] = 0x1.8p-5f * u;
+        c[5] = 0x1.8p-12f * u;
+    }
+    __device__ __forceinline__ void operator()(float h, float l, float (&o)[kTcS]) const {
+        o[0] = __fsub_rn(__fadd_rn(h, c[0]), c[0]);
+        h = __fsub_rn(h, o[0]);
+        o[1] = __fsub_rn(__fadd_rn(h, c[1]), c[1]);
+        h = __fsub_rn(h, o[1]);
+        o[2] = __fsub_rn(__fadd_rn(h, c[2]), c[2]);
+        h = __fadd_rn(__fsub_rn(h, o[2]), l);
+        o[3] = __fsub_rn(__fadd_rn(h, c[3]), c[3]);
+        h = __fsub_rn(h, o[3]);
+        o[4] = __fsub_rn(__fadd_rn(h, c[4]), c[4]);
+        h = __fsub_rn(h, o[4]);
+        o[5] = __fsub_rn(__fadd_rn(h, c[5]), c[5]);
+    }
+};
 
 __device__ __forceinline__ uint32_t pack_bf2(float a, float b) {
     __nv_bfloat162 v = __floats2bfloat162_rn(a, b);  // exact: every slice has <= 8 significant bits
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// element offset of (row, k) in a stage tile [rows][32 real K] of core matrices
+// element offset of (row, k) in a stage tile [rows][16 K] of core matrices
 __device__ __forceinline__ int tile_off(int row, int k) {
-    return (((row >> 3) * 4 + (k >> 3)) << 6) + ((row & 7) << 3) + (k & 7);
+    return (((row >> 3) * 2 + (k >> 3)) << 6) + ((row & 7) << 3) + (k & 7);
 }
+
+// stage counter of a ring of n buffers: index and phase parity
+struct Ring {
+    int i = 0, n;
+    uint32_t ph = 0;
+    __device__ __forceinline__ explicit Ring(int n_) : n(n_) {}
+    __device__ __forceinline__ void next() {
+        if (++i == n) {
+            i = 0;
+            ph ^= 1u;
+        }
+    }
+};
 
 // (-i)^p z
 __device__ __forceinline__ cdf rot_mi(cdf z, int p) {
@@ -262,34 +365,6 @@ __device__ __forceinline__ int exp_bound(float log2_bound) {
     return (int)floorf(log2_bound + 1e-3f) + 1;
 }
 
-struct TcRow {
-    int na, nb;
-    float Q;  // M_aa na^2 + M_bb nb^2
-};
-
-struct TcSmem {
-    int rec[kTcWin];
-    int pairs[kTcGmax];
-    int tidx[kTcGmax][5];  // index of D'_{ijk} for block (i, j) and k = 0..4 (-1 past the class's degree)
-    int eA[kTcM];
-    int eB[kTcEbMax];
-    TcRow rowi[kTcM];
-    int winL, wnpair, wpos, clmin_bits;
-    uint64_t full[kTcNbuf], empty[kTcNbuf], accf, acce, done, psync;
-    uint64_t tfull[kTcTabSlotsMax], tempty[kTcTabSlotsMax];
-    uint32_t tmem;
-    int abort_flag;
-};
-
-// One table slot of a stage: the 16 records' factor tables (copied whole by
-// the bulk-copy engine, tabw float4 each), then the Hermite terms D'_{ijk} of
-// the 16 records as rows [block][density][k = 0..4][record] (one 128-byte
-// bulk copy per row; rows past the block's degree are not written or read).
-__host__ __device__ inline size_t tab_slot_bytes(int tabw, int G, int nd) {
-    const size_t b = (size_t)kTcStageK * tabw * 16 + (size_t)G * nd * 5 * kTcStageK * 8;
-    return (b + 127) / 128 * 128;
-}
-
 __device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(saddr(dst)), "l"(src), "r"(bytes), "r"(saddr(bar))
@@ -303,225 +378,215 @@ __device__ __forceinline__ void mbar_arrive_tx(uint64_t* b, uint32_t tx) {
 }
 
 // index of D'_{p1 p2 p3} (powers of n_1, n_2, n_3) for powers (i, j, k) of (n_a, n_b, n_c)
-__device__ __forceinline__ int term_of(const TcArgs& g, int i, int j, int k) {
-    const int p1 = g.ax == 0 ? i : (g.bx == 0 ? j : k);
-    const int p2 = g.ax == 1 ? i : (g.bx == 1 ? j : k);
+__device__ __forceinline__ int term_of(int ax, int bx, int i, int j, int k) {
+    const int p1 = ax == 0 ? i : (bx == 0 ? j : k);
+    const int p2 = ax == 1 ? i : (bx == 1 ? j : k);
     const int lam = i + j + k;
     return lam_offset(lam) + mono_index(lam, p1, p2);
 }
 
-// A: the four records of group gg (stage-local 4 gg .. 4 gg + 3) for one row,
-// X_r(n_a) Y_r(n_b) sliced, as six 16-byte stores (one core-matrix row per slice)
-__device__ __forceinline__ void form_a(const TcArgs& g, const TcSmem& sm, const float4* tabs, int q, int row,
-                                       int gg, float scA, unsigned char* as) {
-    const TcRow ri = sm.rowi[row];
-    const bool rvalid = ri.na != INT_MIN;
-    const float sa = ri.na < 0 ? -1.f : 1.f, sb = ri.nb < 0 ? -1.f : 1.f;  // X(-n) = conj X(n)
-    const int ia = abs(ri.na), ib = g.offY + abs(ri.nb);
-    float sl[kTcS][8];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int kq = gg * 4 + u;
-        cdf a{{0.f, 0.f}, {0.f, 0.f}};
-        if (rvalid && sm.rec[q * kTcStageK + kq] >= 0) {
-            const float4 xv = tabs[kq * g.tabw + ia], yv = tabs[kq * g.tabw + ib];
-            a = cdf_mul(cdf{{xv.x, xv.y}, {sa * xv.z, sa * xv.w}}, cdf{{yv.x, yv.y}, {sb * yv.z, sb * yv.w}});
-        }
-        float sr[kTcS], si[kTcS];
-        slice6(a.re.hi, a.re.lo, scA, sr);
-        slice6(a.im.hi, a.im.lo, scA, si);
-#pragma unroll
-        for (int s = 0; s < kTcS; ++s) {
-            sl[s][2 * u] = sr[s];
-            sl[s][2 * u + 1] = si[s];
-        }
-    }
-    const int off = tile_off(row, gg * 8);
-#pragma unroll
-    for (int s = 0; s < kTcS; ++s) {
-        uint4 v;
-        v.x = pack_bf2(sl[s][0], sl[s][1]);
-        v.y = pack_bf2(sl[s][2], sl[s][3]);
-        v.z = pack_bf2(sl[s][4], sl[s][5]);
-        v.w = pack_bf2(sl[s][6], sl[s][7]);
-        *reinterpret_cast<uint4*>(as + (size_t)s * kTcAsliceBytes + (size_t)off * 2) = v;
-    }
+// |n|^k for k <= 4, exact
+__device__ __forceinline__ float ipow(float n, int k) {
+    float p = 1.f;
+    for (int q = 0; q < k; ++q) p *= n;
+    return p;
 }
 
-// B: four records (stage-local 4 kg .. 4 kg + 3) of one (block gb, output pair
-// p = n_c nd + d), sliced, in the real form rows (record, re) -> [Re B | Im B],
-// (record, im) -> [-Im B | Re B]: columns gb colw + 2p and + 1, one 16-byte
-// core-matrix row per slice and column.  Blocks past the window's count are zero.
-__device__ __forceinline__ void form_b(const TcArgs& g, const TcSmem& sm, const float4* tabs, const float2* dps,
-                                       int q, int kg, int gb, int p, unsigned char* bs, int bslice) {
-    const int nc = p / g.nd, d = p - nc * g.nd;
-    float s0[kTcS][8], s1[kTcS][8];  // column 2p: (Re, -Im) per record; column 2p + 1: (Im, Re)
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int kq = kg * 4 + u;
-        cdf bv{{0.f, 0.f}, {0.f, 0.f}};
-        if (gb < sm.wnpair && sm.rec[q * kTcStageK + kq] >= 0) {
-            const float4 zv = tabs[kq * g.tabw + g.offZ + nc];
-            const float2* dv = dps + (gb * g.nd + d) * 5 * kTcStageK + kq;
-            const int pr = sm.pairs[gb], nk = sm.winL - (pr & 7) - (pr >> 3);  // k = 0 .. L - i - j
-            df re{0.f, 0.f}, im{0.f, 0.f};
-            float pw = 1.f;
-#pragma unroll
-            for (int kk = 0; kk < 5; ++kk) {
-                if (kk > nk) break;
-                const float2 v = dv[kk * kTcStageK];
-                const df term = df_mulf(df{v.x, v.y}, pw);  // D'_k n_c^k, exact power
-                switch (kk & 3) {                           // (-i)^k
-                    case 0: re = df_add(re, term); break;
-                    case 1: im = df_sub(im, term); break;
-                    case 2: re = df_sub(re, term); break;
-                    default: im = df_add(im, term); break;
-                }
-                pw *= (float)nc;
-            }
-            bv = cdf_mul(cdf{{zv.x, zv.y}, {zv.z, zv.w}}, cdf{re, im});
-        }
-        const float scB = pow2f(6 - sm.eB[gb * g.ncols * g.nd + p]);
-        float sr[kTcS], si[kTcS];
-        slice6(bv.re.hi, bv.re.lo, scB, sr);
-        slice6(bv.im.hi, bv.im.lo, scB, si);
-#pragma unroll
-        for (int s = 0; s < kTcS; ++s) {
-            s0[s][2 * u] = sr[s];
-            s0[s][2 * u + 1] = -si[s];
-            s1[s][2 * u] = si[s];
-            s1[s][2 * u + 1] = sr[s];
-        }
-    }
-    const int c0 = gb * g.colw + 2 * p;
-    const int o0 = tile_off(c0, kg * 8), o1 = tile_off(c0 + 1, kg * 8);
-#pragma unroll
-    for (int s = 0; s < kTcS; ++s) {
-        uint4 v;
-        v.x = pack_bf2(s0[s][0], s0[s][1]);
-        v.y = pack_bf2(s0[s][2], s0[s][3]);
-        v.z = pack_bf2(s0[s][4], s0[s][5]);
-        v.w = pack_bf2(s0[s][6], s0[s][7]);
-        *reinterpret_cast<uint4*>(bs + (size_t)s * bslice + (size_t)o0 * 2) = v;
-        v.x = pack_bf2(s1[s][0], s1[s][1]);
-        v.y = pack_bf2(s1[s][2], s1[s][3]);
-        v.z = pack_bf2(s1[s][4], s1[s][5]);
-        v.w = pack_bf2(s1[s][6], s1[s][7]);
-        *reinterpret_cast<uint4*>(bs + (size_t)s * bslice + (size_t)o1 * 2) = v;
-    }
-}
+// columns of an MMA over nb blocks
+__host__ __device__ __forceinline__ int mma_cols(int nb, int colw) { return (nb * colw + 15) / 16 * 16; }
 
-constexpr int kTcProdWarps = 14;
-constexpr int kTcProdThreads = kTcProdWarps * 32;
-constexpr int kTcMmaWarp = 14;
-constexpr int kTcLoadWarp = 15;
-constexpr int kTcWarps = 16;
-constexpr int kTcEpiWarps = 12;
-constexpr int kTcEpiThreads = kTcEpiWarps * 32;
+constexpr int kTcProdWarps = 16;                    // two groups of eight, stages in turn
+constexpr int kTcGroupWarps = kTcProdWarps / 2;
+constexpr int kTcMmaWarp = 16;
+constexpr int kTcTabWarp = 17;
+constexpr int kTcLoadWarp = 18;
+constexpr int kTcWarps = 19;
 constexpr int kTcThreadsAll = kTcWarps * 32;
-constexpr int kTcTasksMax = 3;        // operand tasks per thread and stage: (512 + 4 G npo) / 448 <= 3
-constexpr int kTcTaskA = 1 << 20;     // task flag: an A task (row | group << 7), else a B task
 
-// Per window (one block each), once per build and density group: the
-// window's smallest width c (every row of A gets the scale exp(-c_min Q))
-// and the column scales of B, |B_ij| <= exp(-c Mcc n^2) sum_k |D'_ijk| n^k,
-// maximised over the window's records, per (block, n_c, density).
-__global__ void __launch_bounds__(256) k_tc_rho_bounds(TcArgs g) {
-    __shared__ int eB[kTcEbMax];
-    __shared__ int tidx[kTcGmax][5];
+// ---- B: window scales and slices, once per build and density group ---------
+
+constexpr int kTcBThreads = 512;
+
+// One block per window.  First the scales: the window's smallest width c
+// (every row of A gets the bound exp(-c_min Q)) and the column bounds of B,
+// |B_ij| <= exp(-c Mcc n^2) sum_k |D'_ijk| n^k maximised over the window's
+// records, per (block, n_c, density).  Then the slices: one thread per four
+// records of one (block, n_c, density), both columns (Re, Im), as halves of
+// 16-byte core-matrix rows; neighbouring lanes take the other half, neighbouring
+// columns and record octets, so a warp's stores of one slice fill 512-byte runs.
+__global__ void __launch_bounds__(kTcBThreads, 2) k_tc_rho_b(TcArgs g) {
+    __shared__ int mx[kTcNmax / 2];  // bits of the column bounds (non-negative floats order as integers)
+    __shared__ int pairs[kTcGmax], tidx[kTcGmax][5];
     __shared__ int clmin_bits;
-    const int w = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+    const int w = g.w0 + blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     const int4 wi = __ldg(g.winfo + w);
-    const int L = wi.x, npair = wi.y, npo = g.nd * g.ncols;
-    for (int i = tid; i < kTcEbMax; i += blockDim.x) eB[i] = -100;
-    if (tid == 0) {
-        for (int b = 0; b < npair; ++b) {
-            const int pr = __ldg(g.wpairs + wi.z + b), i = pr & 7, j = pr >> 3;
-            for (int kk = 0; kk < 5; ++kk) tidx[b][kk] = kk <= L - i - j ? term_of(g, i, j, kk) : -1;
-        }
-        clmin_bits = __float_as_int(INFINITY);
+    const int L = wi.x, npair = wi.y, npo = g.nd * g.ncols, cnt = __ldg(g.wcnt + w);
+    for (int i = tid; i < npair * npo; i += blockDim.x) mx[i] = 0;
+    if (tid < npair) {
+        const int pr = __ldg(g.wpairs + wi.z + tid), i = pr & 7, j = pr >> 3;
+        pairs[tid] = pr;
+        for (int kk = 0; kk < 5; ++kk) tidx[tid][kk] = kk <= L - i - j ? term_of(g.ax, g.bx, i, j, kk) : -1;
     }
+    if (tid == 0) clmin_bits = __float_as_int(INFINITY);
     __syncthreads();
-    const long long cnt = g.dp_stride[L];
-    const float2* dpL = g.Dp + g.dp_base[L];
-    float cmin = INFINITY;
-    for (int k = tid; k < kTcWin; k += blockDim.x) {  // warp-uniform trip count (512 / 256)
-        const int r = __ldg(g.wrec + (size_t)w * kTcWin + k);
-        const float cr = r >= 0 ? __ldg(g.cl + r) : 0.f;
-        if (r >= 0) cmin = fminf(cmin, cr);
-        const long long loc = wi.w + k;
-        for (int gb = 0; gb < npair; ++gb) {
-            for (int d = 0; d < g.nd; ++d) {
-                float cm[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-                if (r >= 0) {
-                    const float2* dp = dpL + (long long)(g.d0 + d) * g.dp_total + loc;
+    const long long stride = g.dp_stride[L];
+    const float2* dpw = g.Dp + g.dp_base[L] + (long long)g.d0 * g.dp_total + wi.w;
+    const long long kb = g.kbase[L] + wi.w;  // the window's first record in the K order
+    constexpr int kIt = kTcWinMax / kTcBThreads;
+    float cr[kIt], cmin = INFINITY;
 #pragma unroll
-                    for (int kk = 0; kk < 5; ++kk) {
-                        const int t = tidx[gb][kk];
-                        if (t >= 0) cm[kk] = fabsf(__ldg(dp + (long long)t * cnt).x) * 1.0001f;
-                    }
-                }
-                for (int nc = 0; nc < g.ncols; ++nc) {
-                    const float x = (float)nc;
-                    const float sv = cm[0] + x * (cm[1] + x * (cm[2] + x * (cm[3] + x * cm[4])));
-                    int eb = r >= 0 && sv > 0.f ? exp_bound(log2f(sv) - cr * g.Mcc * x * x) : -100;
-                    eb = __reduce_max_sync(0xffffffffu, eb);  // warp maximum, one shared atomic per warp
-                    if (lane == 0) atomicMax(&eB[gb * npo + nc * g.nd + d], eb);
+    for (int q = 0; q < kIt; ++q) {
+        const int k = tid + q * kTcBThreads;
+        cr[q] = k < cnt ? __ldg(g.clk + kb + k) : 0.f;
+        if (k < cnt) cmin = fminf(cmin, cr[q]);
+    }
+    for (int gb = 0; gb < npair; ++gb)
+        for (int d = 0; d < g.nd; ++d) {
+            float cm[kIt][5];
+#pragma unroll
+            for (int q = 0; q < kIt; ++q) {
+                const int k = tid + q * kTcBThreads;
+                const float2* dp = dpw + (long long)d * g.dp_total + k;
+#pragma unroll
+                for (int kk = 0; kk < 5; ++kk) {
+                    const int t = tidx[gb][kk];
+                    cm[q][kk] = t >= 0 && k < cnt ? fabsf(__ldg(dp + (long long)t * stride).x) * 1.0001f : 0.f;
                 }
             }
+            for (int nc = 0; nc < g.ncols; ++nc) {
+                const float x = (float)nc, mq = -g.Mcc * x * x;
+                float m = 0.f;
+#pragma unroll
+                for (int q = 0; q < kIt; ++q) {
+                    const float sv = cm[q][0] + x * (cm[q][1] + x * (cm[q][2] + x * (cm[q][3] + x * cm[q][4])));
+                    m = fmaxf(m, sv * exp2f(cr[q] * mq));
+                }
+                const unsigned mb = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+                if (lane == 0 && mb) atomicMax(&mx[gb * npo + nc * g.nd + d], (int)mb);
+            }
         }
-    }
     for (int o = 16; o > 0; o >>= 1) cmin = fminf(cmin, __shfl_xor_sync(0xffffffffu, cmin, o));
     if (lane == 0 && cmin < INFINITY) atomicMin(&clmin_bits, __float_as_int(cmin));
     __syncthreads();
-    for (int i = tid; i < kTcEbMax; i += blockDim.x) g.ebw[(size_t)w * kTcEbMax + i] = eB[i];
     if (tid == 0) g.clw[w] = __int_as_float(clmin_bits);
+    const int nst = (cnt + kTcStageK - 1) / kTcStageK, npc = (npo + 3) / 4, nw = mma_cols(npair, g.colw);
+    uint4* base = g.bs + __ldg(g.boff + w);
+    const int ntask = nst * npair * npc * 16;
+    for (int idx = tid; idx < ntask; idx += kTcBThreads) {
+        int rest = idx >> 4;
+        const int half = idx & 1, oc = (idx >> 3) & 1, p = 4 * (rest % npc) + ((idx >> 1) & 3);
+        rest /= npc;
+        const int gb = rest % npair, q = rest / npair;
+        if (p >= npo) continue;  // columns past the block's outputs are never read back
+        const int nc = p / g.nd, d = p - nc * g.nd;
+        const int pr = pairs[gb], nk = L - (pr & 7) - (pr >> 3);  // k = 0 .. L - i - j
+        const int k0 = q * kTcStageK + oc * 8 + half * 4;
+        const float mb = __int_as_float(mx[gb * npo + p]);
+        const Slicer6 cut(pow2f((mb > 0.f ? exp_bound(log2f(mb)) : -100) - 6));
+        uint32_t s0[kTcS][2], s1[kTcS][2];
+        const float2* dpd = dpw + (long long)d * g.dp_total + k0;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            float o0[2][kTcS], o1[2][kTcS];
+            df re[2], im[2];
+            re[0] = re[1] = im[0] = im[1] = df{0.f, 0.f};
+            float pw = 1.f;
+            for (int kk = 0; kk <= nk; ++kk) {
+                // two records' D'_k (16-byte aligned: classes, windows and halves start at even positions)
+                const float4 v = __ldg(reinterpret_cast<const float4*>(dpd + (long long)tidx[gb][kk] * stride + 2 * u));
+                const df a = df_mulf(df{v.x, v.y}, pw), b = df_mulf(df{v.z, v.w}, pw);  // D'_k n_c^k, exact power
+                switch (kk & 3) {                                                       // (-i)^k
+                    case 0: re[0] = df_add(re[0], a); re[1] = df_add(re[1], b); break;
+                    case 1: im[0] = df_sub(im[0], a); im[1] = df_sub(im[1], b); break;
+                    case 2: re[0] = df_sub(re[0], a); re[1] = df_sub(re[1], b); break;
+                    default: im[0] = df_add(im[0], a); im[1] = df_add(im[1], b); break;
+                }
+                pw *= (float)nc;
+            }
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int k = k0 + 2 * u + e;
+                cdf bv{{0.f, 0.f}, {0.f, 0.f}};
+                if (k < cnt) {
+                    const float4 zv = __ldg(g.tabz + (kb + k) * g.ncols + nc);
+                    bv = cdf_mul(cdf{{zv.x, zv.y}, {zv.z, zv.w}}, cdf{re[e], im[e]});
+                }
+                cut(bv.re.hi, bv.re.lo, o0[e]);
+                cut(bv.im.hi, bv.im.lo, o1[e]);
+            }
+#pragma unroll
+            for (int s = 0; s < kTcS; ++s) {
+                s0[s][u] = pack_bf2(o0[0][s], o0[1][s]);
+                s1[s][u] = pack_bf2(o1[0][s], o1[1][s]);
+            }
+        }
+        const int col = gb * g.colw + 2 * p;
+        uint2* dst = reinterpret_cast<uint2*>(base + (size_t)q * kTcS * nw * 2 + ((col >> 3) * 2 + oc) * 8 + (col & 7)) + half;
+#pragma unroll
+        for (int s = 0; s < kTcS; ++s) {
+            dst[(size_t)s * nw * 4] = make_uint2(s0[s][0], s0[s][1]);
+            dst[(size_t)s * nw * 4 + 2] = make_uint2(s1[s][0], s1[s][1]);
+        }
+    }
 }
 
-__global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int ntslots) {
+// ---- the product ---------------------------------------------------------------
+
+struct TcSmem {
+    uint64_t afull[kTcNbufMax], bfull[kTcNbufMax], empty[kTcNbufMax], accf, acce, done;
+    uint64_t tfull[kTcTabSlotsMax], tempty[kTcTabSlotsMax];
+    uint32_t tmem;
+    int abort_flag;
+};
+
+__host__ __device__ inline size_t tab_slot_bytes(int tws) { return (size_t)kTcStageK * tws * 16; }
+
+// waits (bounded) until the copies counted on the barriers of a ring have
+// landed, `issued` stages into it: nothing is in flight when the CTA exits
+__device__ void ring_settle(uint64_t* bar, int n, long long issued) {
+    for (int b = 0; b < n && b < issued; ++b) {
+        const long long last = issued - 1 - ((issued - 1 - b) % n);  // last stage that used slot b
+        const long long t0 = clock64();
+        while (!mbar_test(bar + b, (uint32_t)((last / n) & 1)) && clock64() - t0 < kTcSpinCycles) {
+        }
+    }
+}
+
+template <int NU>
+__global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf, int ntslots) {
     extern __shared__ __align__(1024) unsigned char tsm[];
-    unsigned char* abuf = tsm;                                                    // [nbuf][S][8192]
-    unsigned char* bbuf = abuf + (size_t)kTcNbuf * kTcS * kTcAsliceBytes;          // [nbuf][S][npad*64]
-    const int bslice = g.npad * 64;
-    unsigned char* tring = bbuf + (size_t)kTcNbuf * kTcS * bslice;                 // [ntslots][slot]
-    const size_t tslot = tab_slot_bytes(g.tabw, g.G, g.nd);
+    unsigned char* abuf = tsm;                                                // [nbuf][S][4096]
+    unsigned char* bbuf = abuf + (size_t)nbuf * kTcS * kTcAsliceBytes;         // [nbuf][S][npad*32]
+    const int bbytes = kTcS * g.npad * 32;
+    unsigned char* tring = bbuf + (size_t)nbuf * bbytes;                       // [ntslots][slot]
+    const size_t tslot = tab_slot_bytes(g.tws);
     TcSmem& sm = *reinterpret_cast<TcSmem*>(tring + (size_t)ntslots * tslot);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int kg = blockIdx.x, mt = blockIdx.y;
-    const int w0 = kg * g.win_per_group, w1 = min(g.nwin, w0 + g.win_per_group);
+    const int j0 = __ldg(g.sched + kg), j1 = __ldg(g.sched + kg + 1);
+    const int* wlist = g.sched + gridDim.x + 1;
     volatile int* abort_flag = &sm.abort_flag;
-    const bool mma_warp = warp == kTcMmaWarp, load_warp = warp == kTcLoadWarp;
-    const bool epi = warp < kTcEpiWarps;  // drains tensor memory: four lane quadrants x three column thirds
 
     if (tid == 0) {
-        for (int b = 0; b < kTcNbuf; ++b) {
-            mbar_init(&sm.full[b], kTcProdWarps);
+        for (int b = 0; b < nbuf; ++b) {
+            mbar_init(&sm.afull[b], kTcGroupWarps);
+            mbar_init(&sm.bfull[b], 1);
             mbar_init(&sm.empty[b], 1);
         }
         for (int b = 0; b < ntslots; ++b) {
             mbar_init(&sm.tfull[b], 1);
-            mbar_init(&sm.tempty[b], kTcProdWarps);
+            mbar_init(&sm.tempty[b], kTcGroupWarps);
         }
         mbar_init(&sm.accf, 1);
-        mbar_init(&sm.acce, kTcEpiWarps);
+        mbar_init(&sm.acce, kTcProdWarps);
         mbar_init(&sm.done, 1);
-        mbar_init(&sm.psync, kTcWarps);
         sm.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (tid < kTcM) {
-        const int m = mt * kTcM + tid;
-        const int2 rw = m < g.nrows ? __ldg(g.rows + m) : make_int2(INT_MIN, 0);
-        TcRow ri;
-        ri.na = rw.x;
-        ri.nb = rw.y;
-        ri.Q = rw.x != INT_MIN ? g.Maa * (float)rw.x * (float)rw.x + g.Mbb * (float)rw.y * (float)rw.y : 0.f;
-        sm.rowi[tid] = ri;
-    }
-    // zero both stage buffers once: padding columns of B are never written
-    for (int i = tid; i < kTcNbuf * kTcS * bslice / 16; i += blockDim.x)
-        reinterpret_cast<uint4*>(bbuf)[i] = make_uint4(0u, 0u, 0u, 0u);
-    if (mma_warp) {
+    // the table slots start finite: records past a window's end are not copied, their A entries meet zeros of B
+    for (int i = tid; i < (int)(ntslots * tslot / 16); i += kTcThreadsAll)
+        reinterpret_cast<uint4*>(tring)[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (warp == kTcMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(&sm.tmem)),
                      "r"(kTcTmemCols)
                      : "memory");
@@ -532,296 +597,238 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int ntslo
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sm.tmem;
-
-    // epilogue roles (warps 0-11): TMEM lanes 32 (w & 3) .. + 31, 8-column chunks c8 = w / 4 (mod 3)
-    const int equad = warp & 3, ewarp3 = warp >> 2, erow = 32 * equad + lane;
-    const uint32_t tlane = (uint32_t)(32 * equad) << 16;
-    const int npo = g.nd * g.ncols;  // complex outputs per block
-    const int nchunk = g.colw / 8;   // 8-column chunks of a block (4 complex outputs each)
-    const uint32_t acc_hi = (uint32_t)(4 * g.npad), acc_lo = acc_hi + (uint32_t)g.colw;
-    if (epi) {
-        for (int c8 = ewarp3; c8 < nchunk; c8 += 3) {
-            const float z[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            tc_st8(tmem + tlane + acc_hi + (uint32_t)(8 * c8), z);
-            tc_st8(tmem + tlane + acc_lo + (uint32_t)(8 * c8), z);
-        }
-        tc_wait_st();
-    }
-    // The operand tasks of a stage, the same for every stage: B tasks (four
-    // records of one (block, output pair)) then A tasks (four records of one
-    // row), dealt to the operand threads in snake order (0..P-1, P-1..0, ...),
-    // so that the heavier B tasks and the A tasks spread evenly.
-    int tk[kTcTasksMax], ntask = 0;
-    {
-        const int nbt = (kTcStageK / 4) * g.G * npo, ntot = nbt + kTcM * 4;
-#pragma unroll
-        for (int e = 0; e < kTcTasksMax; ++e) {
-            const int k = e * kTcProdThreads + ((e & 1) ? kTcProdThreads - 1 - tid : tid);
-            tk[e] = 0;
-            if (!mma_warp && !load_warp && k < ntot) {
-                if (k < nbt) {
-                    const int p = k % npo, t2 = k / npo, gb = t2 % g.G, kgq = t2 / g.G;
-                    tk[e] = kgq | (gb << 2) | (p << 6);
-                } else {
-                    tk[e] = (k - nbt) | kTcTaskA;
-                }
-                ntask = e + 1;
-            }
-        }
-    }
-    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(g.npad >> 3) << 17) |
-                           ((uint32_t)(kTcM >> 4) << 24);
-    long long gs = 0;  // stages so far (every role counts the same)
-    uint32_t ph = 0;
     bool ok = true;
-    for (int w = w0; w < w1 && ok; ++w) {
-        // ---- window records, blocks and scales ----
-        for (int i = tid; i < kTcWin; i += kTcThreadsAll) sm.rec[i] = __ldg(g.wrec + (size_t)w * kTcWin + i);
-        for (int i = tid; i < kTcEbMax; i += kTcThreadsAll) sm.eB[i] = __ldg(g.ebw + (size_t)w * kTcEbMax + i);
-        if (tid == 0) {
-            const int4 wi = __ldg(g.winfo + w);
-            sm.winL = wi.x;
-            sm.wnpair = wi.y;
-            sm.wpos = wi.w;
-            for (int b = 0; b < wi.y; ++b) {
-                const int pr = __ldg(g.wpairs + wi.z + b), i = pr & 7, j = pr >> 3;
-                sm.pairs[b] = pr;
-                for (int kk = 0; kk < 5; ++kk) sm.tidx[b][kk] = kk <= wi.x - i - j ? term_of(g, i, j, kk) : -1;
-            }
-            sm.clmin_bits = __float_as_int(__ldg(g.clw + w));
-        }
-        if (!(ok = prod_sync(&sm.psync, ph, abort_flag, lane, g.spin))) break;
-        const int L = sm.winL, npair = sm.wnpair;
-        const float clmin = __int_as_float(sm.clmin_bits);
-        // ---- stages ----
-        if (load_warp) {
-            // rows of D' a stage needs: (block, density, k <= L - i - j)
-            int nrow = 0;
-            for (int gb = 0; gb < npair; ++gb) nrow += g.nd * (L - (sm.pairs[gb] & 7) - (sm.pairs[gb] >> 3) + 1);
-            const float2* dpL = g.Dp + g.dp_base[L];
-            for (int q = 0; q < kTcStagesPerWin; ++q, ++gs) {
-                const int ts = (int)(gs % ntslots);
-                const long long use = gs / ntslots;
-                if (use > 0) {
-                    ok = __all_sync(0xffffffffu, mbar_wait(&sm.tempty[ts], (uint32_t)((use - 1) & 1), abort_flag, g.spin));
-                    if (!ok) break;
-                }
-                unsigned char* slotp = tring + (size_t)ts * tslot;
-                float2* dps = reinterpret_cast<float2*>(slotp + (size_t)kTcStageK * g.tabw * 16);
-                // A stage holds records from its first entry on, or none (the padding at a
-                // window's end): its D' rows are copied only when it holds some, and then
-                // stay inside the class's 16-padded stride.
-                const int srow = sm.rec[q * kTcStageK] >= 0 ? nrow : 0;
-                if (lane == 0) {
-                    uint32_t nv = 0;
-                    for (int u = 0; u < kTcStageK; ++u) nv += sm.rec[q * kTcStageK + u] >= 0 ? 1u : 0u;
-                    mbar_arrive_tx(&sm.tfull[ts], nv * (uint32_t)g.tabw * 16u + (uint32_t)srow * kTcStageK * 8u);
-                }
-                __syncwarp();
-                // lanes 0-15: the records' factor tables; the rest: 128-byte rows of D'
-                for (int idx = lane; idx < kTcStageK + srow; idx += 32) {
-                    if (idx < kTcStageK) {
-                        const int r = sm.rec[q * kTcStageK + idx];
-                        if (r >= 0)
-                            bulk_copy(slotp + (size_t)idx * g.tabw * 16, g.tab + (size_t)r * g.tabw,
-                                      (uint32_t)g.tabw * 16u, &sm.tfull[ts]);
-                    } else {
-                        int row = idx - kTcStageK, gb = 0;
-                        for (;;) {  // row -> (block, density, k)
-                            const int nkb = L - (sm.pairs[gb] & 7) - (sm.pairs[gb] >> 3) + 1;
-                            if (row < g.nd * nkb) break;
-                            row -= g.nd * nkb;
-                            ++gb;
-                        }
-                        const int pr = sm.pairs[gb], nkb = L - (pr & 7) - (pr >> 3) + 1;
-                        const int d = row / nkb, kk = row - d * nkb;
-                        const long long src = (long long)(g.d0 + d) * g.dp_total +
-                                              (long long)sm.tidx[gb][kk] * g.dp_stride[L] + sm.wpos + q * kTcStageK;
-                        bulk_copy(dps + ((gb * g.nd + d) * 5 + kk) * kTcStageK, dpL + src, kTcStageK * 8u,
-                                  &sm.tfull[ts]);
-                    }
-                }
-                __syncwarp();
-            }
-        } else if (!mma_warp) {
-            for (int q = 0; q < kTcStagesPerWin; ++q, ++gs) {
-                const int slot = (int)(gs & 1), ts = (int)(gs % ntslots);
-                ok = __all_sync(0xffffffffu, mbar_wait(&sm.tfull[ts], (uint32_t)((gs / ntslots) & 1), abort_flag, g.spin));
-                if (!ok) break;
-                if (gs >= kTcNbuf) {
-                    ok = __all_sync(0xffffffffu, mbar_wait(&sm.empty[slot], (uint32_t)(((gs >> 1) - 1) & 1), abort_flag, g.spin));
-                    if (!ok) break;
-                }
-                const unsigned char* slotp = tring + (size_t)ts * tslot;
-                const float4* tabs = reinterpret_cast<const float4*>(slotp);
-                const float2* dps = reinterpret_cast<const float2*>(slotp + (size_t)kTcStageK * g.tabw * 16);
-                unsigned char* as = abuf + (size_t)slot * kTcS * kTcAsliceBytes;
-                unsigned char* bs = bbuf + (size_t)slot * kTcS * bslice;
-#pragma unroll
-                for (int e = 0; e < kTcTasksMax; ++e) {
-                    if (e < ntask) {
-                        const int k = tk[e];
-                        if (k & kTcTaskA) {
-                            const int row = k & (kTcM - 1), gg = (k >> 7) & 3;
-                            form_a(g, sm, tabs, q, row, gg, pow2f(6 - exp_bound(-clmin * sm.rowi[row].Q)), as);
-                        } else {
-                            form_b(g, sm, tabs, dps, q, k & 3, (k >> 2) & 15, k >> 6, bs, bslice);
-                        }
-                    }
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive(&sm.full[slot]);
-                    mbar_arrive(&sm.tempty[ts]);
-                }
-            }
-        } else {
-            if (lane == 0) {
-                const uint32_t a0 = saddr(abuf), b0 = saddr(bbuf);
-                bool first[kTcAcc] = {true, true, true, true};
-                bool mok = true;
-                for (int q = 0; q < kTcStagesPerWin; ++q, ++gs) {
-                    const int slot = (int)(gs & 1);
-                    if (!(mok = mbar_wait(&sm.full[slot], (uint32_t)((gs >> 1) & 1), abort_flag, g.spin))) break;
-                    tc_fence_after();
-                    const uint32_t as = a0 + slot * kTcS * kTcAsliceBytes, bs = b0 + slot * kTcS * bslice;
-#pragma unroll
-                    for (int h = 0; h < 2; ++h)
-#pragma unroll
-                        for (int s = 0; s < kTcS; ++s)
-#pragma unroll
-                            for (int t = 0; s + t < kTcS; ++t) {
-                                const int lv = min(s + t, kTcAcc - 1);
-                                tc_mma(tmem + (uint32_t)(lv * g.npad), sdesc(as + s * kTcAsliceBytes + h * 256),
-                                       sdesc(bs + t * bslice + h * 256), idesc, first[lv] ? 0u : 1u);
-                                first[lv] = false;
-                            }
-                    tc_commit(&sm.empty[slot]);
-                }
-                if (mok) tc_commit(&sm.accf);
-                ok = mok;
-            }
-            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-            gs = __shfl_sync(0xffffffffu, gs, 0);
-        }
-        if (!ok) break;
-        // ---- drain: each block's level sums, scaled and times P_ij, into the double-float sums (warps 0-11) ----
-        if (epi) {
-            ok = __all_sync(0xffffffffu, mbar_wait(&sm.accf, (uint32_t)((w - w0) & 1), abort_flag, g.spin));
-            if (!ok) break;
-            tc_fence_after();
-            const TcRow ri = sm.rowi[erow];
-            const int eAe = exp_bound(-clmin * ri.Q);
-            for (int c8 = ewarp3; c8 < nchunk; c8 += 3) {
-                float H[8], Lo[8];
-                tc_ld8(tmem + tlane + acc_hi + (uint32_t)(8 * c8), H);
-                tc_ld8(tmem + tlane + acc_lo + (uint32_t)(8 * c8), Lo);
-                for (int gb = 0; gb < npair; ++gb) {
-                    const int i = sm.pairs[gb] & 7, j = sm.pairs[gb] >> 3;
-                    float pij = 1.f;  // n_a^i n_b^j, exact
-                    for (int k = 0; k < i; ++k) pij *= (float)ri.na;
-                    for (int k = 0; k < j; ++k) pij *= (float)ri.nb;
-                    float T[kTcAcc][8];
-#pragma unroll
-                    for (int lv = 0; lv < kTcAcc; ++lv)
-                        tc_ld8(tmem + tlane + (uint32_t)(lv * g.npad + gb * g.colw + 8 * c8), T[lv]);
-#pragma unroll
-                    for (int u = 0; u < 8; u += 2) {
-                        const int p = 4 * c8 + u / 2;
-                        if (p < npo) {
-                            cdf v;
-                            v.re = df_add(df_add(two_sum(T[0][u], T[1][u]), df{T[2][u], 0.f}), df{T[3][u], 0.f});
-                            v.im = df_add(df_add(two_sum(T[0][u + 1], T[1][u + 1]), df{T[2][u + 1], 0.f}),
-                                          df{T[3][u + 1], 0.f});
-                            const float sc = pow2f(eAe + sm.eB[gb * npo + p] - 12);  // exact power of two
-                            v = cdf{df_mulf(df{v.re.hi * sc, v.re.lo * sc}, pij),
-                                    df_mulf(df{v.im.hi * sc, v.im.lo * sc}, pij)};
-                            v = rot_mi(v, i + j);
-                            const df re = df_add(df{H[u], Lo[u]}, v.re), im = df_add(df{H[u + 1], Lo[u + 1]}, v.im);
-                            H[u] = re.hi;
-                            Lo[u] = re.lo;
-                            H[u + 1] = im.hi;
-                            Lo[u + 1] = im.lo;
-                        }
-                    }
-                }
-                tc_st8(tmem + tlane + acc_hi + (uint32_t)(8 * c8), H);
-                tc_st8(tmem + tlane + acc_lo + (uint32_t)(8 * c8), Lo);
-            }
-            tc_wait_st();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sm.acce);
-        }
-        // the MMAs of the next window wait for every draining warp
-        if (mma_warp && w + 1 < w1) {
-            ok = __all_sync(0xffffffffu, mbar_wait(&sm.acce, (uint32_t)((w - w0) & 1), abort_flag, g.spin));
-            tc_fence_after();
-        }
-        if (!(ok = prod_sync(&sm.psync, ph, abort_flag, lane, g.spin) && ok)) break;  // window tables reused next window
-    }
-    // ---- partial rows ----
-    if (ok && !*abort_flag && epi) {
-        tc_fence_after();
-        const int mo = mt * kTcM + erow;
-        for (int c8 = ewarp3; c8 < nchunk; c8 += 3) {
-            float H[8], Lo[8];
-            tc_ld8(tmem + tlane + acc_hi + (uint32_t)(8 * c8), H);
-            tc_ld8(tmem + tlane + acc_lo + (uint32_t)(8 * c8), Lo);
-            if (mo < g.nrows) {
-#pragma unroll
-                for (int u = 0; u < 8; u += 2) {
-                    const int p = 4 * c8 + u / 2;
-                    if (p < npo) {
-                        const int nc = p / g.nd, d = p - nc * g.nd;
-                        int idx = __ldg(g.map + (size_t)mo * g.ncols + nc);
-                        if (idx != INT_MIN) {
-                            const bool cj = idx < 0;
-                            if (cj) idx = ~idx;
-                            const double re = (double)H[u] + (double)Lo[u];
-                            const double im = (double)H[u + 1] + (double)Lo[u + 1];
-                            g.out[((long long)(g.d0 + d) * g.ngroups + kg) * g.ng_half + idx] =
-                                make_double2(re, cj ? -im : im);
-                        }
-                    }
-                }
-            }
-        }
-    }
-    if (load_warp && lane == 0) {
-        // bulk copies still in flight (after a failed wait) land before the CTA exits
-        for (int b = 0; b < ntslots && b < gs; ++b) {
-            const long long last = gs - 1 - ((gs - 1 - b) % ntslots);  // last stage that used slot b
-            const long long t0 = clock64();
-            while (!mbar_test(&sm.tfull[b], (uint32_t)((last / ntslots) & 1)) && clock64() - t0 < kTcSpinCycles) {
-            }
-        }
-    }
-    if (mma_warp) {
-        // everything issued completes before tensor memory is freed
+
+    if (warp == kTcTabWarp) {
+        // the stages' X and Y tables: consecutive records of the K order, one bulk copy each
         if (lane == 0) {
+            Ring t(ntslots);
+            long long gt = 0;
+            for (int jw = j0; jw < j1 && ok; ++jw) {
+                const int w = __ldg(wlist + jw), cnt = __ldg(g.wcnt + w);
+                const int4 wi = __ldg(g.winfo + w);
+                const float4* src = g.tabk + (g.kbase[wi.x] + wi.w) * g.tws;
+                for (int k0 = 0; k0 < cnt; k0 += kTcStageK, ++gt, t.next()) {
+                    if (gt >= ntslots && !(ok = mbar_wait(&sm.tempty[t.i], t.ph ^ 1u, abort_flag, g.spin))) break;
+                    const uint32_t bytes = (uint32_t)(min(kTcStageK, cnt - k0) * g.tws) * 16u;
+                    mbar_arrive_tx(&sm.tfull[t.i], bytes);
+                    bulk_copy(tring + (size_t)t.i * tslot, src + (size_t)k0 * g.tws, bytes, &sm.tfull[t.i]);
+                }
+            }
+            ring_settle(sm.tfull, ntslots, gt);
+        }
+        __syncwarp();
+    } else if (warp == kTcLoadWarp) {
+        // the stages' B tiles, one bulk copy each
+        if (lane == 0) {
+            Ring b(nbuf);
+            long long gs = 0;
+            for (int jw = j0; jw < j1 && ok; ++jw) {
+                const int w = __ldg(wlist + jw), nst = (__ldg(g.wcnt + w) + kTcStageK - 1) / kTcStageK;
+                const uint32_t bb = (uint32_t)(kTcS * mma_cols(__ldg(&g.winfo[w].y), g.colw) * 32);
+                const unsigned char* src = reinterpret_cast<const unsigned char*>(g.bs + __ldg(g.boff + w));
+                for (int q = 0; q < nst; ++q, ++gs, b.next()) {
+                    if (gs >= nbuf && !(ok = mbar_wait(&sm.empty[b.i], b.ph ^ 1u, abort_flag, g.spin))) break;
+                    mbar_arrive_tx(&sm.bfull[b.i], bb);
+                    bulk_copy(bbuf + (size_t)b.i * bbytes, src + (size_t)q * bb, bb, &sm.bfull[b.i]);
+                }
+            }
+            ring_settle(sm.bfull, nbuf, gs);
+        }
+        __syncwarp();
+    } else if (warp == kTcMmaWarp) {
+        const uint32_t a0 = saddr(abuf), b0 = saddr(bbuf);
+        Ring b(nbuf);
+        for (int jw = j0; jw < j1 && ok; ++jw) {
+            const int w = __ldg(wlist + jw), nst = (__ldg(g.wcnt + w) + kTcStageK - 1) / kTcStageK;
+            const uint32_t nw = (uint32_t)mma_cols(__ldg(&g.winfo[w].y), g.colw);
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTcM >> 4) << 24);
+            // the window's first MMAs wait for the drain of the previous one
+            if (jw > j0 && !(ok = __all_sync(0xffffffffu, mbar_wait(&sm.acce, (uint32_t)((jw - j0 - 1) & 1), abort_flag, g.spin))))
+                break;
+            tc_fence_after();
+            for (int q = 0; q < nst; ++q, b.next()) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&sm.bfull[b.i], b.ph, abort_flag, g.spin) &&
+                                                 mbar_wait(&sm.afull[b.i], b.ph, abort_flag, g.spin));
+                if (!ok) break;
+                tc_fence_after();
+                if (elect_one()) {
+                    issue_kstep<kTcS, kTcAcc>(tmem, sdesc(a0 + b.i * kTcS * kTcAsliceBytes), kTcAsliceBytes >> 4,
+                                              sdesc(b0 + b.i * bbytes), nw * 2, nw, idesc, q > 0);
+                    tc_commit(&sm.empty[b.i]);
+                    if (q + 1 == nst) tc_commit(&sm.accf);
+                }
+                __syncwarp();
+            }
+        }
+        // everything issued completes before tensor memory is freed
+        if (elect_one()) {
             tc_commit(&sm.done);
             const long long t0 = clock64();
             while (!mbar_test(&sm.done, 0u) && clock64() - t0 < kTcSpinCycles) {
             }
         }
         __syncwarp();
+    } else {
+        // forms row `row` of A for the records 8 oct .. 8 oct + 7 of its group's stages
+        const int grp = warp / kTcGroupWarps, row = tid & (kTcM - 1), oct = (tid >> 7) & 1;
+        const int sl = __ldg(g.slots + mt * kTcM + row);
+        const float fa = (float)(sl & 255), fb = (float)((sl >> 8) & 255);
+        const float Q = g.Maa * fa * fa + g.Mbb * fb * fb;
+        const int rs = 2 * g.tws;  // float2 per record
+        const int xo = oct * 8 * rs + 2 * (sl & 255) + ((sl >> 16) & 1);
+        const int yo = oct * 8 * rs + 2 * (g.offY + ((sl >> 8) & 255)) + ((sl >> 17) & 1);
+        unsigned char* arow = abuf + tile_off(row, oct * 8) * 2;
+        // drains: tensor-memory lanes 32 (warp & 3) .. + 31, 4-column units warp / 4 + 4 x of each block
+        const int eq = warp & 3, es = warp >> 2, erow = 32 * eq + lane;
+        const uint32_t tlane = (uint32_t)(32 * eq) << 16;
+        const int es_slot = __ldg(g.slots + mt * kTcM + erow);
+        const float ea = (float)(es_slot & 255), eb = (float)((es_slot >> 8) & 255);
+        const int ca = (es_slot >> 16) & 1, cb = (es_slot >> 17) & 1;
+        const int nunit = g.colw / 4, npo = g.nd * g.ncols;
+        df S[NU][4];  // double-float sums by sign character: two complex outputs per unit
+#pragma unroll
+        for (int x = 0; x < NU; ++x)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) S[x][v] = df{0.f, 0.f};
+        Ring b(nbuf), t(ntslots);
+        int gs = 0;  // stages so far (mod 2 the group that forms it)
+        bool full = false;  // every buffer used once
+        for (int jw = j0; jw < j1 && ok; ++jw) {
+            const int w = __ldg(wlist + jw), nst = (__ldg(g.wcnt + w) + kTcStageK - 1) / kTcStageK;
+            const Slicer6 cut(pow2f(exp_bound(-__ldg(g.clw + w) * Q) - 6));
+            for (int q = 0; q < nst; ++q, ++gs, b.next(), t.next()) {
+                full = full || gs >= nbuf;
+                if ((gs & 1) != grp) continue;
+                ok = __all_sync(0xffffffffu, mbar_wait(&sm.tfull[t.i], t.ph, abort_flag, g.spin));
+                if (!ok) break;
+                const float2* tb = reinterpret_cast<const float2*>(tring + (size_t)t.i * tslot);
+                uint32_t pk[kTcS][4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    float o[2][kTcS];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const float2 x = tb[(2 * u + e) * rs + xo], y = tb[(2 * u + e) * rs + yo];
+                        const df a = df_mul_u(df{x.x, x.y}, df{y.x, y.y});
+                        cut(a.hi, a.lo, o[e]);
+                    }
+#pragma unroll
+                    for (int s = 0; s < kTcS; ++s) pk[s][u] = pack_bf2(o[0][s], o[1][s]);
+                }
+                if (full) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(&sm.empty[b.i], b.ph ^ 1u, abort_flag, g.spin));
+                    if (!ok) break;
+                }
+                unsigned char* as = arow + (size_t)b.i * kTcS * kTcAsliceBytes;
+#pragma unroll
+                for (int s = 0; s < kTcS; ++s)
+                    *reinterpret_cast<uint4*>(as + (size_t)s * kTcAsliceBytes) =
+                        make_uint4(pk[s][0], pk[s][1], pk[s][2], pk[s][3]);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(&sm.afull[b.i]);
+                    mbar_arrive(&sm.tempty[t.i]);
+                }
+            }
+            if (!ok) break;
+            // ---- drain: each block's level sums, times (-i)^{i+j} n_a^i n_b^j, into the sums by character ----
+            ok = __all_sync(0xffffffffu, mbar_wait(&sm.accf, (uint32_t)((jw - j0) & 1), abort_flag, g.spin));
+            if (!ok) break;
+            tc_fence_after();
+            const int4 wi = __ldg(g.winfo + w);
+            const uint32_t nw = (uint32_t)mma_cols(wi.y, g.colw);
+            for (int gb = 0; gb < wi.y; ++gb) {
+                const int pr = __ldg(g.wpairs + wi.z + gb), i = pr & 7, j = pr >> 3;
+                // type (ta, tb) of lane ^ mask adds to this lane's character; i^{ta - i} = i^{ca} times a real sign
+                const int mask = (i & 1) | ((j & 1) << 1);
+                float f = ipow(ea, i) * ipow(eb, j);
+                if ((((i >> 1) + (j >> 1) + (ca & i) + (cb & j)) & 1) != 0) f = -f;
+#pragma unroll
+                for (int x = 0; x < NU; ++x) {
+                    const int un = es + 4 * x;
+                    if (un < nunit) {
+                        float T[5][4];
+                        tc_ld_levels4(tmem + tlane + (uint32_t)(gb * g.colw + 4 * un), nw, T);
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) {
+                            df l = level_sum(T[0][v], T[1][v], T[2][v], T[3][v], T[4][v]);
+                            if (mask) {
+                                l.hi = __shfl_xor_sync(0xffffffffu, l.hi, mask);
+                                l.lo = __shfl_xor_sync(0xffffffffu, l.lo, mask);
+                            }
+                            S[x][v] = df_add(S[x][v], df_mulf_u(l, f));
+                        }
+                    }
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.acce);
+        }
+        // ---- partial rows: characters back to the signs of (n_a, n_b) ----
+        if (ok && !*abort_flag) {
+            const bool da = (es_slot >> 18) & 1, db = (es_slot >> 19) & 1, valid = (es_slot >> 20) & 1;
+            const int na = da && (lane & 1) ? -(es_slot & 255) : (es_slot & 255);
+            const int nb = db && (lane & 2) ? -((es_slot >> 8) & 255) : ((es_slot >> 8) & 255);
+            const int* mrow = g.map + ((size_t)(na + g.nam) * (2 * g.nbm + 1) + (nb + g.nbm)) * g.ncols;
+#pragma unroll
+            for (int x = 0; x < NU; ++x) {
+                const int un = es + 4 * x;
+                if (un < nunit) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        // i^{ca + cb}, then the sign sums over the two characters of each axis
+                        const cdf z = rot_mi(cdf{S[x][2 * h], S[x][2 * h + 1]}, 4 - ca - cb);
+                        df c[2] = {z.re, z.im};
+#pragma unroll
+                        for (int r = 0; r < 2; ++r) {
+                            df o{__shfl_xor_sync(0xffffffffu, c[r].hi, 1), __shfl_xor_sync(0xffffffffu, c[r].lo, 1)};
+                            if (da) c[r] = (lane & 1) ? df_sub(o, c[r]) : df_add(c[r], o);
+                            o = df{__shfl_xor_sync(0xffffffffu, c[r].hi, 2), __shfl_xor_sync(0xffffffffu, c[r].lo, 2)};
+                            if (db) c[r] = (lane & 2) ? df_sub(o, c[r]) : df_add(c[r], o);
+                        }
+                        const int p = 2 * un + h;
+                        if (valid && p < npo) {
+                            const int nc = p / g.nd, d = p - nc * g.nd;
+                            int idx = __ldg(mrow + nc);
+                            if (idx != INT_MIN) {
+                                const bool cj = idx < 0;
+                                if (cj) idx = ~idx;
+                                const double re = (double)c[0].hi + (double)c[0].lo;
+                                const double im = (double)c[1].hi + (double)c[1].lo;
+                                g.out[((long long)(g.d0 + d) * g.out_rows + g.out_row0 + kg) * g.ng_half + idx] =
+                                    make_double2(re, cj ? -im : im);
+                            }
+                        }
+                    }
+                }
+            }
+        }
     }
     tc_fence_before();
     __syncthreads();
     if (*abort_flag && tid == 0) atomicOr(g.err, 1);
-    if (mma_warp) {
-        __syncwarp();
+    if (warp == kTcMmaWarp) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols) : "memory");
     }
 }
 
-// per-record factor tables X(0..na), Y(0..nb), Z(0..nc) in FP64, kept as double-float
-__global__ void k_tc_tables(const PairWalk* __restrict__ walk, long long npairs, int ax, int bx, int cx, int nna,
-                            int nnb, int nnc, double Maa, double Mbb, double Mcc, float4* __restrict__ tab,
-                            float* __restrict__ cl) {
+// c log2(e) of each record: the windows sort by it
+__global__ void k_tc_width(const PairWalk* __restrict__ walk, long long npairs, float* __restrict__ cl) {
+    const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r < npairs) cl[r] = (float)(walk[r].c * 1.4426950408889634);
+}
+
+// Per-record factor tables in FP64, kept as double-float: X(0..na), Y(0..nb)
+// with tws entries per record, in record order (the back-contraction's tiles)
+// and in the K order (the structure-factor stages), so that a tile or a stage
+// is one contiguous copy; Z(0..nc) in the K order.
+__global__ void k_tc_tables(const PairWalk* __restrict__ walk, long long npairs, const int* __restrict__ kpos, int ax,
+                            int bx, int cx, int nna, int nnb, int nnc, int tws, double Maa, double Mbb, double Mcc,
+                            float4* __restrict__ tab, float4* __restrict__ tabk, float4* __restrict__ tabz) {
     const int tabw = nna + nnb + nnc;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= npairs * tabw) return;
@@ -850,16 +857,22 @@ __global__ void k_tc_tables(const PairWalk* __restrict__ walk, long long npairs,
     double s, c;
     sincospi(2.0 * th, &s, &c);
     const df re = df_from_double(gval * c), im = df_from_double(-gval * s);
-    tab[t] = make_float4(re.hi, re.lo, im.hi, im.lo);
-    if (e == 0) cl[r] = (float)(w.c * 1.4426950408889634);
+    const float4 v = make_float4(re.hi, re.lo, im.hi, im.lo);
+    const long long k = kpos[r];
+    if (e < nna + nnb) {
+        tab[r * tws + e] = v;
+        tabk[k * tws + e] = v;
+    } else {
+        tabz[k * nnc + n] = v;
+    }
 }
 
-// shared memory of one CTA with `nts` table slots (at least 120 KB, so that a
-// second CTA never shares an SM: each one takes all 512 tensor-memory
-// columns, and a second would wait in tcgen05.alloc)
-size_t tc_smem_bytes(int npad, int tabw, int G, int nd, int nts) {
-    const size_t need = (size_t)kTcNbuf * kTcS * kTcAsliceBytes + (size_t)kTcNbuf * kTcS * npad * 64 +
-                        (size_t)nts * tab_slot_bytes(tabw, G, nd) + sizeof(TcSmem) + 64;
+// shared memory of one CTA with nbuf stage buffers and nts table slots (at
+// least 120 KB, so that a second CTA never shares an SM: each one takes all
+// 512 tensor-memory columns, and a second would wait in tcgen05.alloc)
+size_t tc_smem_bytes(int npad, int tws, int nbuf, int nts) {
+    const size_t need = (size_t)nbuf * kTcS * (kTcAsliceBytes + (size_t)npad * 32) + (size_t)nts * tab_slot_bytes(tws) +
+                        sizeof(TcSmem) + 64;
     return std::max<size_t>(need, 120 * 1024);
 }
 
@@ -878,17 +891,29 @@ int tc_upload(ftcj_plan* P, T** ptr, const std::vector<T>& v) {
 
 int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
+
+// the product kernel whose drain warps hold a block of colw columns in registers
+const void* tc_rho_kernel(int colw) {
+    switch ((colw + 15) / 16) {
+        case 1: return (const void*)k_tc_rho<1>;
+        case 2: return (const void*)k_tc_rho<2>;
+        case 3: return (const void*)k_tc_rho<3>;
+        case 4: return (const void*)k_tc_rho<4>;
+        case 5: return (const void*)k_tc_rho<5>;
+        default: return (const void*)k_tc_rho<6>;
+    }
+}
+
 // column layout for nd densities and ncols values of n_c: real columns per
-// block (a multiple of 8) and the largest block count G whose level
-// accumulators (4 x G x colw, rounded to 16) and double-float sums (2 colw)
-// fit the 512 tensor-memory columns; G = 0 when not even one block fits
+// block (a multiple of 8) and the largest block count G whose columns fit the
+// MMA width; G = 0 when not even one block fits
 void tc_columns(int nd, int ncols, int* colw, int* G, int* npad) {
     *colw = round_up(2 * nd * ncols, 8);
     *G = 0;
     *npad = 0;
     for (int gg = kTcGmax; gg >= 1; --gg) {
-        const int np = round_up(gg * *colw, 16);
-        if (np <= kTcNmma && 4 * np + 2 * *colw <= kTcTmemCols && gg * nd * ncols <= kTcEbMax) {
+        const int np = mma_cols(gg, *colw);
+        if (np <= kTcNmax) {
             *G = gg;
             *npad = np;
             return;
@@ -896,48 +921,86 @@ void tc_columns(int nd, int ncols, int* colw, int* G, int* npad) {
     }
 }
 
+// The slots of a set of points (|n_a|, |n_b|), in groups of four lanes: the
+// types (ta, tb) of one point (bit 0 ta, bit 1 tb) where both indices are
+// positive; where one is zero its only type is the real part, and two such
+// points share a group (the free bit says which); the origin takes one more.
+// quads: the same groups for the back-contraction's operand former (bit 0:
+// both indices positive, bit 1: n_b = 0, then two indices of 8 bits).
+void tc_slots(const std::set<std::pair<int, int>>& pts, std::vector<int>& slots, std::vector<int>& quads) {
+    std::vector<int> axa, axb;  // n_a > 0, n_b = 0 and n_a = 0, n_b > 0
+    bool origin = false;
+    slots.clear();
+    quads.clear();
+    for (const auto& q : pts) {
+        if (q.first > 0 && q.second > 0) {
+            for (int t = 0; t < 4; ++t) slots.push_back(slot_pack(q.first, q.second, t & 1, t >> 1, 1, 1, 1));
+            quads.push_back(1 | (q.first << 2) | (q.second << 10));
+        } else if (q.first > 0) {
+            axa.push_back(q.first);
+        } else if (q.second > 0) {
+            axb.push_back(q.second);
+        } else {
+            origin = true;
+        }
+    }
+    for (size_t k = 0; k < axa.size(); k += 2) {
+        const bool two = k + 1 < axa.size();
+        const int n[2] = {axa[k], two ? axa[k + 1] : axa[k]};
+        for (int t = 0; t < 4; ++t) slots.push_back(slot_pack(n[t >> 1], 0, t & 1, 0, 1, 0, t < 2 || two));
+        quads.push_back(2 | (n[0] << 2) | (n[1] << 10));
+    }
+    for (size_t k = 0; k < axb.size(); k += 2) {
+        const bool two = k + 1 < axb.size();
+        const int n[2] = {axb[k], two ? axb[k + 1] : axb[k]};
+        for (int t = 0; t < 4; ++t) slots.push_back(slot_pack(0, n[t & 1], 0, t >> 1, 0, 1, !(t & 1) || two));
+        quads.push_back(0 | (n[0] << 2) | (n[1] << 10));
+    }
+    if (origin) {
+        for (int t = 0; t < 4; ++t) slots.push_back(slot_pack(0, 0, 0, 0, 0, 0, t == 0));
+        quads.push_back(0);
+    }
+}
 
 // ---- the back-contraction (Alg. S1) in the same separable form -------------
 //
 // The walks' back-contraction sums, over the stored half sphere,
 //   J'_{r,ijk} = Re sum_n (-i)^{i+j+k} n_a^i n_b^j n_c^k X_r(n_a) Y_r(n_b) Z_r(n_c) W(n).
-// On the grid of rows m = (n_a, n_b) and columns n_c >= 0 (a stored point -n
-// enters as conj W, since the conjugate of the summand at -n is the summand
-// at n with conj W) this is
+// On the grid of (n_a, n_b) and n_c >= 0 (a stored point -n enters as conj W,
+// since the conjugate of the summand at -n is the summand at n with conj W)
+// this is, with the real products X_ta Y_tb of the structure-factor pass,
 //   J'_{r,ijk} = Re (-i)^k sum_{n_c} n_c^k Z_r(n_c) U_ij[r, n_c],
-//   U_ij[r, n_c] = sum_m A^T[r, m] V_ij[m, n_c],
-//   A^T[r, m] = X_r(n_a) Y_r(n_b),  V_ij = (-i)^{i+j} n_a^i n_b^j W(m, n_c),
-// a complex matrix product with M = 128 records of one class, K = the rows
-// (real and imaginary parts), N = (i, j) blocks x densities x n_c.  V_ij does
+//   U_ij[r, n_c] = sum_slots X_r,ta(|n_a|) Y_r,tb(|n_b|) V_ij[slot, n_c],
+//   V_ij = i^{ta+tb} (-i)^{i+j} |n_a|^i |n_b|^j sum_{s_a,s_b} s_a^{ta+i} s_b^{tb+j} W(s_a |n_a|, s_b |n_b|, n_c),
+// a matrix product with M = 128 records of one class, real A^T, K = the
+// slots, N = (i, j) blocks x densities x (Re, Im) of n_c: half the
+// multiply-adds and A^T entries of the complex form over signed rows.  V_ij does
 // not depend on the record: it is sliced once per build (k_tc_vbound,
 // k_tc_vslice) into stage tiles in global memory that bulk copies bring into
 // shared memory, and only A^T is formed in the kernel, from the 128 records'
-// factor tables staged once per work item.  Every entry of A^T has modulus
-// <= 1 (scale 2^1 for all of them); each column of V_ij gets its own scale
-// over all rows, so that entries far out in the sphere (where W has decayed)
-// sit many bits below their column's scale.  Seven slices (products with
-// s + t <= 6, 28 per k-step) keep the truncation below 2^-45 of the scales.
-// The rows are cut into parts of at most 512 (1024 real K terms), each a
-// work item of its own: within a part, levels 0-3 are exact (the level-3 sums
-// stay below 1024 x 14720 < 2^24 in units of 2^-21: |A| <= 1 bounds the
-// leading slice of A by 32) and only levels 4-6 share the rounded fifth
-// accumulator.  The tensor core's FP32 accumulation does not round to
+// factor tables.  Every entry of A^T has modulus <= 1 (bound 2^1 for all of
+// them); each column of V_ij gets its own bound over all slots, so that entries
+// far out in the sphere (where W has decayed) sit many bits below their
+// column's bound.  Seven slices (products with s + t <= 6, 28 per k-step) keep
+// the truncation below 2^-45 of the bounds.  The slots are cut into parts of at
+// most 1024, each a work unit of its own: within a part, levels 0-3 are exact
+// (the level-3 sums stay below 1024 x 14848 < 2^24 in units of 2^-21: |A| <= 1
+// bounds the leading slice of A by 32) and only levels 4-6 share the rounded
+// fifth accumulator.  The tensor core's FP32 accumulation does not round to
 // nearest, so the rounded accumulator's error grows with the number of MMAs
 // that add into it and with its size; keeping level 3 out of it keeps that
-// error ~2^-7 of the four-accumulator scheme's.  The level sums go straight
+// error ~2^-7 of a four-accumulator scheme's.  The level sums go straight
 // to the epilogue, which forms the part's J' for k <= L - i - j in
 // double-float and writes it as one of the partial FP64 sums the J -> AO map
 // adds.
 
-constexpr int kTcJStageM = 8;        // rows per stage: one MMA k-step of 16 real K
+constexpr int kTcJStageM = 16;       // slots per stage: one MMA k-step
 constexpr int kTcJS = 7;             // slices per operand
 constexpr int kTcJProducts = kTcJS * (kTcJS + 1) / 2;  // slice products formed: s + t <= 6
-constexpr int kTcJPartStages = 64;   // stages per row part at most: 512 rows, one exact accumulation
-constexpr int kTcJPartRows = kTcJPartStages * kTcJStageM;
+constexpr int kTcJPartStages = 64;   // stages per part at most: 1024 slots, one exact accumulation
 constexpr int kTcJAcc = 5;           // accumulators: levels 0-3 exact, levels 4-6 rounded
 constexpr int kTcJNmax = 96;         // MMA N at most: five level accumulators in the 512 columns
-constexpr int kTcJAsliceBytes = kTcM * 2 * kTcJStageM * 2;  // 128 records x 16 real K x bf16
-constexpr int kTcJTasks = kTcM * kTcJStageM;                  // (record, row) entries of a stage
+constexpr int kTcJAsliceBytes = kTcM * kTcJStageM * 2;        // 128 records x 16 K x bf16
 constexpr int kTcPairsAll = 15;      // (i, j) with i + j <= 4
 
 __host__ __device__ constexpr int pair_index(int i, int j) { return i * 5 - i * (i - 1) / 2 + j; }
@@ -951,49 +1014,55 @@ __device__ __forceinline__ void pair_of_index(int pr, int& i, int& j) {
     j = pr;
 }
 
-// Seven slices of x = hi + lo (|x| < 2^e, sc = 2^(6-e)): o[s] = m_s 2^(-7s),
-// integers |m_s| <= 64, x = 2^(e-6) sum_s o[s] up to 2^(e-51).  As in the
-// six-slice split, but the low part joins at slice 3 through an error-free
-// sum, so that none of its bits above 2^-45 (in units of o[0]) is lost.
-__device__ __forceinline__ void slice7(float hi, float lo, float sc, float (&o)[kTcJS]) {
-    float h = hi * sc;
-    const float l = lo * sc;
-    o[0] = (h + 0x1.8p23f) - 0x1.8p23f;
-    h -= o[0];
-    o[1] = (h + 0x1.8p16f) - 0x1.8p16f;
-    h -= o[1];
-    o[2] = (h + 0x1.8p9f) - 0x1.8p9f;
-    h -= o[2];
-    const df j = two_sum(h, l);  // h + l = j.hi + j.lo exactly
-    o[3] = (j.hi + 0x1.8p2f) - 0x1.8p2f;
-    h = (j.hi - o[3]) + j.lo;
-    o[4] = (h + 0x1.8p-5f) - 0x1.8p-5f;
-    h -= o[4];
-    o[5] = (h + 0x1.8p-12f) - 0x1.8p-12f;
-    h -= o[5];
-    o[6] = (h + 0x1.8p-19f) - 0x1.8p-19f;
-}
-
-// element offset of (row, k) in a stage tile [rows][16 real K] of core matrices
-__device__ __forceinline__ int tile_off16(int row, int k) {
-    return (((row >> 3) * 2 + (k >> 3)) << 6) + ((row & 7) << 3) + (k & 7);
-}
-
-// K-major, no swizzle: K-adjacent core matrices 128 B apart, 8-row groups 256 B apart
-__device__ __forceinline__ uint64_t sdesc16(uint32_t addr) {
-    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(128u >> 4) << 16) | ((uint64_t)(256u >> 4) << 32) |
-           (1ull << 46);
-}
+// Seven slices of x = h + l (|x| < 2^e): o[s] = m_s u 2^(-7s), u = 2^(e-6),
+// integers |m_s| <= 64, x = sum_s o[s] up to 2^(e-51).  As in the six-slice
+// split, but the low part joins at slice 3 through an error-free sum, so that
+// none of its bits above 2^-45 u is lost.
+struct Slicer7 {
+    float c[kTcJS];
+    __device__ __forceinline__ explicit Slicer7(float u) {
+        c[0] = 0x1.8p23f * u;
+        c[1] = 0x1.8p16f * u;
+        c[2] = 0x1.8p9f * u;
+        c[3] = 0x1.8p2f * u;
+        c[4] = 0x1.8p-5f * u;
+        c[5] = 0x1.8p-12f * u;
+        c[6] = 0x1.8p-19f * u;
+    }
+    __device__ __forceinline__ void operator()(float h, float l, float (&o)[kTcJS]) const {
+        o[0] = __fsub_rn(__fadd_rn(h, c[0]), c[0]);
+        h = __fsub_rn(h, o[0]);
+        o[1] = __fsub_rn(__fadd_rn(h, c[1]), c[1]);
+        h = __fsub_rn(h, o[1]);
+        o[2] = __fsub_rn(__fadd_rn(h, c[2]), c[2]);
+        h = __fsub_rn(h, o[2]);
+        const df j = two_sum(h, l);  // h + l = j.hi + j.lo exactly
+        o[3] = __fsub_rn(__fadd_rn(j.hi, c[3]), c[3]);
+        h = __fadd_rn(__fsub_rn(j.hi, o[3]), j.lo);
+        o[4] = __fsub_rn(__fadd_rn(h, c[4]), c[4]);
+        h = __fsub_rn(h, o[4]);
+        o[5] = __fsub_rn(__fadd_rn(h, c[5]), c[5]);
+        h = __fsub_rn(h, o[5]);
+        o[6] = __fsub_rn(__fadd_rn(h, c[6]), c[6]);
+    }
+};
 
 struct TcJArgs {
-    const int2* rows;       // (n_a, n_b) per row (the structure-factor pass's rows)
-    const int* map;         // [rows][ncols]: half-sphere index, ~index where the stored point is -n, INT_MIN none
+    const int* slots;       // the structure-factor pass's slots
+    const int* quads;       // their groups of four
+    const int* map;         // as in TcArgs
     const double2* W;       // potential W(G) on the half sphere, [dens][ng_half]
-    const int4* items;      // work items: class L | row part << 8, blocks, first block index into ipairs, first record
+    const int* sched;       // [grid + 1] offsets, then unit ids grouped by CTA
+    const int4* units;      // work units: class L | part << 8, first block group, block groups, first record
+    const int2* groups;     // block groups: first index into ipairs, blocks
     const int* ipairs;      // (i | j << 3) of each block
-    const float4* tab;      // per record [tabw]: X(0..), Y(0..), Z(0..) as complex double-float
-    __nv_bfloat16* vs;      // sliced V_ij: [15 (i, j)][stage][slice][colw x 16 real K] stage tiles
-    int* ev;                // column scales of V_ij: [15][nd][ncols]
+    const long long* voff;  // start of each block group's V tiles in vs (elements)
+    const int* vplace;      // [15 (i, j)][kNclass]: block group << 8 | place of the block in it, -1 none
+    const float4* tab;      // X(0..), Y(0..) as complex double-float, [tws] per record
+    const float4* tabz;     // Z(0..), [ncols] per record in the K order
+    const int* kpos;        // position of each record in the K order of all classes
+    __nv_bfloat16* vs;      // sliced V_ij: [block group][stage][slice][columns of its MMA x 16 K] stage tiles
+    int* ev;                // column bounds of V_ij: [15][nd][ncols]
     double* Jp;             // partial back-contraction sums [dens][part][term] in the split form's class layout
     long long ng_half;
     long long jp_total;     // doubles per density of Jp
@@ -1001,32 +1070,47 @@ struct TcJArgs {
     long long term_base[kNclass];
     int* err;               // device error word (bit 0: a bounded wait gave up)
     int ax, bx, cx;
-    int tabw, offY, offZ;
+    int nam, nbm;
+    int tws, offY;          // table entries per record (odd: conflict-free across records), start of Y
     int ncols, nd, d0;
     int gw;                 // real columns per density: 2 ncols rounded up to 8
     int colw;               // real columns per block: nd gw
-    int npad;               // MMA N of a full item: blocks x colw rounded up to 16 (<= 128)
-    int nrows, nstage, nitems;
-    int nparts, spp;        // row parts, stages per part
+    int npad;               // MMA N of a full unit: blocks x colw rounded up to 16
+    int nslots, nstage;     // slots, stages of 16
+    int nparts, spp;        // slot parts, stages per part
     long long spin;         // clock cycles a wait between roles may take before it gives up
 };
 
-// column scales: the exponent bound of max over the rows of |n_a^i n_b^j W(m, n_c)|
+// V_ij of one slot and column, without the factor i^{ta+tb} (-i)^{i+j}
+__device__ __forceinline__ cdf v_entry(const TcJArgs& g, int slot, int i, int j, int d, int nc) {
+    cdf v{{0.f, 0.f}, {0.f, 0.f}};
+    const int sl = slot < g.nslots ? __ldg(g.slots + slot) : 0;
+    if (!((sl >> 20) & 1)) return v;
+    const int na = sl & 255, nb = (sl >> 8) & 255, pa = ((sl >> 16) + i) & 1, pb = ((sl >> 17) + j) & 1;
+    for (int sa = 0; sa <= (na > 0 ? 1 : 0); ++sa)
+        for (int sb = 0; sb <= (nb > 0 ? 1 : 0); ++sb) {
+            const int idx = __ldg(g.map + ((size_t)((sa ? -na : na) + g.nam) * (2 * g.nbm + 1) +
+                                           (sb ? -nb : nb) + g.nbm) * g.ncols + nc);
+            if (idx == INT_MIN) continue;
+            const double2 w = __ldg(g.W + (long long)(g.d0 + d) * g.ng_half + (idx < 0 ? ~idx : idx));
+            cdf t{split_double(w.x), split_double(idx < 0 ? -w.y : w.y)};
+            if ((pa & sa) ^ (pb & sb)) t = cdf{df_neg(t.re), df_neg(t.im)};
+            v = cdf_add(v, t);
+        }
+    const float p = ipow((float)na, i) * ipow((float)nb, j);  // exact
+    return cdf{df_mulf(v.re, p), df_mulf(v.im, p)};
+}
+
+// column bounds: the exponent bound of max over the slots of |Re V_ij|, |Im V_ij|
 __global__ void __launch_bounds__(256) k_tc_vbound(TcJArgs g) {
     const int col = blockIdx.x;  // ((i, j) nd + d) ncols + n_c
     const int nc = col % g.ncols, d = (col / g.ncols) % g.nd, pr = col / (g.ncols * g.nd);
     int i, j;
     pair_of_index(pr, i, j);
     float mx = 0.f;
-    for (int m = threadIdx.x; m < g.nrows; m += blockDim.x) {
-        const int2 rw = __ldg(g.rows + m);
-        const int idx = __ldg(g.map + (size_t)m * g.ncols + nc);
-        if (idx == INT_MIN) continue;
-        const double2 w = __ldg(g.W + (long long)(g.d0 + d) * g.ng_half + (idx < 0 ? ~idx : idx));
-        float p = 1.f;
-        for (int k = 0; k < i; ++k) p *= (float)abs(rw.x);
-        for (int k = 0; k < j; ++k) p *= (float)abs(rw.y);
-        mx = fmaxf(mx, p * (float)fmax(fabs(w.x), fabs(w.y)));
+    for (int m = threadIdx.x; m < g.nslots; m += blockDim.x) {
+        const cdf v = v_entry(g, m, i, j, d, nc);
+        mx = fmaxf(mx, fmaxf(fabsf(v.re.hi), fabsf(v.im.hi)));
     }
     __shared__ float red[256];
     red[threadIdx.x] = mx;
@@ -1039,13 +1123,12 @@ __global__ void __launch_bounds__(256) k_tc_vbound(TcJArgs g) {
     if (threadIdx.x == 0) g.ev[col] = red[0] > 0.f ? exp_bound(log2f(red[0] * 1.0001f)) : -100;
 }
 
-// V_ij sliced into stage tiles: tile (i, j), stage q, slice s holds column
-// d gw + 2 n_c + part and K = (row, re/im) in the real form rows
-// (m, re) -> [Re V | Im V], (m, im) -> [-Im V | Re V]; columns past 2 ncols
-// stay zero from the allocation.
+// V_ij sliced into stage tiles: block group, stage q, slice s holds the columns
+// of its blocks, d gw + 2 n_c (Re) and + 1 (Im) within a block, and K = slot;
+// one thread per two slots; columns past 2 ncols are never read back.
 __global__ void __launch_bounds__(256) k_tc_vslice(TcJArgs g) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long per_pair = (long long)g.nstage * kTcJStageM * g.nd * g.ncols;
+    const long long per_pair = (long long)g.nstage * (kTcJStageM / 2) * g.nd * g.ncols;
     if (t >= kTcPairsAll * per_pair) return;
     const int pr = (int)(t / per_pair);
     long long rem = t - pr * per_pair;
@@ -1053,116 +1136,79 @@ __global__ void __launch_bounds__(256) k_tc_vslice(TcJArgs g) {
     rem /= g.ncols;
     const int d = (int)(rem % g.nd);
     rem /= g.nd;
-    const int ml = (int)(rem % kTcJStageM), q = (int)(rem / kTcJStageM);
-    const int m = q * kTcJStageM + ml;
+    const int m2 = (int)(rem % (kTcJStageM / 2)), q = (int)(rem / (kTcJStageM / 2));
     int i, j;
     pair_of_index(pr, i, j);
-    cdf v{{0.f, 0.f}, {0.f, 0.f}};
-    if (m < g.nrows) {
-        const int2 rw = __ldg(g.rows + m);
-        const int idx = __ldg(g.map + (size_t)m * g.ncols + nc);
-        if (idx != INT_MIN) {
-            const double2 w = __ldg(g.W + (long long)(g.d0 + d) * g.ng_half + (idx < 0 ? ~idx : idx));
-            float p = 1.f;  // n_a^i n_b^j, exact
-            for (int k = 0; k < i; ++k) p *= (float)rw.x;
-            for (int k = 0; k < j; ++k) p *= (float)rw.y;
-            const cdf wv{split_double(w.x), split_double(idx < 0 ? -w.y : w.y)};
-            v = rot_mi(cdf{df_mulf(wv.re, p), df_mulf(wv.im, p)}, i + j);
-        }
-    }
-    const float sc = pow2f(6 - g.ev[(pr * g.nd + d) * g.ncols + nc]);
-    float sr[kTcJS], si[kTcJS];
-    slice7(v.re.hi, v.re.lo, sc, sr);
-    slice7(v.im.hi, v.im.lo, sc, si);
-    const int c0 = d * g.gw + 2 * nc;
-    __nv_bfloat16* base = g.vs + ((size_t)pr * g.nstage + q) * kTcJS * (size_t)g.colw * 16;
-    const int o0 = tile_off16(c0, 2 * ml), o1 = tile_off16(c0 + 1, 2 * ml);
+    const Slicer7 cut(pow2f(g.ev[(pr * g.nd + d) * g.ncols + nc] - 6));
+    float sr[2][kTcJS], si[2][kTcJS];
 #pragma unroll
-    for (int s = 0; s < kTcJS; ++s) {
-        __nv_bfloat16* bs = base + (size_t)s * g.colw * 16;
-        *reinterpret_cast<uint32_t*>(bs + o0) = pack_bf2(sr[s], -si[s]);
-        *reinterpret_cast<uint32_t*>(bs + o1) = pack_bf2(si[s], sr[s]);
+    for (int e = 0; e < 2; ++e) {
+        const int slot = q * kTcJStageM + 2 * m2 + e;
+        const int sl = slot < g.nslots ? __ldg(g.slots + slot) : 0;
+        const cdf v = rot_mi(v_entry(g, slot, i, j, d, nc), i + j + 8 - ((sl >> 16) & 1) - ((sl >> 17) & 1));
+        cut(v.re.hi, v.re.lo, sr[e]);
+        cut(v.im.hi, v.im.lo, si[e]);
+    }
+    // every block group that holds (i, j), at most one per class
+    for (int L = 0; L < kNclass; ++L) {
+        const int pl = __ldg(g.vplace + pr * kNclass + L);
+        if (pl < 0) continue;
+        const int gi = pl >> 8, nw = mma_cols(__ldg(&g.groups[gi].y), g.colw);
+        const int c0 = (pl & 255) * g.colw + d * g.gw + 2 * nc;
+        const int o0 = tile_off(c0, 2 * m2), o1 = tile_off(c0 + 1, 2 * m2);
+        __nv_bfloat16* bs = g.vs + __ldg(g.voff + gi) + (size_t)q * kTcJS * nw * 16;
+#pragma unroll
+        for (int s = 0; s < kTcJS; ++s, bs += nw * 16) {
+            *reinterpret_cast<uint32_t*>(bs + o0) = pack_bf2(sr[0][s], sr[1][s]);
+            *reinterpret_cast<uint32_t*>(bs + o1) = pack_bf2(si[0][s], si[1][s]);
+        }
     }
 }
 
 struct TcJSmem {
-    int rec[kTcM];
-    int pairs[kTcGmax];
-    int tidx[kTcGmax][5];  // index of J'_{ijk} for block (i, j) and k = 0..4 (-1 past the class's degree)
-    int2 rowi[kTcJPartRows];  // the part's rows
-    int iL, inb, ipart;
-    uint64_t full[kTcNbuf], empty[kTcNbuf], bfull[kTcNbuf], tfull, accf, acce, done, psync;
+    uint64_t afull[kTcNbufMax], bfull[kTcNbufMax], empty[kTcNbufMax], tfull, tempty, accf, acce, done;
     uint32_t tmem;
     int abort_flag;
 };
 
-// index of J'_{p1 p2 p3} (powers of n_1, n_2, n_3) for powers (i, j, k) of (n_a, n_b, n_c)
-__device__ __forceinline__ int term_of_j(const TcJArgs& g, int i, int j, int k) {
-    const int p1 = g.ax == 0 ? i : (g.bx == 0 ? j : k);
-    const int p2 = g.ax == 1 ? i : (g.bx == 1 ? j : k);
-    const int lam = i + j + k;
-    return lam_offset(lam) + mono_index(lam, p1, p2);
-}
-
-// A^T entry (record r, stage row ml): X_r(n_a) Y_r(n_b) sliced, one 4-byte
-// store (re, im) per slice; a warp's 32 entries (8 records x 4 rows) fill
-// eight core-matrix rows, 128 contiguous bytes
-__device__ __forceinline__ void form_aj(const TcJArgs& g, const TcJSmem& sm, const float4* tabs, int q, int k,
-                                        unsigned char* as) {
-    const int ml = (k & 3) | (((k >> 5) & 1) << 2);
-    const int r = ((k >> 2) & 7) | ((k >> 6) << 3);
-    const int m = q * kTcJStageM + ml;  // q: stage of the part
-    cdf a{{0.f, 0.f}, {0.f, 0.f}};
-    if (sm.rowi[m].x != INT_MIN && sm.rec[r] >= 0) {
-        const int2 rw = sm.rowi[m];
-        const float4 xv = tabs[r * g.tabw + abs(rw.x)], yv = tabs[r * g.tabw + g.offY + abs(rw.y)];
-        const float sa = rw.x < 0 ? -1.f : 1.f, sb = rw.y < 0 ? -1.f : 1.f;  // X(-n) = conj X(n)
-        a = cdf_mul(cdf{{xv.x, xv.y}, {sa * xv.z, sa * xv.w}}, cdf{{yv.x, yv.y}, {sb * yv.z, sb * yv.w}});
-    }
-    float sr[kTcJS], si[kTcJS];
-    slice7(a.re.hi, a.re.lo, 0x1p5f, sr);  // |A| <= 1 < 2^1
-    slice7(a.im.hi, a.im.lo, 0x1p5f, si);
-    const int off = tile_off16(r, 2 * ml);
-#pragma unroll
-    for (int s = 0; s < kTcJS; ++s)
-        *reinterpret_cast<uint32_t*>(as + (size_t)s * kTcJAsliceBytes + (size_t)off * 2) = pack_bf2(sr[s], si[s]);
-}
-
-// Persistent over the work items (class, group of (i, j) blocks, 128
-// records, row part), with the structure-factor kernel's roles: warps 0-13
-// form the A^T slices of each 8-row stage, lane 0 of warp 14 issues the MMAs, warp 15
-// brings the item's factor tables (once per item) and the V_ij stage tiles
-// in with bulk copies; warps 0-11 then form J' from tensor memory (lane
-// quadrant w & 3, (block, density) groups w / 4 mod 3).  Waits are bounded
-// as in the structure-factor kernel.
-__global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g) {
+// Persistent over work units (class, slot part, 128 records), each running
+// its (i, j) block groups in turn on the same staged factor tables, dealt to
+// the CTAs at plan time (largest first, least loaded).  The structure-factor
+// kernel's roles: warps 0-15, two groups in turn, form the A^T slices of each
+// 16-slot stage, one thread per record and eight slots (two point groups: two
+// 16-byte table reads and four real products each, one 16-byte core-matrix row
+// per slice), lane 0 of warp 16 issues the MMAs, warp 17 brings the factor
+// tables and warp 18 the V_ij stage tiles in with bulk copies; warps 0-15 then
+// form J' from tensor memory (lane quadrant w & 3, (block, density) pairs
+// w / 4 mod 4).  Waits are bounded as in the structure-factor kernel.
+__global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) {
     extern __shared__ __align__(1024) unsigned char tsm[];
-    const int bslice = g.npad * 32;
+    const int bbytes = kTcJS * g.npad * 32;
     unsigned char* abuf = tsm;                                                     // [nbuf][S][4096]
-    unsigned char* bbuf = abuf + (size_t)kTcNbuf * kTcJS * kTcJAsliceBytes;          // [nbuf][S][npad x 32]
-    float4* tabs = reinterpret_cast<float4*>(bbuf + (size_t)kTcNbuf * kTcJS * bslice);  // [128][tabw]
-    TcJSmem& sm = *reinterpret_cast<TcJSmem*>(tabs + (size_t)kTcM * g.tabw);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    unsigned char* bbuf = abuf + (size_t)nbuf * kTcJS * kTcJAsliceBytes;             // [nbuf][S][npad x 32]
+    float4* tabs = reinterpret_cast<float4*>(bbuf + (size_t)nbuf * bbytes);         // [128][tws]: X, Y
+    TcJSmem& sm = *reinterpret_cast<TcJSmem*>(tabs + (size_t)kTcM * g.tws);
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     volatile int* abort_flag = &sm.abort_flag;
-    const bool mma_warp = warp == kTcMmaWarp, load_warp = warp == kTcLoadWarp, epi = warp < kTcEpiWarps;
     if (tid == 0) {
-        for (int b = 0; b < kTcNbuf; ++b) {
-            mbar_init(&sm.full[b], kTcProdWarps);
-            mbar_init(&sm.empty[b], 1);
+        for (int b = 0; b < nbuf; ++b) {
+            mbar_init(&sm.afull[b], kTcGroupWarps);
             mbar_init(&sm.bfull[b], 1);
+            mbar_init(&sm.empty[b], 1);
         }
         mbar_init(&sm.tfull, 1);
+        mbar_init(&sm.tempty, kTcProdWarps);
         mbar_init(&sm.accf, 1);
-        mbar_init(&sm.acce, kTcEpiWarps);
+        mbar_init(&sm.acce, kTcProdWarps);
         mbar_init(&sm.done, 1);
-        mbar_init(&sm.psync, kTcWarps);
         sm.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // columns of B past an item's blocks are never read into an output: clear them once
-    for (int i = tid; i < kTcNbuf * kTcJS * bslice / 16; i += kTcThreadsAll)
+    // finite start: columns of B past a unit's blocks and rows of A past its records are never read into an output
+    for (int i = tid; i < nbuf * bbytes / 16; i += kTcThreadsAll)
         reinterpret_cast<uint4*>(bbuf)[i] = make_uint4(0u, 0u, 0u, 0u);
-    if (mma_warp) {
+    for (int i = tid; i < kTcM * g.tws; i += kTcThreadsAll) tabs[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (warp == kTcMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(&sm.tmem)),
                      "r"(kTcTmemCols)
                      : "memory");
@@ -1173,217 +1219,253 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g) {
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sm.tmem;
-    const int equad = warp & 3, ethird = warp >> 2, erow = 32 * equad + lane;
-    const uint32_t tlane = (uint32_t)(32 * equad) << 16;
-    long long gs = 0;  // stages so far (every role counts the same)
-    int nit = 0;       // items finished
-    int ntab = 0;      // table loads issued (load warp)
-    uint32_t ph = 0;
+    const int j0 = __ldg(g.sched + blockIdx.x), j1 = __ldg(g.sched + blockIdx.x + 1);
+    const int* ulist = g.sched + gridDim.x + 1;
     bool ok = true;
-    for (int it = blockIdx.x; it < g.nitems; it += gridDim.x) {
-        // ---- the item: class, blocks, records ----
-        const int4 in = __ldg(g.items + it);
-        const int iL = in.x & 255, part = in.x >> 8;
-        if (tid == 0) {
-            sm.iL = iL;
-            sm.inb = in.y;
-            sm.ipart = part;
-            for (int b = 0; b < in.y; ++b) {
-                const int pr = __ldg(g.ipairs + in.z + b), i = pr & 7, j = pr >> 3;
-                sm.pairs[b] = pr;
-                for (int kk = 0; kk < 5; ++kk) sm.tidx[b][kk] = kk <= iL - i - j ? term_of_j(g, i, j, kk) : -1;
-            }
-        }
-        if (tid < kTcM) sm.rec[tid] = (long long)in.w + tid < g.cls_start[iL + 1] ? in.w + tid : -1;
-        for (int m = tid; m < kTcJPartRows; m += kTcThreadsAll) {
-            const int mg = part * g.spp * kTcJStageM + m;
-            sm.rowi[m] = m < g.spp * kTcJStageM && mg < g.nrows ? __ldg(g.rows + mg) : make_int2(INT_MIN, 0);
-        }
-        if (!(ok = prod_sync(&sm.psync, ph, abort_flag, lane, g.spin))) break;
-        const int L = sm.iL, nb = sm.inb, q0 = sm.ipart * g.spp, nst = min(g.spp, g.nstage - q0);
-        if (load_warp) {
-            // the records' factor tables, then every stage's V_ij tiles
-            if (lane == 0) {
-                uint32_t nv = 0;
-                for (int r = 0; r < kTcM; ++r) nv += sm.rec[r] >= 0 ? 1u : 0u;
-                mbar_arrive_tx(&sm.tfull, nv * (uint32_t)g.tabw * 16u);
-            }
-            __syncwarp();
-            for (int r = lane; r < kTcM; r += 32)
-                if (sm.rec[r] >= 0)
-                    bulk_copy(tabs + (size_t)r * g.tabw, g.tab + (size_t)sm.rec[r] * g.tabw, (uint32_t)g.tabw * 16u,
-                              &sm.tfull);
-            ++ntab;
-            const uint32_t blk = (uint32_t)g.colw * 32u;  // bytes of one block's slice of a stage
-            for (int q = 0; q < nst; ++q, ++gs) {
-                const int slot = (int)(gs & 1);
-                if (gs >= kTcNbuf) {
-                    ok = __all_sync(0xffffffffu, mbar_wait(&sm.empty[slot], (uint32_t)(((gs >> 1) - 1) & 1), abort_flag, g.spin));
-                    if (!ok) break;
-                }
-                unsigned char* bs = bbuf + (size_t)slot * kTcJS * bslice;
-                if (lane == 0) mbar_arrive_tx(&sm.bfull[slot], (uint32_t)(nb * kTcJS) * blk);
-                __syncwarp();
-                for (int c = lane; c < nb * kTcJS; c += 32) {
-                    const int gb = c / kTcJS, s = c - gb * kTcJS;
-                    const int pr = sm.pairs[gb];
-                    const size_t src =
-                        (((size_t)pair_index(pr & 7, pr >> 3) * g.nstage + q0 + q) * kTcJS + s) * g.colw * 16;
-                    bulk_copy(bs + (size_t)s * bslice + (size_t)gb * blk, g.vs + src, blk, &sm.bfull[slot]);
-                }
-                __syncwarp();
-            }
-        } else if (!mma_warp) {
-            ok = __all_sync(0xffffffffu, mbar_wait(&sm.tfull, (uint32_t)(nit & 1), abort_flag, g.spin));
-            if (ok) {
-                for (int q = 0; q < nst; ++q, ++gs) {
-                    const int slot = (int)(gs & 1);
-                    if (gs >= kTcNbuf) {
-                        ok = __all_sync(0xffffffffu,
-                                        mbar_wait(&sm.empty[slot], (uint32_t)(((gs >> 1) - 1) & 1), abort_flag, g.spin));
-                        if (!ok) break;
-                    }
-                    unsigned char* as = abuf + (size_t)slot * kTcJS * kTcJAsliceBytes;
-                    for (int k = tid; k < kTcJTasks; k += kTcProdThreads) form_aj(g, sm, tabs, q, k, as);
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&sm.full[slot]);
-                }
-            }
-        } else {
-            if (lane == 0) {
-                const uint32_t a0 = saddr(abuf), b0 = saddr(bbuf);
-                const int nw = min(g.npad, (nb * g.colw + 15) / 16 * 16);
-                const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(nw >> 3) << 17) |
-                                       ((uint32_t)(kTcM >> 4) << 24);
-                bool first[kTcJAcc] = {true, true, true, true, true};
-                bool mok = true;
-                if (nit > 0) mok = mbar_wait(&sm.acce, (uint32_t)((nit - 1) & 1), abort_flag, g.spin);  // tensor memory drained
-                tc_fence_after();
-                for (int q = 0; q < nst && mok; ++q, ++gs) {
-                    const int slot = (int)(gs & 1);
-                    if (!(mok = mbar_wait(&sm.full[slot], (uint32_t)((gs >> 1) & 1), abort_flag, g.spin))) break;
-                    if (!(mok = mbar_wait(&sm.bfull[slot], (uint32_t)((gs >> 1) & 1), abort_flag, g.spin))) break;
-                    tc_fence_after();
-                    const uint32_t as = a0 + slot * kTcJS * kTcJAsliceBytes, bs = b0 + slot * kTcJS * bslice;
-#pragma unroll
-                    for (int s = 0; s < kTcJS; ++s)
-#pragma unroll
-                        for (int t = 0; s + t < kTcJS; ++t) {
-                            const int lv = min(s + t, kTcJAcc - 1);
-                            tc_mma(tmem + (uint32_t)(lv * g.npad), sdesc16(as + s * kTcJAsliceBytes),
-                                   sdesc16(bs + t * bslice), idesc, first[lv] ? 0u : 1u);
-                            first[lv] = false;
-                        }
-                    tc_commit(&sm.empty[slot]);
-                }
-                if (mok) tc_commit(&sm.accf);
-                ok = mok;
-            }
-            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-            gs = __shfl_sync(0xffffffffu, gs, 0);
-        }
-        if (!ok) break;
-        // ---- J'_{r,ijk} = Re (-i)^k sum_{n_c} n_c^k Z_r(n_c) U_ij[r, n_c] (warps 0-11) ----
-        if (epi) {
-            ok = __all_sync(0xffffffffu, mbar_wait(&sm.accf, (uint32_t)(nit & 1), abort_flag, g.spin));
-            if (!ok) break;
-            tc_fence_after();
-            const int r = sm.rec[erow];
-            const long long cnt = g.cls_start[L + 1] - g.cls_start[L];
-            for (int grp = ethird; grp < nb * g.nd; grp += 3) {
-                const int gb = grp / g.nd, d = grp - gb * g.nd;
-                const int pr = sm.pairs[gb], i = pr & 7, j = pr >> 3, nk = L - i - j;
-                const int* evp = g.ev + (pair_index(i, j) * g.nd + d) * g.ncols;
-                cdf J[5];
-#pragma unroll
-                for (int kk = 0; kk < 5; ++kk) J[kk] = cdf{{0.f, 0.f}, {0.f, 0.f}};
-                for (int c8 = 0; c8 < g.gw / 8; ++c8) {
-                    float T[kTcJAcc][8];
-#pragma unroll
-                    for (int lv = 0; lv < kTcJAcc; ++lv)
-                        tc_ld8(tmem + tlane + (uint32_t)(lv * g.npad + gb * g.colw + d * g.gw + 8 * c8), T[lv]);
-                    if (r < 0) continue;
-#pragma unroll
-                    for (int u = 0; u < 8; u += 2) {
-                        const int nc = 4 * c8 + u / 2;
-                        if (nc < g.ncols) {
-                            cdf v;
-                            v.re = df_add(df_add(df_add(two_sum(T[0][u], T[1][u]), df{T[2][u], 0.f}), df{T[3][u], 0.f}),
-                                          df{T[4][u], 0.f});
-                            v.im = df_add(df_add(df_add(two_sum(T[0][u + 1], T[1][u + 1]), df{T[2][u + 1], 0.f}),
-                                                 df{T[3][u + 1], 0.f}),
-                                          df{T[4][u + 1], 0.f});
-                            const float sc = pow2f(1 + __ldg(evp + nc) - 12);  // exact power of two
-                            v = cdf{df{v.re.hi * sc, v.re.lo * sc}, df{v.im.hi * sc, v.im.lo * sc}};
-                            const float4 zv = tabs[erow * g.tabw + g.offZ + nc];
-                            const cdf zu = cdf_mul(cdf{{zv.x, zv.y}, {zv.z, zv.w}}, v);
-                            float pw = 1.f;  // n_c^k, exact
-#pragma unroll
-                            for (int kk = 0; kk < 5; ++kk) {
-                                if (kk <= nk) J[kk] = cdf{df_add(J[kk].re, df_mulf(zu.re, pw)), df_add(J[kk].im, df_mulf(zu.im, pw))};
-                                pw *= (float)nc;
-                            }
-                        }
-                    }
-                }
-                if (r >= 0) {
-                    double* jp = g.Jp + ((long long)(g.d0 + d) * g.nparts + sm.ipart) * g.jp_total + g.term_base[L] +
-                                 (r - g.cls_start[L]);
-#pragma unroll
-                    for (int kk = 0; kk < 5; ++kk)
-                        if (kk <= nk) {
-                            const df re = rot_mi(J[kk], kk).re;
-                            jp[(long long)sm.tidx[gb][kk] * cnt] = (double)re.hi + (double)re.lo;
-                        }
-                }
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sm.acce);
-        }
-        ++nit;
-        // the tables, records and blocks are rewritten by the next item
-        if (!(ok = prod_sync(&sm.psync, ph, abort_flag, lane, g.spin) && ok)) break;
-    }
-    if (load_warp && lane == 0) {
-        // bulk copies still in flight (after a failed wait) land before the CTA exits
-        for (int b = 0; b < kTcNbuf && b < gs; ++b) {
-            const long long last = gs - 1 - ((gs - 1 - b) % kTcNbuf);
-            const long long t0 = clock64();
-            while (!mbar_test(&sm.bfull[b], (uint32_t)((last >> 1) & 1)) && clock64() - t0 < kTcSpinCycles) {
-            }
-        }
-        if (ntab > 0) {
-            const long long t0 = clock64();
-            while (!mbar_test(&sm.tfull, (uint32_t)((ntab - 1) & 1)) && clock64() - t0 < kTcSpinCycles) {
-            }
-        }
-    }
-    if (mma_warp) {
-        // everything issued completes before tensor memory is freed
+
+    if (warp == kTcTabWarp) {
+        // the units' factor tables: consecutive records, one bulk copy each
         if (lane == 0) {
+            long long nu = 0;
+            for (int ju = j0; ju < j1; ++ju, ++nu) {
+                const int4 un = __ldg(g.units + __ldg(ulist + ju));
+                const int nv = (int)min((long long)kTcM, g.cls_start[(un.x & 255) + 1] - un.w);
+                if (nu > 0 && !mbar_wait(&sm.tempty, (uint32_t)((nu - 1) & 1), abort_flag, g.spin)) break;
+                const uint32_t bytes = (uint32_t)(nv * g.tws) * 16u;
+                mbar_arrive_tx(&sm.tfull, bytes);
+                bulk_copy(tabs, g.tab + (size_t)un.w * g.tws, bytes, &sm.tfull);
+            }
+            ring_settle(&sm.tfull, 1, nu);
+        }
+        __syncwarp();
+    } else if (warp == kTcLoadWarp) {
+        // the stages' V_ij tiles, one bulk copy each
+        if (lane == 0) {
+            Ring b(nbuf);
+            long long gs = 0;
+            for (int ju = j0; ju < j1 && ok; ++ju) {
+                const int4 un = __ldg(g.units + __ldg(ulist + ju));
+                const int q0 = (un.x >> 8) * g.spp, nst = min(g.spp, g.nstage - q0);
+                for (int gi = 0; gi < un.z && ok; ++gi) {
+                    const uint32_t bytes = (uint32_t)(kTcJS * mma_cols(__ldg(&g.groups[un.y + gi].y), g.colw) * 32);
+                    const unsigned char* src = reinterpret_cast<const unsigned char*>(g.vs + __ldg(g.voff + un.y + gi)) +
+                                               (size_t)q0 * bytes;
+                    for (int q = 0; q < nst; ++q, ++gs, b.next()) {
+                        if (gs >= nbuf && !(ok = mbar_wait(&sm.empty[b.i], b.ph ^ 1u, abort_flag, g.spin))) break;
+                        mbar_arrive_tx(&sm.bfull[b.i], bytes);
+                        bulk_copy(bbuf + (size_t)b.i * bbytes, src + (size_t)q * bytes, bytes, &sm.bfull[b.i]);
+                    }
+                }
+            }
+            ring_settle(sm.bfull, nbuf, gs);
+        }
+        __syncwarp();
+    } else if (warp == kTcMmaWarp) {
+        const uint32_t a0 = saddr(abuf), b0 = saddr(bbuf);
+        Ring b(nbuf);
+        int ng = 0;  // block groups issued
+        for (int ju = j0; ju < j1 && ok; ++ju) {
+            const int4 un = __ldg(g.units + __ldg(ulist + ju));
+            const int nst = min(g.spp, g.nstage - (un.x >> 8) * g.spp);
+            for (int gi = 0; gi < un.z && ok; ++gi, ++ng) {
+                const uint32_t nw = (uint32_t)mma_cols(__ldg(&g.groups[un.y + gi].y), g.colw);
+                const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTcM >> 4) << 24);
+                // tensor memory drained
+                if (ng > 0 && !(ok = __all_sync(0xffffffffu, mbar_wait(&sm.acce, (uint32_t)((ng - 1) & 1), abort_flag, g.spin))))
+                    break;
+                tc_fence_after();
+                for (int q = 0; q < nst; ++q, b.next()) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(&sm.bfull[b.i], b.ph, abort_flag, g.spin) &&
+                                                     mbar_wait(&sm.afull[b.i], b.ph, abort_flag, g.spin));
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (elect_one()) {
+                        issue_kstep<kTcJS, kTcJAcc>(tmem, sdesc(a0 + b.i * kTcJS * kTcJAsliceBytes), kTcJAsliceBytes >> 4,
+                                                    sdesc(b0 + b.i * bbytes), nw * 2, nw, idesc, q > 0);
+                        tc_commit(&sm.empty[b.i]);
+                        if (q + 1 == nst) tc_commit(&sm.accf);
+                    }
+                    __syncwarp();
+                }
+            }
+        }
+        // everything issued completes before tensor memory is freed
+        if (elect_one()) {
             tc_commit(&sm.done);
             const long long t0 = clock64();
             while (!mbar_test(&sm.done, 0u) && clock64() - t0 < kTcSpinCycles) {
             }
         }
         __syncwarp();
+    } else {
+        // operand role: record rec, slots 8 oct .. 8 oct + 7 (two point groups) of its group's stages
+        const int grp = warp / kTcGroupWarps, rec = tid & (kTcM - 1), oct = (tid >> 7) & 1;
+        const float4* trec = tabs + (size_t)rec * g.tws;
+        unsigned char* arow = abuf + tile_off(rec, oct * 8) * 2;
+        const Slicer7 cut(0x1p-5f);  // |A| <= 1 < 2^1
+        // epilogue role
+        const int eq = warp & 3, es = warp >> 2, erow = 32 * eq + lane;
+        const uint32_t tlane = (uint32_t)(32 * eq) << 16;
+        const int nquad = g.nslots / 4;
+        Ring b(nbuf);
+        int gs = 0, ng = 0, nu = 0;
+        bool full = false;  // every buffer used once
+        for (int ju = j0; ju < j1 && ok; ++ju, ++nu) {
+            const int4 un = __ldg(g.units + __ldg(ulist + ju));
+            const int L = un.x & 255, part = un.x >> 8, q0 = part * g.spp, nst = min(g.spp, g.nstage - q0);
+            const long long r = (long long)un.w + erow;
+            const bool rvalid = r < g.cls_start[L + 1];
+            const long long cnt = g.cls_start[L + 1] - g.cls_start[L];
+            if (!(ok = __all_sync(0xffffffffu, mbar_wait(&sm.tfull, (uint32_t)(nu & 1), abort_flag, g.spin)))) break;
+            for (int gi = 0; gi < un.z && ok; ++gi, ++ng) {
+                for (int q = 0; q < nst; ++q, ++gs, b.next()) {
+                    full = full || gs >= nbuf;
+                    if ((gs & 1) != grp) continue;
+                    const int qd = (q0 + q) * 4 + oct * 2;
+                    uint32_t pk[kTcJS][4];
+#pragma unroll
+                    for (int v = 0; v < 2; ++v) {
+                        const int info = qd + v < nquad ? __ldg(g.quads + qd + v) : 0;
+                        const int n0 = (info >> 2) & 255, n1 = (info >> 10) & 255;
+                        // the four products of the point group, in slot order; with one index zero its factor is 1
+                        df a[4];
+                        if (info & 1) {
+                            const float4 x = trec[n0], y = trec[g.offY + n1];
+                            const df x0{x.x, x.y}, x1{x.z, x.w}, y0{y.x, y.y}, y1{y.z, y.w};
+                            a[0] = df_mul_u(x0, y0);
+                            a[1] = df_mul_u(x1, y0);
+                            a[2] = df_mul_u(x0, y1);
+                            a[3] = df_mul_u(x1, y1);
+                        } else {
+                            const int off = info & 2 ? 0 : g.offY;
+                            const float4 x = trec[off + n0], y = trec[off + n1];
+                            const bool ab = info & 2;
+                            a[0] = df{x.x, x.y};
+                            a[1] = ab ? df{x.z, x.w} : df{y.x, y.y};
+                            a[2] = ab ? df{y.x, y.y} : df{x.z, x.w};
+                            a[3] = df{y.z, y.w};
+                        }
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            float o0[kTcJS], o1[kTcJS];
+                            cut(a[2 * h].hi, a[2 * h].lo, o0);
+                            cut(a[2 * h + 1].hi, a[2 * h + 1].lo, o1);
+#pragma unroll
+                            for (int s = 0; s < kTcJS; ++s) pk[s][2 * v + h] = pack_bf2(o0[s], o1[s]);
+                        }
+                    }
+                    if (full) {
+                        ok = __all_sync(0xffffffffu, mbar_wait(&sm.empty[b.i], b.ph ^ 1u, abort_flag, g.spin));
+                        if (!ok) break;
+                    }
+                    unsigned char* as = arow + (size_t)b.i * kTcJS * kTcJAsliceBytes;
+#pragma unroll
+                    for (int s = 0; s < kTcJS; ++s)
+                        *reinterpret_cast<uint4*>(as + (size_t)s * kTcJAsliceBytes) =
+                            make_uint4(pk[s][0], pk[s][1], pk[s][2], pk[s][3]);
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&sm.afull[b.i]);
+                }
+                if (!ok) break;
+                // the last reads of the unit's tables are done
+                if (gi + 1 == un.z) {
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&sm.tempty);
+                }
+                // ---- J'_{r,ijk} = Re (-i)^k sum_{n_c} n_c^k Z_r(n_c) U_ij[r, n_c] ----
+                ok = __all_sync(0xffffffffu, mbar_wait(&sm.accf, (uint32_t)(ng & 1), abort_flag, g.spin));
+                if (!ok) break;
+                tc_fence_after();
+                const int2 gr = __ldg(g.groups + un.y + gi);
+                const uint32_t nw = (uint32_t)mma_cols(gr.y, g.colw);
+                const float4* zrec = g.tabz + (size_t)__ldg(g.kpos + (rvalid ? r : un.w)) * g.ncols;
+                for (int pd = es; pd < gr.y * g.nd; pd += kTcProdWarps / 4) {
+                    const int gb = pd / g.nd, d = pd - gb * g.nd;
+                    const int pr = __ldg(g.ipairs + gr.x + gb), i = pr & 7, j = pr >> 3, nk = L - i - j;
+                    df J[5];
+#pragma unroll
+                    for (int kk = 0; kk < 5; ++kk) J[kk] = df{0.f, 0.f};
+                    for (int c4 = 0; c4 < g.gw / 4; ++c4) {
+                        float T[kTcJAcc][4];
+                        float4 zv[2];
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) zv[u] = __ldg(zrec + min(2 * c4 + u, g.ncols - 1));
+                        tc_ld_levels4(tmem + tlane + (uint32_t)(gb * g.colw + d * g.gw + 4 * c4), nw, T);
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            const int nc = 2 * c4 + u;
+                            if (nc < g.ncols) {
+                                const cdf v{level_sum(T[0][2 * u], T[1][2 * u], T[2][2 * u], T[3][2 * u], T[4][2 * u]),
+                                            level_sum(T[0][2 * u + 1], T[1][2 * u + 1], T[2][2 * u + 1],
+                                                      T[3][2 * u + 1], T[4][2 * u + 1])};
+                                const cdf zu = cdf_mul_u(cdf{{zv[u].x, zv[u].y}, {zv[u].z, zv[u].w}}, v);
+                                float pw = 1.f;  // n_c^k, exact; Re (-i)^k zu is +-Re (k even) or +-Im (k odd)
+#pragma unroll
+                                for (int kk = 0; kk < 5; ++kk) {
+                                    if (kk <= nk) J[kk] = df_add(J[kk], df_mulf_u(kk & 1 ? zu.im : zu.re, pw));
+                                    pw *= (float)nc;
+                                }
+                            }
+                        }
+                    }
+                    if (rvalid) {
+                        double* jp = g.Jp + ((long long)(g.d0 + d) * g.nparts + part) * g.jp_total + g.term_base[L] +
+                                     (r - g.cls_start[L]);
+#pragma unroll
+                        for (int kk = 0; kk < 5; ++kk)
+                            if (kk <= nk) {
+                                const double v = (double)J[kk].hi + (double)J[kk].lo;
+                                jp[(long long)term_of(g.ax, g.bx, i, j, kk) * cnt] = kk == 2 || kk == 3 ? -v : v;
+                            }
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sm.acce);
+            }
+        }
     }
     tc_fence_before();
     __syncthreads();
     if (*abort_flag && tid == 0) atomicOr(g.err, 1);
-    if (mma_warp) {
-        __syncwarp();
+    if (warp == kTcMmaWarp) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols) : "memory");
     }
 }
 
-size_t tc_j_smem_bytes(int npad, int tabw) {
-    const size_t need = (size_t)kTcNbuf * kTcJS * kTcJAsliceBytes + (size_t)kTcNbuf * kTcJS * npad * 32 +
-                        (size_t)kTcM * tabw * 16 + sizeof(TcJSmem) + 64;
+size_t tc_j_smem_bytes(int npad, int tws, int nbuf) {
+    const size_t need = (size_t)nbuf * kTcJS * (kTcJAsliceBytes + (size_t)npad * 32) + (size_t)kTcM * tws * 16 +
+                        sizeof(TcJSmem) + 64;
     return std::max<size_t>(need, 120 * 1024);
+}
+
+// work dealt to nbin bins, largest first, each to the least loaded bin (ties
+// to the lower one): nbin + 1 offsets, then the item ids of each bin
+std::vector<int> deal(const std::vector<double>& cost, int nbin) {
+    std::vector<int> order(cost.size());
+    for (size_t k = 0; k < order.size(); ++k) order[k] = (int)k;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
+    std::vector<std::vector<int>> lists(nbin);
+    using Slot = std::pair<double, int>;
+    std::priority_queue<Slot, std::vector<Slot>, std::greater<Slot>> heap;
+    for (int b = 0; b < nbin; ++b) heap.push({0.0, b});
+    for (int k : order) {
+        const Slot s = heap.top();
+        heap.pop();
+        lists[s.second].push_back(k);
+        heap.push({s.first + cost[k], s.second});
+    }
+    std::vector<int> out;
+    int off = 0;
+    for (const auto& l : lists) {
+        out.push_back(off);
+        off += (int)l.size();
+    }
+    out.push_back(off);
+    for (const auto& l : lists) out.insert(out.end(), l.begin(), l.end());
+    return out;
 }
 
 }  // namespace
@@ -1397,9 +1479,9 @@ long long tc_spin(const ftcj_plan* P) {
 
 int setup_tc_j(ftcj_plan* P);
 
-// Plan-time set-up of the tensor-core form: the column axis, the rows and
-// their half-sphere map, the factor tables, the windows (class, block group,
-// 512 records sorted by width) and the partial-row count.
+// Plan-time set-up of the tensor-core form: the column axis, the slots and the
+// half-sphere map, the factor tables, the windows (class, block group, records
+// sorted by width), their deal to CTA groups and the B tiles.
 int setup_tc(ftcj_plan* P) {
     if (!P->ortho) return fail(FTCJ_EUNSUPPORTED, "the tensor-core contraction needs an orthorhombic cell");
     if (P->precision != FTCJ_PREC_SPLIT)
@@ -1409,10 +1491,14 @@ int setup_tc(ftcj_plan* P) {
     const int64_t ngh = P->ng_half;
     int64_t recs_by_class[kNclass];
     for (int L = 0; L < kNclass; ++L) recs_by_class[L] = P->class_start[L + 1] - P->class_start[L];
-    // the column axis: operand work ~ row tiles x (record passes x 128 rows + B entries), per density group
+    // the column axis: SM cycles ~ row tiles x record passes x (the 21 slice products of a k-step, reading 4 KB of A
+    // about three times in four and 32 B per column of B from shared memory at 128 B per cycle, and the forming of
+    // A), per density group
     struct AxisPlan {
-        std::vector<std::pair<int, int>> rows;
-        int ncols = 0, nd = 0, colw = 0, G = 0, npad = 0;
+        std::set<std::pair<int, int>> pts;
+        std::vector<int> slots, quads;
+        size_t rows = 0;
+        int ncols = 0, nd = 0, colw = 0, G = 0, npad = 0, nam = 0, nbm = 0;
     } best;
     int best_c = -1;
     double best_cost = 1e300;
@@ -1426,22 +1512,26 @@ int setup_tc(ftcj_plan* P) {
             if (n[c] < 0)
                 for (int x = 0; x < 3; ++x) n[x] = -n[x];
             rs.insert({n[a], n[b]});
+            ap.pts.insert({std::abs(n[a]), std::abs(n[b])});
+            ap.nam = std::max(ap.nam, std::abs(n[a]));
+            ap.nbm = std::max(ap.nbm, std::abs(n[b]));
             ncmax = std::max(ncmax, n[c]);
         }
+        ap.rows = rs.size();
         ap.ncols = ncmax + 1;
         for (ap.nd = P->max_dens; ap.nd >= 1; --ap.nd) {
             tc_columns(ap.nd, ap.ncols, &ap.colw, &ap.G, &ap.npad);
             if (ap.G > 0) break;
         }
         if (ap.nd < 1 || ap.G < 1) continue;
-        ap.rows.assign(rs.begin(), rs.end());
-        const double mt = (double)((ap.rows.size() + kTcM - 1) / kTcM);
+        tc_slots(ap.pts, ap.slots, ap.quads);
+        const double mt = (double)((ap.slots.size() + kTcM - 1) / kTcM);
         const double launches = (double)((P->max_dens + ap.nd - 1) / ap.nd);
         double work = 0.0;
         for (int L = 0; L < kNclass; ++L) {
             const int nb = (L + 1) * (L + 2) / 2;
-            const double passes = (double)((nb + ap.G - 1) / ap.G);
-            work += (double)recs_by_class[L] * (passes * kTcM + 1.5 * nb * ap.nd * ap.ncols);
+            for (int g0 = 0; g0 < nb; g0 += ap.G)
+                work += (double)recs_by_class[L] * (500.0 + 21.0 * (24.0 + 0.25 * mma_cols(std::min(ap.G, nb - g0), ap.colw)));
         }
         const double cost = launches * mt * work;
         if (cost < best_cost) {
@@ -1460,71 +1550,85 @@ int setup_tc(ftcj_plan* P) {
     P->tc_colw = best.colw;
     P->tc_G = best.G;
     P->tc_npad = best.npad;
-    P->tc_rows = (int)best.rows.size();
-    P->tc_mtiles = (P->tc_rows + kTcM - 1) / kTcM;
-    // half-sphere map: row (n_a, n_b), column n_c >= 0
-    std::vector<int> map((size_t)P->tc_rows * P->tc_ncols, INT_MIN);
-    {
-        std::vector<std::pair<int, int>>& rows = best.rows;
-        for (int64_t q = 0; q < ngh; ++q) {
-            int n[3] = {P->gvec[3 * q], P->gvec[3 * q + 1], P->gvec[3 * q + 2]};
-            bool cj = false;
-            if (n[c] < 0) {
-                for (int x = 0; x < 3; ++x) n[x] = -n[x];
-                cj = true;
-            }
-            const auto it = std::lower_bound(rows.begin(), rows.end(), std::make_pair(n[a], n[b]));
-            const size_t rix = (size_t)(it - rows.begin());
-            map[rix * P->tc_ncols + n[c]] = cj ? ~(int)q : (int)q;
+    P->tc_rows = (int)best.rows;
+    P->tc_nslots = (int)best.slots.size();
+    P->tc_mtiles = std::max(1, (P->tc_nslots + kTcM - 1) / kTcM);
+    P->tc_nna = best.nam + 1;
+    P->tc_nnb = best.nbm + 1;
+    std::vector<int> slots = best.slots;
+    slots.resize((size_t)P->tc_mtiles * kTcM, 0);
+    // half-sphere map: (n_a, n_b) and n_c >= 0
+    std::vector<int> map((size_t)(2 * best.nam + 1) * (2 * best.nbm + 1) * P->tc_ncols, INT_MIN);
+    for (int64_t q = 0; q < ngh; ++q) {
+        int n[3] = {P->gvec[3 * q], P->gvec[3 * q + 1], P->gvec[3 * q + 2]};
+        bool cj = false;
+        if (n[c] < 0) {
+            for (int x = 0; x < 3; ++x) n[x] = -n[x];
+            cj = true;
         }
+        const size_t rix = (size_t)(n[a] + best.nam) * (2 * best.nbm + 1) + (size_t)(n[b] + best.nbm);
+        map[rix * P->tc_ncols + n[c]] = cj ? ~(int)q : (int)q;
     }
-    std::vector<int2> rowv(best.rows.size());
-    int nam = 0, nbm = 0;
-    for (size_t i = 0; i < best.rows.size(); ++i) {
-        rowv[i] = make_int2(best.rows[i].first, best.rows[i].second);
-        nam = std::max(nam, std::abs(best.rows[i].first));
-        nbm = std::max(nbm, std::abs(best.rows[i].second));
-    }
-    P->tc_nna = nam + 1;
-    P->tc_nnb = nbm + 1;
-    // factor tables first: the windows below sort records by their width
-    const int tabw = P->tc_nna + P->tc_nnb + P->tc_ncols;
-    P->tc_tabw = tabw;
-    const size_t ntab = (size_t)std::max<int64_t>(P->npairs, 1) * tabw;
-    FTCJ_CUDA(cudaMalloc(&P->d_tc_tab, sizeof(float4) * ntab));
-    P->device_bytes += sizeof(float4) * ntab;
-    FTCJ_CUDA(cudaMalloc(&P->d_tc_cl, sizeof(float) * std::max<int64_t>(P->npairs, 1)));
-    P->device_bytes += sizeof(float) * std::max<int64_t>(P->npairs, 1);
+    // the windows sort records by their width
+    const int tws = (P->tc_nna + P->tc_nnb) | 1;
+    P->tc_tws = tws;
+    const size_t nrec = (size_t)std::max<int64_t>(P->npairs, 1);
     FTCJ_CUDA(cudaMalloc(&P->d_tc_err, sizeof(int)));
     FTCJ_CUDA(cudaMemset(P->d_tc_err, 0, sizeof(int)));
-    std::vector<float> clh((size_t)std::max<int64_t>(P->npairs, 1), 0.f);
+    FTCJ_CUDA(cudaMalloc(&P->d_tc_cl, sizeof(float) * nrec));
+    P->device_bytes += sizeof(float) * nrec;
+    std::vector<float> clh(nrec, 0.f);
     if (P->npairs > 0) {
-        const long long n = P->npairs * (long long)tabw;
-        k_tc_tables<<<(unsigned)((n + 255) / 256), 256>>>(P->d_walk, P->npairs, a, b, c, P->tc_nna, P->tc_nnb,
-                                                        P->tc_ncols, P->M[4 * a], P->M[4 * b], P->M[4 * c],
-                                                        reinterpret_cast<float4*>(P->d_tc_tab), P->d_tc_cl);
+        k_tc_width<<<(unsigned)((P->npairs + 255) / 256), 256>>>(P->d_walk, P->npairs, P->d_tc_cl);
         FTCJ_CUDA(cudaGetLastError());
         FTCJ_CUDA(cudaMemcpy(clh.data(), P->d_tc_cl, sizeof(float) * P->npairs, cudaMemcpyDeviceToHost));
     }
-    // windows: for each class L, its (i, j) blocks in groups of G, and the
-    // class's records sorted by width c = 1/4p in blocks of 512 (the K order of
-    // the matrix product; records of similar width have entries of similar size)
-    std::vector<int> wrec, wpairs;
-    std::vector<int4> winfo;
-    std::vector<int> pos((size_t)std::max<int64_t>(P->npairs, 1), 0);
     // Hermite terms in the K order: [dens][class][term][position], each class's stride a multiple of 16
     P->tc_dp_total = 0;
     for (int L = 0; L < kNclass; ++L) {
         P->tc_dp_base[L] = P->tc_dp_total;
-        P->tc_dp_stride[L] = (recs_by_class[L] + kTcStageK - 1) / kTcStageK * kTcStageK;
+        P->tc_dp_stride[L] = (recs_by_class[L] + 15) / 16 * 16;
         P->tc_dp_total += (long long)nterms(L) * P->tc_dp_stride[L];
     }
+    // K order: the records of a class sorted by width c = 1/4p (records of similar width have entries of similar size)
+    std::vector<std::vector<int>> order(kNclass);
+    std::vector<int> pos(nrec, 0), kpos(nrec, 0);
+    std::vector<float> clk(nrec, 0.f);
     for (int L = 0; L < kNclass; ++L) {
-        std::vector<int> recs;
+        std::vector<int>& recs = order[L];
         for (int64_t r = P->class_start[L]; r < P->class_start[L + 1]; ++r) recs.push_back((int)r);
-        if (recs.empty()) continue;
         std::stable_sort(recs.begin(), recs.end(), [&](int x, int y) { return clh[x] < clh[y]; });
-        for (size_t k = 0; k < recs.size(); ++k) pos[recs[k]] = (int)k;
+        for (size_t k = 0; k < recs.size(); ++k) {
+            pos[recs[k]] = (int)k;
+            kpos[recs[k]] = (int)(P->class_start[L] + (int64_t)k);
+            clk[P->class_start[L] + k] = clh[recs[k]];
+        }
+    }
+    // Records per window: a window costs one drain of tensor memory (~7% of a 1024-record window of 96 columns),
+    // a CTA group holds at least four windows where there are enough records, so that the deal comes out even
+    const int groups_max = std::max(1, P->num_sms / P->tc_mtiles);
+    auto windows = [&](int wlen) {
+        int64_t n = 0;
+        for (int L = 0; L < kNclass; ++L) {
+            const int nb = (L + 1) * (L + 2) / 2;
+            n += (recs_by_class[L] + wlen - 1) / wlen * ((nb + P->tc_G - 1) / P->tc_G);
+        }
+        return n;
+    };
+    P->tc_wlen = kTcWinMax;
+    while (P->tc_wlen > 128 && windows(P->tc_wlen) < 4 * (int64_t)groups_max) P->tc_wlen /= 2;
+    const int wlen = P->tc_wlen;
+    // windows: for each class L, its (i, j) blocks in groups of G, the class's records wlen at a time
+    struct Win {
+        int4 info;
+        int cnt;
+        double cost;
+    };
+    std::vector<Win> wins;
+    std::vector<int> wpairs;
+    for (int L = 0; L < kNclass; ++L) {
+        const std::vector<int>& recs = order[L];
+        if (recs.empty()) continue;
         std::vector<int> blocks;
         for (int i = 0; i <= L; ++i)
             for (int j = 0; i + j <= L; ++j) blocks.push_back(i | (j << 3));
@@ -1532,81 +1636,146 @@ int setup_tc(ftcj_plan* P) {
             const int nb = (int)std::min<size_t>(P->tc_G, blocks.size() - g0);
             const int first = (int)wpairs.size();
             wpairs.insert(wpairs.end(), blocks.begin() + g0, blocks.begin() + g0 + nb);
-            for (size_t r0 = 0; r0 < recs.size(); r0 += kTcWin) {
-                winfo.push_back(make_int4(L, nb, first, (int)r0));
-                for (int k = 0; k < kTcWin; ++k) wrec.push_back(r0 + k < recs.size() ? recs[r0 + k] : -1);
+            for (size_t r0 = 0; r0 < recs.size(); r0 += wlen) {
+                const int cnt = (int)std::min<size_t>(wlen, recs.size() - r0);
+                const double nst = (double)((cnt + kTcStageK - 1) / kTcStageK);
+                wins.push_back({make_int4(L, nb, first, (int)r0), cnt,
+                                nst * (500.0 + 21.0 * (24.0 + 0.25 * mma_cols(nb, P->tc_colw))) + 70.0 * nb * P->tc_colw});
             }
         }
     }
-    if (winfo.empty()) {  // no records: one empty window keeps the launch shape valid
-        winfo.push_back(make_int4(0, 0, 0, 0));
-        wrec.assign(kTcWin, -1);
+    // Passes: the B tiles of a pass's windows fill one workspace, bounded so that a large system reuses it
+    // instead of growing it; each pass deals its windows to CTA groups, one CTA per SM over all (group, row
+    // tile) pairs, so that the grid is a single wave (a partial second wave would double the pass)
+    const int nwin = (int)wins.size();
+    P->tc_nwin = nwin;
+    std::vector<int4> winfo((size_t)std::max(1, nwin), make_int4(0, 0, 0, 0));
+    std::vector<int> wcnt((size_t)std::max(1, nwin), 0);
+    std::vector<long long> boff((size_t)std::max(1, nwin), 0);
+    P->tc_passes.clear();
+    P->tc_out_rows = 0;
+    long long bmax = 1;
+    std::vector<int> sched;
+    for (int w0 = 0; w0 < nwin;) {
+        long long off = 0;
+        int w1 = w0;
+        while (w1 < nwin) {
+            const Win& w = wins[w1];
+            const long long n = (long long)((w.cnt + kTcStageK - 1) / kTcStageK) * kTcS * mma_cols(w.info.y, P->tc_colw) * 2;
+            if (w1 > w0 && (off + n) * 16 > kTcBWorkMax) break;
+            winfo[w1] = w.info;
+            wcnt[w1] = w.cnt;
+            boff[w1] = off;
+            off += n;
+            ++w1;
+        }
+        bmax = std::max(bmax, off);
+        const int ng = std::min(groups_max, w1 - w0);
+        std::vector<double> cost;
+        for (int w = w0; w < w1; ++w) cost.push_back(wins[w].cost);
+        std::vector<int> s = deal(cost, ng);
+        for (size_t k = (size_t)ng + 1; k < s.size(); ++k) s[k] += w0;
+        P->tc_passes.push_back({w0, w1 - w0, ng, P->tc_out_rows, (int)sched.size()});
+        sched.insert(sched.end(), s.begin(), s.end());
+        P->tc_out_rows += ng;
+        w0 = w1;
     }
-    P->tc_nwin = (int)winfo.size();
-    // MMA work of one pass: per window and row tile, 32 stages x 2 k-steps x 21 slice products of
-    // M = 128 rows, N = the window's columns, K = 16, for every density group
+    P->tc_out_rows = std::max(1, P->tc_out_rows);
+    // MMA work of one pass: per window and row tile, its stages x 21 slice products of M = 128 rows,
+    // N = the window's columns, K = 16, for every density group
     P->tc_mma_flops = 0;
     for (int d0 = 0; d0 < P->max_dens; d0 += P->tc_nd) {
-        const int ndg = std::min(P->tc_nd, P->max_dens - d0);
-        const int colw = round_up(2 * ndg * P->tc_ncols, 8), np = round_up(P->tc_G * colw, 16);
-        for (const int4& wi : winfo) {
-            const long long nw = std::min(np, round_up(std::max(1, wi.y) * colw, 16));
-            P->tc_mma_flops += (long long)P->tc_mtiles * kTcStagesPerWin * 2 * 21 * 2LL * kTcM * nw * 16;
-        }
+        const int colw = round_up(2 * std::min(P->tc_nd, P->max_dens - d0) * P->tc_ncols, 8);
+        for (const Win& w : wins)
+            P->tc_mma_flops += (long long)P->tc_mtiles * ((w.cnt + kTcStageK - 1) / kTcStageK) * 21 * 2LL * kTcM *
+                               mma_cols(w.info.y, colw) * 16;
     }
-    // window groups: one CTA per SM over all (group, row tile) pairs, so the
-    // grid is a single wave of equal CTAs (a partial second wave would double the pass)
-    const int want = std::max(1, std::min(P->tc_nwin, P->num_sms / std::max(1, P->tc_mtiles)));
-    P->tc_wpg = std::max(1, (P->tc_nwin + want - 1) / want);
-    P->tc_ngroups = (P->tc_nwin + P->tc_wpg - 1) / P->tc_wpg;
-    // table slots in flight: as many as shared memory holds, 2 to 4
+    // stage buffers and table slots: four buffers where at least three slots fit beside them, else fewer
     int dev = 0, optin = 0;
     FTCJ_CUDA(cudaGetDevice(&dev));
     FTCJ_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     P->tc_tslots = 0;
-    for (int nts = kTcTabSlotsMax; nts >= 2 && !P->tc_tslots; --nts)
-        if (tc_smem_bytes(P->tc_npad, tabw, P->tc_G, P->tc_nd, nts) <= (size_t)optin) P->tc_tslots = nts;
+    for (int nbuf = kTcNbufMax; nbuf >= 2 && !P->tc_tslots; --nbuf)
+        for (int nts = kTcTabSlotsMax; nts >= (nbuf > 2 ? 3 : 1) && !P->tc_tslots; --nts)
+            if (tc_smem_bytes(P->tc_npad, tws, nbuf, nts) <= (size_t)optin) {
+                P->tc_nbuf = nbuf;
+                P->tc_tslots = nts;
+            }
     if (!P->tc_tslots)
         return fail(FTCJ_EUNSUPPORTED, "the G sphere is too long for the tensor-core kernel's shared-memory tables");
     int rc;
-    int2* rows_dev = nullptr;
-    if ((rc = tc_upload(P, &rows_dev, rowv))) return rc;
-    P->d_tc_rows = rows_dev;
+    if ((rc = tc_upload(P, &P->d_tc_slots, slots))) return rc;
+    if ((rc = tc_upload(P, &P->d_tc_quads, best.quads))) return rc;
     if ((rc = tc_upload(P, &P->d_tc_map, map))) return rc;
-    if ((rc = tc_upload(P, &P->d_tc_kappa, wrec))) return rc;
     if ((rc = tc_upload(P, &P->d_tc_wpairs, wpairs))) return rc;
     if ((rc = tc_upload(P, &P->d_tc_pos, pos))) return rc;
+    if ((rc = tc_upload(P, &P->d_tc_kpos, kpos))) return rc;
+    FTCJ_CUDA(cudaMemcpy(P->d_tc_cl, clk.data(), sizeof(float) * nrec, cudaMemcpyHostToDevice));
+    FTCJ_CUDA(cudaMalloc(&P->d_tc_tab, sizeof(float4) * nrec * tws));
+    FTCJ_CUDA(cudaMalloc(&P->d_tc_tabk, sizeof(float4) * nrec * tws));
+    FTCJ_CUDA(cudaMalloc(&P->d_tc_tabz, sizeof(float4) * nrec * P->tc_ncols));
+    P->device_bytes += sizeof(float4) * nrec * (2 * (size_t)tws + P->tc_ncols);
+    // the odd stride's spare entry is copied along but never read
+    FTCJ_CUDA(cudaMemset(P->d_tc_tab, 0, sizeof(float4) * nrec * tws));
+    FTCJ_CUDA(cudaMemset(P->d_tc_tabk, 0, sizeof(float4) * nrec * tws));
+    if (P->npairs > 0) {
+        const long long n = P->npairs * (long long)(P->tc_nna + P->tc_nnb + P->tc_ncols);
+        k_tc_tables<<<(unsigned)((n + 255) / 256), 256>>>(
+            P->d_walk, P->npairs, P->d_tc_kpos, a, b, c, P->tc_nna, P->tc_nnb, P->tc_ncols, tws, P->M[4 * a],
+            P->M[4 * b], P->M[4 * c], reinterpret_cast<float4*>(P->d_tc_tab), reinterpret_cast<float4*>(P->d_tc_tabk),
+            reinterpret_cast<float4*>(P->d_tc_tabz));
+        FTCJ_CUDA(cudaGetLastError());
+    }
+    if ((rc = tc_upload(P, &P->d_tc_wcnt, wcnt))) return rc;
+    if ((rc = tc_upload(P, &P->d_tc_boff, boff))) return rc;
+    if ((rc = tc_upload(P, &P->d_tc_sched, sched))) return rc;
     int4* winfo_dev = nullptr;
     if ((rc = tc_upload(P, &winfo_dev, winfo))) return rc;
     P->d_tc_winfo = winfo_dev;
-    if ((rc = tc_upload(P, &P->d_tc_ebw, std::vector<int>((size_t)P->tc_nwin * kTcEbMax, -100)))) return rc;
-    if ((rc = tc_upload(P, &P->d_tc_clw, std::vector<float>((size_t)P->tc_nwin, 0.f)))) return rc;
-    if ((rc = allow_dynamic_smem((const void*)k_tc_rho, tc_smem_bytes(P->tc_npad, tabw, P->tc_G, P->tc_nd, P->tc_tslots))))
-        return rc;
+    if ((rc = tc_upload(P, &P->d_tc_clw, std::vector<float>((size_t)std::max(1, nwin), 0.f)))) return rc;
+    if (cudaMalloc(&P->d_tc_b, (size_t)bmax * 16) != cudaSuccess) {
+        cudaGetLastError();
+        P->d_tc_b = nullptr;
+        return fail(FTCJ_ENOMEM, "cudaMalloc of the tensor-core operand tiles failed");
+    }
+    P->device_bytes += (size_t)bmax * 16;
+    // columns between a window's blocks and the MMA's multiple of 16 are never written nor read back: finite once
+    FTCJ_CUDA(cudaMemset(P->d_tc_b, 0, (size_t)bmax * 16));
+    // calls with fewer densities run the instantiation of their own block width
+    for (int nd = 1; nd <= P->tc_nd; ++nd)
+        if ((rc = allow_dynamic_smem(tc_rho_kernel(round_up(2 * nd * P->tc_ncols, 8)),
+                                     tc_smem_bytes(P->tc_npad, tws, P->tc_nbuf, P->tc_tslots))))
+            return rc;
     return setup_tc_j(P);
 }
 
 int launch_tc_rho(ftcj_plan* P, int ndens, cudaStream_t s) {
     if (P->ng_half == 0 || P->npairs == 0) {
-        FTCJ_CUDA(cudaMemsetAsync(P->d_rho_part, 0, sizeof(double2) * (size_t)ndens * P->tc_ngroups * P->ng_half, s));
+        FTCJ_CUDA(cudaMemsetAsync(P->d_rho_part, 0, sizeof(double2) * (size_t)ndens * P->tc_out_rows * P->ng_half, s));
         return FTCJ_OK;
     }
     TcArgs g;
-    g.rows = reinterpret_cast<const int2*>(P->d_tc_rows);
+    g.slots = P->d_tc_slots;
     g.map = P->d_tc_map;
-    g.wrec = P->d_tc_kappa;
     g.winfo = reinterpret_cast<const int4*>(P->d_tc_winfo);
+    g.wcnt = P->d_tc_wcnt;
+    g.boff = P->d_tc_boff;
     g.wpairs = P->d_tc_wpairs;
-    g.tab = reinterpret_cast<const float4*>(P->d_tc_tab);
-    g.cl = P->d_tc_cl;
+    g.tabk = reinterpret_cast<const float4*>(P->d_tc_tabk);
+    g.tabz = reinterpret_cast<const float4*>(P->d_tc_tabz);
+    g.clk = P->d_tc_cl;
+    for (int cc = 0; cc < kNclass; ++cc) g.kbase[cc] = P->class_start[cc];
     g.Dp = reinterpret_cast<const float2*>(P->d_Dp);
     g.dp_total = P->tc_dp_total;
     for (int cc = 0; cc < kNclass; ++cc) {
         g.dp_base[cc] = P->tc_dp_base[cc];
         g.dp_stride[cc] = P->tc_dp_stride[cc];
     }
+    g.bs = reinterpret_cast<uint4*>(P->d_tc_b);
+    g.clw = P->d_tc_clw;
     g.out = reinterpret_cast<double2*>(P->d_rho_part);
     g.ng_half = P->ng_half;
+    g.out_rows = P->tc_out_rows;
     g.err = P->d_tc_err;
     g.Maa = (float)P->M[4 * P->tc_axis[0]];
     g.Mbb = (float)P->M[4 * P->tc_axis[1]];
@@ -1614,48 +1783,50 @@ int launch_tc_rho(ftcj_plan* P, int ndens, cudaStream_t s) {
     g.ax = P->tc_axis[0];
     g.bx = P->tc_axis[1];
     g.cx = P->tc_axis[2];
-    g.tabw = P->tc_tabw;
+    g.nam = P->tc_nna - 1;
+    g.nbm = P->tc_nnb - 1;
+    g.tws = P->tc_tws;
     g.offY = P->tc_nna;
-    g.offZ = P->tc_nna + P->tc_nnb;
     g.ncols = P->tc_ncols;
-    g.G = P->tc_G;
-    g.nwin = P->tc_nwin;
-    g.win_per_group = P->tc_wpg;
-    g.ngroups = P->tc_ngroups;
-    g.nrows = P->tc_rows;
+    g.nslots = P->tc_nslots;
     g.spin = tc_spin(P);
-    g.ebw = P->d_tc_ebw;
-    g.clw = P->d_tc_clw;
-    const size_t smem = tc_smem_bytes(P->tc_npad, P->tc_tabw, P->tc_G, P->tc_nd, P->tc_tslots);
+    const size_t smem = tc_smem_bytes(P->tc_npad, g.tws, P->tc_nbuf, P->tc_tslots);
     for (int d0 = 0; d0 < ndens; d0 += P->tc_nd) {
         g.d0 = d0;
         g.nd = std::min(P->tc_nd, ndens - d0);
-        int colw, Gx, npad;
-        tc_columns(g.nd, g.ncols, &colw, &Gx, &npad);
-        // the plan's block count G is kept; a smaller last density group only narrows each block
-        g.colw = colw;
-        g.npad = round_up(P->tc_G * colw, 16);
-        k_tc_rho_bounds<<<(unsigned)P->tc_nwin, 256, 0, s>>>(g);
-        FTCJ_CUDA(cudaGetLastError());
-        k_tc_rho<<<dim3((unsigned)P->tc_ngroups, (unsigned)P->tc_mtiles), kTcThreadsAll, smem, s>>>(g, P->tc_tslots);
-        FTCJ_CUDA(cudaGetLastError());
+        // the plan's block count G is kept; a smaller density group only narrows each block
+        g.colw = round_up(2 * g.nd * g.ncols, 8);
+        g.npad = mma_cols(P->tc_G, g.colw);
+        for (const TcPass& ps : P->tc_passes) {
+            g.w0 = ps.w0;
+            g.out_row0 = ps.out_row0;
+            g.sched = P->d_tc_sched + ps.sched;
+            k_tc_rho_b<<<(unsigned)ps.nwin, kTcBThreads, 0, s>>>(g);
+            FTCJ_CUDA(cudaGetLastError());
+            const dim3 grid((unsigned)ps.ngroups, (unsigned)P->tc_mtiles);
+            int nbuf = P->tc_nbuf, nts = P->tc_tslots;
+            void* args[] = {&g, &nbuf, &nts};
+            FTCJ_CUDA(cudaLaunchKernel(tc_rho_kernel(g.colw), grid, dim3(kTcThreadsAll), args, smem, s));
+        }
     }
     return FTCJ_OK;
 }
 
-int tc_rho_launches(const ftcj_plan* P, int nd) { return 2 * ((nd + P->tc_nd - 1) / P->tc_nd); }
+int tc_rho_launches(const ftcj_plan* P, int nd) {
+    return 2 * (int)std::max<size_t>(1, P->tc_passes.size()) * ((nd + P->tc_nd - 1) / P->tc_nd);
+}
 
 // Plan-time set-up of the tensor-core back-contraction: densities per
-// launch, (i, j) blocks per work item, the items and the V_ij tile buffer.
-// tc_j stays false, and the split walk runs the back-contraction, where the
-// rows exceed one exact accumulation, one density's columns exceed the MMA
-// width, or the factor tables exceed shared memory.
+// launch, (i, j) blocks per group, the work units, their deal to the CTAs and
+// the V_ij tile buffer.  tc_j stays false, and the split walk runs the
+// back-contraction, where one density's columns exceed the MMA width or the
+// factor tables exceed shared memory.
 int setup_tc_j(ftcj_plan* P) {
     P->tc_j = false;
     const int gw = round_up(2 * P->tc_ncols, 8);
     int64_t tiles[kNclass];
     for (int L = 0; L < kNclass; ++L) tiles[L] = (P->class_start[L + 1] - P->class_start[L] + kTcM - 1) / kTcM;
-    // densities per launch: the fewest A^T formations (items x launches)
+    // densities per launch: the fewest A^T formations (tiles x block groups x launches)
     int nd_best = 0, G_best = 0;
     double cost_best = 1e300;
     for (int nd = 1; nd <= P->max_dens; ++nd) {
@@ -1675,32 +1846,67 @@ int setup_tc_j(ftcj_plan* P) {
         }
     }
     if (!nd_best) return FTCJ_OK;
-    const int npad = round_up(G_best * nd_best * gw, 16);
+    const int npad = mma_cols(G_best, nd_best * gw);
     int dev = 0, optin = 0;
     FTCJ_CUDA(cudaGetDevice(&dev));
     FTCJ_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    if (tc_j_smem_bytes(npad, P->tc_tabw) > (size_t)optin) return FTCJ_OK;
-    // row parts of at most 64 stages, as even as the stage count allows
-    const int nstage = (P->tc_rows + kTcJStageM - 1) / kTcJStageM;
-    const int spp = (nstage + (nstage + kTcJPartStages - 1) / kTcJPartStages - 1) /
-                    ((nstage + kTcJPartStages - 1) / kTcJPartStages);
-    const int nparts = (nstage + spp - 1) / spp;  // every part holds at least one stage
-    // work items, the costliest classes first: (class, block group, 128 records, row part)
-    std::vector<int4> items;
+    // as many stage buffers as fit beside the tables
+    const int tws = P->tc_tws;
+    int nbuf = kTcNbufMax;
+    while (nbuf > 2 && tc_j_smem_bytes(npad, tws, nbuf) > (size_t)optin) --nbuf;
+    if (tc_j_smem_bytes(npad, tws, nbuf) > (size_t)optin) return FTCJ_OK;
+    P->tc_jnbuf = nbuf;
+    // slot parts of at most 64 stages, as even as the stage count allows
+    const int nstage = (P->tc_nslots + kTcJStageM - 1) / kTcJStageM;
+    const int nsplit = std::max(1, (nstage + kTcJPartStages - 1) / kTcJPartStages);
+    const int spp = std::max(1, (nstage + nsplit - 1) / nsplit);
+    const int nparts = std::max(1, (nstage + spp - 1) / spp);  // every part holds at least one stage
+    std::vector<int2> groups;
     std::vector<int> ipairs;
+    std::vector<int4> units;
+    std::vector<double> cost;
+    std::vector<int> vplace((size_t)kTcPairsAll * kNclass, -1);
+    std::vector<long long> voff;
+    long long nvs = 0;
+    P->tc_j_mma_flops = 0;
+    // a unit holds all block groups of its class, or one group each where there are too few units to fill the GPU
+    int64_t whole = 0;
+    for (int L = 0; L < kNclass; ++L) whole += tiles[L] * nparts;
+    const bool split_groups = whole < 4 * (int64_t)P->num_sms;
     for (int L = kNclass - 1; L >= 0; --L) {
         if (!tiles[L]) continue;
         std::vector<int> blocks;
         for (int i = 0; i <= L; ++i)
             for (int j = 0; i + j <= L; ++j) blocks.push_back(i | (j << 3));
+        const int first = (int)groups.size();
         for (size_t g0 = 0; g0 < blocks.size(); g0 += G_best) {
             const int nb = (int)std::min<size_t>(G_best, blocks.size() - g0);
-            const int first = (int)ipairs.size();
+            for (int k = 0; k < nb; ++k)
+                vplace[(size_t)pair_index(blocks[g0 + k] & 7, blocks[g0 + k] >> 3) * kNclass + L] =
+                    (int)groups.size() << 8 | k;
+            voff.push_back(nvs);
+            nvs += (long long)nstage * kTcJS * mma_cols(nb, nd_best * gw) * 16;
+            groups.push_back(make_int2((int)ipairs.size(), nb));
             ipairs.insert(ipairs.end(), blocks.begin() + g0, blocks.begin() + g0 + nb);
-            for (int64_t t = 0; t < tiles[L]; ++t)
-                for (int h = 0; h < nparts; ++h)
-                    items.push_back(make_int4(L | (h << 8), nb, first, (int)(P->class_start[L] + t * kTcM)));
         }
+        const int ngr = (int)groups.size() - first;
+        for (int64_t t = 0; t < tiles[L]; ++t)
+            for (int h = 0; h < nparts; ++h) {
+                const int nst = std::min(spp, nstage - h * spp);
+                for (int g0 = 0; g0 < ngr; g0 += split_groups ? 1 : ngr) {
+                    const int n = split_groups ? 1 : ngr;
+                    double cc = 2000.0;
+                    for (int k = 0; k < n; ++k) {
+                        const int nb = groups[first + g0 + k].y;
+                        cc += nst * (28.0 * (25.0 + 0.25 * mma_cols(nb, nd_best * gw)) + 500.0) + 110.0 * nb * nd_best * gw;
+                        for (int d0 = 0; d0 < P->max_dens; d0 += nd_best)
+                            P->tc_j_mma_flops += (long long)nst * kTcJProducts * 2LL * kTcM *
+                                                 mma_cols(nb, std::min(nd_best, P->max_dens - d0) * gw) * 16;
+                    }
+                    units.push_back(make_int4(L | (h << 8), first + g0, n, (int)(P->class_start[L] + t * kTcM)));
+                    cost.push_back(cc);
+                }
+            }
     }
     P->tc_jnd = nd_best;
     P->tc_jgw = gw;
@@ -1709,31 +1915,27 @@ int setup_tc_j(ftcj_plan* P) {
     P->tc_jnstage = nstage;
     P->tc_jparts = nparts;
     P->tc_jspp = spp;
-    P->tc_jnitems = (int)items.size();
-    // MMA work of one back-contraction over max_dens densities: per item and stage 21 slice
-    // products of M = 128 records, N = the item's columns, K = 16
-    P->tc_j_mma_flops = 0;
-    for (int d0 = 0; d0 < P->max_dens; d0 += nd_best) {
-        const int colw = std::min(nd_best, P->max_dens - d0) * gw, np = round_up(G_best * colw, 16);
-        for (const int4& it : items) {
-            const int part = it.x >> 8, nst = std::min(spp, nstage - part * spp);
-            P->tc_j_mma_flops +=
-                (long long)nst * kTcJProducts * 2LL * kTcM * std::min(np, round_up(it.y * colw, 16)) * 16;
-        }
-    }
+    P->tc_jgrid = std::max(1, std::min(P->num_sms, (int)units.size()));
+    const std::vector<int> sched = deal(cost, P->tc_jgrid);
     int rc;
-    int4* items_dev = nullptr;
-    if ((rc = tc_upload(P, &items_dev, items))) return rc;
-    P->d_tc_jitems = items_dev;
+    int4* units_dev = nullptr;
+    if ((rc = tc_upload(P, &units_dev, units))) return rc;
+    P->d_tc_jitems = units_dev;
+    int2* groups_dev = nullptr;
+    if ((rc = tc_upload(P, &groups_dev, groups))) return rc;
+    P->d_tc_jgroups = groups_dev;
     if ((rc = tc_upload(P, &P->d_tc_jpairs, ipairs))) return rc;
-    const size_t nvs = (size_t)kTcPairsAll * P->tc_jnstage * kTcJS * (size_t)nd_best * gw * 16;
-    FTCJ_CUDA(cudaMalloc(&P->d_tc_vs, sizeof(__nv_bfloat16) * nvs));
-    P->device_bytes += sizeof(__nv_bfloat16) * nvs;
-    FTCJ_CUDA(cudaMemset(P->d_tc_vs, 0, sizeof(__nv_bfloat16) * nvs));
+    if ((rc = tc_upload(P, &P->d_tc_jsched, sched))) return rc;
+    if ((rc = tc_upload(P, &P->d_tc_voff, voff))) return rc;
+    if ((rc = tc_upload(P, &P->d_tc_vplace, vplace))) return rc;
+    nvs = std::max(nvs, 1LL);
+    FTCJ_CUDA(cudaMalloc(&P->d_tc_vs, sizeof(__nv_bfloat16) * (size_t)nvs));
+    P->device_bytes += sizeof(__nv_bfloat16) * (size_t)nvs;
+    FTCJ_CUDA(cudaMemset(P->d_tc_vs, 0, sizeof(__nv_bfloat16) * (size_t)nvs));
     const size_t nev = (size_t)kTcPairsAll * nd_best * P->tc_ncols;
     FTCJ_CUDA(cudaMalloc(&P->d_tc_ev, sizeof(int) * nev));
     P->device_bytes += sizeof(int) * nev;
-    if ((rc = allow_dynamic_smem((const void*)k_tc_j, tc_j_smem_bytes(npad, P->tc_tabw)))) return rc;
+    if ((rc = allow_dynamic_smem((const void*)k_tc_j, tc_j_smem_bytes(npad, tws, nbuf)))) return rc;
     P->tc_j = true;
     return FTCJ_OK;
 }
@@ -1744,12 +1946,19 @@ int launch_tc_j(ftcj_plan* P, int ndens, const double* W, cudaStream_t s) {
         return FTCJ_OK;
     }
     TcJArgs g;
-    g.rows = reinterpret_cast<const int2*>(P->d_tc_rows);
+    g.slots = P->d_tc_slots;
+    g.quads = P->d_tc_quads;
     g.map = P->d_tc_map;
     g.W = reinterpret_cast<const double2*>(W);
-    g.items = reinterpret_cast<const int4*>(P->d_tc_jitems);
+    g.sched = P->d_tc_jsched;
+    g.units = reinterpret_cast<const int4*>(P->d_tc_jitems);
+    g.groups = reinterpret_cast<const int2*>(P->d_tc_jgroups);
     g.ipairs = P->d_tc_jpairs;
+    g.voff = P->d_tc_voff;
+    g.vplace = P->d_tc_vplace;
     g.tab = reinterpret_cast<const float4*>(P->d_tc_tab);
+    g.tabz = reinterpret_cast<const float4*>(P->d_tc_tabz);
+    g.kpos = P->d_tc_kpos;
     g.vs = reinterpret_cast<__nv_bfloat16*>(P->d_tc_vs);
     g.ev = P->d_tc_ev;
     g.Jp = P->d_Jp;
@@ -1761,31 +1970,30 @@ int launch_tc_j(ftcj_plan* P, int ndens, const double* W, cudaStream_t s) {
     g.ax = P->tc_axis[0];
     g.bx = P->tc_axis[1];
     g.cx = P->tc_axis[2];
-    g.tabw = P->tc_tabw;
+    g.nam = P->tc_nna - 1;
+    g.nbm = P->tc_nnb - 1;
+    g.tws = P->tc_tws;
     g.offY = P->tc_nna;
-    g.offZ = P->tc_nna + P->tc_nnb;
     g.ncols = P->tc_ncols;
     g.gw = P->tc_jgw;
-    g.nrows = P->tc_rows;
+    g.nslots = P->tc_nslots;
     g.nstage = P->tc_jnstage;
-    g.nitems = P->tc_jnitems;
     g.nparts = P->tc_jparts;
     g.spin = tc_spin(P);
     g.spp = P->tc_jspp;
-    const size_t smem = tc_j_smem_bytes(P->tc_jnpad, P->tc_tabw);
-    const int grid = std::max(1, std::min(P->num_sms, P->tc_jnitems));
+    const size_t smem = tc_j_smem_bytes(P->tc_jnpad, P->tc_tws, P->tc_jnbuf);
     for (int d0 = 0; d0 < ndens; d0 += P->tc_jnd) {
         g.d0 = d0;
         g.nd = std::min(P->tc_jnd, ndens - d0);
         // the plan's block count is kept; a smaller last density group only narrows each block
         g.colw = g.nd * g.gw;
-        g.npad = round_up(P->tc_jG * g.colw, 16);
+        g.npad = mma_cols(P->tc_jG, g.colw);
         k_tc_vbound<<<(unsigned)(kTcPairsAll * g.nd * g.ncols), 256, 0, s>>>(g);
         FTCJ_CUDA(cudaGetLastError());
-        const long long nv = (long long)kTcPairsAll * g.nstage * kTcJStageM * g.nd * g.ncols;
+        const long long nv = (long long)kTcPairsAll * g.nstage * (kTcJStageM / 2) * g.nd * g.ncols;
         k_tc_vslice<<<(unsigned)((nv + 255) / 256), 256, 0, s>>>(g);
         FTCJ_CUDA(cudaGetLastError());
-        k_tc_j<<<(unsigned)grid, kTcThreadsAll, smem, s>>>(g);
+        k_tc_j<<<(unsigned)P->tc_jgrid, kTcThreadsAll, smem, s>>>(g, P->tc_jnbuf);
         FTCJ_CUDA(cudaGetLastError());
     }
     return FTCJ_OK;
