@@ -252,6 +252,7 @@ def measure_form(ctx, w, wname, form):
     plan = ftcj.Plan.from_workload(w, precision=prec, pair_gcut_eps=eps, contraction=contraction,
                                    shard_count=world if sharded else 0, shard_index=rank if sharded else 0)
     info = plan.info
+    contraction = info["contraction"]  # the FP64 form runs it too where it applies
     Dk = ctx["Dk"]
     nd = w.ndens
     Jk = torch.empty_like(Dk)
@@ -352,11 +353,13 @@ def measure_form(ctx, w, wname, form):
         tc = {}
         for key, kern, mma, t_ms, note in (
                 ("tc_rho", "k_tc_rho", float(info["tc_mma_flops"]) * reps, rho_pass_ms,
-                 "21 bf16 slice products per product exact to 2^-41 (6 slices a side), real form of the "
-                 "complex product (4 real per complex multiply-add)"),
+                 ("36 bf16 slice products per product (8 slices a side)" if pipe == "fp64" else
+                  "21 bf16 slice products per product exact to 2^-41 (6 slices a side)") +
+                 ", real products of the sign-symmetric rows (2 real per complex multiply-add)"),
                 ("tc_j", "k_tc_j", float(info["tc_j_mma_flops"]) * reps, j_pass_ms,
-                 "28 bf16 slice products per product exact to 2^-45 (7 slices a side), real form of the "
-                 "complex product")):
+                 ("36 bf16 slice products per product (8 slices a side)" if pipe == "fp64" else
+                  "28 bf16 slice products per product exact to 2^-45 (7 slices a side)") +
+                 ", real products of the sign-symmetric rows")):
             if mma <= 0:
                 continue
             tc[kern] = {"bound": "tensor", "kernel": kern, "pass_ms": t_ms,

@@ -255,8 +255,10 @@ struct ftcj_plan {
     void* d_tc_tab = nullptr;    // float4 [npairs][tws], record order
     void* d_tc_tabk = nullptr;   // the same in the K order of all classes
     void* d_tc_tabz = nullptr;   // float4 [npairs][ncols], K order
+    void* d_tc_tabz3 = nullptr;  // the same in triple-float (FP64 form)
     float* d_tc_cl = nullptr;    // [npairs] widths, K order
     int* d_tc_kpos = nullptr;    // [npairs] position of each record in that order
+    int* d_tc_korder = nullptr;  // [npairs] class-local record of each position (FP64 form)
     int* d_tc_err = nullptr;     // device error word of the bounded waits
     int* d_tc_pos = nullptr;     // [npairs]: position of each record in its class's K order
     float* d_tc_clw = nullptr;   // [nwin]: the windows' smallest widths
@@ -265,7 +267,8 @@ struct ftcj_plan {
     bool tc_j = false;
     int tc_jnd = 0, tc_jgw = 0, tc_jG = 0, tc_jnpad = 0;  // densities per launch, columns per density, blocks per group, MMA N
     int tc_jnstage = 0, tc_jgrid = 0, tc_jnbuf = 0;         // 16-slot stages, CTAs, stage buffers
-    int tc_jparts = 0, tc_jspp = 0;                         // slot parts (one exact accumulation each), stages per part
+    int tc_jparts = 0, tc_jspp = 0;                         // partial arrays of J' (slot parts x column splits), stages per part
+    int tc_jsub = 1;                                        // column splits of the epilogue
     int64_t tc_j_mma_flops = 0;                             // bf16 MMA flops of one pass over max_dens densities
     void* d_tc_jitems = nullptr;   // int4 [units]: class | part << 8, first block group, block groups, first record
     void* d_tc_jgroups = nullptr;  // int2 [groups]: first block, blocks
@@ -357,6 +360,7 @@ bool split_grad_walk_exact(const ftcj_plan* P);
 
 // --- tensor-core separable contraction (tc.cu) ---
 int setup_tc(ftcj_plan* P);
+void release_tc(ftcj_plan* P);  // back to a plan without the tensor-core form
 int launch_tc_rho(ftcj_plan* P, int ndens, cudaStream_t s);
 int tc_rho_launches(const ftcj_plan* P, int nd);
 int launch_tc_j(ftcj_plan* P, int ndens, const double* W, cudaStream_t s);

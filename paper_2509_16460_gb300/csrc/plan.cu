@@ -301,13 +301,10 @@ void free_device(ftcj_plan* P) {
                     P->d_gvec, P->d_vg, P->d_tw, P->d_Tmat, P->d_D0n, P->d_J0n, P->d_cbuf0, P->d_cbuf1,
                     P->d_Dp, P->d_Jp, P->d_rho_part, P->d_rho, P->d_W, P->d_Epart, P->d_Dk_stage,
                     P->d_Jk_stage, P->d_EJ_stage, P->d_check, P->d_split_init, P->d_split_const, P->d_Jg,
-                    P->d_maps, P->d_map_off, P->d_sched, P->d_rec_gcut, P->d_tc_slots, P->d_tc_quads,
-                    P->d_tc_map, P->d_tc_tab, P->d_tc_tabk, P->d_tc_tabz, P->d_tc_kpos, P->d_tc_cl, P->d_tc_err, P->d_tc_wpairs,
-                    P->d_tc_winfo, P->d_tc_wcnt, P->d_tc_boff, P->d_tc_sched, P->d_tc_b, P->d_tc_pos,
-                    P->d_tc_jitems, P->d_tc_jgroups, P->d_tc_jpairs, P->d_tc_jsched, P->d_tc_vs, P->d_tc_ev,
-                    P->d_tc_clw, P->d_tc_voff, P->d_tc_vplace};
+                    P->d_maps, P->d_map_off, P->d_sched, P->d_rec_gcut};
     for (void* p : ptrs)
         if (p) cudaFree(p);
+    release_tc(P);
     free_gpw(P);
     if (P->dd) {
         free_device(P->dd);
@@ -548,6 +545,24 @@ int create(const ftcj_cell* cell, const ftcj_basis* basis, const int kmesh[3], c
     if ((rc = build_rho_schedule(P))) return rc;
     if (P->tc && !P->ortho) return fail(FTCJ_EUNSUPPORTED, "the tensor-core contraction needs an orthorhombic cell");
     if (P->tc && (rc = setup_tc(P))) return rc;
+    // The FP64 form runs the same separable contraction where the cell is orthorhombic, with operands cut finely
+    // enough for its errors to stay below FP64 accumulation's (tc.cu): GB300 has 64 FP32 lanes and far more tensor
+    // throughput for each FP64 lane that the walks would use (both passes: slab of 940 AOs, walks 36.7 ms, contraction
+    // 1.55 ms; diamond cell 2.02 and 0.30 ms; 18 AOs 0.33 and 0.08 ms).
+    // A caller's own walk shape, |n_i| above 63 (powers of n exact in FP32 no longer), spheres wider than the MMA
+    // and plans short of memory keep the walks.
+    if (P->precision == FTCJ_PREC_FP64 && P->ortho && !P->d_rec_gcut && prm->chunk_points <= 0 && prm->rho_blocks <= 0 &&
+        P->n_abs_max <= kSplitNmax && P->npairs > 0 && P->ng_half > 0) {
+        const size_t bytes = P->device_bytes;
+        P->tc = true;
+        rc = setup_tc(P);
+        if (rc == FTCJ_EUNSUPPORTED || rc == FTCJ_ENOMEM) {
+            release_tc(P);
+            P->device_bytes = bytes;
+        } else if (rc) {
+            return rc;
+        }
+    }
     P->rho_rows = P->tc ? P->tc_out_rows : P->npb;
 
     size_t nn = (size_t)P->nao * P->nao;

@@ -82,6 +82,7 @@
 #include <cmath>
 #include <queue>
 #include <set>
+#include <type_traits>
 #include <vector>
 
 #include "df.cuh"
@@ -92,10 +93,9 @@ namespace {
 
 constexpr int kTcM = 128;                      // rows per tile (MMA M)
 constexpr int kTcStageK = 16;                  // records per stage: one MMA k-step
-constexpr int kTcWinMax = 1024;                // records per exact-accumulation window at most
-constexpr int kTcNmax = 96;                    // MMA N at most: five level accumulators in the 512 columns
-constexpr int kTcS = 6;                        // slices per operand
-constexpr int kTcAcc = 5;                      // accumulators: levels 0-3 exact, levels 4, 5 rounded
+constexpr int kTcWinMax = 1024;                // records per exact-accumulation window at most (FP64 form: half)
+constexpr int kTcNmax = 96;                    // MMA N at most in the split form: five accumulators in 512 columns
+constexpr int kTcNmax64 = 64;                  // in the FP64 form: eight
 constexpr int kTcTmemCols = 512;
 constexpr int kTcGmax = 15;                    // (i, j) blocks per window at most (class 4 has 15)
 constexpr int kTcNbufMax = 4;                  // stage buffers at most
@@ -120,11 +120,14 @@ struct TcArgs {
     const long long* boff;  // [nwin]: start of the window's B tiles in bs (16-byte units)
     const int* sched;    // [ngroups + 1] offsets, then window ids grouped by CTA group
     const int* wpairs;   // (i | j << 3) of each block
-    const float4* tabk;  // X(0..), Y(0..) as complex double-float, [tws] per record in the K order of all classes
-    const float4* tabz;  // Z(0..), [ncols] per record in the same order
+    const void* tabk;    // X(0..), Y(0..) as complex double-float or double (16 bytes either way), [tws] per record in
+                         // the K order of all classes
+    const void* tabz;    // Z(0..), [ncols] per record in the same order
     const float* clk;    // c log2(e) in the same order
     long long kbase[kNclass];  // first record of each class in that order
-    const float2* Dp;    // Hermite densities (double-float) in the K order: [dens][class][term][position]
+    const void* Dp;      // Hermite densities: split form double-float in the K order, [dens][class][term][position];
+                         // FP64 form doubles in record order, [dens][class][term][record]
+    const int* korder;   // FP64 form: class-local record of each position of the K order of all classes
     long long dp_total;
     long long dp_base[kNclass];
     long long dp_stride[kNclass];
@@ -279,12 +282,98 @@ __device__ __forceinline__ void tc_ld_levels4(uint32_t taddr, uint32_t npad, flo
         for (int i = 0; i < 4; ++i) v[l][i] = __uint_as_float(r[4 * l + i]);
 }
 
-// the sum of the five level sums of one real output, double-float (|lo| may
-// exceed ulp(hi)/2 by a few units)
-__device__ __forceinline__ df level_sum(float t0, float t1, float t2, float t3, float t4) {
-    const df a = two_sum(t0, t1), b = two_sum(t2, t3);
+__device__ __forceinline__ void tc_ld_levels4(uint32_t taddr, uint32_t npad, float (&v)[8][4]) {
+    uint32_t r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%32];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%33];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%8,%9,%10,%11}, [%34];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%12,%13,%14,%15}, [%35];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%16,%17,%18,%19}, [%36];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%20,%21,%22,%23}, [%37];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%24,%25,%26,%27}, [%38];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%28,%29,%30,%31}, [%39];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr), "r"(taddr + npad), "r"(taddr + 2 * npad), "r"(taddr + 3 * npad), "r"(taddr + 4 * npad),
+          "r"(taddr + 5 * npad), "r"(taddr + 6 * npad), "r"(taddr + 7 * npad)
+        : "memory");
+#pragma unroll
+    for (int l = 0; l < 8; ++l)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[l][i] = __uint_as_float(r[4 * l + i]);
+}
+
+// Triple-float: the unevaluated sum of three FP32 numbers, about 70 bits; the
+// FP64 form adds its level sums in it on the FP32 pipe, 64 times the FP64 rate.
+struct tf {
+    float h, m, l;
+};
+
+__device__ __forceinline__ tf tf_add(tf a, tf b) {
+    const df s = two_sum(a.h, b.h), t = two_sum(a.m, b.m), u = two_sum(t.hi, s.lo);
+    const float l = __fadd_rn(__fadd_rn(a.l, b.l), __fadd_rn(t.lo, u.lo));
+    const df h = fast_two_sum(s.hi, u.hi), m = two_sum(h.lo, l);
+    return tf{h.hi, m.hi, m.lo};
+}
+
+__device__ __forceinline__ tf tf_mulf(tf a, float f) {
+    const float p = __fmul_rn(a.h, f), q = __fmul_rn(a.m, f);
+    const float e = __fmaf_rn(a.h, f, -p);
+    const df s = two_sum(e, q);
+    return tf{p, s.hi, __fadd_rn(s.lo, __fmaf_rn(a.l, f, __fmaf_rn(a.m, f, -q)))};
+}
+
+__device__ __forceinline__ tf tf_mul(tf a, tf b) {
+    const float p = __fmul_rn(a.h, b.h), q = __fmul_rn(a.h, b.m), r = __fmul_rn(a.m, b.h);
+    const float e = __fmaf_rn(a.h, b.h, -p);
+    const df s = two_sum(q, r), t = two_sum(s.hi, e);
+    float l = __fmaf_rn(a.m, b.m, __fadd_rn(__fmaf_rn(a.h, b.m, -q), __fmaf_rn(a.m, b.h, -r)));
+    l = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, l));
+    return tf{p, t.hi, __fadd_rn(l, __fadd_rn(s.lo, t.lo))};
+}
+
+__device__ __forceinline__ tf tf_neg(tf a) { return tf{-a.h, -a.m, -a.l}; }
+
+__device__ __forceinline__ double tf_double(tf a) { return widen(a.h) + (widen(a.m) + widen(a.l)); }
+
+// Operations that the kernels need on their sums, double-float or triple-float
+__device__ __forceinline__ df sum_zero(df) { return df{0.f, 0.f}; }
+__device__ __forceinline__ tf sum_zero(tf) { return tf{0.f, 0.f, 0.f}; }
+__device__ __forceinline__ df sum_neg(df a) { return df_neg(a); }
+__device__ __forceinline__ tf sum_neg(tf a) { return tf{-a.h, -a.m, -a.l}; }
+__device__ __forceinline__ df sum_add(df a, df b) { return df_add(a, b); }
+__device__ __forceinline__ tf sum_add(tf a, tf b) { return tf_add(a, b); }
+__device__ __forceinline__ df sum_mulf(df a, float f) { return df_mulf_u(a, f); }
+__device__ __forceinline__ tf sum_mulf(tf a, float f) { return tf_mulf(a, f); }
+__device__ __forceinline__ double sum_double(df a) { return (double)a.hi + (double)a.lo; }
+__device__ __forceinline__ double sum_double(tf a) { return tf_double(a); }
+__device__ __forceinline__ df sum_xor(df a, int mask) {
+    return df{__shfl_xor_sync(0xffffffffu, a.hi, mask), __shfl_xor_sync(0xffffffffu, a.lo, mask)};
+}
+__device__ __forceinline__ tf sum_xor(tf a, int mask) {
+    return tf{__shfl_xor_sync(0xffffffffu, a.h, mask), __shfl_xor_sync(0xffffffffu, a.m, mask),
+              __shfl_xor_sync(0xffffffffu, a.l, mask)};
+}
+
+// the level sums of one real output (column v of the levels read), in double-
+// float (|lo| may exceed ulp(hi)/2 by a few units) and in triple-float
+__device__ __forceinline__ df level_sum(const float (&t)[5][4], int v) {
+    const df a = two_sum(t[0][v], t[1][v]), b = two_sum(t[2][v], t[3][v]);
     const df s = two_sum(a.hi, b.hi);
-    return df{s.hi, __fadd_rn(__fadd_rn(s.lo, a.lo), __fadd_rn(b.lo, t4))};
+    return df{s.hi, __fadd_rn(__fadd_rn(s.lo, a.lo), __fadd_rn(b.lo, t[4][v]))};
+}
+__device__ __forceinline__ tf level_sum(const float (&t)[8][4], int v) {
+    const df a = two_sum(t[0][v], t[1][v]), b = two_sum(t[2][v], t[3][v]), c = two_sum(t[4][v], t[5][v]);
+    const df s = two_sum(a.hi, b.hi);
+    const df m1 = two_sum(s.lo, a.lo), m2 = two_sum(m1.hi, b.lo), m3 = two_sum(m2.hi, c.hi);
+    const float l = __fadd_rn(__fadd_rn(__fadd_rn(m1.lo, m2.lo), m3.lo),
+                              __fadd_rn(c.lo, __fadd_rn(t[6][v], t[7][v])));
+    const df m = two_sum(m3.hi, l);
+    return tf{s.hi, m.hi, m.lo};
 }
 
 // ---- operand slices ---------------------------------------------------------
@@ -302,7 +391,7 @@ __device__ __forceinline__ float pow2f(int k) {
 // nearest even, no fast-math reassociation); slices 0-2 peel the high part
 // exactly, the low part joins at slice 3 with one rounding below 2^(e-45).
 struct Slicer6 {
-    float c[kTcS];
+    float c[6];
     __device__ __forceinline__ explicit Slicer6(float u) {
         c[0] = 0x1.8p23f * u;
         c[1] = 0x1.8p16f * u;
@@ -311,7 +400,7 @@ struct Slicer6 {
         c[4] = 0x1.8p-5f * u;
         c[5] = 0x1.8p-12f * u;
     }
-    __device__ __forceinline__ void operator()(float h, float l, float (&o)[kTcS]) const {
+    __device__ __forceinline__ void operator()(float h, float l, float (&o)[6]) const {
         o[0] = __fsub_rn(__fadd_rn(h, c[0]), c[0]);
         h = __fsub_rn(h, o[0]);
         o[1] = __fsub_rn(__fadd_rn(h, c[1]), c[1]);
@@ -329,6 +418,79 @@ struct Slicer6 {
 __device__ __forceinline__ uint32_t pack_bf2(float a, float b) {
     __nv_bfloat162 v = __floats2bfloat162_rn(a, b);  // exact: every slice has <= 8 significant bits
     return *reinterpret_cast<uint32_t*>(&v);
+}
+
+// Seven slices of x = h + l (|x| < 2^e): o[s] = m_s u 2^(-7s), u = 2^(e-6),
+// integers |m_s| <= 64, x = sum_s o[s] up to 2^(e-51).  As in the six-slice
+// split, but the low part joins at slice 3 through an error-free sum, so that
+// none of its bits above 2^-45 u is lost.
+struct Slicer7 {
+    float c[7];
+    __device__ __forceinline__ explicit Slicer7(float u) {
+        c[0] = 0x1.8p23f * u;
+        c[1] = 0x1.8p16f * u;
+        c[2] = 0x1.8p9f * u;
+        c[3] = 0x1.8p2f * u;
+        c[4] = 0x1.8p-5f * u;
+        c[5] = 0x1.8p-12f * u;
+        c[6] = 0x1.8p-19f * u;
+    }
+    __device__ __forceinline__ void operator()(float h, float l, float (&o)[7]) const {
+        o[0] = __fsub_rn(__fadd_rn(h, c[0]), c[0]);
+        h = __fsub_rn(h, o[0]);
+        o[1] = __fsub_rn(__fadd_rn(h, c[1]), c[1]);
+        h = __fsub_rn(h, o[1]);
+        o[2] = __fsub_rn(__fadd_rn(h, c[2]), c[2]);
+        h = __fsub_rn(h, o[2]);
+        const df j = two_sum(h, l);  // h + l = j.hi + j.lo exactly
+        o[3] = __fsub_rn(__fadd_rn(j.hi, c[3]), c[3]);
+        h = __fadd_rn(__fsub_rn(j.hi, o[3]), j.lo);
+        o[4] = __fsub_rn(__fadd_rn(h, c[4]), c[4]);
+        h = __fsub_rn(h, o[4]);
+        o[5] = __fsub_rn(__fadd_rn(h, c[5]), c[5]);
+        h = __fsub_rn(h, o[5]);
+        o[6] = __fsub_rn(__fadd_rn(h, c[6]), c[6]);
+    }
+};
+
+// The FP64 form's slices: x (|x| < 2^e) in fixed point to 2^(e-55), truncated,
+// cut into eight 7-bit digits m_s in [-64, 64], x = 2^(e-6) sum_s m_s 2^(-7s),
+// with integer operations alone (GB300 has 64 FP32 and 32 integer lanes for
+// each FP64 one).  The word holds the digits plus 64 each, digit s at bit
+// 7 (7 - s); |x| <= 2^e (1 - 2^-11) keeps the word below 2^56 + 2^49.
+__device__ __forceinline__ unsigned long long fixed8(double x, int e) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+    // an exponent far below e, zero and subnormals among them, shifts everything out
+    const int r = min(e + 1022 - (int)((u >> 52) & 0x7ff), 63);
+    const unsigned long long f = (((u & 0xfffffffffffffULL) | 0x10000000000000ULL) << 2) >> r;
+    constexpr unsigned long long bias = 64ULL * (((1ULL << 56) - 1) / 127);  // 64 in every digit
+    const unsigned long long neg = (unsigned long long)((long long)u >> 63);
+    return (f ^ neg) + (bias - neg);
+}
+
+// The digits of two words as bf16 pairs, digit s times 2^(-7s): 128 + u is the
+// bf16 with u in its mantissa field (u = 128, digit 0 only, carries into the
+// exponent: 256), and 192 = 128 + 64 comes off in one exact FMA.  A byte
+// permutation puts 16 bits of each word side by side, so that one shift and one
+// mask serve both.
+__device__ __forceinline__ uint32_t digit_fma(uint32_t v, float w) {
+    const __nv_bfloat162 r = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&v), __float2bfloat162_rn(w),
+                                     __float2bfloat162_rn(-192.f * w));
+    return *reinterpret_cast<const uint32_t*>(&r);
+}
+__device__ __forceinline__ void digit_pairs(unsigned long long a, unsigned long long b, uint32_t (&o)[8]) {
+    const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32), bl = (uint32_t)b, bh = (uint32_t)(b >> 32);
+    constexpr uint32_t kMask = 0x007f007fu, kOne = 0x43004300u;
+    const uint32_t w0 = __byte_perm(al, bl, 0x5410);  // bits 0-15
+    o[7] = digit_fma((w0 & kMask) | kOne, 0x1p-49f);
+    o[6] = digit_fma(((w0 >> 7) & kMask) | kOne, 0x1p-42f);
+    o[5] = digit_fma(((__byte_perm(al, bl, 0x6521) >> 6) & kMask) | kOne, 0x1p-35f);  // bits 8-23
+    o[4] = digit_fma(((__byte_perm(al, bl, 0x7632) >> 5) & kMask) | kOne, 0x1p-28f);  // bits 16-31
+    o[3] = digit_fma((__byte_perm(__funnelshift_r(al, ah, 28), __funnelshift_r(bl, bh, 28), 0x5410) & kMask) | kOne,
+                     0x1p-21f);
+    o[2] = digit_fma(((__byte_perm(ah, bh, 0x5410) >> 3) & kMask) | kOne, 0x1p-14f);
+    o[1] = digit_fma(((__byte_perm(ah, bh, 0x6521) >> 2) & kMask) | kOne, 0x1p-7f);
+    o[0] = digit_fma(((__byte_perm(ah, bh, 0x7632) >> 1) & 0x00ff00ffu) + kOne, 1.f);
 }
 
 // element offset of (row, k) in a stage tile [rows][16 K] of core matrices
@@ -395,6 +557,67 @@ __device__ __forceinline__ float ipow(float n, int k) {
 // columns of an MMA over nb blocks
 __host__ __device__ __forceinline__ int mma_cols(int nb, int colw) { return (nb * colw + 15) / 16 * 16; }
 
+// ---- the two precisions of the product -----------------------------------------
+//
+// S slices per operand, ACC level accumulators, Comp the table component (a
+// real or imaginary part), Sum the type that adds level sums.  pair() multiplies
+// the X and Y parts of two K entries and cuts both products; a row's bound 2^e
+// is in the slices (split form) or comes back through row_scale (FP64 form,
+// whose A digits carry only 2^(-7s)).
+
+template <int NS, class Cutter>
+struct SplitPrec {
+    static constexpr int S = NS, ACC = 5;  // levels 0-3 exact, the rest in a rounded fifth accumulator
+    using Comp = float2;
+    using Sum = df;
+    struct Cut {
+        Cutter c;
+        __device__ __forceinline__ explicit Cut(int e) : c(pow2f(e - 6)) {}
+        __device__ __forceinline__ void pair(df a, df b, uint32_t (&o)[S]) const {
+            float oa[S], ob[S];
+            c(a.hi, a.lo, oa);
+            c(b.hi, b.lo, ob);
+#pragma unroll
+            for (int s = 0; s < S; ++s) o[s] = pack_bf2(oa[s], ob[s]);
+        }
+    };
+    using Entry = df;
+    __device__ static __forceinline__ Entry product(float2 x, float2 y) { return df_mul_u(df{x.x, x.y}, df{y.x, y.y}); }
+    __device__ static __forceinline__ Entry entry(float2 x) { return df{x.x, x.y}; }
+    __device__ static __forceinline__ float row_scale(int) { return 1.f; }
+    static constexpr int kWin = kTcWinMax, kNmax = kTcNmax;
+};
+using PrecRho = SplitPrec<6, Slicer6>;
+using PrecJ = SplitPrec<7, Slicer7>;
+
+// Eight slices, 36 products s + t <= 7, every level in an accumulator of its
+// own: 64^2 x 8 products x 512 K terms = 2^24 keeps all of them exact over a
+// window of 512, and 56 bits below the bounds of the window leave the sums with
+// a smaller error than FP64 accumulation.
+struct Prec64 {
+    static constexpr int S = 8, ACC = 8;
+    using Comp = double;
+    using Sum = tf;
+    struct Cut {
+        int e;
+        __device__ __forceinline__ explicit Cut(int e_) : e(e_) {}
+        __device__ __forceinline__ void pair(double a, double b, uint32_t (&o)[S]) const {
+            digit_pairs(fixed8(a, e), fixed8(b, e), o);
+        }
+    };
+    using Entry = double;
+    __device__ static __forceinline__ Entry product(double x, double y) { return x * y; }
+    __device__ static __forceinline__ Entry entry(double x) { return x; }
+    __device__ static __forceinline__ float row_scale(int e) { return pow2f(e - 6); }
+    static constexpr int kWin = kTcWinMax / 2, kNmax = kTcNmax64;
+};
+
+// the exponent of a bound (log2), not below -60 in the FP64 form, where the last slice sits 2^-55 under it
+template <class P>
+__device__ __forceinline__ int bound_exp(float log2_bound) {
+    return P::S == 8 ? max(exp_bound(log2_bound), -60) : exp_bound(log2_bound);
+}
+
 constexpr int kTcProdWarps = 16;                    // two groups of eight, stages in turn
 constexpr int kTcGroupWarps = kTcProdWarps / 2;
 constexpr int kTcMmaWarp = 16;
@@ -414,7 +637,10 @@ constexpr int kTcBThreads = 512;
 // records of one (block, n_c, density), both columns (Re, Im), as halves of
 // 16-byte core-matrix rows; neighbouring lanes take the other half, neighbouring
 // columns and record octets, so a warp's stores of one slice fill 512-byte runs.
-__global__ void __launch_bounds__(kTcBThreads, 2) k_tc_rho_b(TcArgs g) {
+template <class P>
+__global__ void __launch_bounds__(kTcBThreads, P::S == 8 ? 1 : 2) k_tc_rho_b(TcArgs g) {
+    constexpr bool kF64 = P::S == 8;
+    constexpr int kS = P::S;
     __shared__ int mx[kTcNmax / 2];  // bits of the column bounds (non-negative floats order as integers)
     __shared__ int pairs[kTcGmax], tidx[kTcGmax][5];
     __shared__ int clmin_bits;
@@ -430,15 +656,19 @@ __global__ void __launch_bounds__(kTcBThreads, 2) k_tc_rho_b(TcArgs g) {
     if (tid == 0) clmin_bits = __float_as_int(INFINITY);
     __syncthreads();
     const long long stride = g.dp_stride[L];
-    const float2* dpw = g.Dp + g.dp_base[L] + (long long)g.d0 * g.dp_total + wi.w;
+    // split form: this window's positions; FP64 form: the class's records
+    const float2* dpw = reinterpret_cast<const float2*>(g.Dp) + g.dp_base[L] + (long long)g.d0 * g.dp_total + wi.w;
+    const double* dp64 = reinterpret_cast<const double*>(g.Dp) + g.dp_base[L] + (long long)g.d0 * g.dp_total;
     const long long kb = g.kbase[L] + wi.w;  // the window's first record in the K order
-    constexpr int kIt = kTcWinMax / kTcBThreads;
+    constexpr int kIt = P::kWin / kTcBThreads;
     float cr[kIt], cmin = INFINITY;
+    int ko[kIt];
 #pragma unroll
     for (int q = 0; q < kIt; ++q) {
         const int k = tid + q * kTcBThreads;
         cr[q] = k < cnt ? __ldg(g.clk + kb + k) : 0.f;
         if (k < cnt) cmin = fminf(cmin, cr[q]);
+        ko[q] = kF64 && k < cnt ? __ldg(g.korder + kb + k) : 0;
     }
     for (int gb = 0; gb < npair; ++gb)
         for (int d = 0; d < g.nd; ++d) {
@@ -446,11 +676,13 @@ __global__ void __launch_bounds__(kTcBThreads, 2) k_tc_rho_b(TcArgs g) {
 #pragma unroll
             for (int q = 0; q < kIt; ++q) {
                 const int k = tid + q * kTcBThreads;
-                const float2* dp = dpw + (long long)d * g.dp_total + k;
 #pragma unroll
                 for (int kk = 0; kk < 5; ++kk) {
                     const int t = tidx[gb][kk];
-                    cm[q][kk] = t >= 0 && k < cnt ? fabsf(__ldg(dp + (long long)t * stride).x) * 1.0001f : 0.f;
+                    cm[q][kk] = 0.f;
+                    if (t < 0 || k >= cnt) continue;
+                    const long long off = (long long)d * g.dp_total + (long long)t * stride;
+                    cm[q][kk] = 1.0001f * (kF64 ? fabsf((float)__ldg(dp64 + off + ko[q])) : fabsf(__ldg(dpw + off + k).x));
                 }
             }
             for (int nc = 0; nc < g.ncols; ++nc) {
@@ -482,48 +714,94 @@ __global__ void __launch_bounds__(kTcBThreads, 2) k_tc_rho_b(TcArgs g) {
         const int pr = pairs[gb], nk = L - (pr & 7) - (pr >> 3);  // k = 0 .. L - i - j
         const int k0 = q * kTcStageK + oc * 8 + half * 4;
         const float mb = __int_as_float(mx[gb * npo + p]);
-        const Slicer6 cut(pow2f((mb > 0.f ? exp_bound(log2f(mb)) : -100) - 6));
-        uint32_t s0[kTcS][2], s1[kTcS][2];
-        const float2* dpd = dpw + (long long)d * g.dp_total + k0;
+        const int eb = mb > 0.f ? bound_exp<P>(log2f(mb)) : -60;
+        uint32_t s0[kS][2], s1[kS][2];
+        if constexpr (kF64) {
+            const float sc = pow2f(eb - 6);  // B's digits carry their column's bound
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            float o0[2][kTcS], o1[2][kTcS];
-            df re[2], im[2];
-            re[0] = re[1] = im[0] = im[1] = df{0.f, 0.f};
-            float pw = 1.f;
-            for (int kk = 0; kk <= nk; ++kk) {
-                // two records' D'_k (16-byte aligned: classes, windows and halves start at even positions)
-                const float4 v = __ldg(reinterpret_cast<const float4*>(dpd + (long long)tidx[gb][kk] * stride + 2 * u));
-                const df a = df_mulf(df{v.x, v.y}, pw), b = df_mulf(df{v.z, v.w}, pw);  // D'_k n_c^k, exact power
-                switch (kk & 3) {                                                       // (-i)^k
-                    case 0: re[0] = df_add(re[0], a); re[1] = df_add(re[1], b); break;
-                    case 1: im[0] = df_sub(im[0], a); im[1] = df_sub(im[1], b); break;
-                    case 2: re[0] = df_sub(re[0], a); re[1] = df_sub(re[1], b); break;
-                    default: im[0] = df_add(im[0], a); im[1] = df_add(im[1], b); break;
+            for (int u = 0; u < 2; ++u) {
+                unsigned long long fr[2], fi[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int k = k0 + 2 * u + e;
+                    double br = 0.0, bi = 0.0;
+                    if (k < cnt) {
+                        const double* dp = dp64 + (long long)d * g.dp_total + __ldg(g.korder + kb + k);
+                        const double2 z = __ldg(reinterpret_cast<const double2*>(g.tabz) + (kb + k) * g.ncols + nc);
+                        // sum_k D'_k (-i n_c)^k: terms of even k real, of odd k imaginary (few FP64 instructions:
+                        // the pipe has 2 lanes per SM)
+                        double re = __ldg(dp + (long long)tidx[gb][0] * stride);
+                        if (nk == 0) {
+                            br = z.x * re;
+                            bi = z.y * re;
+                        } else {
+                            const double x = widen((float)nc);
+                            double im = -x * __ldg(dp + (long long)tidx[gb][1] * stride);
+                            if (nk > 1) re = fma(-widen((float)(nc * nc)), __ldg(dp + (long long)tidx[gb][2] * stride), re);
+                            if (nk > 2) im = fma(widen((float)(nc * nc * nc)), __ldg(dp + (long long)tidx[gb][3] * stride), im);
+                            if (nk > 3)
+                                re = fma(widen((float)(nc * nc * nc * nc)), __ldg(dp + (long long)tidx[gb][4] * stride), re);
+                            br = z.x * re - z.y * im;
+                            bi = z.x * im + z.y * re;
+                        }
+                    }
+                    fr[e] = fixed8(br, eb);
+                    fi[e] = fixed8(bi, eb);
                 }
-                pw *= (float)nc;
-            }
+                float w = sc;
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int k = k0 + 2 * u + e;
-                cdf bv{{0.f, 0.f}, {0.f, 0.f}};
-                if (k < cnt) {
-                    const float4 zv = __ldg(g.tabz + (kb + k) * g.ncols + nc);
-                    bv = cdf_mul(cdf{{zv.x, zv.y}, {zv.z, zv.w}}, cdf{re[e], im[e]});
+                for (int s = 0; s < kS; ++s, w *= 0x1p-7f) {
+                    const int sh = 7 * (7 - s);
+                    auto digit = [&](unsigned long long f) {
+                        return (float)((int)((f >> sh) & (s == 0 ? 0xffULL : 0x7fULL)) - 64) * w;
+                    };
+                    s0[s][u] = pack_bf2(digit(fr[0]), digit(fr[1]));
+                    s1[s][u] = pack_bf2(digit(fi[0]), digit(fi[1]));
                 }
-                cut(bv.re.hi, bv.re.lo, o0[e]);
-                cut(bv.im.hi, bv.im.lo, o1[e]);
             }
+        } else {
+            const typename P::Cut cut(eb);
+            const float2* dpd = dpw + (long long)d * g.dp_total + k0;
 #pragma unroll
-            for (int s = 0; s < kTcS; ++s) {
-                s0[s][u] = pack_bf2(o0[0][s], o0[1][s]);
-                s1[s][u] = pack_bf2(o1[0][s], o1[1][s]);
+            for (int u = 0; u < 2; ++u) {
+                df re[2], im[2];
+                re[0] = re[1] = im[0] = im[1] = df{0.f, 0.f};
+                float pw = 1.f;
+                for (int kk = 0; kk <= nk; ++kk) {
+                    // two records' D'_k (16-byte aligned: classes, windows and halves start at even positions)
+                    const float4 v = __ldg(reinterpret_cast<const float4*>(dpd + (long long)tidx[gb][kk] * stride + 2 * u));
+                    const df a = df_mulf(df{v.x, v.y}, pw), b = df_mulf(df{v.z, v.w}, pw);  // D'_k n_c^k, exact power
+                    switch (kk & 3) {                                                       // (-i)^k
+                        case 0: re[0] = df_add(re[0], a); re[1] = df_add(re[1], b); break;
+                        case 1: im[0] = df_sub(im[0], a); im[1] = df_sub(im[1], b); break;
+                        case 2: re[0] = df_sub(re[0], a); re[1] = df_sub(re[1], b); break;
+                        default: im[0] = df_add(im[0], a); im[1] = df_add(im[1], b); break;
+                    }
+                    pw *= (float)nc;
+                }
+                cdf bv[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int k = k0 + 2 * u + e;
+                    bv[e] = cdf{{0.f, 0.f}, {0.f, 0.f}};
+                    if (k < cnt) {
+                        const float4 zv = __ldg(reinterpret_cast<const float4*>(g.tabz) + (kb + k) * g.ncols + nc);
+                        bv[e] = cdf_mul(cdf{{zv.x, zv.y}, {zv.z, zv.w}}, cdf{re[e], im[e]});
+                    }
+                }
+                uint32_t o[kS];
+                cut.pair(bv[0].re, bv[1].re, o);
+#pragma unroll
+                for (int s = 0; s < kS; ++s) s0[s][u] = o[s];
+                cut.pair(bv[0].im, bv[1].im, o);
+#pragma unroll
+                for (int s = 0; s < kS; ++s) s1[s][u] = o[s];
             }
         }
         const int col = gb * g.colw + 2 * p;
-        uint2* dst = reinterpret_cast<uint2*>(base + (size_t)q * kTcS * nw * 2 + ((col >> 3) * 2 + oc) * 8 + (col & 7)) + half;
+        uint2* dst = reinterpret_cast<uint2*>(base + (size_t)q * kS * nw * 2 + ((col >> 3) * 2 + oc) * 8 + (col & 7)) + half;
 #pragma unroll
-        for (int s = 0; s < kTcS; ++s) {
+        for (int s = 0; s < kS; ++s) {
             dst[(size_t)s * nw * 4] = make_uint2(s0[s][0], s0[s][1]);
             dst[(size_t)s * nw * 4 + 2] = make_uint2(s1[s][0], s1[s][1]);
         }
@@ -552,12 +830,12 @@ __device__ void ring_settle(uint64_t* bar, int n, long long issued) {
     }
 }
 
-template <int NU>
+template <class P, int NU>
 __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf, int ntslots) {
     extern __shared__ __align__(1024) unsigned char tsm[];
     unsigned char* abuf = tsm;                                                // [nbuf][S][4096]
-    unsigned char* bbuf = abuf + (size_t)nbuf * kTcS * kTcAsliceBytes;         // [nbuf][S][npad*32]
-    const int bbytes = kTcS * g.npad * 32;
+    unsigned char* bbuf = abuf + (size_t)nbuf * P::S * kTcAsliceBytes;         // [nbuf][S][npad*32]
+    const int bbytes = P::S * g.npad * 32;
     unsigned char* tring = bbuf + (size_t)nbuf * bbytes;                       // [ntslots][slot]
     const size_t tslot = tab_slot_bytes(g.tws);
     TcSmem& sm = *reinterpret_cast<TcSmem*>(tring + (size_t)ntslots * tslot);
@@ -607,7 +885,7 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf,
             for (int jw = j0; jw < j1 && ok; ++jw) {
                 const int w = __ldg(wlist + jw), cnt = __ldg(g.wcnt + w);
                 const int4 wi = __ldg(g.winfo + w);
-                const float4* src = g.tabk + (g.kbase[wi.x] + wi.w) * g.tws;
+                const float4* src = reinterpret_cast<const float4*>(g.tabk) + (g.kbase[wi.x] + wi.w) * g.tws;
                 for (int k0 = 0; k0 < cnt; k0 += kTcStageK, ++gt, t.next()) {
                     if (gt >= ntslots && !(ok = mbar_wait(&sm.tempty[t.i], t.ph ^ 1u, abort_flag, g.spin))) break;
                     const uint32_t bytes = (uint32_t)(min(kTcStageK, cnt - k0) * g.tws) * 16u;
@@ -625,7 +903,7 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf,
             long long gs = 0;
             for (int jw = j0; jw < j1 && ok; ++jw) {
                 const int w = __ldg(wlist + jw), nst = (__ldg(g.wcnt + w) + kTcStageK - 1) / kTcStageK;
-                const uint32_t bb = (uint32_t)(kTcS * mma_cols(__ldg(&g.winfo[w].y), g.colw) * 32);
+                const uint32_t bb = (uint32_t)(P::S * mma_cols(__ldg(&g.winfo[w].y), g.colw) * 32);
                 const unsigned char* src = reinterpret_cast<const unsigned char*>(g.bs + __ldg(g.boff + w));
                 for (int q = 0; q < nst; ++q, ++gs, b.next()) {
                     if (gs >= nbuf && !(ok = mbar_wait(&sm.empty[b.i], b.ph ^ 1u, abort_flag, g.spin))) break;
@@ -653,7 +931,7 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf,
                 if (!ok) break;
                 tc_fence_after();
                 if (elect_one()) {
-                    issue_kstep<kTcS, kTcAcc>(tmem, sdesc(a0 + b.i * kTcS * kTcAsliceBytes), kTcAsliceBytes >> 4,
+                    issue_kstep<P::S, P::ACC>(tmem, sdesc(a0 + b.i * P::S * kTcAsliceBytes), kTcAsliceBytes >> 4,
                                               sdesc(b0 + b.i * bbytes), nw * 2, nw, idesc, q > 0);
                     tc_commit(&sm.empty[b.i]);
                     if (q + 1 == nst) tc_commit(&sm.accf);
@@ -675,7 +953,7 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf,
         const int sl = __ldg(g.slots + mt * kTcM + row);
         const float fa = (float)(sl & 255), fb = (float)((sl >> 8) & 255);
         const float Q = g.Maa * fa * fa + g.Mbb * fb * fb;
-        const int rs = 2 * g.tws;  // float2 per record
+        const int rs = 2 * g.tws;  // components per record
         const int xo = oct * 8 * rs + 2 * (sl & 255) + ((sl >> 16) & 1);
         const int yo = oct * 8 * rs + 2 * (g.offY + ((sl >> 8) & 255)) + ((sl >> 17) & 1);
         unsigned char* arow = abuf + tile_off(row, oct * 8) * 2;
@@ -686,43 +964,41 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf,
         const float ea = (float)(es_slot & 255), eb = (float)((es_slot >> 8) & 255);
         const int ca = (es_slot >> 16) & 1, cb = (es_slot >> 17) & 1;
         const int nunit = g.colw / 4, npo = g.nd * g.ncols;
-        df S[NU][4];  // double-float sums by sign character: two complex outputs per unit
+        typename P::Sum S[NU][4];  // sums by sign character: two complex outputs per unit
 #pragma unroll
         for (int x = 0; x < NU; ++x)
 #pragma unroll
-            for (int v = 0; v < 4; ++v) S[x][v] = df{0.f, 0.f};
+            for (int v = 0; v < 4; ++v) S[x][v] = sum_zero(typename P::Sum());
+        const float eQ = g.Maa * ea * ea + g.Mbb * eb * eb;
         Ring b(nbuf), t(ntslots);
         int gs = 0;  // stages so far (mod 2 the group that forms it)
         bool full = false;  // every buffer used once
         for (int jw = j0; jw < j1 && ok; ++jw) {
             const int w = __ldg(wlist + jw), nst = (__ldg(g.wcnt + w) + kTcStageK - 1) / kTcStageK;
-            const Slicer6 cut(pow2f(exp_bound(-__ldg(g.clw + w) * Q) - 6));
+            const float cl = __ldg(g.clw + w);
+            const typename P::Cut cut(bound_exp<P>(-cl * Q));
             for (int q = 0; q < nst; ++q, ++gs, b.next(), t.next()) {
                 full = full || gs >= nbuf;
                 if ((gs & 1) != grp) continue;
                 ok = __all_sync(0xffffffffu, mbar_wait(&sm.tfull[t.i], t.ph, abort_flag, g.spin));
                 if (!ok) break;
-                const float2* tb = reinterpret_cast<const float2*>(tring + (size_t)t.i * tslot);
-                uint32_t pk[kTcS][4];
+                const typename P::Comp* tb = reinterpret_cast<const typename P::Comp*>(tring + (size_t)t.i * tslot);
+                uint32_t pk[P::S][4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    float o[2][kTcS];
+                    uint32_t o[P::S];
+                    cut.pair(P::product(tb[2 * u * rs + xo], tb[2 * u * rs + yo]),
+                             P::product(tb[(2 * u + 1) * rs + xo], tb[(2 * u + 1) * rs + yo]), o);
 #pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const float2 x = tb[(2 * u + e) * rs + xo], y = tb[(2 * u + e) * rs + yo];
-                        const df a = df_mul_u(df{x.x, x.y}, df{y.x, y.y});
-                        cut(a.hi, a.lo, o[e]);
-                    }
-#pragma unroll
-                    for (int s = 0; s < kTcS; ++s) pk[s][u] = pack_bf2(o[0][s], o[1][s]);
+                    for (int s = 0; s < P::S; ++s) pk[s][u] = o[s];
                 }
                 if (full) {
                     ok = __all_sync(0xffffffffu, mbar_wait(&sm.empty[b.i], b.ph ^ 1u, abort_flag, g.spin));
                     if (!ok) break;
                 }
-                unsigned char* as = arow + (size_t)b.i * kTcS * kTcAsliceBytes;
+                unsigned char* as = arow + (size_t)b.i * P::S * kTcAsliceBytes;
 #pragma unroll
-                for (int s = 0; s < kTcS; ++s)
+                for (int s = 0; s < P::S; ++s)
                     *reinterpret_cast<uint4*>(as + (size_t)s * kTcAsliceBytes) =
                         make_uint4(pk[s][0], pk[s][1], pk[s][2], pk[s][3]);
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -739,26 +1015,24 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf,
             tc_fence_after();
             const int4 wi = __ldg(g.winfo + w);
             const uint32_t nw = (uint32_t)mma_cols(wi.y, g.colw);
+            const float rsc = P::row_scale(bound_exp<P>(-cl * eQ));
             for (int gb = 0; gb < wi.y; ++gb) {
                 const int pr = __ldg(g.wpairs + wi.z + gb), i = pr & 7, j = pr >> 3;
                 // type (ta, tb) of lane ^ mask adds to this lane's character; i^{ta - i} = i^{ca} times a real sign
                 const int mask = (i & 1) | ((j & 1) << 1);
-                float f = ipow(ea, i) * ipow(eb, j);
+                float f = ipow(ea, i) * ipow(eb, j) * rsc;
                 if ((((i >> 1) + (j >> 1) + (ca & i) + (cb & j)) & 1) != 0) f = -f;
 #pragma unroll
                 for (int x = 0; x < NU; ++x) {
                     const int un = es + 4 * x;
                     if (un < nunit) {
-                        float T[5][4];
+                        float T[P::ACC][4];
                         tc_ld_levels4(tmem + tlane + (uint32_t)(gb * g.colw + 4 * un), nw, T);
 #pragma unroll
                         for (int v = 0; v < 4; ++v) {
-                            df l = level_sum(T[0][v], T[1][v], T[2][v], T[3][v], T[4][v]);
-                            if (mask) {
-                                l.hi = __shfl_xor_sync(0xffffffffu, l.hi, mask);
-                                l.lo = __shfl_xor_sync(0xffffffffu, l.lo, mask);
-                            }
-                            S[x][v] = df_add(S[x][v], df_mulf_u(l, f));
+                            typename P::Sum l = level_sum(T, v);
+                            if (mask) l = sum_xor(l, mask);
+                            S[x][v] = sum_add(S[x][v], sum_mulf(l, f));
                         }
                     }
                 }
@@ -780,14 +1054,21 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf,
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         // i^{ca + cb}, then the sign sums over the two characters of each axis
-                        const cdf z = rot_mi(cdf{S[x][2 * h], S[x][2 * h + 1]}, 4 - ca - cb);
-                        df c[2] = {z.re, z.im};
+                        typename P::Sum c[2] = {S[x][2 * h], S[x][2 * h + 1]};
+                        if (ca + cb == 1) {
+                            const typename P::Sum t = c[0];
+                            c[0] = sum_neg(c[1]);
+                            c[1] = t;
+                        } else if (ca + cb == 2) {
+                            c[0] = sum_neg(c[0]);
+                            c[1] = sum_neg(c[1]);
+                        }
 #pragma unroll
                         for (int r = 0; r < 2; ++r) {
-                            df o{__shfl_xor_sync(0xffffffffu, c[r].hi, 1), __shfl_xor_sync(0xffffffffu, c[r].lo, 1)};
-                            if (da) c[r] = (lane & 1) ? df_sub(o, c[r]) : df_add(c[r], o);
-                            o = df{__shfl_xor_sync(0xffffffffu, c[r].hi, 2), __shfl_xor_sync(0xffffffffu, c[r].lo, 2)};
-                            if (db) c[r] = (lane & 2) ? df_sub(o, c[r]) : df_add(c[r], o);
+                            typename P::Sum o = sum_xor(c[r], 1);
+                            if (da) c[r] = (lane & 1) ? sum_add(o, sum_neg(c[r])) : sum_add(c[r], o);
+                            o = sum_xor(c[r], 2);
+                            if (db) c[r] = (lane & 2) ? sum_add(o, sum_neg(c[r])) : sum_add(c[r], o);
                         }
                         const int p = 2 * un + h;
                         if (valid && p < npo) {
@@ -796,8 +1077,7 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf,
                             if (idx != INT_MIN) {
                                 const bool cj = idx < 0;
                                 if (cj) idx = ~idx;
-                                const double re = (double)c[0].hi + (double)c[0].lo;
-                                const double im = (double)c[1].hi + (double)c[1].lo;
+                                const double re = sum_double(c[0]), im = sum_double(c[1]);
                                 g.out[((long long)(g.d0 + d) * g.out_rows + g.out_row0 + kg) * g.ng_half + idx] =
                                     make_double2(re, cj ? -im : im);
                             }
@@ -822,13 +1102,15 @@ __global__ void k_tc_width(const PairWalk* __restrict__ walk, long long npairs, 
     if (r < npairs) cl[r] = (float)(walk[r].c * 1.4426950408889634);
 }
 
-// Per-record factor tables in FP64, kept as double-float: X(0..na), Y(0..nb)
+// Per-record factor tables in FP64, kept as double-float or double: X(0..na), Y(0..nb)
 // with tws entries per record, in record order (the back-contraction's tiles)
 // and in the K order (the structure-factor stages), so that a tile or a stage
 // is one contiguous copy; Z(0..nc) in the K order.
+template <bool F64>
 __global__ void k_tc_tables(const PairWalk* __restrict__ walk, long long npairs, const int* __restrict__ kpos, int ax,
                             int bx, int cx, int nna, int nnb, int nnc, int tws, double Maa, double Mbb, double Mcc,
-                            float4* __restrict__ tab, float4* __restrict__ tabk, float4* __restrict__ tabz) {
+                            float4* __restrict__ tab, float4* __restrict__ tabk, float4* __restrict__ tabz,
+                            float4* __restrict__ tabz3) {  // F64: tab, tabk, tabz as double2; Z also as triple-float
     const int tabw = nna + nnb + nnc;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= npairs * tabw) return;
@@ -856,35 +1138,55 @@ __global__ void k_tc_tables(const PairWalk* __restrict__ walk, long long npairs,
     th -= rint(th);
     double s, c;
     sincospi(2.0 * th, &s, &c);
-    const df re = df_from_double(gval * c), im = df_from_double(-gval * s);
-    const float4 v = make_float4(re.hi, re.lo, im.hi, im.lo);
+    float4 v;
+    if (F64) {
+        const double2 z = make_double2(gval * c, -gval * s);
+        v = *reinterpret_cast<const float4*>(&z);
+    } else {
+        const df re = df_from_double(gval * c), im = df_from_double(-gval * s);
+        v = make_float4(re.hi, re.lo, im.hi, im.lo);
+    }
     const long long k = kpos[r];
     if (e < nna + nnb) {
         tab[r * tws + e] = v;
         tabk[k * tws + e] = v;
     } else {
         tabz[k * nnc + n] = v;
+        if (F64) {
+            const double z[2] = {gval * c, -gval * s};
+            for (int q = 0; q < 2; ++q) {
+                const float h = (float)z[q], m = (float)(z[q] - (double)h);
+                tabz3[2 * (k * nnc + n) + q] = make_float4(h, m, (float)(z[q] - (double)h - (double)m), 0.f);
+            }
+        }
     }
 }
 
 // shared memory of one CTA with nbuf stage buffers and nts table slots (at
 // least 120 KB, so that a second CTA never shares an SM: each one takes all
 // 512 tensor-memory columns, and a second would wait in tcgen05.alloc)
-size_t tc_smem_bytes(int npad, int tws, int nbuf, int nts) {
-    const size_t need = (size_t)nbuf * kTcS * (kTcAsliceBytes + (size_t)npad * 32) + (size_t)nts * tab_slot_bytes(tws) +
+size_t tc_smem_bytes(int slices, int npad, int tws, int nbuf, int nts) {
+    const size_t need = (size_t)nbuf * slices * (kTcAsliceBytes + (size_t)npad * 32) + (size_t)nts * tab_slot_bytes(tws) +
                         sizeof(TcSmem) + 64;
     return std::max<size_t>(need, 120 * 1024);
 }
 
+int tc_alloc(ftcj_plan* P, void** ptr, size_t bytes) {
+    const cudaError_t e = cudaMalloc(ptr, std::max<size_t>(bytes, 16));
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        *ptr = nullptr;
+        return fail(FTCJ_ENOMEM, std::string("cudaMalloc of ") + std::to_string(bytes) +
+                                     " bytes failed: " + cudaGetErrorString(e));
+    }
+    P->device_bytes += std::max<size_t>(bytes, 16);
+    return FTCJ_OK;
+}
+
 template <class T>
 int tc_upload(ftcj_plan* P, T** ptr, const std::vector<T>& v) {
-    const size_t n = std::max<size_t>(v.size(), 1);
-    cudaError_t e = cudaMalloc((void**)ptr, sizeof(T) * n);
-    if (e != cudaSuccess) {
-        *ptr = nullptr;
-        return fail(FTCJ_ENOMEM, std::string("cudaMalloc failed: ") + cudaGetErrorString(e));
-    }
-    P->device_bytes += sizeof(T) * n;
+    const int rc = tc_alloc(P, (void**)ptr, sizeof(T) * std::max<size_t>(v.size(), 1));
+    if (rc) return rc;
     if (!v.empty()) FTCJ_CUDA(cudaMemcpy(*ptr, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice));
     return FTCJ_OK;
 }
@@ -893,27 +1195,36 @@ int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
 
 // the product kernel whose drain warps hold a block of colw columns in registers
-const void* tc_rho_kernel(int colw) {
-    switch ((colw + 15) / 16) {
-        case 1: return (const void*)k_tc_rho<1>;
-        case 2: return (const void*)k_tc_rho<2>;
-        case 3: return (const void*)k_tc_rho<3>;
-        case 4: return (const void*)k_tc_rho<4>;
-        case 5: return (const void*)k_tc_rho<5>;
-        default: return (const void*)k_tc_rho<6>;
+const void* tc_rho_kernel(bool f64, int colw) {
+    const int nu = (colw + 15) / 16;
+    if (f64) {
+        switch (nu) {
+            case 1: return (const void*)k_tc_rho<Prec64, 1>;
+            case 2: return (const void*)k_tc_rho<Prec64, 2>;
+            case 3: return (const void*)k_tc_rho<Prec64, 3>;
+            default: return (const void*)k_tc_rho<Prec64, 4>;
+        }
+    }
+    switch (nu) {
+        case 1: return (const void*)k_tc_rho<PrecRho, 1>;
+        case 2: return (const void*)k_tc_rho<PrecRho, 2>;
+        case 3: return (const void*)k_tc_rho<PrecRho, 3>;
+        case 4: return (const void*)k_tc_rho<PrecRho, 4>;
+        case 5: return (const void*)k_tc_rho<PrecRho, 5>;
+        default: return (const void*)k_tc_rho<PrecRho, 6>;
     }
 }
 
 // column layout for nd densities and ncols values of n_c: real columns per
 // block (a multiple of 8) and the largest block count G whose columns fit the
 // MMA width; G = 0 when not even one block fits
-void tc_columns(int nd, int ncols, int* colw, int* G, int* npad) {
+void tc_columns(int nmax, int nd, int ncols, int* colw, int* G, int* npad) {
     *colw = round_up(2 * nd * ncols, 8);
     *G = 0;
     *npad = 0;
     for (int gg = kTcGmax; gg >= 1; --gg) {
         const int np = mma_cols(gg, *colw);
-        if (np <= kTcNmax) {
+        if (np <= nmax) {
             *G = gg;
             *npad = np;
             return;
@@ -995,11 +1306,6 @@ void tc_slots(const std::set<std::pair<int, int>>& pts, std::vector<int>& slots,
 // adds.
 
 constexpr int kTcJStageM = 16;       // slots per stage: one MMA k-step
-constexpr int kTcJS = 7;             // slices per operand
-constexpr int kTcJProducts = kTcJS * (kTcJS + 1) / 2;  // slice products formed: s + t <= 6
-constexpr int kTcJPartStages = 64;   // stages per part at most: 1024 slots, one exact accumulation
-constexpr int kTcJAcc = 5;           // accumulators: levels 0-3 exact, levels 4-6 rounded
-constexpr int kTcJNmax = 96;         // MMA N at most: five level accumulators in the 512 columns
 constexpr int kTcJAsliceBytes = kTcM * kTcJStageM * 2;        // 128 records x 16 K x bf16
 constexpr int kTcPairsAll = 15;      // (i, j) with i + j <= 4
 
@@ -1014,39 +1320,6 @@ __device__ __forceinline__ void pair_of_index(int pr, int& i, int& j) {
     j = pr;
 }
 
-// Seven slices of x = h + l (|x| < 2^e): o[s] = m_s u 2^(-7s), u = 2^(e-6),
-// integers |m_s| <= 64, x = sum_s o[s] up to 2^(e-51).  As in the six-slice
-// split, but the low part joins at slice 3 through an error-free sum, so that
-// none of its bits above 2^-45 u is lost.
-struct Slicer7 {
-    float c[kTcJS];
-    __device__ __forceinline__ explicit Slicer7(float u) {
-        c[0] = 0x1.8p23f * u;
-        c[1] = 0x1.8p16f * u;
-        c[2] = 0x1.8p9f * u;
-        c[3] = 0x1.8p2f * u;
-        c[4] = 0x1.8p-5f * u;
-        c[5] = 0x1.8p-12f * u;
-        c[6] = 0x1.8p-19f * u;
-    }
-    __device__ __forceinline__ void operator()(float h, float l, float (&o)[kTcJS]) const {
-        o[0] = __fsub_rn(__fadd_rn(h, c[0]), c[0]);
-        h = __fsub_rn(h, o[0]);
-        o[1] = __fsub_rn(__fadd_rn(h, c[1]), c[1]);
-        h = __fsub_rn(h, o[1]);
-        o[2] = __fsub_rn(__fadd_rn(h, c[2]), c[2]);
-        h = __fsub_rn(h, o[2]);
-        const df j = two_sum(h, l);  // h + l = j.hi + j.lo exactly
-        o[3] = __fsub_rn(__fadd_rn(j.hi, c[3]), c[3]);
-        h = __fadd_rn(__fsub_rn(j.hi, o[3]), j.lo);
-        o[4] = __fsub_rn(__fadd_rn(h, c[4]), c[4]);
-        h = __fsub_rn(h, o[4]);
-        o[5] = __fsub_rn(__fadd_rn(h, c[5]), c[5]);
-        h = __fsub_rn(h, o[5]);
-        o[6] = __fsub_rn(__fadd_rn(h, c[6]), c[6]);
-    }
-};
-
 struct TcJArgs {
     const int* slots;       // the structure-factor pass's slots
     const int* quads;       // their groups of four
@@ -1058,8 +1331,9 @@ struct TcJArgs {
     const int* ipairs;      // (i | j << 3) of each block
     const long long* voff;  // start of each block group's V tiles in vs (elements)
     const int* vplace;      // [15 (i, j)][kNclass]: block group << 8 | place of the block in it, -1 none
-    const float4* tab;      // X(0..), Y(0..) as complex double-float, [tws] per record
-    const float4* tabz;     // Z(0..), [ncols] per record in the K order
+    const void* tab;        // X(0..), Y(0..) as complex double-float or double, [tws] per record
+    const void* tabz;       // Z(0..), [ncols] per record in the K order: complex double-float, or triple-float as two
+                            // float4 (FP64 form)
     const int* kpos;        // position of each record in the K order of all classes
     __nv_bfloat16* vs;      // sliced V_ij: [block group][stage][slice][columns of its MMA x 16 K] stage tiles
     int* ev;                // column bounds of V_ij: [15][nd][ncols]
@@ -1077,31 +1351,49 @@ struct TcJArgs {
     int colw;               // real columns per block: nd gw
     int npad;               // MMA N of a full unit: blocks x colw rounded up to 16
     int nslots, nstage;     // slots, stages of 16
-    int nparts, spp;        // slot parts, stages per part
+    int nparts, spp;        // partial arrays of J' (slot parts x nsub), stages per part
+    int nsub;               // a block's columns are split over this many of the four warps of a lane quadrant
     long long spin;         // clock cycles a wait between roles may take before it gives up
 };
 
-// V_ij of one slot and column, without the factor i^{ta+tb} (-i)^{i+j}
-__device__ __forceinline__ cdf v_entry(const TcJArgs& g, int slot, int i, int j, int d, int nc) {
+// V_ij of one slot and column, without the factor i^{ta+tb} (-i)^{i+j}: in
+// double-float, or in FP64 (exact sign sums up to one rounding each)
+template <class P>
+__device__ __forceinline__ auto v_entry(const TcJArgs& g, int slot, int i, int j, int d, int nc) {
+    constexpr bool kF64 = P::S == 8;
     cdf v{{0.f, 0.f}, {0.f, 0.f}};
+    double2 v64 = make_double2(0.0, 0.0);
     const int sl = slot < g.nslots ? __ldg(g.slots + slot) : 0;
-    if (!((sl >> 20) & 1)) return v;
     const int na = sl & 255, nb = (sl >> 8) & 255, pa = ((sl >> 16) + i) & 1, pb = ((sl >> 17) + j) & 1;
-    for (int sa = 0; sa <= (na > 0 ? 1 : 0); ++sa)
-        for (int sb = 0; sb <= (nb > 0 ? 1 : 0); ++sb) {
-            const int idx = __ldg(g.map + ((size_t)((sa ? -na : na) + g.nam) * (2 * g.nbm + 1) +
-                                           (sb ? -nb : nb) + g.nbm) * g.ncols + nc);
-            if (idx == INT_MIN) continue;
-            const double2 w = __ldg(g.W + (long long)(g.d0 + d) * g.ng_half + (idx < 0 ? ~idx : idx));
-            cdf t{split_double(w.x), split_double(idx < 0 ? -w.y : w.y)};
-            if ((pa & sa) ^ (pb & sb)) t = cdf{df_neg(t.re), df_neg(t.im)};
-            v = cdf_add(v, t);
-        }
+    if ((sl >> 20) & 1) {
+        for (int sa = 0; sa <= (na > 0 ? 1 : 0); ++sa)
+            for (int sb = 0; sb <= (nb > 0 ? 1 : 0); ++sb) {
+                const int idx = __ldg(g.map + ((size_t)((sa ? -na : na) + g.nam) * (2 * g.nbm + 1) +
+                                               (sb ? -nb : nb) + g.nbm) * g.ncols + nc);
+                if (idx == INT_MIN) continue;
+                double2 w = __ldg(g.W + (long long)(g.d0 + d) * g.ng_half + (idx < 0 ? ~idx : idx));
+                if (idx < 0) w.y = -w.y;
+                const bool neg = (pa & sa) ^ (pb & sb);
+                if constexpr (kF64) {
+                    v64.x += neg ? -w.x : w.x;
+                    v64.y += neg ? -w.y : w.y;
+                } else {
+                    cdf t{split_double(w.x), split_double(w.y)};
+                    if (neg) t = cdf{df_neg(t.re), df_neg(t.im)};
+                    v = cdf_add(v, t);
+                }
+            }
+    }
     const float p = ipow((float)na, i) * ipow((float)nb, j);  // exact
-    return cdf{df_mulf(v.re, p), df_mulf(v.im, p)};
+    if constexpr (kF64) return make_double2(v64.x * (double)p, v64.y * (double)p);
+    else return cdf{df_mulf(v.re, p), df_mulf(v.im, p)};
 }
 
+__device__ __forceinline__ float v_abs(cdf v) { return fmaxf(fabsf(v.re.hi), fabsf(v.im.hi)); }
+__device__ __forceinline__ float v_abs(double2 v) { return fmaxf(fabsf((float)v.x), fabsf((float)v.y)); }
+
 // column bounds: the exponent bound of max over the slots of |Re V_ij|, |Im V_ij|
+template <class P>
 __global__ void __launch_bounds__(256) k_tc_vbound(TcJArgs g) {
     const int col = blockIdx.x;  // ((i, j) nd + d) ncols + n_c
     const int nc = col % g.ncols, d = (col / g.ncols) % g.nd, pr = col / (g.ncols * g.nd);
@@ -1109,8 +1401,7 @@ __global__ void __launch_bounds__(256) k_tc_vbound(TcJArgs g) {
     pair_of_index(pr, i, j);
     float mx = 0.f;
     for (int m = threadIdx.x; m < g.nslots; m += blockDim.x) {
-        const cdf v = v_entry(g, m, i, j, d, nc);
-        mx = fmaxf(mx, fmaxf(fabsf(v.re.hi), fabsf(v.im.hi)));
+        mx = fmaxf(mx, v_abs(v_entry<P>(g, m, i, j, d, nc)));
     }
     __shared__ float red[256];
     red[threadIdx.x] = mx;
@@ -1120,13 +1411,15 @@ __global__ void __launch_bounds__(256) k_tc_vbound(TcJArgs g) {
         __syncthreads();
     }
     // |Re V|, |Im V| <= mx up to the FP32 rounding of the bound
-    if (threadIdx.x == 0) g.ev[col] = red[0] > 0.f ? exp_bound(log2f(red[0] * 1.0001f)) : -100;
+    if (threadIdx.x == 0) g.ev[col] = red[0] > 0.f ? bound_exp<P>(log2f(red[0] * 1.0001f)) : -60;
 }
 
 // V_ij sliced into stage tiles: block group, stage q, slice s holds the columns
 // of its blocks, d gw + 2 n_c (Re) and + 1 (Im) within a block, and K = slot;
 // one thread per two slots; columns past 2 ncols are never read back.
+template <class P>
 __global__ void __launch_bounds__(256) k_tc_vslice(TcJArgs g) {
+    constexpr int kS = P::S;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long per_pair = (long long)g.nstage * (kTcJStageM / 2) * g.nd * g.ncols;
     if (t >= kTcPairsAll * per_pair) return;
@@ -1139,15 +1432,41 @@ __global__ void __launch_bounds__(256) k_tc_vslice(TcJArgs g) {
     const int m2 = (int)(rem % (kTcJStageM / 2)), q = (int)(rem / (kTcJStageM / 2));
     int i, j;
     pair_of_index(pr, i, j);
-    const Slicer7 cut(pow2f(g.ev[(pr * g.nd + d) * g.ncols + nc] - 6));
-    float sr[2][kTcJS], si[2][kTcJS];
+    const int ev = g.ev[(pr * g.nd + d) * g.ncols + nc];
+    uint32_t sr[kS], si[kS];
+    if constexpr (P::S == 8) {
+        unsigned long long fr[2], fi[2];
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-        const int slot = q * kTcJStageM + 2 * m2 + e;
-        const int sl = slot < g.nslots ? __ldg(g.slots + slot) : 0;
-        const cdf v = rot_mi(v_entry(g, slot, i, j, d, nc), i + j + 8 - ((sl >> 16) & 1) - ((sl >> 17) & 1));
-        cut(v.re.hi, v.re.lo, sr[e]);
-        cut(v.im.hi, v.im.lo, si[e]);
+        for (int e = 0; e < 2; ++e) {
+            const int slot = q * kTcJStageM + 2 * m2 + e;
+            const int sl = slot < g.nslots ? __ldg(g.slots + slot) : 0;
+            const double2 v = v_entry<P>(g, slot, i, j, d, nc);
+            const int rot = (i + j + 8 - ((sl >> 16) & 1) - ((sl >> 17) & 1)) & 3;  // times (-i)^rot
+            const double re = rot & 1 ? v.y : v.x, im = rot & 1 ? -v.x : v.y;
+            fr[e] = fixed8(rot & 2 ? -re : re, ev);
+            fi[e] = fixed8(rot & 2 ? -im : im, ev);
+        }
+        float w = pow2f(ev - 6);
+#pragma unroll
+        for (int s = 0; s < kS; ++s, w *= 0x1p-7f) {
+            const int sh = 7 * (7 - s);
+            auto digit = [&](unsigned long long f) {
+                return (float)((int)((f >> sh) & (s == 0 ? 0xffULL : 0x7fULL)) - 64) * w;
+            };
+            sr[s] = pack_bf2(digit(fr[0]), digit(fr[1]));
+            si[s] = pack_bf2(digit(fi[0]), digit(fi[1]));
+        }
+    } else {
+        const typename P::Cut cut(ev);
+        cdf v[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int slot = q * kTcJStageM + 2 * m2 + e;
+            const int sl = slot < g.nslots ? __ldg(g.slots + slot) : 0;
+            v[e] = rot_mi(v_entry<P>(g, slot, i, j, d, nc), i + j + 8 - ((sl >> 16) & 1) - ((sl >> 17) & 1));
+        }
+        cut.pair(v[0].re, v[1].re, sr);
+        cut.pair(v[0].im, v[1].im, si);
     }
     // every block group that holds (i, j), at most one per class
     for (int L = 0; L < kNclass; ++L) {
@@ -1156,11 +1475,11 @@ __global__ void __launch_bounds__(256) k_tc_vslice(TcJArgs g) {
         const int gi = pl >> 8, nw = mma_cols(__ldg(&g.groups[gi].y), g.colw);
         const int c0 = (pl & 255) * g.colw + d * g.gw + 2 * nc;
         const int o0 = tile_off(c0, 2 * m2), o1 = tile_off(c0 + 1, 2 * m2);
-        __nv_bfloat16* bs = g.vs + __ldg(g.voff + gi) + (size_t)q * kTcJS * nw * 16;
+        __nv_bfloat16* bs = g.vs + __ldg(g.voff + gi) + (size_t)q * kS * nw * 16;
 #pragma unroll
-        for (int s = 0; s < kTcJS; ++s, bs += nw * 16) {
-            *reinterpret_cast<uint32_t*>(bs + o0) = pack_bf2(sr[0][s], sr[1][s]);
-            *reinterpret_cast<uint32_t*>(bs + o1) = pack_bf2(si[0][s], si[1][s]);
+        for (int s = 0; s < kS; ++s, bs += nw * 16) {
+            *reinterpret_cast<uint32_t*>(bs + o0) = sr[s];
+            *reinterpret_cast<uint32_t*>(bs + o1) = si[s];
         }
     }
 }
@@ -1179,13 +1498,14 @@ struct TcJSmem {
 // 16-byte table reads and four real products each, one 16-byte core-matrix row
 // per slice), lane 0 of warp 16 issues the MMAs, warp 17 brings the factor
 // tables and warp 18 the V_ij stage tiles in with bulk copies; warps 0-15 then
-// form J' from tensor memory (lane quadrant w & 3, (block, density) pairs
-// w / 4 mod 4).  Waits are bounded as in the structure-factor kernel.
+// form J' from tensor memory (lane quadrant w & 3; (block, density) pairs,
+// their columns split further where a group has fewer than four, w / 4 mod 4).  Waits are bounded as in the structure-factor kernel.
+template <class P>
 __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) {
     extern __shared__ __align__(1024) unsigned char tsm[];
-    const int bbytes = kTcJS * g.npad * 32;
+    const int bbytes = P::S * g.npad * 32;
     unsigned char* abuf = tsm;                                                     // [nbuf][S][4096]
-    unsigned char* bbuf = abuf + (size_t)nbuf * kTcJS * kTcJAsliceBytes;             // [nbuf][S][npad x 32]
+    unsigned char* bbuf = abuf + (size_t)nbuf * P::S * kTcJAsliceBytes;             // [nbuf][S][npad x 32]
     float4* tabs = reinterpret_cast<float4*>(bbuf + (size_t)nbuf * bbytes);         // [128][tws]: X, Y
     TcJSmem& sm = *reinterpret_cast<TcJSmem*>(tabs + (size_t)kTcM * g.tws);
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -1233,7 +1553,7 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) 
                 if (nu > 0 && !mbar_wait(&sm.tempty, (uint32_t)((nu - 1) & 1), abort_flag, g.spin)) break;
                 const uint32_t bytes = (uint32_t)(nv * g.tws) * 16u;
                 mbar_arrive_tx(&sm.tfull, bytes);
-                bulk_copy(tabs, g.tab + (size_t)un.w * g.tws, bytes, &sm.tfull);
+                bulk_copy(tabs, reinterpret_cast<const float4*>(g.tab) + (size_t)un.w * g.tws, bytes, &sm.tfull);
             }
             ring_settle(&sm.tfull, 1, nu);
         }
@@ -1247,7 +1567,7 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) 
                 const int4 un = __ldg(g.units + __ldg(ulist + ju));
                 const int q0 = (un.x >> 8) * g.spp, nst = min(g.spp, g.nstage - q0);
                 for (int gi = 0; gi < un.z && ok; ++gi) {
-                    const uint32_t bytes = (uint32_t)(kTcJS * mma_cols(__ldg(&g.groups[un.y + gi].y), g.colw) * 32);
+                    const uint32_t bytes = (uint32_t)(P::S * mma_cols(__ldg(&g.groups[un.y + gi].y), g.colw) * 32);
                     const unsigned char* src = reinterpret_cast<const unsigned char*>(g.vs + __ldg(g.voff + un.y + gi)) +
                                                (size_t)q0 * bytes;
                     for (int q = 0; q < nst; ++q, ++gs, b.next()) {
@@ -1280,7 +1600,7 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) 
                     if (!ok) break;
                     tc_fence_after();
                     if (elect_one()) {
-                        issue_kstep<kTcJS, kTcJAcc>(tmem, sdesc(a0 + b.i * kTcJS * kTcJAsliceBytes), kTcJAsliceBytes >> 4,
+                        issue_kstep<P::S, P::ACC>(tmem, sdesc(a0 + b.i * P::S * kTcJAsliceBytes), kTcJAsliceBytes >> 4,
                                                     sdesc(b0 + b.i * bbytes), nw * 2, nw, idesc, q > 0);
                         tc_commit(&sm.empty[b.i]);
                         if (q + 1 == nst) tc_commit(&sm.accf);
@@ -1300,9 +1620,11 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) 
     } else {
         // operand role: record rec, slots 8 oct .. 8 oct + 7 (two point groups) of its group's stages
         const int grp = warp / kTcGroupWarps, rec = tid & (kTcM - 1), oct = (tid >> 7) & 1;
-        const float4* trec = tabs + (size_t)rec * g.tws;
+        using Comp = typename P::Comp;
+        using Entry = typename P::Entry;
+        const Comp* trec = reinterpret_cast<const Comp*>(tabs + (size_t)rec * g.tws);  // two components per entry
         unsigned char* arow = abuf + tile_off(rec, oct * 8) * 2;
-        const Slicer7 cut(0x1p-5f);  // |A| <= 1 < 2^1
+        const typename P::Cut cut(1);  // |A| <= 1 < 2^1
         // epilogue role
         const int eq = warp & 3, es = warp >> 2, erow = 32 * eq + lane;
         const uint32_t tlane = (uint32_t)(32 * eq) << 16;
@@ -1322,45 +1644,45 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) 
                     full = full || gs >= nbuf;
                     if ((gs & 1) != grp) continue;
                     const int qd = (q0 + q) * 4 + oct * 2;
-                    uint32_t pk[kTcJS][4];
+                    uint32_t pk[P::S][4];
 #pragma unroll
                     for (int v = 0; v < 2; ++v) {
                         const int info = qd + v < nquad ? __ldg(g.quads + qd + v) : 0;
                         const int n0 = (info >> 2) & 255, n1 = (info >> 10) & 255;
                         // the four products of the point group, in slot order; with one index zero its factor is 1
-                        df a[4];
+                        Entry a[4];
                         if (info & 1) {
-                            const float4 x = trec[n0], y = trec[g.offY + n1];
-                            const df x0{x.x, x.y}, x1{x.z, x.w}, y0{y.x, y.y}, y1{y.z, y.w};
-                            a[0] = df_mul_u(x0, y0);
-                            a[1] = df_mul_u(x1, y0);
-                            a[2] = df_mul_u(x0, y1);
-                            a[3] = df_mul_u(x1, y1);
+                            const Comp x0 = trec[2 * n0], x1 = trec[2 * n0 + 1];
+                            const Comp y0 = trec[2 * (g.offY + n1)], y1 = trec[2 * (g.offY + n1) + 1];
+                            a[0] = P::product(x0, y0);
+                            a[1] = P::product(x1, y0);
+                            a[2] = P::product(x0, y1);
+                            a[3] = P::product(x1, y1);
                         } else {
                             const int off = info & 2 ? 0 : g.offY;
-                            const float4 x = trec[off + n0], y = trec[off + n1];
                             const bool ab = info & 2;
-                            a[0] = df{x.x, x.y};
-                            a[1] = ab ? df{x.z, x.w} : df{y.x, y.y};
-                            a[2] = ab ? df{y.x, y.y} : df{x.z, x.w};
-                            a[3] = df{y.z, y.w};
+                            const Entry x0 = P::entry(trec[2 * (off + n0)]), x1 = P::entry(trec[2 * (off + n0) + 1]);
+                            const Entry y0 = P::entry(trec[2 * (off + n1)]), y1 = P::entry(trec[2 * (off + n1) + 1]);
+                            a[0] = x0;
+                            a[1] = ab ? x1 : y0;
+                            a[2] = ab ? y0 : x1;
+                            a[3] = y1;
                         }
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
-                            float o0[kTcJS], o1[kTcJS];
-                            cut(a[2 * h].hi, a[2 * h].lo, o0);
-                            cut(a[2 * h + 1].hi, a[2 * h + 1].lo, o1);
+                            uint32_t o[P::S];
+                            cut.pair(a[2 * h], a[2 * h + 1], o);
 #pragma unroll
-                            for (int s = 0; s < kTcJS; ++s) pk[s][2 * v + h] = pack_bf2(o0[s], o1[s]);
+                            for (int s = 0; s < P::S; ++s) pk[s][2 * v + h] = o[s];
                         }
                     }
                     if (full) {
                         ok = __all_sync(0xffffffffu, mbar_wait(&sm.empty[b.i], b.ph ^ 1u, abort_flag, g.spin));
                         if (!ok) break;
                     }
-                    unsigned char* as = arow + (size_t)b.i * kTcJS * kTcJAsliceBytes;
+                    unsigned char* as = arow + (size_t)b.i * P::S * kTcJAsliceBytes;
 #pragma unroll
-                    for (int s = 0; s < kTcJS; ++s)
+                    for (int s = 0; s < P::S; ++s)
                         *reinterpret_cast<uint4*>(as + (size_t)s * kTcJAsliceBytes) =
                             make_uint4(pk[s][0], pk[s][1], pk[s][2], pk[s][3]);
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -1379,28 +1701,52 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) 
                 tc_fence_after();
                 const int2 gr = __ldg(g.groups + un.y + gi);
                 const uint32_t nw = (uint32_t)mma_cols(gr.y, g.colw);
-                const float4* zrec = g.tabz + (size_t)__ldg(g.kpos + (rvalid ? r : un.w)) * g.ncols;
-                for (int pd = es; pd < gr.y * g.nd; pd += kTcProdWarps / 4) {
-                    const int gb = pd / g.nd, d = pd - gb * g.nd;
+                const float4* zrec =
+                    reinterpret_cast<const float4*>(g.tabz) +
+                    (size_t)__ldg(g.kpos + (rvalid ? r : un.w)) * g.ncols * (P::S == 8 ? 2 : 1);
+                for (int ps = es; ps < gr.y * g.nd * g.nsub; ps += kTcProdWarps / 4) {
+                    const int pd = ps / g.nsub, sub = ps - pd * g.nsub, gb = pd / g.nd, d = pd - gb * g.nd;
                     const int pr = __ldg(g.ipairs + gr.x + gb), i = pr & 7, j = pr >> 3, nk = L - i - j;
-                    df J[5];
+                    typename P::Sum J[5];
 #pragma unroll
-                    for (int kk = 0; kk < 5; ++kk) J[kk] = df{0.f, 0.f};
-                    for (int c4 = 0; c4 < g.gw / 4; ++c4) {
-                        float T[kTcJAcc][4];
-                        float4 zv[2];
+                    for (int kk = 0; kk < 5; ++kk) J[kk] = sum_zero(typename P::Sum());
+                    for (int c4 = sub; c4 < g.gw / 4; c4 += g.nsub) {
+                        float T[P::ACC][4];
+                        typename P::Sum zr[2], zi[2];  // Z: double-float in one float4, triple-float in two
 #pragma unroll
-                        for (int u = 0; u < 2; ++u) zv[u] = __ldg(zrec + min(2 * c4 + u, g.ncols - 1));
+                        for (int u = 0; u < 2; ++u) {
+                            const int nc = min(2 * c4 + u, g.ncols - 1);
+                            if constexpr (P::S == 8) {
+                                const float4 a = __ldg(zrec + 2 * nc), b = __ldg(zrec + 2 * nc + 1);
+                                zr[u] = tf{a.x, a.y, a.z};
+                                zi[u] = tf{b.x, b.y, b.z};
+                            } else {
+                                const float4 a = __ldg(zrec + nc);
+                                zr[u] = df{a.x, a.y};
+                                zi[u] = df{a.z, a.w};
+                            }
+                        }
                         tc_ld_levels4(tmem + tlane + (uint32_t)(gb * g.colw + d * g.gw + 4 * c4), nw, T);
 #pragma unroll
                         for (int u = 0; u < 2; ++u) {
                             const int nc = 2 * c4 + u;
-                            if (nc < g.ncols) {
-                                const cdf v{level_sum(T[0][2 * u], T[1][2 * u], T[2][2 * u], T[3][2 * u], T[4][2 * u]),
-                                            level_sum(T[0][2 * u + 1], T[1][2 * u + 1], T[2][2 * u + 1],
-                                                      T[3][2 * u + 1], T[4][2 * u + 1])};
-                                const cdf zu = cdf_mul_u(cdf{{zv[u].x, zv[u].y}, {zv[u].z, zv[u].w}}, v);
-                                float pw = 1.f;  // n_c^k, exact; Re (-i)^k zu is +-Re (k even) or +-Im (k odd)
+                            if (nc >= g.ncols) continue;
+                            const auto vr = level_sum(T, 2 * u), vi = level_sum(T, 2 * u + 1);
+                            // n_c^k exact; Re (-i)^k zu is +-Re (k even) or +-Im (k odd)
+                            if constexpr (P::S == 8) {
+                                const tf re = tf_add(tf_mul(zr[u], vr), tf_neg(tf_mul(zi[u], vi)));
+                                J[0] = tf_add(J[0], re);
+                                if (nk > 0) {
+                                    const tf im = tf_add(tf_mul(zr[u], vi), tf_mul(zi[u], vr));
+                                    const float x = (float)nc;
+                                    J[1] = tf_add(J[1], tf_mulf(im, x));
+                                    if (nk > 1) J[2] = tf_add(J[2], tf_mulf(re, x * x));
+                                    if (nk > 2) J[3] = tf_add(J[3], tf_mulf(im, x * x * x));
+                                    if (nk > 3) J[4] = tf_add(J[4], tf_mulf(re, x * x * x * x));
+                                }
+                            } else {
+                                const cdf zu = cdf_mul_u(cdf{zr[u], zi[u]}, cdf{vr, vi});
+                                float pw = 1.f;
 #pragma unroll
                                 for (int kk = 0; kk < 5; ++kk) {
                                     if (kk <= nk) J[kk] = df_add(J[kk], df_mulf_u(kk & 1 ? zu.im : zu.re, pw));
@@ -1410,12 +1756,12 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) 
                         }
                     }
                     if (rvalid) {
-                        double* jp = g.Jp + ((long long)(g.d0 + d) * g.nparts + part) * g.jp_total + g.term_base[L] +
+                        double* jp = g.Jp + ((long long)(g.d0 + d) * g.nparts + part * g.nsub + sub) * g.jp_total + g.term_base[L] +
                                      (r - g.cls_start[L]);
 #pragma unroll
                         for (int kk = 0; kk < 5; ++kk)
                             if (kk <= nk) {
-                                const double v = (double)J[kk].hi + (double)J[kk].lo;
+                                const double v = sum_double(sum_mulf(J[kk], P::row_scale(1)));  // exact power of two
                                 jp[(long long)term_of(g.ax, g.bx, i, j, kk) * cnt] = kk == 2 || kk == 3 ? -v : v;
                             }
                     }
@@ -1435,8 +1781,8 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) 
     }
 }
 
-size_t tc_j_smem_bytes(int npad, int tws, int nbuf) {
-    const size_t need = (size_t)nbuf * kTcJS * (kTcJAsliceBytes + (size_t)npad * 32) + (size_t)kTcM * tws * 16 +
+size_t tc_j_smem_bytes(int slices, int npad, int tws, int nbuf) {
+    const size_t need = (size_t)nbuf * slices * (kTcJAsliceBytes + (size_t)npad * 32) + (size_t)kTcM * tws * 16 +
                         sizeof(TcJSmem) + 64;
     return std::max<size_t>(need, 120 * 1024);
 }
@@ -1470,7 +1816,21 @@ std::vector<int> deal(const std::vector<double>& cost, int nbin) {
 
 }  // namespace
 
-int tc_supported(const ftcj_plan* P) { return P->ortho ? 1 : 0; }
+void release_tc(ftcj_plan* P) {
+    void** ptrs[] = {(void**)&P->d_tc_slots, (void**)&P->d_tc_quads, (void**)&P->d_tc_map, (void**)&P->d_tc_wpairs,
+                     &P->d_tc_winfo, (void**)&P->d_tc_wcnt, (void**)&P->d_tc_boff, (void**)&P->d_tc_sched, &P->d_tc_b,
+                     &P->d_tc_tab, &P->d_tc_tabk, &P->d_tc_tabz, &P->d_tc_tabz3, (void**)&P->d_tc_cl, (void**)&P->d_tc_kpos,
+                     (void**)&P->d_tc_korder, (void**)&P->d_tc_err, (void**)&P->d_tc_pos, (void**)&P->d_tc_clw,
+                     &P->d_tc_jitems, &P->d_tc_jgroups, (void**)&P->d_tc_jpairs, (void**)&P->d_tc_jsched, &P->d_tc_vs,
+                     (void**)&P->d_tc_voff, (void**)&P->d_tc_vplace, (void**)&P->d_tc_ev};
+    for (void** p : ptrs) {
+        if (*p) cudaFree(*p);
+        *p = nullptr;
+    }
+    P->tc = P->tc_j = false;
+    P->tc_dp_total = 0;
+    P->tc_passes.clear();
+}
 
 // clock-cycle budget of one wait between the kernels' roles
 long long tc_spin(const ftcj_plan* P) {
@@ -1484,16 +1844,19 @@ int setup_tc_j(ftcj_plan* P);
 // sorted by width), their deal to CTA groups and the B tiles.
 int setup_tc(ftcj_plan* P) {
     if (!P->ortho) return fail(FTCJ_EUNSUPPORTED, "the tensor-core contraction needs an orthorhombic cell");
-    if (P->precision != FTCJ_PREC_SPLIT)
-        return fail(FTCJ_EUNSUPPORTED, "the tensor-core contraction is part of the split-precision form");
+    const bool f64 = P->precision == FTCJ_PREC_FP64;
+    const int nmax = f64 ? Prec64::kNmax : PrecRho::kNmax, slices = f64 ? Prec64::S : PrecRho::S;
+    const int nprod = slices * (slices + 1) / 2;
     if (P->d_rec_gcut) return fail(FTCJ_EUNSUPPORTED, "the tensor-core contraction walks the whole sphere");
     if (P->npairs >= (1 << 24)) return fail(FTCJ_EUNSUPPORTED, "more than 2^24 pair records");
     const int64_t ngh = P->ng_half;
     int64_t recs_by_class[kNclass];
     for (int L = 0; L < kNclass; ++L) recs_by_class[L] = P->class_start[L + 1] - P->class_start[L];
-    // the column axis: SM cycles ~ row tiles x record passes x (the 21 slice products of a k-step, reading 4 KB of A
-    // about three times in four and 32 B per column of B from shared memory at 128 B per cycle, and the forming of
-    // A), per density group
+    // The column axis: SM cycles of both passes, per density group.  Structure factors: per 16 records and row tile
+    // the slice products (A read about three times in four, 32 B per column of B, at 128 B per cycle) and the forming
+    // of A, and per entry of B its forming; back-contraction: the same per 16 slots and record tile, and per (record,
+    // block, n_c) the epilogue.  The per-entry costs are measured ones.
+    const double kB = f64 ? 5.0 : 3.7, kE = f64 ? 5.0 : 2.9;
     struct AxisPlan {
         std::set<std::pair<int, int>> pts;
         std::vector<int> slots, quads;
@@ -1520,20 +1883,24 @@ int setup_tc(ftcj_plan* P) {
         ap.rows = rs.size();
         ap.ncols = ncmax + 1;
         for (ap.nd = P->max_dens; ap.nd >= 1; --ap.nd) {
-            tc_columns(ap.nd, ap.ncols, &ap.colw, &ap.G, &ap.npad);
+            tc_columns(nmax, ap.nd, ap.ncols, &ap.colw, &ap.G, &ap.npad);
             if (ap.G > 0) break;
         }
         if (ap.nd < 1 || ap.G < 1) continue;
         tc_slots(ap.pts, ap.slots, ap.quads);
         const double mt = (double)((ap.slots.size() + kTcM - 1) / kTcM);
         const double launches = (double)((P->max_dens + ap.nd - 1) / ap.nd);
-        double work = 0.0;
+        double cost = 0.0;
         for (int L = 0; L < kNclass; ++L) {
             const int nb = (L + 1) * (L + 2) / 2;
-            for (int g0 = 0; g0 < nb; g0 += ap.G)
-                work += (double)recs_by_class[L] * (500.0 + 21.0 * (24.0 + 0.25 * mma_cols(std::min(ap.G, nb - g0), ap.colw)));
+            const double rows16 = (double)recs_by_class[L] / 16.0, nst = (double)ap.slots.size() / 16.0;
+            for (int g0 = 0; g0 < nb; g0 += ap.G) {
+                const double stage = 500.0 + nprod * (24.0 + 0.25 * mma_cols(std::min(ap.G, nb - g0), ap.colw));
+                cost += rows16 * stage * (mt + nst / 8.0);  // a record tile of the back-contraction is 128 records
+            }
+            cost += (double)recs_by_class[L] * nb * ap.nd * ap.ncols * (kB + kE);
         }
-        const double cost = launches * mt * work;
+        cost *= launches;
         if (cost < best_cost) {
             best_cost = cost;
             best_c = c;
@@ -1573,10 +1940,10 @@ int setup_tc(ftcj_plan* P) {
     const int tws = (P->tc_nna + P->tc_nnb) | 1;
     P->tc_tws = tws;
     const size_t nrec = (size_t)std::max<int64_t>(P->npairs, 1);
-    FTCJ_CUDA(cudaMalloc(&P->d_tc_err, sizeof(int)));
+    int rc;
+    if ((rc = tc_alloc(P, (void**)&P->d_tc_err, sizeof(int)))) return rc;
     FTCJ_CUDA(cudaMemset(P->d_tc_err, 0, sizeof(int)));
-    FTCJ_CUDA(cudaMalloc(&P->d_tc_cl, sizeof(float) * nrec));
-    P->device_bytes += sizeof(float) * nrec;
+    if ((rc = tc_alloc(P, (void**)&P->d_tc_cl, sizeof(float) * nrec))) return rc;
     std::vector<float> clh(nrec, 0.f);
     if (P->npairs > 0) {
         k_tc_width<<<(unsigned)((P->npairs + 255) / 256), 256>>>(P->d_walk, P->npairs, P->d_tc_cl);
@@ -1592,7 +1959,7 @@ int setup_tc(ftcj_plan* P) {
     }
     // K order: the records of a class sorted by width c = 1/4p (records of similar width have entries of similar size)
     std::vector<std::vector<int>> order(kNclass);
-    std::vector<int> pos(nrec, 0), kpos(nrec, 0);
+    std::vector<int> pos(nrec, 0), kpos(nrec, 0), korder(nrec, 0);
     std::vector<float> clk(nrec, 0.f);
     for (int L = 0; L < kNclass; ++L) {
         std::vector<int>& recs = order[L];
@@ -1602,6 +1969,7 @@ int setup_tc(ftcj_plan* P) {
             pos[recs[k]] = (int)k;
             kpos[recs[k]] = (int)(P->class_start[L] + (int64_t)k);
             clk[P->class_start[L] + k] = clh[recs[k]];
+            korder[P->class_start[L] + k] = (int)(recs[k] - P->class_start[L]);
         }
     }
     // Records per window: a window costs one drain of tensor memory (~7% of a 1024-record window of 96 columns),
@@ -1615,7 +1983,7 @@ int setup_tc(ftcj_plan* P) {
         }
         return n;
     };
-    P->tc_wlen = kTcWinMax;
+    P->tc_wlen = f64 ? Prec64::kWin : PrecRho::kWin;
     while (P->tc_wlen > 128 && windows(P->tc_wlen) < 4 * (int64_t)groups_max) P->tc_wlen /= 2;
     const int wlen = P->tc_wlen;
     // windows: for each class L, its (i, j) blocks in groups of G, the class's records wlen at a time
@@ -1640,7 +2008,7 @@ int setup_tc(ftcj_plan* P) {
                 const int cnt = (int)std::min<size_t>(wlen, recs.size() - r0);
                 const double nst = (double)((cnt + kTcStageK - 1) / kTcStageK);
                 wins.push_back({make_int4(L, nb, first, (int)r0), cnt,
-                                nst * (500.0 + 21.0 * (24.0 + 0.25 * mma_cols(nb, P->tc_colw))) + 70.0 * nb * P->tc_colw});
+                                nst * (500.0 + nprod * (24.0 + 0.25 * mma_cols(nb, P->tc_colw))) + 70.0 * nb * P->tc_colw});
             }
         }
     }
@@ -1661,7 +2029,7 @@ int setup_tc(ftcj_plan* P) {
         int w1 = w0;
         while (w1 < nwin) {
             const Win& w = wins[w1];
-            const long long n = (long long)((w.cnt + kTcStageK - 1) / kTcStageK) * kTcS * mma_cols(w.info.y, P->tc_colw) * 2;
+            const long long n = (long long)((w.cnt + kTcStageK - 1) / kTcStageK) * slices * mma_cols(w.info.y, P->tc_colw) * 2;
             if (w1 > w0 && (off + n) * 16 > kTcBWorkMax) break;
             winfo[w1] = w.info;
             wcnt[w1] = w.cnt;
@@ -1681,13 +2049,13 @@ int setup_tc(ftcj_plan* P) {
         w0 = w1;
     }
     P->tc_out_rows = std::max(1, P->tc_out_rows);
-    // MMA work of one pass: per window and row tile, its stages x 21 slice products of M = 128 rows,
+    // MMA work of one pass: per window and row tile, its stages x the slice products of M = 128 rows,
     // N = the window's columns, K = 16, for every density group
     P->tc_mma_flops = 0;
     for (int d0 = 0; d0 < P->max_dens; d0 += P->tc_nd) {
         const int colw = round_up(2 * std::min(P->tc_nd, P->max_dens - d0) * P->tc_ncols, 8);
         for (const Win& w : wins)
-            P->tc_mma_flops += (long long)P->tc_mtiles * ((w.cnt + kTcStageK - 1) / kTcStageK) * 21 * 2LL * kTcM *
+            P->tc_mma_flops += (long long)P->tc_mtiles * ((w.cnt + kTcStageK - 1) / kTcStageK) * nprod * 2LL * kTcM *
                                mma_cols(w.info.y, colw) * 16;
     }
     // stage buffers and table slots: four buffers where at least three slots fit beside them, else fewer
@@ -1697,33 +2065,34 @@ int setup_tc(ftcj_plan* P) {
     P->tc_tslots = 0;
     for (int nbuf = kTcNbufMax; nbuf >= 2 && !P->tc_tslots; --nbuf)
         for (int nts = kTcTabSlotsMax; nts >= (nbuf > 2 ? 3 : 1) && !P->tc_tslots; --nts)
-            if (tc_smem_bytes(P->tc_npad, tws, nbuf, nts) <= (size_t)optin) {
+            if (tc_smem_bytes(slices, P->tc_npad, tws, nbuf, nts) <= (size_t)optin) {
                 P->tc_nbuf = nbuf;
                 P->tc_tslots = nts;
             }
     if (!P->tc_tslots)
         return fail(FTCJ_EUNSUPPORTED, "the G sphere is too long for the tensor-core kernel's shared-memory tables");
-    int rc;
     if ((rc = tc_upload(P, &P->d_tc_slots, slots))) return rc;
     if ((rc = tc_upload(P, &P->d_tc_quads, best.quads))) return rc;
     if ((rc = tc_upload(P, &P->d_tc_map, map))) return rc;
     if ((rc = tc_upload(P, &P->d_tc_wpairs, wpairs))) return rc;
     if ((rc = tc_upload(P, &P->d_tc_pos, pos))) return rc;
     if ((rc = tc_upload(P, &P->d_tc_kpos, kpos))) return rc;
+    if (f64 && (rc = tc_upload(P, &P->d_tc_korder, korder))) return rc;
     FTCJ_CUDA(cudaMemcpy(P->d_tc_cl, clk.data(), sizeof(float) * nrec, cudaMemcpyHostToDevice));
-    FTCJ_CUDA(cudaMalloc(&P->d_tc_tab, sizeof(float4) * nrec * tws));
-    FTCJ_CUDA(cudaMalloc(&P->d_tc_tabk, sizeof(float4) * nrec * tws));
-    FTCJ_CUDA(cudaMalloc(&P->d_tc_tabz, sizeof(float4) * nrec * P->tc_ncols));
-    P->device_bytes += sizeof(float4) * nrec * (2 * (size_t)tws + P->tc_ncols);
+    if ((rc = tc_alloc(P, &P->d_tc_tab, sizeof(float4) * nrec * tws))) return rc;
+    if ((rc = tc_alloc(P, &P->d_tc_tabk, sizeof(float4) * nrec * tws))) return rc;
+    if ((rc = tc_alloc(P, &P->d_tc_tabz, sizeof(float4) * nrec * P->tc_ncols))) return rc;
+    if (f64 && (rc = tc_alloc(P, &P->d_tc_tabz3, 2 * sizeof(float4) * nrec * P->tc_ncols))) return rc;
     // the odd stride's spare entry is copied along but never read
     FTCJ_CUDA(cudaMemset(P->d_tc_tab, 0, sizeof(float4) * nrec * tws));
     FTCJ_CUDA(cudaMemset(P->d_tc_tabk, 0, sizeof(float4) * nrec * tws));
     if (P->npairs > 0) {
         const long long n = P->npairs * (long long)(P->tc_nna + P->tc_nnb + P->tc_ncols);
-        k_tc_tables<<<(unsigned)((n + 255) / 256), 256>>>(
+        auto* tables = f64 ? k_tc_tables<true> : k_tc_tables<false>;
+        tables<<<(unsigned)((n + 255) / 256), 256>>>(
             P->d_walk, P->npairs, P->d_tc_kpos, a, b, c, P->tc_nna, P->tc_nnb, P->tc_ncols, tws, P->M[4 * a],
             P->M[4 * b], P->M[4 * c], reinterpret_cast<float4*>(P->d_tc_tab), reinterpret_cast<float4*>(P->d_tc_tabk),
-            reinterpret_cast<float4*>(P->d_tc_tabz));
+            reinterpret_cast<float4*>(P->d_tc_tabz), reinterpret_cast<float4*>(P->d_tc_tabz3));
         FTCJ_CUDA(cudaGetLastError());
     }
     if ((rc = tc_upload(P, &P->d_tc_wcnt, wcnt))) return rc;
@@ -1733,18 +2102,13 @@ int setup_tc(ftcj_plan* P) {
     if ((rc = tc_upload(P, &winfo_dev, winfo))) return rc;
     P->d_tc_winfo = winfo_dev;
     if ((rc = tc_upload(P, &P->d_tc_clw, std::vector<float>((size_t)std::max(1, nwin), 0.f)))) return rc;
-    if (cudaMalloc(&P->d_tc_b, (size_t)bmax * 16) != cudaSuccess) {
-        cudaGetLastError();
-        P->d_tc_b = nullptr;
-        return fail(FTCJ_ENOMEM, "cudaMalloc of the tensor-core operand tiles failed");
-    }
-    P->device_bytes += (size_t)bmax * 16;
+    if ((rc = tc_alloc(P, &P->d_tc_b, (size_t)bmax * 16))) return rc;
     // columns between a window's blocks and the MMA's multiple of 16 are never written nor read back: finite once
     FTCJ_CUDA(cudaMemset(P->d_tc_b, 0, (size_t)bmax * 16));
     // calls with fewer densities run the instantiation of their own block width
     for (int nd = 1; nd <= P->tc_nd; ++nd)
-        if ((rc = allow_dynamic_smem(tc_rho_kernel(round_up(2 * nd * P->tc_ncols, 8)),
-                                     tc_smem_bytes(P->tc_npad, tws, P->tc_nbuf, P->tc_tslots))))
+        if ((rc = allow_dynamic_smem(tc_rho_kernel(f64, round_up(2 * nd * P->tc_ncols, 8)),
+                                     tc_smem_bytes(slices, P->tc_npad, tws, P->tc_nbuf, P->tc_tslots))))
             return rc;
     return setup_tc_j(P);
 }
@@ -1761,15 +2125,17 @@ int launch_tc_rho(ftcj_plan* P, int ndens, cudaStream_t s) {
     g.wcnt = P->d_tc_wcnt;
     g.boff = P->d_tc_boff;
     g.wpairs = P->d_tc_wpairs;
-    g.tabk = reinterpret_cast<const float4*>(P->d_tc_tabk);
-    g.tabz = reinterpret_cast<const float4*>(P->d_tc_tabz);
+    const bool f64 = P->precision == FTCJ_PREC_FP64;
+    g.tabk = P->d_tc_tabk;
+    g.tabz = P->d_tc_tabz;
+    g.korder = P->d_tc_korder;
     g.clk = P->d_tc_cl;
     for (int cc = 0; cc < kNclass; ++cc) g.kbase[cc] = P->class_start[cc];
-    g.Dp = reinterpret_cast<const float2*>(P->d_Dp);
-    g.dp_total = P->tc_dp_total;
+    g.Dp = P->d_Dp;
+    g.dp_total = f64 ? P->total_terms : P->tc_dp_total;
     for (int cc = 0; cc < kNclass; ++cc) {
-        g.dp_base[cc] = P->tc_dp_base[cc];
-        g.dp_stride[cc] = P->tc_dp_stride[cc];
+        g.dp_base[cc] = f64 ? P->term_base[cc] : P->tc_dp_base[cc];
+        g.dp_stride[cc] = f64 ? P->class_start[cc + 1] - P->class_start[cc] : P->tc_dp_stride[cc];
     }
     g.bs = reinterpret_cast<uint4*>(P->d_tc_b);
     g.clw = P->d_tc_clw;
@@ -1790,7 +2156,7 @@ int launch_tc_rho(ftcj_plan* P, int ndens, cudaStream_t s) {
     g.ncols = P->tc_ncols;
     g.nslots = P->tc_nslots;
     g.spin = tc_spin(P);
-    const size_t smem = tc_smem_bytes(P->tc_npad, g.tws, P->tc_nbuf, P->tc_tslots);
+    const size_t smem = tc_smem_bytes(f64 ? Prec64::S : PrecRho::S, P->tc_npad, g.tws, P->tc_nbuf, P->tc_tslots);
     for (int d0 = 0; d0 < ndens; d0 += P->tc_nd) {
         g.d0 = d0;
         g.nd = std::min(P->tc_nd, ndens - d0);
@@ -1801,12 +2167,13 @@ int launch_tc_rho(ftcj_plan* P, int ndens, cudaStream_t s) {
             g.w0 = ps.w0;
             g.out_row0 = ps.out_row0;
             g.sched = P->d_tc_sched + ps.sched;
-            k_tc_rho_b<<<(unsigned)ps.nwin, kTcBThreads, 0, s>>>(g);
+            if (f64) k_tc_rho_b<Prec64><<<(unsigned)ps.nwin, kTcBThreads, 0, s>>>(g);
+            else k_tc_rho_b<PrecRho><<<(unsigned)ps.nwin, kTcBThreads, 0, s>>>(g);
             FTCJ_CUDA(cudaGetLastError());
             const dim3 grid((unsigned)ps.ngroups, (unsigned)P->tc_mtiles);
             int nbuf = P->tc_nbuf, nts = P->tc_tslots;
             void* args[] = {&g, &nbuf, &nts};
-            FTCJ_CUDA(cudaLaunchKernel(tc_rho_kernel(g.colw), grid, dim3(kTcThreadsAll), args, smem, s));
+            FTCJ_CUDA(cudaLaunchKernel(tc_rho_kernel(f64, g.colw), grid, dim3(kTcThreadsAll), args, smem, s));
         }
     }
     return FTCJ_OK;
@@ -1823,6 +2190,9 @@ int tc_rho_launches(const ftcj_plan* P, int nd) {
 // factor tables exceed shared memory.
 int setup_tc_j(ftcj_plan* P) {
     P->tc_j = false;
+    const bool f64 = P->precision == FTCJ_PREC_FP64;
+    const int nmax = f64 ? Prec64::kNmax : PrecJ::kNmax, slices = f64 ? Prec64::S : PrecJ::S;
+    const int nprod = slices * (slices + 1) / 2, part_stages = (f64 ? Prec64::kWin : PrecJ::kWin) / kTcJStageM;
     const int gw = round_up(2 * P->tc_ncols, 8);
     int64_t tiles[kNclass];
     for (int L = 0; L < kNclass; ++L) tiles[L] = (P->class_start[L + 1] - P->class_start[L] + kTcM - 1) / kTcM;
@@ -1831,8 +2201,8 @@ int setup_tc_j(ftcj_plan* P) {
     double cost_best = 1e300;
     for (int nd = 1; nd <= P->max_dens; ++nd) {
         const int colw = nd * gw;
-        if (colw > kTcJNmax) break;
-        const int G = std::min(kTcGmax, kTcJNmax / colw);
+        if (colw > nmax) break;
+        const int G = std::min(kTcGmax, nmax / colw);
         double items = 0.0;
         for (int L = 0; L < kNclass; ++L) {
             const int nb = (L + 1) * (L + 2) / 2;
@@ -1853,12 +2223,12 @@ int setup_tc_j(ftcj_plan* P) {
     // as many stage buffers as fit beside the tables
     const int tws = P->tc_tws;
     int nbuf = kTcNbufMax;
-    while (nbuf > 2 && tc_j_smem_bytes(npad, tws, nbuf) > (size_t)optin) --nbuf;
-    if (tc_j_smem_bytes(npad, tws, nbuf) > (size_t)optin) return FTCJ_OK;
+    while (nbuf > 2 && tc_j_smem_bytes(slices, npad, tws, nbuf) > (size_t)optin) --nbuf;
+    if (tc_j_smem_bytes(slices, npad, tws, nbuf) > (size_t)optin) return FTCJ_OK;
     P->tc_jnbuf = nbuf;
-    // slot parts of at most 64 stages, as even as the stage count allows
+    // slot parts of one exact accumulation each (1024 slots, 512 in the FP64 form), as even as the stage count allows
     const int nstage = (P->tc_nslots + kTcJStageM - 1) / kTcJStageM;
-    const int nsplit = std::max(1, (nstage + kTcJPartStages - 1) / kTcJPartStages);
+    const int nsplit = std::max(1, (nstage + part_stages - 1) / part_stages);
     const int spp = std::max(1, (nstage + nsplit - 1) / nsplit);
     const int nparts = std::max(1, (nstage + spp - 1) / spp);  // every part holds at least one stage
     std::vector<int2> groups;
@@ -1885,7 +2255,7 @@ int setup_tc_j(ftcj_plan* P) {
                 vplace[(size_t)pair_index(blocks[g0 + k] & 7, blocks[g0 + k] >> 3) * kNclass + L] =
                     (int)groups.size() << 8 | k;
             voff.push_back(nvs);
-            nvs += (long long)nstage * kTcJS * mma_cols(nb, nd_best * gw) * 16;
+            nvs += (long long)nstage * slices * mma_cols(nb, nd_best * gw) * 16;
             groups.push_back(make_int2((int)ipairs.size(), nb));
             ipairs.insert(ipairs.end(), blocks.begin() + g0, blocks.begin() + g0 + nb);
         }
@@ -1898,9 +2268,9 @@ int setup_tc_j(ftcj_plan* P) {
                     double cc = 2000.0;
                     for (int k = 0; k < n; ++k) {
                         const int nb = groups[first + g0 + k].y;
-                        cc += nst * (28.0 * (25.0 + 0.25 * mma_cols(nb, nd_best * gw)) + 500.0) + 110.0 * nb * nd_best * gw;
+                        cc += nst * (nprod * (25.0 + 0.25 * mma_cols(nb, nd_best * gw)) + 500.0) + 110.0 * nb * nd_best * gw;
                         for (int d0 = 0; d0 < P->max_dens; d0 += nd_best)
-                            P->tc_j_mma_flops += (long long)nst * kTcJProducts * 2LL * kTcM *
+                            P->tc_j_mma_flops += (long long)nst * nprod * 2LL * kTcM *
                                                  mma_cols(nb, std::min(nd_best, P->max_dens - d0) * gw) * 16;
                     }
                     units.push_back(make_int4(L | (h << 8), first + g0, n, (int)(P->class_start[L] + t * kTcM)));
@@ -1913,7 +2283,8 @@ int setup_tc_j(ftcj_plan* P) {
     P->tc_jG = G_best;
     P->tc_jnpad = npad;
     P->tc_jnstage = nstage;
-    P->tc_jparts = nparts;
+    P->tc_jsub = std::max(1, 4 / (G_best * nd_best) == 3 ? 2 : 4 / (G_best * nd_best));
+    P->tc_jparts = nparts * P->tc_jsub;
     P->tc_jspp = spp;
     P->tc_jgrid = std::max(1, std::min(P->num_sms, (int)units.size()));
     const std::vector<int> sched = deal(cost, P->tc_jgrid);
@@ -1929,13 +2300,11 @@ int setup_tc_j(ftcj_plan* P) {
     if ((rc = tc_upload(P, &P->d_tc_voff, voff))) return rc;
     if ((rc = tc_upload(P, &P->d_tc_vplace, vplace))) return rc;
     nvs = std::max(nvs, 1LL);
-    FTCJ_CUDA(cudaMalloc(&P->d_tc_vs, sizeof(__nv_bfloat16) * (size_t)nvs));
-    P->device_bytes += sizeof(__nv_bfloat16) * (size_t)nvs;
+    if ((rc = tc_alloc(P, &P->d_tc_vs, sizeof(__nv_bfloat16) * (size_t)nvs))) return rc;
     FTCJ_CUDA(cudaMemset(P->d_tc_vs, 0, sizeof(__nv_bfloat16) * (size_t)nvs));
     const size_t nev = (size_t)kTcPairsAll * nd_best * P->tc_ncols;
-    FTCJ_CUDA(cudaMalloc(&P->d_tc_ev, sizeof(int) * nev));
-    P->device_bytes += sizeof(int) * nev;
-    if ((rc = allow_dynamic_smem((const void*)k_tc_j, tc_j_smem_bytes(npad, tws, nbuf)))) return rc;
+    if ((rc = tc_alloc(P, (void**)&P->d_tc_ev, sizeof(int) * nev))) return rc;
+    if ((rc = allow_dynamic_smem(f64 ? (const void*)k_tc_j<Prec64> : (const void*)k_tc_j<PrecJ>, tc_j_smem_bytes(slices, npad, tws, nbuf)))) return rc;
     P->tc_j = true;
     return FTCJ_OK;
 }
@@ -1945,6 +2314,7 @@ int launch_tc_j(ftcj_plan* P, int ndens, const double* W, cudaStream_t s) {
         FTCJ_CUDA(cudaMemsetAsync(P->d_Jp, 0, sizeof(double) * (size_t)ndens * P->tc_jparts * P->total_terms, s));
         return FTCJ_OK;
     }
+    const bool f64 = P->precision == FTCJ_PREC_FP64;
     TcJArgs g;
     g.slots = P->d_tc_slots;
     g.quads = P->d_tc_quads;
@@ -1956,8 +2326,8 @@ int launch_tc_j(ftcj_plan* P, int ndens, const double* W, cudaStream_t s) {
     g.ipairs = P->d_tc_jpairs;
     g.voff = P->d_tc_voff;
     g.vplace = P->d_tc_vplace;
-    g.tab = reinterpret_cast<const float4*>(P->d_tc_tab);
-    g.tabz = reinterpret_cast<const float4*>(P->d_tc_tabz);
+    g.tab = P->d_tc_tab;
+    g.tabz = f64 ? P->d_tc_tabz3 : P->d_tc_tabz;
     g.kpos = P->d_tc_kpos;
     g.vs = reinterpret_cast<__nv_bfloat16*>(P->d_tc_vs);
     g.ev = P->d_tc_ev;
@@ -1979,21 +2349,27 @@ int launch_tc_j(ftcj_plan* P, int ndens, const double* W, cudaStream_t s) {
     g.nslots = P->tc_nslots;
     g.nstage = P->tc_jnstage;
     g.nparts = P->tc_jparts;
+    g.nsub = P->tc_jsub;
     g.spin = tc_spin(P);
     g.spp = P->tc_jspp;
-    const size_t smem = tc_j_smem_bytes(P->tc_jnpad, P->tc_tws, P->tc_jnbuf);
+    const size_t smem = tc_j_smem_bytes(f64 ? Prec64::S : PrecJ::S, P->tc_jnpad, P->tc_tws, P->tc_jnbuf);
     for (int d0 = 0; d0 < ndens; d0 += P->tc_jnd) {
         g.d0 = d0;
         g.nd = std::min(P->tc_jnd, ndens - d0);
         // the plan's block count is kept; a smaller last density group only narrows each block
         g.colw = g.nd * g.gw;
         g.npad = mma_cols(P->tc_jG, g.colw);
-        k_tc_vbound<<<(unsigned)(kTcPairsAll * g.nd * g.ncols), 256, 0, s>>>(g);
+        const unsigned nbound = (unsigned)(kTcPairsAll * g.nd * g.ncols);
+        if (f64) k_tc_vbound<Prec64><<<nbound, 256, 0, s>>>(g);
+        else k_tc_vbound<PrecJ><<<nbound, 256, 0, s>>>(g);
         FTCJ_CUDA(cudaGetLastError());
         const long long nv = (long long)kTcPairsAll * g.nstage * (kTcJStageM / 2) * g.nd * g.ncols;
-        k_tc_vslice<<<(unsigned)((nv + 255) / 256), 256, 0, s>>>(g);
+        const unsigned nslice = (unsigned)((nv + 255) / 256);
+        if (f64) k_tc_vslice<Prec64><<<nslice, 256, 0, s>>>(g);
+        else k_tc_vslice<PrecJ><<<nslice, 256, 0, s>>>(g);
         FTCJ_CUDA(cudaGetLastError());
-        k_tc_j<<<(unsigned)P->tc_jgrid, kTcThreadsAll, smem, s>>>(g, P->tc_jnbuf);
+        if (f64) k_tc_j<Prec64><<<(unsigned)P->tc_jgrid, kTcThreadsAll, smem, s>>>(g, P->tc_jnbuf);
+        else k_tc_j<PrecJ><<<(unsigned)P->tc_jgrid, kTcThreadsAll, smem, s>>>(g, P->tc_jnbuf);
         FTCJ_CUDA(cudaGetLastError());
     }
     return FTCJ_OK;
