@@ -220,6 +220,24 @@ int default_split_chunk(ftcj_plan* P) {
     return build_walk(P);
 }
 
+// Shorter walk chunks for plans of few tiles: a block walks its chunk's points
+// one after another, so a plan with fewer tiles than the GPU has room for is
+// bound by that walk's latency while SMs stand idle.  Without a chunk of the
+// caller's the sphere is cut into as many chunks as give each SM about four
+// blocks, at least 48 points each (a chunk start costs about 15 points: walk
+// state, Hermite terms, partial sums) and never shorter than a line.
+int balance_chunks(ftcj_plan* P) {
+    const int64_t tiles = (int64_t)P->tiles.size(), want = 4 * (int64_t)P->num_sms;
+    if (tiles == 0 || tiles * (int64_t)P->chunks.size() >= want) return FTCJ_OK;
+    const int64_t nch = (want + tiles - 1) / tiles;
+    int longest = 1;
+    for (const WLine& l : P->lines) longest = std::max(longest, l.hi - l.lo + 1);
+    const int chunk = (int)std::max<int64_t>({(P->ng_half + nch - 1) / nch, 48, longest});
+    if (chunk >= P->max_chunk_pts) return FTCJ_OK;
+    P->chunk_max = chunk;
+    return build_walk(P);
+}
+
 template <class T>
 int dalloc(ftcj_plan* P, T** ptr, size_t count) {
     if (count == 0) count = 1;
@@ -491,8 +509,6 @@ int create(const ftcj_cell* cell, const ftcj_basis* basis, const int kmesh[3], c
 
     if ((rc = upload(P, &P->d_groups, P->groups))) return rc;
     if ((rc = upload(P, &P->d_members, P->members))) return rc;
-    if ((rc = upload(P, &P->d_lines, P->lines))) return rc;
-    if ((rc = upload(P, &P->d_chunks, P->chunks))) return rc;
     if ((rc = upload(P, &P->d_gvec, P->gvec))) return rc;
     if ((rc = dalloc(P, &P->d_vg, (size_t)P->ng_half))) return rc;
     if ((rc = dalloc(P, &P->d_tw, (size_t)3 * 16 * 16 * 2))) return rc;
@@ -516,6 +532,9 @@ int create(const ftcj_cell* cell, const ftcj_basis* basis, const int kmesh[3], c
             P->tiles.push_back({c, (int)f, cnt, INFINITY});
         }
     if ((rc = upload(P, &P->d_tiles, P->tiles))) return rc;
+    if (prm->chunk_points <= 0 && (rc = balance_chunks(P))) return rc;
+    if ((rc = upload(P, &P->d_lines, P->lines))) return rc;
+    if ((rc = upload(P, &P->d_chunks, P->chunks))) return rc;
     if ((rc = upload_walk_tables(P))) return rc;
     if ((rc = upload_hermite_tables(P))) return rc;
     if ((rc = build_maps(P))) return rc;
@@ -529,6 +548,10 @@ int create(const ftcj_cell* cell, const ftcj_basis* basis, const int kmesh[3], c
     }
     int nch = std::max<int>(1, (int)P->chunks.size());
     P->npb = std::max(1, std::min<int>((int)std::max<size_t>(1, P->tiles.size()), P->num_sms * bps / nch));
+    // several short chunks of few tiles: one block per (tile, chunk), dealt by the hardware, comes out more even than
+    // one wave of blocks of which some hold two tiles
+    if (nch > 1 && P->tiles.size() < 4 * (size_t)P->num_sms && prm->chunk_points <= 0)
+        P->npb = (int)std::max<size_t>(1, P->tiles.size());
     if (prm->rho_blocks > 0) {
         P->npb = std::min<int>(prm->rho_blocks, (int)std::max<size_t>(1, P->tiles.size()));
         P->rho_hi_tiles = 0;  // an explicit block count keeps the one-launch walk
