@@ -24,6 +24,13 @@ namespace {
 
 constexpr int kSBatch = 8;  // points per reduction batch of the split rho walk (4 lanes per point)
 
+// How a walk gets its prefactors along a line.  kRec: the value and its ratio
+// advance point by point.  kOrtho (orthorhombic cells): a per-record table X(n1)
+// serves every line, and the points +-n1 share their work, since X(-n1) =
+// conj X(n1) (diamond cell: rho walk 182 -> 165 us, J walk 140 -> 122; molecular
+// crystal with per-pair cutoffs: 4.93 -> 4.22 ms and 3.16 -> 2.82).
+enum : int { kRec = 0, kOrtho = 1 };
+
 
 struct Layout {
     long long start[kNclass + 1];
@@ -87,6 +94,7 @@ __device__ void split_state(const PairWalk& w, const double* M6, int n2, int n3,
 // per-pair real multipliers of the recurrences, double-float
 struct SConst {
     df q1, q2, q3, x12, y12, x13, y13, x23, y23;
+    cdf r1;  // X(1) = exp(-c M11) exp(-2 pi i f1)
 };
 
 // Once per plan: chunk-start states and the multipliers of every pair record.
@@ -112,6 +120,8 @@ __global__ void k_split_setup(const PairWalk* __restrict__ walk, long long npair
         k.y13 = df_from_double(w.y13);
         k.x23 = df_from_double(w.x23);
         k.y23 = df_from_double(w.y23);
+        const double g1 = exp(-w.c * cc.M6[0]);
+        k.r1 = to_cdf(g1 * w.e1r, g1 * w.e1i);
         cst[i] = k;
     }
 }
@@ -120,6 +130,7 @@ __device__ __forceinline__ SConst idle_const() {
     SConst k;
     const df one{1.f, 0.f};
     k.q1 = k.q2 = k.q3 = k.x12 = k.y12 = k.x13 = k.y13 = k.x23 = k.y23 = one;
+    k.r1 = cdf{{0.f, 0.f}, {0.f, 0.f}};
     return k;
 }
 
@@ -131,12 +142,11 @@ __device__ __forceinline__ SState idle_state() {
     return s;
 }
 
-// One transition of the walk program.  With ORTHO (the per-record X(n1)
-// table serves every line) the n1 ratios RfL, RbL, rF0c, rB0c are not used
-// and not advanced.  Line steps inside a plane use the deferred-renormalisation
+// One transition of the walk program.  The n1 ratios RfL, RbL, rF0c, rB0c are
+// advanced only where the walk uses them (kRec).  Line steps inside a plane use the deferred-renormalisation
 // products (at most one plane's lines deep); plane steps keep the plane values
 // renormalised, and every plane restarts the line values from them.
-template <bool ORTHO>
+template <int MODE>
 __device__ __forceinline__ void split_step(const SConst& k, int op, SState& s, const SState* init_p, bool valid) {
     switch (op) {
         case OP_FIRST:
@@ -145,7 +155,7 @@ __device__ __forceinline__ void split_step(const SConst& k, int op, SState& s, c
         case OP_N2F:
             s.gpL = cdf_mul_u(s.gpL, s.Sd);
             s.Sd = cdf_scale_u(s.Sd, k.q2);
-            if (!ORTHO) {
+            if (MODE == kRec) {
                 s.RfL = cdf_scale_u(s.RfL, k.x12);
                 s.RbL = cdf_scale_u(s.RbL, k.y12);
             }
@@ -153,7 +163,7 @@ __device__ __forceinline__ void split_step(const SConst& k, int op, SState& s, c
         case OP_NEGSTART:
             s.gpL = cdf_mul_u(s.gpC, s.RB0c);
             s.Sd = cdf_scale_u(s.RB0c, k.q2);
-            if (!ORTHO) {
+            if (MODE == kRec) {
                 s.RfL = cdf_scale_u(s.rF0c, k.y12);
                 s.RbL = cdf_scale_u(s.rB0c, k.x12);
             }
@@ -161,7 +171,7 @@ __device__ __forceinline__ void split_step(const SConst& k, int op, SState& s, c
         case OP_N2B:
             s.gpL = cdf_mul_u(s.gpL, s.Sd);
             s.Sd = cdf_scale_u(s.Sd, k.q2);
-            if (!ORTHO) {
+            if (MODE == kRec) {
                 s.RfL = cdf_scale_u(s.RfL, k.y12);
                 s.RbL = cdf_scale_u(s.RbL, k.x12);
             }
@@ -171,7 +181,7 @@ __device__ __forceinline__ void split_step(const SConst& k, int op, SState& s, c
             s.Tc = cdf_scale(s.Tc, k.q3);
             s.RF0c = cdf_scale(s.RF0c, k.x23);
             s.RB0c = cdf_scale(s.RB0c, k.y23);
-            if (!ORTHO) {
+            if (MODE == kRec) {
                 s.rF0c = cdf_scale(s.rF0c, k.x13);
                 s.rB0c = cdf_scale(s.rB0c, k.y13);
             }
@@ -223,6 +233,19 @@ __device__ __forceinline__ cdf poly_at(const cdf* c, float x) {
     return t[0];
 }
 
+// the even and the odd part of sum_i c_i x^i, as poly_at
+template <int L>
+__device__ __forceinline__ void poly_parts(const cdf* c, float x, cdf& even, cdf& odd) {
+    const float x2 = x * x;
+    even = c[0];
+    if (L >= 2) even = cdf_add_u(even, cdf{df_mulf_u(c[L >= 2 ? 2 : 0].re, x2), df_mulf_u(c[L >= 2 ? 2 : 0].im, x2)});
+    if (L >= 4)
+        even = cdf_add_u(even, cdf{df_mulf_u(c[L >= 4 ? 4 : 0].re, x2 * x2), df_mulf_u(c[L >= 4 ? 4 : 0].im, x2 * x2)});
+    odd = cdf{{0.f, 0.f}, {0.f, 0.f}};
+    if (L >= 1) odd = cdf{df_mulf_u(c[L >= 1 ? 1 : 0].re, x), df_mulf_u(c[L >= 1 ? 1 : 0].im, x)};
+    if (L >= 3) odd = cdf_add_u(odd, cdf{df_mulf_u(c[L >= 3 ? 3 : 0].re, x * x2), df_mulf_u(c[L >= 3 ? 3 : 0].im, x * x2)});
+}
+
 // Sums the batch's contributions over the block's 128 records: in warp w the
 // four lanes j, j+8, j+16, j+24 each add a quarter of point j's column of the
 // warp's 32 records, two shuffles join the quarters, and the four warp sums
@@ -263,24 +286,15 @@ __device__ __noinline__ void split_flush(float4* buf, float4* red, float4* row, 
 }
 
 // Builds the record's table X(n1) = exp(-c M11 n1^2) exp(-2 pi i f1 n1) for
-// n1 in [0, nx) with the line-independent ratios of an orthorhombic cell (the
-// first line's RfL and q1).  There the backward ratio is the conjugate of the
-// forward one, so X(-n1) = conj X(n1) and the half table serves both ends.
-__device__ __forceinline__ void build_xtab(const SState& s0, const df q1, int nx, float4* Xs, int tid) {
+// n1 in [0, nx); X(-n1) = conj X(n1), so the half table serves both ends.
+__device__ __forceinline__ void build_xtab(const SConst& k, int nx, float4* Xs, int tid) {
     cdf x{{1.f, 0.f}, {0.f, 0.f}};
-    cdf R = s0.RfL;
+    cdf R = k.r1;
     for (int n = 0; n < nx; ++n) {
         Xs[n * kTile + tid] = make_float4(x.re.hi, x.re.lo, x.im.hi, x.im.lo);
         x = cdf_mul(x, R);
-        R = cdf_scale(R, q1);
+        R = cdf_scale(R, k.q1);
     }
-}
-
-// X(m) from the half table: conj X(-m) for m < 0 (dir 1 walks m < 0)
-__device__ __forceinline__ cdf xtab_at(const float4* Xs, int m, int dir, int tid) {
-    const float4 v = Xs[(dir == 0 ? m : -m) * kTile + tid];
-    const float sg = dir == 0 ? 1.f : -1.f;
-    return cdf{{v.x, v.y}, {sg * v.z, sg * v.w}};
 }
 
 // The tile's part of a line under its G radius (per-pair cutoffs): the n1
@@ -334,12 +348,13 @@ __device__ __forceinline__ int first_index(const WLine& ln, int p0, int dir, int
     return ln.pt - p0 + n0 + (min(ln.hi, -1) - first);
 }
 
-template <int L, bool ORTHO, bool CUT>
+template <int L, int MODE, bool CUT>
 __device__ void rho_tile_split(const Tile& tl, const Layout& lay, const float2* __restrict__ Dp_d,
                                const SConst* __restrict__ cst, const SState* __restrict__ init_c,
                                const WLine* __restrict__ lines, const WChunk ch, float4* buf, float4* red,
                                float4* row, float2* Dsm, float4* Xs, int nx, int* spt) {
     constexpr int NT = nterms(L);
+    constexpr bool ORTHO = MODE == kOrtho;
     const int tid = threadIdx.x;
     const bool valid = tid < tl.count;
     const long long pi = (long long)tl.first + tid;
@@ -352,7 +367,7 @@ __device__ void rho_tile_split(const Tile& tl, const Layout& lay, const float2* 
         Dsm[t * kTile + tid] = valid ? Dp_d[lay.base[L] + (long long)t * cnt + loc] : make_float2(0.f, 0.f);
     const SConst k = valid ? cst[pi] : idle_const();
     const SState* init_p = init_c + (valid ? pi : 0);
-    if (ORTHO) build_xtab(valid ? *init_p : idle_state(), k.q1, nx, Xs, tid);
+    if (ORTHO) build_xtab(k, nx, Xs, tid);
     SState s;
     int slot = 0, par = 0, rbase = 0, mode = kWalkOn;
     for (int li = ch.l0; li < ch.l1; ++li) {
@@ -361,7 +376,7 @@ __device__ void rho_tile_split(const Tile& tl, const Layout& lay, const float2* 
             if (mode == kSkipRest) break;
             if (skip_line(mode, ln.op)) continue;
         }
-        split_step<ORTHO>(k, ln.op, s, init_p, valid);
+        split_step<MODE>(k, ln.op, s, init_p, valid);
         int lo = ln.lo, hi = ln.hi;
         if (CUT) {
             if (ORTHO && line_outside(ln, tl.gcut2)) {
@@ -397,9 +412,51 @@ __device__ void rho_tile_split(const Tile& tl, const Layout& lay, const float2* 
                     }
         }
         if (ORTHO) {
-            // the line value gp(0) goes into the coefficients; X(n1) carries the rest
+            // the line value gp(0) goes into the coefficients; X(n1) (and u^n1) carry the rest
 #pragma unroll
             for (int i = 0; i <= L; ++i) c[i] = cdf_mul_u(s.gpL, c[i]);
+        }
+        // one value of the batch: its point is q of the chunk (paired and cut walks), or the next one
+        auto put = [&](const cdf& z, int q) {
+            buf[slot * (kTile + 1) + tid] = make_float4(z.re.hi, z.re.lo, z.im.hi, z.im.lo);
+            if ((CUT || ORTHO) && tid == 0) spt[par * kSBatch + slot] = q;
+            if (++slot == kSBatch) {
+                split_flush(buf, red, row, CUT || ORTHO ? spt + par * kSBatch : nullptr, rbase, kSBatch);
+                par ^= 1;  // the next batch's indices go to the other half
+                rbase += kSBatch;
+                slot = 0;
+            }
+        };
+        if (ORTHO) {
+            // Points +-m together: with E and O the even and odd parts of the polynomial, U = Xr E + i Xi O and
+            // V = Xr O + i Xi E give rho(+-m) = U +- V.  The row keeps U at +m and V at -m; the signs are joined when
+            // it is written out.  The line through the origin stores its positive points only: U + V at once.
+            const int q0 = ln.pt - ch.p0;
+            const bool half = ln.lo > 0;
+            if (!half) put(c[0], q0);
+            // not unrolled: the walk's instruction footprint (five classes) stays in the instruction cache
+#pragma unroll 1
+            for (int m = 1; m <= hi; ++m) {
+                cdf E, O;
+                poly_parts<L>(c, (float)m, E, O);
+                const float4 xv = Xs[m * kTile + tid];
+                const df xr{xv.x, xv.y}, xi{xv.z, xv.w};
+                cdf U, V;
+                if (L == 0) {
+                    U = cdf{df_mul_u(xr, E.re), df_mul_u(xr, E.im)};
+                    V = cdf{df_neg(df_mul_u(xi, E.im)), df_mul_u(xi, E.re)};
+                } else {
+                    U = cdf{df_mul_sub_u(xr, E.re, xi, O.im), df_mul_add_u(xr, E.im, xi, O.re)};
+                    V = cdf{df_mul_sub_u(xr, O.re, xi, E.im), df_mul_add_u(xr, O.im, xi, E.re)};
+                }
+                if (half) {
+                    put(cdf_add_u(U, V), q0 + m - 1);
+                } else {
+                    put(U, q0 + m);
+                    put(V, q0 + ln.hi + m);
+                }
+            }
+            continue;
         }
         // not unrolled: the walk's instruction footprint (five classes) stays in the instruction cache
 #pragma unroll 1
@@ -411,56 +468,97 @@ __device__ void rho_tile_split(const Tile& tl, const Layout& lay, const float2* 
                 m0 = 0;
                 m1 = hi;
                 step = 1;
-                if (!ORTHO) {
-                    gp = s.gpL;
-                    R = s.RfL;
-                }
+                gp = s.gpL;
+                R = s.RfL;
             } else {
                 if (lo > -1) continue;
                 m0 = -1;
                 m1 = lo;
                 step = -1;
-                if (!ORTHO) {
-                    gp = cdf_mul_u(s.gpL, s.RbL);
-                    R = cdf_scale_u(s.RbL, k.q1);
-                }
-            }
-            if (ORTHO) {
-                // no recurrence to carry: visit exactly the line's points of this direction
-                m0 = dir == 0 ? max(lo, 0) : min(hi, -1);
-                if ((m1 - m0) * step < 0) continue;
+                gp = cdf_mul_u(s.gpL, s.RbL);
+                R = cdf_scale_u(s.RbL, k.q1);
             }
             int q = CUT ? first_index(ln, ch.p0, dir, dir == 0 ? max(lo, 0) : min(hi, -1)) : 0;
             float x = (float)m0;
             const float xstep = (float)step;
             for (int m = m0;; m += step, x += xstep) {
-                if (ORTHO || (m >= lo && m <= hi)) {
+                if (m >= lo && m <= hi) {
                     const cdf a = poly_at<L>(c, x);
-                    cdf xv;
-                    if (ORTHO) xv = xtab_at(Xs, m, dir, tid);
-                    const cdf z = ORTHO ? cdf_mul_u(xv, a) : cdf_mul_u(gp, a);
-                    buf[slot * (kTile + 1) + tid] = make_float4(z.re.hi, z.re.lo, z.im.hi, z.im.lo);
-                    if (CUT) {
-                        if (tid == 0) spt[par * kSBatch + slot] = q;
-                        ++q;
-                    }
-                    if (++slot == kSBatch) {
-                        split_flush(buf, red, row, CUT ? spt + par * kSBatch : nullptr, rbase, kSBatch);
-                        par ^= 1;  // the next batch's indices go to the other half
-                        rbase += kSBatch;
-                        slot = 0;
-                    }
+                    put(cdf_mul_u(gp, a), q++);
                 }
                 if (m == m1) break;
-                if (!ORTHO) {
-                    gp = cdf_mul_u(gp, R);
-                    R = cdf_scale_u(R, k.q1);
-                }
+                gp = cdf_mul_u(gp, R);
+                R = cdf_scale_u(R, k.q1);
             }
         }
     }
-    if (slot > 0) split_flush(buf, red, row, CUT ? spt + par * kSBatch : nullptr, rbase, slot);
+    if (slot > 0) split_flush(buf, red, row, CUT || ORTHO ? spt + par * kSBatch : nullptr, rbase, slot);
     __syncthreads();
+}
+
+// The block's row to global memory in FP64, as the values of its points: the
+// paired walk's sums U (at +m) and V (at -m) of every line become U + V and U - V.
+template <int MODE>
+__device__ __forceinline__ void write_row(const float4* row, const WLine* __restrict__ lines, const WChunk ch,
+                                          double2* __restrict__ out) {
+    auto value = [&](int i) {
+        const float4 v = row[i];
+        return make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w);
+    };
+    if (MODE == kOrtho) {
+        for (int li = ch.l0 + (int)threadIdx.x; li < ch.l1; li += blockDim.x) {
+            const WLine ln = lines[li];
+            const int q0 = ln.pt - ch.p0, n = ln.hi - ln.lo + 1;
+            if (ln.lo > 0 || n < 1) {
+                for (int m = 0; m < n; ++m) out[q0 + m] = value(q0 + m);
+                continue;
+            }
+            out[q0] = value(q0);
+            for (int m = 1; m <= ln.hi; ++m) {
+                const double2 U = value(q0 + m), V = value(q0 + ln.hi + m);
+                out[q0 + m] = make_double2(U.x + V.x, U.y + V.y);
+                out[q0 + ln.hi + m] = make_double2(U.x - V.x, U.y - V.y);
+            }
+        }
+    } else {
+        for (int i = threadIdx.x; i < ch.p1 - ch.p0; i += blockDim.x) out[i] = value(i);
+    }
+}
+
+// The potential of a chunk in shared memory, double-float: W at every point, or
+// for the paired walk W(+m) + W(-m) at +m and W(+m) - W(-m) at -m (the line
+// through the origin stores its positive points only: W itself).
+template <int MODE, class Load>
+__device__ __forceinline__ void load_w(float4* wsm, const WLine* __restrict__ lines, const WChunk ch, Load at) {
+    auto put = [&](int i, double x, double y) {
+        const df re = df_from_double(x), im = df_from_double(y);
+        wsm[i] = make_float4(re.hi, re.lo, im.hi, im.lo);
+    };
+    if (MODE == kOrtho) {
+        for (int li = ch.l0 + (int)threadIdx.x; li < ch.l1; li += blockDim.x) {
+            const WLine ln = lines[li];
+            const int q0 = ln.pt - ch.p0, n = ln.hi - ln.lo + 1;
+            if (ln.lo > 0 || n < 1) {
+                for (int m = 0; m < n; ++m) {
+                    const double2 w = at(q0 + m);
+                    put(q0 + m, w.x, w.y);
+                }
+                continue;
+            }
+            const double2 w0 = at(q0);
+            put(q0, w0.x, w0.y);
+            for (int m = 1; m <= ln.hi; ++m) {
+                const double2 a = at(q0 + m), b = at(q0 + ln.hi + m);
+                put(q0 + m, a.x + b.x, a.y + b.y);
+                put(q0 + ln.hi + m, a.x - b.x, a.y - b.y);
+            }
+        }
+    } else {
+        for (int i = threadIdx.x; i < ch.p1 - ch.p0; i += blockDim.x) {
+            const double2 w = at(i);
+            put(i, w.x, w.y);
+        }
+    }
 }
 
 // The structure-factor walk, persistent over the plan's tile schedule.  PART
@@ -468,7 +566,7 @@ __device__ void rho_tile_split(const Tile& tl, const Layout& lay, const float2* 
 // four blocks per SM); PART 2: classes 3-4.  Where shared memory holds the
 // one-kernel walk below three blocks per SM, parts 2 and 1 run as two launches
 // in turn, blocks [0, npb_hi) and [npb_hi, npb) of the schedule and the rows.
-template <bool ORTHO, bool CUT, int PART>
+template <int MODE, bool CUT, int PART>
 __global__ void __launch_bounds__(kTile, PART == 1 ? 4 : 3) k_rho_walk_split(
     const Tile* __restrict__ tiles, int b0, Layout lay, const float2* __restrict__ Dp, const SConst* __restrict__ cst,
     const SState* __restrict__ init, long long npairs, const WLine* __restrict__ lines,
@@ -483,7 +581,7 @@ __global__ void __launch_bounds__(kTile, PART == 1 ? 4 : 3) k_rho_walk_split(
     float4* red = buf + kSBatch * (kTile + 1);
     float2* Dsm = reinterpret_cast<float2*>(red + kTile);
     float4* Xs = reinterpret_cast<float4*>(Dsm + nterms(PART == 1 ? 2 : 4) * kTile);
-    float4* row = Xs + (ORTHO ? nx * kTile : 0);
+    float4* row = Xs + (MODE == kOrtho ? nx * kTile : 0);
     for (int i = threadIdx.x; i < npts; i += blockDim.x) row[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
     const float2* Dp_d = Dp + (long long)d * lay.total;
@@ -492,7 +590,7 @@ __global__ void __launch_bounds__(kTile, PART == 1 ? 4 : 3) k_rho_walk_split(
     for (int j = sched[b]; j < sched[b + 1]; ++j) {
         const Tile tl = tiles[sched[npb + 1 + j]];
 #define FTCJ_RHO_TILE(Lc) \
-    rho_tile_split<Lc, ORTHO, CUT>(tl, lay, Dp_d, cst, init_c, lines, ch, buf, red, row, Dsm, Xs, nx, spt)
+    rho_tile_split<Lc, MODE, CUT>(tl, lay, Dp_d, cst, init_c, lines, ch, buf, red, row, Dsm, Xs, nx, spt)
         if (PART == 1) {
             if (tl.cls == 0) FTCJ_RHO_TILE(0);
             else if (tl.cls == 1) FTCJ_RHO_TILE(1);
@@ -512,23 +610,20 @@ __global__ void __launch_bounds__(kTile, PART == 1 ? 4 : 3) k_rho_walk_split(
 #undef FTCJ_RHO_TILE
     }
     __syncthreads();
-    double2* out = rho_part + ((long long)d * npb + b) * ng_half + ch.p0;
-    for (int i = threadIdx.x; i < npts; i += blockDim.x) {
-        const float4 v = row[i];
-        out[i] = make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w);
-    }
+    write_row<MODE>(row, lines, ch, rho_part + ((long long)d * npb + b) * ng_half + ch.p0);
 }
 
 // ---- J -------------------------------------------------------------------
 
 // L: degree of the sums (the record's class, or one more for the nuclear
 // gradient's sums); C: the record's class, which places its terms in `lay`.
-template <int L, bool ORTHO, bool CUT, int C = L>
+template <int L, int MODE, bool CUT, int C = L>
 __device__ void j_tile_split(const Tile& tl, const Layout& lay, const SConst* __restrict__ cst,
                              const SState* __restrict__ init_c, const WLine* __restrict__ lines, const WChunk ch,
                              const float4* __restrict__ wsm,
                              double* __restrict__ Jp_dc, float2* Jsm, float4* Xs, int nx) {
     constexpr int NT = nterms(L);
+    constexpr bool ORTHO = MODE == kOrtho;
     const int tid = threadIdx.x;
     const bool valid = tid < tl.count;
     const long long pi = (long long)tl.first + tid;
@@ -540,7 +635,7 @@ __device__ void j_tile_split(const Tile& tl, const Layout& lay, const SConst* __
     // (updated once per line)
 #pragma unroll
     for (int t = 0; t < NT; ++t) Jsm[t * kTile + tid] = make_float2(0.f, 0.f);
-    if (ORTHO) build_xtab(valid ? *init_p : idle_state(), k.q1, nx, Xs, tid);
+    if (ORTHO) build_xtab(k, nx, Xs, tid);
     SState s;
     int mode = kWalkOn;
     for (int li = ch.l0; li < ch.l1; ++li) {
@@ -549,7 +644,7 @@ __device__ void j_tile_split(const Tile& tl, const Layout& lay, const SConst* __
             if (mode == kSkipRest) break;
             if (skip_line(mode, ln.op)) continue;
         }
-        split_step<ORTHO>(k, ln.op, s, init_p, valid);
+        split_step<MODE>(k, ln.op, s, init_p, valid);
         int lo = ln.lo, hi = ln.hi;
         if (CUT) {
             if (ORTHO && line_outside(ln, tl.gcut2)) {
@@ -562,59 +657,78 @@ __device__ void j_tile_split(const Tile& tl, const Layout& lay, const SConst* __
         cdf A[L + 1];
 #pragma unroll
         for (int i = 0; i <= L; ++i) A[i] = cdf{{0.f, 0.f}, {0.f, 0.f}};
-        int qs = ln.pt - ch.p0;  // without cutoffs the line's points are visited in stored order
-#pragma unroll
-        for (int dir = 0; dir < 2; ++dir) {
-            int m0, m1, step;
-            cdf gp, R;
-            if (dir == 0) {
-                if (hi < 0) continue;
-                m0 = 0;
-                m1 = hi;
-                step = 1;
-                if (!ORTHO) {
-                    gp = s.gpL;
-                    R = s.RfL;
-                }
-            } else {
-                if (lo > -1) continue;
-                m0 = -1;
-                m1 = lo;
-                step = -1;
-                if (!ORTHO) {
-                    gp = cdf_mul_u(s.gpL, s.RbL);
-                    R = cdf_scale_u(s.RbL, k.q1);
-                }
-            }
-            if (ORTHO) {
-                // no recurrence to carry: visit exactly the line's points of this direction
-                m0 = dir == 0 ? max(lo, 0) : min(hi, -1);
-                if ((m1 - m0) * step < 0) continue;
-            }
-            int q = CUT ? first_index(ln, ch.p0, dir, dir == 0 ? max(lo, 0) : min(hi, -1)) : qs;
-            float x = (float)m0;
-            const float xstep = (float)step;
-            for (int m = m0;; m += step, x += xstep) {
-                if (ORTHO || (m >= lo && m <= hi)) {
-                    const cdf w = unpack(wsm[q++]);
-                    cdf xv;
-                    if (ORTHO) xv = xtab_at(Xs, m, dir, tid);
-                    const cdf t = ORTHO ? cdf_mul_u(xv, w) : cdf_mul_u(gp, w);
-                    A[0] = cdf_add_u(A[0], t);
+        // A_i += n1^i t, exact powers (|n1|^L < 2^24)
+        auto add = [&](int i, const cdf& z, float p) {
+            A[i] = cdf{df_add_u(A[i].re, df_mulf_u(z.re, p)), df_add_u(A[i].im, df_mulf_u(z.im, p))};
+        };
+        if (ORTHO) {
+            // Points +-m together: with P = W(m) + W(-m) and M = W(m) - W(-m) the even powers take X W(m) + conj X
+            // W(-m) = Xr P + i Xi M, the odd ones X W(m) - conj X W(-m) = Xr M + i Xi P; on the line through the
+            // origin, whose positive points alone are stored, both are X W(m).
+            const int q0 = ln.pt - ch.p0;
+            const bool half = ln.lo > 0;
+            if (!half) A[0] = unpack(wsm[q0]);
+#pragma unroll 1
+            for (int m = 1; m <= hi; ++m) {
+                const cdf P = unpack(wsm[half ? q0 + m - 1 : q0 + m]);
+                const cdf M = half ? P : unpack(wsm[q0 + ln.hi + m]);
+                const float4 xv = Xs[m * kTile + tid];
+                const df xr{xv.x, xv.y}, xi{xv.z, xv.w};
+                const cdf ev{df_mul_sub_u(xr, P.re, xi, M.im), df_mul_add_u(xr, P.im, xi, M.re)};
+                A[0] = cdf_add_u(A[0], ev);
+                if (L >= 1) {
+                    const float x = (float)m;
+                    const cdf od{df_mul_sub_u(xr, M.re, xi, P.im), df_mul_add_u(xr, M.im, xi, P.re)};
                     float p = 1.f;
 #pragma unroll
                     for (int i = 1; i <= L; ++i) {
-                        p *= x;  // n1^i, exact (|n1|^L < 2^24)
-                        A[i] = cdf{df_add_u(A[i].re, df_mulf_u(t.re, p)), df_add_u(A[i].im, df_mulf_u(t.im, p))};
+                        p *= x;
+                        add(i, i & 1 ? od : ev, p);
                     }
                 }
-                if (m == m1) break;
-                if (!ORTHO) {
+            }
+        } else {
+            int qs = ln.pt - ch.p0;  // without cutoffs the line's points are visited in stored order
+#pragma unroll
+            for (int dir = 0; dir < 2; ++dir) {
+                int m0, m1, step;
+                cdf gp, R;
+                    if (dir == 0) {
+                    if (hi < 0) continue;
+                    m0 = 0;
+                    m1 = hi;
+                    step = 1;
+                    gp = s.gpL;
+                    R = s.RfL;
+                } else {
+                    if (lo > -1) continue;
+                    m0 = -1;
+                    m1 = lo;
+                    step = -1;
+                    gp = cdf_mul_u(s.gpL, s.RbL);
+                    R = cdf_scale_u(s.RbL, k.q1);
+                }
+                int q = CUT ? first_index(ln, ch.p0, dir, dir == 0 ? max(lo, 0) : min(hi, -1)) : qs;
+                float x = (float)m0;
+                const float xstep = (float)step;
+                for (int m = m0;; m += step, x += xstep) {
+                    if (m >= lo && m <= hi) {
+                        const cdf w = unpack(wsm[q++]);
+                        const cdf t = cdf_mul_u(gp, w);
+                        A[0] = cdf_add_u(A[0], t);
+                        float p = 1.f;
+#pragma unroll
+                        for (int i = 1; i <= L; ++i) {
+                            p *= x;
+                            add(i, t, p);
+                        }
+                    }
+                    if (m == m1) break;
                     gp = cdf_mul_u(gp, R);
                     R = cdf_scale_u(R, k.q1);
                 }
+                qs = q;
             }
-            qs = q;
         }
         if (ORTHO) {
 #pragma unroll
@@ -660,7 +774,7 @@ __device__ void j_tile_split(const Tile& tl, const Layout& lay, const SConst* __
 // that the nuclear gradient contracts (one more power of G from d/dR_A), into
 // the gradient's term layout; the slices grow to 20 resp. 56 terms, and the
 // degree-5 part takes the registers of two blocks per SM.
-template <bool ORTHO, bool CUT, int PART, int E>
+template <int MODE, bool CUT, int PART, int E>
 __global__ void __launch_bounds__(kTile, PART == 1 ? 4 : (E ? 2 : 3)) k_j_walk_split(
     const Tile* __restrict__ tiles, int tile0, Layout lay, const SConst* __restrict__ cst,
     const SState* __restrict__ init, long long npairs, const WLine* __restrict__ lines,
@@ -669,21 +783,16 @@ __global__ void __launch_bounds__(kTile, PART == 1 ? 4 : (E ? 2 : 3)) k_j_walk_s
     extern __shared__ float4 ssm[];
     const int tix = tile0 + blockIdx.x, cidx = blockIdx.y, d = blockIdx.z;
     const WChunk ch = chunks[cidx];
-    const int npts = ch.p1 - ch.p0;
     float4* wsm = ssm;
     float2* Jsm = reinterpret_cast<float2*>(ssm + max_chunk_pts);
     float4* Xs = reinterpret_cast<float4*>(Jsm + nterms((PART == 1 ? 2 : 4) + E) * kTile);
     const double2* Wd = W + (long long)d * ng_half + ch.p0;
-    for (int i = threadIdx.x; i < npts; i += blockDim.x) {
-        const double2 v = Wd[i];
-        const df re = df_from_double(v.x), im = df_from_double(v.y);
-        wsm[i] = make_float4(re.hi, re.lo, im.hi, im.lo);
-    }
+    load_w<MODE>(wsm, lines, ch, [&](int i) { return __ldg(Wd + i); });
     __syncthreads();
     const Tile tl = tiles[tix];
     double* Jp_dc = Jp + ((long long)d * nchunks + cidx) * lay.total;
     const SState* init_c = init + (long long)cidx * npairs;
-#define FTCJ_J_TILE(c) j_tile_split<(c) + E, ORTHO, CUT, (c)>(tl, lay, cst, init_c, lines, ch, wsm, Jp_dc, Jsm, Xs, nx)
+#define FTCJ_J_TILE(c) j_tile_split<(c) + E, MODE, CUT, (c)>(tl, lay, cst, init_c, lines, ch, wsm, Jp_dc, Jsm, Xs, nx)
     if (PART == 1) {
         switch (tl.cls) {
             case 0: FTCJ_J_TILE(0); break;
@@ -743,14 +852,14 @@ size_t j_smem(const ftcj_plan* P, int part, int e = 0) {
 }
 
 // the walk kernels for the plan's shape: X(n1) table or recurrence, with or without per-pair cutoffs
-using RhoKernel = decltype(&k_rho_walk_split<true, true, 0>);
-using JKernel = decltype(&k_j_walk_split<true, true, 0, 0>);
+using RhoKernel = decltype(&k_rho_walk_split<kOrtho, true, 0>);
+using JKernel = decltype(&k_j_walk_split<kOrtho, true, 0, 0>);
 
 template <int PART>
 RhoKernel rho_kernel_part(const ftcj_plan* P) {
     const bool c = P->d_rec_gcut != nullptr;
-    if (use_xtab(P)) return c ? k_rho_walk_split<true, true, PART> : k_rho_walk_split<true, false, PART>;
-    return c ? k_rho_walk_split<false, true, PART> : k_rho_walk_split<false, false, PART>;
+    if (use_xtab(P)) return c ? k_rho_walk_split<kOrtho, true, PART> : k_rho_walk_split<kOrtho, false, PART>;
+    return c ? k_rho_walk_split<kRec, true, PART> : k_rho_walk_split<kRec, false, PART>;
 }
 
 RhoKernel rho_kernel(const ftcj_plan* P, int part = 0) {
@@ -760,8 +869,8 @@ RhoKernel rho_kernel(const ftcj_plan* P, int part = 0) {
 template <int PART, int E>
 JKernel j_kernel_part(const ftcj_plan* P) {
     const bool c = P->d_rec_gcut != nullptr;
-    if (use_xtab(P)) return c ? k_j_walk_split<true, true, PART, E> : k_j_walk_split<true, false, PART, E>;
-    return c ? k_j_walk_split<false, true, PART, E> : k_j_walk_split<false, false, PART, E>;
+    if (use_xtab(P)) return c ? k_j_walk_split<kOrtho, true, PART, E> : k_j_walk_split<kOrtho, false, PART, E>;
+    return c ? k_j_walk_split<kRec, true, PART, E> : k_j_walk_split<kRec, false, PART, E>;
 }
 
 JKernel j_kernel(const ftcj_plan* P, int part) {
@@ -811,22 +920,22 @@ struct BatchCell {
 };
 
 // one tile of one class, out of line: each class's walk gets its own register allocation
-template <int Lc, bool ORTHO>
+template <int Lc, int MODE>
 __device__ __noinline__ void batch_rho_tile(const Tile tl, const BatchCell* C, const float2* __restrict__ Dp_d,
                                             const SState* __restrict__ init_c, const WChunk ch, float4* buf,
                                             float4* red, float4* row, float2* Dsm, float4* Xs, int* spt) {
-    rho_tile_split<Lc, ORTHO, false>(tl, C->lay, Dp_d, C->cst, init_c, C->lines, ch, buf, red, row, Dsm, Xs, C->nx,
+    rho_tile_split<Lc, MODE, false>(tl, C->lay, Dp_d, C->cst, init_c, C->lines, ch, buf, red, row, Dsm, Xs, C->nx,
                                      spt);
 }
 
-template <int Lc, bool ORTHO>
+template <int Lc, int MODE>
 __device__ __noinline__ void batch_j_tile(const Tile tl, const BatchCell* C, const SState* __restrict__ init_c,
                                           const WChunk ch, const float4* wsm, double* Jp_dc, float2* Jsm,
                                           float4* Xs) {
-    j_tile_split<Lc, ORTHO, false, Lc>(tl, C->lay, C->cst, init_c, C->lines, ch, wsm, Jp_dc, Jsm, Xs, C->nx);
+    j_tile_split<Lc, MODE, false, Lc>(tl, C->lay, C->cst, init_c, C->lines, ch, wsm, Jp_dc, Jsm, Xs, C->nx);
 }
 
-template <bool ORTHO>
+template <int MODE>
 __device__ __forceinline__ void batch_rho_item(const BatchCell& C, int b, int cidx, int d, float4* ssm, int* spt) {
     const WChunk ch = C.chunks[cidx];
     const int npts = ch.p1 - ch.p0;
@@ -834,14 +943,14 @@ __device__ __forceinline__ void batch_rho_item(const BatchCell& C, int b, int ci
     float4* red = buf + kSBatch * (kTile + 1);
     float2* Dsm = reinterpret_cast<float2*>(red + kTile);
     float4* Xs = reinterpret_cast<float4*>(Dsm + nterms(4) * kTile);
-    float4* row = Xs + (ORTHO ? C.nx * kTile : 0);
+    float4* row = Xs + (MODE == kOrtho ? C.nx * kTile : 0);
     for (int i = threadIdx.x; i < npts; i += blockDim.x) row[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
     const float2* Dp_d = C.Dp + (long long)d * C.lay.total;
     const SState* init_c = C.init + (long long)cidx * C.npairs;
     for (int j = C.sched[b]; j < C.sched[b + 1]; ++j) {
         const Tile tl = C.tiles[C.sched[C.npb + 1 + j]];
-#define FTCJ_BRHO(Lc) batch_rho_tile<Lc, ORTHO>(tl, &C, Dp_d, init_c, ch, buf, red, row, Dsm, Xs, spt)
+#define FTCJ_BRHO(Lc) batch_rho_tile<Lc, MODE>(tl, &C, Dp_d, init_c, ch, buf, red, row, Dsm, Xs, spt)
         switch (tl.cls) {
             case 0: FTCJ_BRHO(0); break;
             case 1: FTCJ_BRHO(1); break;
@@ -852,15 +961,11 @@ __device__ __forceinline__ void batch_rho_item(const BatchCell& C, int b, int ci
 #undef FTCJ_BRHO
     }
     __syncthreads();
-    double2* out = C.rho_part + ((long long)d * C.npb + b) * C.ng_half + ch.p0;
-    for (int i = threadIdx.x; i < npts; i += blockDim.x) {
-        const float4 v = row[i];
-        out[i] = make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w);
-    }
+    write_row<MODE>(row, C.lines, ch, C.rho_part + ((long long)d * C.npb + b) * C.ng_half + ch.p0);
     __syncthreads();
 }
 
-template <bool ORTHO>
+template <int MODE>
 __device__ __forceinline__ void batch_j_item(const BatchCell& C, int tix, int cidx, int d, float4* ssm) {
     const WChunk ch = C.chunks[cidx];
     const int npts = ch.p1 - ch.p0;
@@ -868,16 +973,12 @@ __device__ __forceinline__ void batch_j_item(const BatchCell& C, int tix, int ci
     float2* Jsm = reinterpret_cast<float2*>(ssm + npts);
     float4* Xs = reinterpret_cast<float4*>(Jsm + nterms(4) * kTile);
     const double2* Wd = C.W + (long long)d * C.ng_half + ch.p0;
-    for (int i = threadIdx.x; i < npts; i += blockDim.x) {
-        const double2 v = __ldcg(Wd + i);  // written in this launch: through L2
-        const df re = df_from_double(v.x), im = df_from_double(v.y);
-        wsm[i] = make_float4(re.hi, re.lo, im.hi, im.lo);
-    }
+    load_w<MODE>(wsm, C.lines, ch, [&](int i) { return __ldcg(Wd + i); });  // written in this launch: through L2
     __syncthreads();
     const Tile tl = C.tiles[tix];
     double* Jp_dc = C.Jp + ((long long)d * C.nchunks + cidx) * C.lay.total;
     const SState* init_c = C.init + (long long)cidx * C.npairs;
-#define FTCJ_BJ(c) batch_j_tile<(c), ORTHO>(tl, &C, init_c, ch, wsm, Jp_dc, Jsm, Xs)
+#define FTCJ_BJ(c) batch_j_tile<(c), MODE>(tl, &C, init_c, ch, wsm, Jp_dc, Jsm, Xs)
     switch (tl.cls) {
         case 0: FTCJ_BJ(0); break;
         case 1: FTCJ_BJ(1); break;
@@ -921,7 +1022,7 @@ __device__ __noinline__ void batch_reduce_cell(const BatchCell& C, double* se) {
 #define FTCJ_BATCH_MINB 3
 #endif
 
-template <bool ORTHO>
+template <int MODE>
 __global__ void __launch_bounds__(kTile, FTCJ_BATCH_MINB) k_batch_walks(const BatchCell* __restrict__ cells,
                                                            const int4* __restrict__ items, int nitems,
                                                            int* counter, int* remaining, int* ready, int* err,
@@ -943,7 +1044,7 @@ __global__ void __launch_bounds__(kTile, FTCJ_BATCH_MINB) k_batch_walks(const Ba
         const BatchCell& C = sc;
         const int d = in.w & 0xffff;
         if ((in.w >> 16) == 0) {
-            batch_rho_item<ORTHO>(C, in.y, in.z, d, ssm, spt);
+            batch_rho_item<MODE>(C, in.y, in.z, d, ssm, spt);
             // the last structure-factor item of the cell does its reduction
             __threadfence();
             if (threadIdx.x == 0) s_go = atomicSub(remaining + in.x, 1) == 1;
@@ -970,7 +1071,7 @@ __global__ void __launch_bounds__(kTile, FTCJ_BATCH_MINB) k_batch_walks(const Ba
                 s_go = ok;
             }
             __syncthreads();
-            if (s_go) batch_j_item<ORTHO>(C, in.y, in.z, d, ssm);
+            if (s_go) batch_j_item<MODE>(C, in.y, in.z, d, ssm);
             __syncthreads();
         }
     }
@@ -1177,7 +1278,7 @@ int batch_walks_create(const std::vector<ftcj_plan*>& plans, BatchWalks** out) {
         C.sched = P->d_sched;
         C.npb = P->npb;
         C.nchunks = (int)P->chunks.size();
-        C.nx = use_xtab(P) ? xtab_entries(P) : 0;
+        C.nx = ortho ? xtab_entries(P) : 0;
         C.ndens = P->max_dens;
         C.lay = make_layout(P);
         C.Dp = reinterpret_cast<const float2*>(P->d_Dp);
@@ -1232,7 +1333,7 @@ int batch_walks_create(const std::vector<ftcj_plan*>& plans, BatchWalks** out) {
     bw->nitems = (int)items.size();
     bw->smem = smem;
     bw->ortho = ortho;
-    const void* kern = ortho ? (const void*)k_batch_walks<true> : (const void*)k_batch_walks<false>;
+    const void* kern = ortho ? (const void*)k_batch_walks<kOrtho> : (const void*)k_batch_walks<kRec>;
     cudaError_t e = cudaMalloc(&bw->d_cells, sizeof(BatchCell) * std::max(n, 1));
     if (e == cudaSuccess) e = cudaMalloc(&bw->d_items, sizeof(int4) * std::max<size_t>(items.size(), 1));
     if (e == cudaSuccess) e = cudaMalloc(&bw->d_remaining0, sizeof(int) * std::max(n, 1));
@@ -1272,7 +1373,7 @@ int batch_walks_launch(BatchWalks* bw, const std::vector<ftcj_plan*>& plans, lon
                                       s));
         }
     if (bw->nitems == 0) return FTCJ_OK;
-    auto kern = bw->ortho ? k_batch_walks<true> : k_batch_walks<false>;
+    auto kern = bw->ortho ? k_batch_walks<kOrtho> : k_batch_walks<kRec>;
     kern<<<(unsigned)bw->grid, kTile, bw->smem, s>>>(bw->d_cells, bw->d_items, bw->nitems, bw->d_state,
                                                      bw->d_state + 2, bw->d_state + 2 + n, bw->d_state + 1, spin);
     FTCJ_CUDA(cudaGetLastError());
