@@ -174,6 +174,7 @@ struct ftcj_plan {
     int chunk_max;        // G points per walk chunk (a plan parameter)
     int max_chunk_pts;
     int n1_min, n1_max;
+    int xtab64 = 0;  // FP64 walks: entries of the per-record X(n1) table (0: recurrences)
     int n_abs_max;  // largest |n_i| of the sphere's G = sum_i n_i b_i
     // pairs
     int64_t npairs, npairs_ordered;

@@ -21,6 +21,7 @@
 // (deterministic, no atomics).
 // J: the thread accumulates sum over a line of t(n1) n1^i, then folds the
 // line into J'_ijk with n2^j n3^k; nothing is shared between threads.
+#include <algorithm>
 #include <cmath>
 
 #include "ftcj_internal.h"
@@ -136,6 +137,26 @@ __device__ __forceinline__ PairWalk idle_walk() {
     return w;
 }
 
+// The per-record table of the walks along a line: X(n1) = exp(-c M11 n1^2)
+// exp(-2 pi i f1 n1), n1 in [0, nx), X(-n1) = conj X(n1).  A line's factor is
+// then g(0) X(n1) u^n1 with the real u = exp(-2c (M12 n2 + M13 n3)): per point
+// one multiplication for u^n1 and two to apply it, where the recurrences of the
+// Gaussian, its ratio and the phase take eight.  The FP64 pipe (2 lanes per SM)
+// is what the walks wait for, so its instructions per (record, point) set the
+// time: structure factors 9 + 2L instead of 17 + 2L, back-contraction 7 + 3L
+// instead of 14 + 2L (triclinic cell, 383 AOs: 3.00 -> 2.07 and 2.67 -> 1.60 ms).
+__device__ __forceinline__ double build_xtab(const PairWalk& w, double M11, int nx, double2* Xs, int tid) {
+    const double g1 = exp(-w.c * M11);
+    double xr = 1.0, xi = 0.0, rr = g1 * w.e1r, ri = g1 * w.e1i;
+    for (int n = 0; n < nx; ++n) {
+        Xs[n * kTile + tid] = make_double2(xr, xi);
+        cmul(xr, xi, rr, ri, xr, xi);
+        rr *= w.q1;
+        ri *= w.q1;
+    }
+    return 1.0 / g1;  // u = rF / g1
+}
+
 // products n2^j n3^k for j + k <= L
 template <int L>
 __device__ __forceinline__ void powers23(int n2, int n3, double pq[L + 1][L + 1]) {
@@ -210,10 +231,10 @@ __device__ __forceinline__ void rho_flush(double2* buf, double2* red, double2* r
     }
 }
 
-template <int L, bool CUT>
+template <int L, bool CUT, bool XT>
 __device__ void rho_tile(const double* M6, const Tile& tl, const Layout& lay, const double* __restrict__ Dp_d,
                          const PairWalk* __restrict__ walk, const WLine* __restrict__ lines, const WChunk ch,
-                         double2* buf, double2* red, double2* row, int* spt) {
+                         double2* buf, double2* red, double2* row, int* spt, double2* Xs, int nx) {
     constexpr int NT = nterms(L);
     const int tid = threadIdx.x;
     const bool valid = tid < tl.count;
@@ -224,9 +245,20 @@ __device__ void rho_tile(const double* M6, const Tile& tl, const Layout& lay, co
 #pragma unroll
     for (int t = 0; t < NT; ++t) D[t] = valid ? Dp_d[lay.base[L] + (long long)t * cnt + loc] : 0.0;
     const PairWalk w = valid ? walk[pi] : idle_walk();
+    const double ig = XT ? build_xtab(w, M6[0], nx, Xs, tid) : 0.0;
     WalkState s;
     int slot = 0, par = 0;
     int rbase = 0;
+    auto put = [&](const WLine& ln, int m, double zr, double zi) {
+        buf[slot * (kTile + 1) + tid] = make_double2(zr, zi);
+        if (CUT && tid == 0) spt[par * kBatch + slot] = point_index(ln, ch.p0, m);
+        if (++slot == kBatch) {
+            rho_flush(buf, red, row, CUT ? spt + par * kBatch : nullptr, rbase, kBatch);
+            rbase += kBatch;
+            slot = 0;
+            par ^= 1;
+        }
+    };
     for (int li = ch.l0; li < ch.l1; ++li) {
         const WLine ln = lines[li];
         state_step(w, M6, ln.op, ln.n2, ln.n3, s);
@@ -261,6 +293,37 @@ __device__ void rho_tile(const double* M6, const Tile& tl, const Layout& lay, co
                         ++t;
                     }
         }
+        if (XT) {
+            // the line value goes into the coefficients, X(n1) u^n1 carries the rest
+            const double g0r = s.gL * s.phLr, g0i = s.gL * s.phLi;
+#pragma unroll
+            for (int i = 0; i <= L; ++i) cmul(cr[i], ci[i], g0r, g0i, cr[i], ci[i]);
+#pragma unroll 1
+            for (int dir = 0; dir < 2; ++dir) {
+                const double f = (dir ? s.rB : s.rF) * ig, sg = dir ? -1.0 : 1.0;
+                const int last = dir ? -lo : hi, first = dir ? max(1, -hi) : max(0, lo);
+                double t = 1.0;
+                for (int m = 1; m < first; ++m) t *= f;  // a line that does not reach n1 = 0
+                for (int m = first; m <= last; ++m) {
+                    if (m == 0) {
+                        put(ln, 0, cr[0], ci[0]);
+                        continue;
+                    }
+                    t *= f;
+                    const double x = sg * (double)m;
+                    double ar = cr[L], ai = ci[L];
+#pragma unroll
+                    for (int i = L - 1; i >= 0; --i) {
+                        ar = fma(ar, x, cr[i]);
+                        ai = fma(ai, x, ci[i]);
+                    }
+                    const double2 X = Xs[m * kTile + tid];
+                    const double wr = t * X.x, wi = dir ? -t * X.y : t * X.y;
+                    put(ln, dir ? -m : m, wr * ar - wi * ai, wr * ai + wi * ar);
+                }
+            }
+            continue;
+        }
         // forward half of the line: n1 = 0, 1, ..., hi
         if (hi >= 0) {
             double g = s.gL, r = s.rF, pr = s.phLr, pim = s.phLi, x = 0.0;
@@ -273,14 +336,7 @@ __device__ void rho_tile(const double* M6, const Tile& tl, const Layout& lay, co
                         ai = fma(ai, x, ci[i]);
                     }
                     const double gr = g * pr, gi = g * pim;
-                    buf[slot * (kTile + 1) + tid] = make_double2(gr * ar - gi * ai, gr * ai + gi * ar);
-                    if (CUT && tid == 0) spt[par * kBatch + slot] = point_index(ln, ch.p0, m);
-                    if (++slot == kBatch) {
-                        rho_flush(buf, red, row, CUT ? spt + par * kBatch : nullptr, rbase, kBatch);
-                        rbase += kBatch;
-                        slot = 0;
-                        par ^= 1;
-                    }
+                    put(ln, m, gr * ar - gi * ai, gr * ai + gi * ar);
                 }
                 g *= r;
                 r *= w.q1;
@@ -301,14 +357,7 @@ __device__ void rho_tile(const double* M6, const Tile& tl, const Layout& lay, co
                         ai = fma(ai, x, ci[i]);
                     }
                     const double gr = g * pr, gi = g * pim;
-                    buf[slot * (kTile + 1) + tid] = make_double2(gr * ar - gi * ai, gr * ai + gi * ar);
-                    if (CUT && tid == 0) spt[par * kBatch + slot] = point_index(ln, ch.p0, m);
-                    if (++slot == kBatch) {
-                        rho_flush(buf, red, row, CUT ? spt + par * kBatch : nullptr, rbase, kBatch);
-                        rbase += kBatch;
-                        slot = 0;
-                        par ^= 1;
-                    }
+                    put(ln, m, gr * ar - gi * ai, gr * ai + gi * ar);
                 }
                 g *= r;
                 r *= w.q1;
@@ -321,13 +370,13 @@ __device__ void rho_tile(const double* M6, const Tile& tl, const Layout& lay, co
     __syncthreads();
 }
 
-template <bool CUT>
+template <bool CUT, bool XT>
 __global__ void __launch_bounds__(kTile) k_rho_walk(const Tile* __restrict__ tiles, int ntiles, Layout lay,
                                                     const double* __restrict__ Dp, const PairWalk* __restrict__ walk,
                                                     const WLine* __restrict__ lines,
                                                     const WChunk* __restrict__ chunks, int npb,
                                                     double2* __restrict__ rho_part, long long ng_half, CellConst cc,
-                                                    const int* __restrict__ sched) {
+                                                    const int* __restrict__ sched, int nx) {
     extern __shared__ double2 smem[];
     __shared__ int spt[2 * kBatch];  // point indices of the current and the previous batch (per-pair cutoffs)
     const int b = blockIdx.x, cidx = blockIdx.y, d = blockIdx.z;
@@ -335,7 +384,8 @@ __global__ void __launch_bounds__(kTile) k_rho_walk(const Tile* __restrict__ til
     const int npts = ch.p1 - ch.p0;
     double2* buf = smem;
     double2* red = buf + kBatch * (kTile + 1);
-    double2* row = red + kTile;
+    double2* Xs = red + kTile;
+    double2* row = Xs + (XT ? nx * kTile : 0);
     for (int i = threadIdx.x; i < npts; i += blockDim.x) row[i] = make_double2(0.0, 0.0);
     __syncthreads();
     const double* Dp_d = Dp + (long long)d * lay.total;
@@ -343,11 +393,11 @@ __global__ void __launch_bounds__(kTile) k_rho_walk(const Tile* __restrict__ til
     for (int j = sched[b]; j < sched[b + 1]; ++j) {
         const Tile tl = tiles[sched[npb + 1 + j]];
         switch (tl.cls) {
-            case 0: rho_tile<0, CUT>(cc.M6, tl, lay, Dp_d, walk, lines, ch, buf, red, row, spt); break;
-            case 1: rho_tile<1, CUT>(cc.M6, tl, lay, Dp_d, walk, lines, ch, buf, red, row, spt); break;
-            case 2: rho_tile<2, CUT>(cc.M6, tl, lay, Dp_d, walk, lines, ch, buf, red, row, spt); break;
-            case 3: rho_tile<3, CUT>(cc.M6, tl, lay, Dp_d, walk, lines, ch, buf, red, row, spt); break;
-            default: rho_tile<4, CUT>(cc.M6, tl, lay, Dp_d, walk, lines, ch, buf, red, row, spt); break;
+            case 0: rho_tile<0, CUT, XT>(cc.M6, tl, lay, Dp_d, walk, lines, ch, buf, red, row, spt, Xs, nx); break;
+            case 1: rho_tile<1, CUT, XT>(cc.M6, tl, lay, Dp_d, walk, lines, ch, buf, red, row, spt, Xs, nx); break;
+            case 2: rho_tile<2, CUT, XT>(cc.M6, tl, lay, Dp_d, walk, lines, ch, buf, red, row, spt, Xs, nx); break;
+            case 3: rho_tile<3, CUT, XT>(cc.M6, tl, lay, Dp_d, walk, lines, ch, buf, red, row, spt, Xs, nx); break;
+            default: rho_tile<4, CUT, XT>(cc.M6, tl, lay, Dp_d, walk, lines, ch, buf, red, row, spt, Xs, nx); break;
         }
     }
     __syncthreads();
@@ -438,10 +488,10 @@ __global__ void __launch_bounds__(256) k_energy_final(const double* __restrict__
 
 // L is the polynomial degree walked (the record's class, or class + 1 for the
 // gradient); the term layout is that of the record's class tl.cls.
-template <int L, bool CUT>
+template <int L, bool CUT, bool XT>
 __device__ void j_tile(const double* M6, const Tile& tl, const Layout& lay, const PairWalk* __restrict__ walk,
                        const WLine* __restrict__ lines, const WChunk ch, const double2* __restrict__ wsm,
-                       const double* __restrict__ pw, int n1min, double* __restrict__ Jp_dc) {
+                       const double* __restrict__ pw, int n1min, double* __restrict__ Jp_dc, double2* Xs, int nx) {
     constexpr int NT = nterms(L);
     const int tid = threadIdx.x;
     const bool valid = tid < tl.count;
@@ -449,6 +499,7 @@ __device__ void j_tile(const double* M6, const Tile& tl, const Layout& lay, cons
     const long long cnt = lay.start[tl.cls + 1] - lay.start[tl.cls];
     const long long loc = pi - lay.start[tl.cls];
     const PairWalk w = valid ? walk[pi] : idle_walk();
+    const double ig = XT ? build_xtab(w, M6[0], nx, Xs, tid) : 0.0;
     double J[NT];
 #pragma unroll
     for (int t = 0; t < NT; ++t) J[t] = 0.0;
@@ -465,49 +516,85 @@ __device__ void j_tile(const double* M6, const Tile& tl, const Layout& lay, cons
             Ar[i] = 0.0;
             Ai[i] = 0.0;
         }
-        int q = point_index(ln, ch.p0, max(lo, 0));
-        if (hi >= 0) {
-            double g = s.gL, r = s.rF, pr = s.phLr, pim = s.phLi;
-            for (int m = 0; m <= hi; ++m) {
-                if (m >= lo) {
+        if (XT) {
+#pragma unroll 1
+            for (int dir = 0; dir < 2; ++dir) {
+                const double f = (dir ? s.rB : s.rF) * ig;
+                const int last = dir ? -lo : hi, first = dir ? max(1, -hi) : max(0, lo);
+                if (first > last) continue;
+                int q = point_index(ln, ch.p0, dir ? -first : first);
+                double t = 1.0;
+                for (int m = 1; m < first; ++m) t *= f;  // a line that does not reach n1 = 0
+                for (int m = first; m <= last; ++m) {
                     const double2 W = wsm[q++];
-                    const double gr = g * pr, gi = g * pim;
-                    const double tr = gr * W.x - gi * W.y, ti = gr * W.y + gi * W.x;
-                    Ar[0] += tr;
-                    Ai[0] += ti;
-                    const double* pwm = pw + (m - n1min) * kPw;
+                    if (m == 0) {
+                        Ar[0] += W.x;
+                        Ai[0] += W.y;
+                        continue;
+                    }
+                    t *= f;
+                    const double2 X = Xs[m * kTile + tid];
+                    const double Xi = dir ? -X.y : X.y;
+                    const double yr = X.x * W.x - Xi * W.y, yi = X.x * W.y + Xi * W.x;
+                    Ar[0] = fma(t, yr, Ar[0]);
+                    Ai[0] = fma(t, yi, Ai[0]);
+                    const double* pwm = pw + ((dir ? -m : m) - n1min) * kPw;
 #pragma unroll
                     for (int i = 1; i <= L; ++i) {
-                        Ar[i] = fma(tr, pwm[i], Ar[i]);
-                        Ai[i] = fma(ti, pwm[i], Ai[i]);
+                        const double p = t * pwm[i];
+                        Ar[i] = fma(p, yr, Ar[i]);
+                        Ai[i] = fma(p, yi, Ai[i]);
                     }
                 }
-                g *= r;
-                r *= w.q1;
-                cmul(pr, pim, w.e1r, w.e1i, pr, pim);
             }
-        }
-        if (lo <= -1) {
-            q = point_index(ln, ch.p0, min(hi, -1));
-            double g = s.gL * s.rB, r = s.rB * w.q1, pr, pim;
-            cmul(s.phLr, s.phLi, w.e1r, -w.e1i, pr, pim);
-            for (int m = -1; m >= lo; --m) {
-                if (m <= hi) {
-                    const double2 W = wsm[q++];
-                    const double gr = g * pr, gi = g * pim;
-                    const double tr = gr * W.x - gi * W.y, ti = gr * W.y + gi * W.x;
-                    Ar[0] += tr;
-                    Ai[0] += ti;
-                    const double* pwm = pw + (m - n1min) * kPw;
+            const double g0r = s.gL * s.phLr, g0i = s.gL * s.phLi;
 #pragma unroll
-                    for (int i = 1; i <= L; ++i) {
-                        Ar[i] = fma(tr, pwm[i], Ar[i]);
-                        Ai[i] = fma(ti, pwm[i], Ai[i]);
+            for (int i = 0; i <= L; ++i) cmul(Ar[i], Ai[i], g0r, g0i, Ar[i], Ai[i]);
+        } else {
+            int q = point_index(ln, ch.p0, max(lo, 0));
+            if (hi >= 0) {
+                double g = s.gL, r = s.rF, pr = s.phLr, pim = s.phLi;
+                for (int m = 0; m <= hi; ++m) {
+                    if (m >= lo) {
+                        const double2 W = wsm[q++];
+                        const double gr = g * pr, gi = g * pim;
+                        const double tr = gr * W.x - gi * W.y, ti = gr * W.y + gi * W.x;
+                        Ar[0] += tr;
+                        Ai[0] += ti;
+                        const double* pwm = pw + (m - n1min) * kPw;
+    #pragma unroll
+                        for (int i = 1; i <= L; ++i) {
+                            Ar[i] = fma(tr, pwm[i], Ar[i]);
+                            Ai[i] = fma(ti, pwm[i], Ai[i]);
+                        }
                     }
+                    g *= r;
+                    r *= w.q1;
+                    cmul(pr, pim, w.e1r, w.e1i, pr, pim);
                 }
-                g *= r;
-                r *= w.q1;
-                cmul(pr, pim, w.e1r, -w.e1i, pr, pim);
+            }
+            if (lo <= -1) {
+                q = point_index(ln, ch.p0, min(hi, -1));
+                double g = s.gL * s.rB, r = s.rB * w.q1, pr, pim;
+                cmul(s.phLr, s.phLi, w.e1r, -w.e1i, pr, pim);
+                for (int m = -1; m >= lo; --m) {
+                    if (m <= hi) {
+                        const double2 W = wsm[q++];
+                        const double gr = g * pr, gi = g * pim;
+                        const double tr = gr * W.x - gi * W.y, ti = gr * W.y + gi * W.x;
+                        Ar[0] += tr;
+                        Ai[0] += ti;
+                        const double* pwm = pw + (m - n1min) * kPw;
+    #pragma unroll
+                        for (int i = 1; i <= L; ++i) {
+                            Ar[i] = fma(tr, pwm[i], Ar[i]);
+                            Ai[i] = fma(ti, pwm[i], Ai[i]);
+                        }
+                    }
+                    g *= r;
+                    r *= w.q1;
+                    cmul(pr, pim, w.e1r, -w.e1i, pr, pim);
+                }
             }
         }
         // J'_ijk += Re[(-i)^{i+j+k} A_i] n2^j n3^k
@@ -540,18 +627,20 @@ __device__ void j_tile(const double* M6, const Tile& tl, const Layout& lay, cons
 
 // EXTRA = 0: the back-contraction of degree L; EXTRA = 1: degree L + 1, the
 // sums the nuclear gradient needs (one more power of G from d/dR).
-template <int EXTRA, bool CUT>
+template <int EXTRA, bool CUT, bool XT>
 __global__ void __launch_bounds__(kTile) k_j_walk(const Tile* __restrict__ tiles, Layout lay,
                                                   const PairWalk* __restrict__ walk, const WLine* __restrict__ lines,
                                                   const WChunk* __restrict__ chunks, int nchunks,
                                                   const double2* __restrict__ W, long long ng_half, int n1min,
-                                                  int n1cnt, int max_chunk_pts, double* __restrict__ Jp, CellConst cc) {
+                                                  int n1cnt, int max_chunk_pts, double* __restrict__ Jp, CellConst cc,
+                                                  int nx) {
     extern __shared__ double2 smem[];
     const int tix = blockIdx.x, cidx = blockIdx.y, d = blockIdx.z;
     const WChunk ch = chunks[cidx];
     const int npts = ch.p1 - ch.p0;
     double2* wsm = smem;
     double* pw = reinterpret_cast<double*>(smem + max_chunk_pts);
+    double2* Xs = smem + max_chunk_pts + (n1cnt * kPw + 1) / 2;
     const double2* Wd = W + (long long)d * ng_half + ch.p0;
     for (int i = threadIdx.x; i < npts; i += blockDim.x) wsm[i] = Wd[i];
     for (int i = threadIdx.x; i < n1cnt * kPw; i += blockDim.x) {
@@ -564,13 +653,13 @@ __global__ void __launch_bounds__(kTile) k_j_walk(const Tile* __restrict__ tiles
     const Tile tl = tiles[tix];
     double* Jp_dc = Jp + ((long long)d * nchunks + cidx) * lay.total;
     switch (tl.cls + EXTRA) {
-        case 0: j_tile<0, CUT>(cc.M6, tl, lay, walk, lines, ch, wsm, pw, n1min, Jp_dc); break;
-        case 1: j_tile<1, CUT>(cc.M6, tl, lay, walk, lines, ch, wsm, pw, n1min, Jp_dc); break;
-        case 2: j_tile<2, CUT>(cc.M6, tl, lay, walk, lines, ch, wsm, pw, n1min, Jp_dc); break;
-        case 3: j_tile<3, CUT>(cc.M6, tl, lay, walk, lines, ch, wsm, pw, n1min, Jp_dc); break;
-        case 4: j_tile<4, CUT>(cc.M6, tl, lay, walk, lines, ch, wsm, pw, n1min, Jp_dc); break;
+        case 0: j_tile<0, CUT, XT>(cc.M6, tl, lay, walk, lines, ch, wsm, pw, n1min, Jp_dc, Xs, nx); break;
+        case 1: j_tile<1, CUT, XT>(cc.M6, tl, lay, walk, lines, ch, wsm, pw, n1min, Jp_dc, Xs, nx); break;
+        case 2: j_tile<2, CUT, XT>(cc.M6, tl, lay, walk, lines, ch, wsm, pw, n1min, Jp_dc, Xs, nx); break;
+        case 3: j_tile<3, CUT, XT>(cc.M6, tl, lay, walk, lines, ch, wsm, pw, n1min, Jp_dc, Xs, nx); break;
+        case 4: j_tile<4, CUT, XT>(cc.M6, tl, lay, walk, lines, ch, wsm, pw, n1min, Jp_dc, Xs, nx); break;
         default:
-            if (EXTRA) j_tile<5, CUT>(cc.M6, tl, lay, walk, lines, ch, wsm, pw, n1min, Jp_dc);
+            if (EXTRA) j_tile<5, CUT, XT>(cc.M6, tl, lay, walk, lines, ch, wsm, pw, n1min, Jp_dc, Xs, nx);
             break;
     }
 }
@@ -600,30 +689,73 @@ Layout make_grad_layout(const ftcj_plan* P) {
     return l;
 }
 
-size_t rho_smem_bytes(const ftcj_plan* P) {
-    return sizeof(double2) * ((size_t)kBatch * (kTile + 1) + kTile + (size_t)std::max(P->max_chunk_pts, 1));
+// Entries of the X(n1) table, 0 where the walks run the recurrences: where a
+// line's factors exp(-c M11 n1^2) and u^n1, whose product alone is bounded by
+// the plan's checks, could leave FP64's range, or the table shared memory.
+int xtab_entries(const ftcj_plan* P) {
+    const int nx = std::max(-P->n1_min, P->n1_max) + 1;
+    if (nx > 32) return 0;
+    double amin = INFINITY, e = 0.0;
+    for (const GroupDev& g : P->groups) amin = std::min(amin, g.alpha);
+    for (const WLine& l : P->lines)
+        if (l.lo <= l.hi) {
+            const double n = std::max(std::abs(l.lo), std::abs(l.hi));
+            e = std::max(e, std::max(P->M[0] * n * n, 2.0 * std::fabs(P->M[1] * l.n2 + P->M[2] * l.n3) * n));
+        }
+    return e / (8.0 * amin) <= 300.0 ? nx : 0;
 }
 
-size_t j_smem_bytes(const ftcj_plan* P) {
-    int n1cnt = P->n1_max - P->n1_min + 1;
-    return sizeof(double2) * (size_t)std::max(P->max_chunk_pts, 1) + sizeof(double) * kPw * (size_t)n1cnt;
+size_t rho_smem_bytes(const ftcj_plan* P, int nx) {
+    return sizeof(double2) * ((size_t)kBatch * (kTile + 1) + kTile + (size_t)nx * kTile +
+                              (size_t)std::max(P->max_chunk_pts, 1));
+}
+
+size_t j_smem_bytes(const ftcj_plan* P, int nx) {
+    const size_t n1cnt = (size_t)(P->n1_max - P->n1_min + 1);
+    return sizeof(double2) * ((size_t)std::max(P->max_chunk_pts, 1) + (n1cnt * kPw + 1) / 2 + (size_t)nx * kTile);
+}
+
+using RhoKernel = decltype(&k_rho_walk<false, false>);
+using JKernel = decltype(&k_j_walk<0, false, false>);
+
+RhoKernel rho_kernel(const ftcj_plan* P) {
+    const bool c = P->d_rec_gcut != nullptr;
+    if (P->xtab64 > 0) return c ? k_rho_walk<true, true> : k_rho_walk<false, true>;
+    return c ? k_rho_walk<true, false> : k_rho_walk<false, false>;
+}
+
+template <int EXTRA>
+JKernel j_kernel(const ftcj_plan* P) {
+    const bool c = P->d_rec_gcut != nullptr;
+    if (P->xtab64 > 0) return c ? k_j_walk<EXTRA, true, true> : k_j_walk<EXTRA, false, true>;
+    return c ? k_j_walk<EXTRA, true, false> : k_j_walk<EXTRA, false, false>;
 }
 
 }  // namespace
 
 int upload_walk_tables(ftcj_plan* P) {
-    int rc = allow_dynamic_smem((const void*)k_rho_walk<false>, rho_smem_bytes(P));
-    if (!rc) rc = allow_dynamic_smem((const void*)k_rho_walk<true>, rho_smem_bytes(P));
-    if (!rc) rc = allow_dynamic_smem((const void*)k_j_walk<0, false>, j_smem_bytes(P));
-    if (!rc) rc = allow_dynamic_smem((const void*)k_j_walk<0, true>, j_smem_bytes(P));
-    if (!rc) rc = allow_dynamic_smem((const void*)k_j_walk<1, false>, j_smem_bytes(P));
-    if (!rc) rc = allow_dynamic_smem((const void*)k_j_walk<1, true>, j_smem_bytes(P));
+    int dev = 0, optin = 0;
+    FTCJ_CUDA(cudaGetDevice(&dev));
+    FTCJ_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    // the table only where two blocks still share an SM (both walks; a quarter of it per chunk point and table entry)
+    P->xtab64 = xtab_entries(P);
+    if (std::max(rho_smem_bytes(P, P->xtab64), j_smem_bytes(P, P->xtab64)) > (size_t)optin / 2) P->xtab64 = 0;
+    const size_t rs = rho_smem_bytes(P, P->xtab64), js = j_smem_bytes(P, P->xtab64);
+    int rc = FTCJ_OK;
+    for (const void* k : {(const void*)k_rho_walk<false, false>, (const void*)k_rho_walk<true, false>,
+                          (const void*)k_rho_walk<false, true>, (const void*)k_rho_walk<true, true>})
+        if (!rc) rc = allow_dynamic_smem(k, rs);
+    for (const void* k : {(const void*)k_j_walk<0, false, false>, (const void*)k_j_walk<0, true, false>,
+                          (const void*)k_j_walk<1, false, false>, (const void*)k_j_walk<1, true, false>,
+                          (const void*)k_j_walk<0, false, true>, (const void*)k_j_walk<0, true, true>,
+                          (const void*)k_j_walk<1, false, true>, (const void*)k_j_walk<1, true, true>})
+        if (!rc) rc = allow_dynamic_smem(k, js);
     return rc;
 }
 
 int rho_walk_blocks_per_sm(ftcj_plan* P, int* out) {
     int n = 0;
-    FTCJ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_rho_walk<false>, kTile, rho_smem_bytes(P)));
+    FTCJ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, rho_kernel(P), kTile, rho_smem_bytes(P, P->xtab64)));
     *out = n > 0 ? n : 1;
     return FTCJ_OK;
 }
@@ -641,11 +773,10 @@ int launch_rho_walk(ftcj_plan* P, int ndens, cudaStream_t s) {
         return FTCJ_OK;
     }
     dim3 g(P->npb, (unsigned)P->chunks.size(), ndens);
-    auto kern = P->d_rec_gcut ? k_rho_walk<true> : k_rho_walk<false>;
-    kern<<<g, kTile, rho_smem_bytes(P), s>>>(P->d_tiles, (int)P->tiles.size(), make_layout(P), P->d_Dp,
+    rho_kernel(P)<<<g, kTile, rho_smem_bytes(P, P->xtab64), s>>>(P->d_tiles, (int)P->tiles.size(), make_layout(P), P->d_Dp,
                                                    P->d_walk, P->d_lines, P->d_chunks, P->npb,
                                                    reinterpret_cast<double2*>(P->d_rho_part), P->ng_half, P->cc,
-                                                   P->d_sched);
+                                                   P->d_sched, P->xtab64);
     FTCJ_CUDA(cudaGetLastError());
     return FTCJ_OK;
 }
@@ -682,10 +813,9 @@ int launch_j_walk(ftcj_plan* P, int ndens, const double* W, cudaStream_t s) {
     }
     dim3 g((unsigned)P->tiles.size(), nch, ndens);
     int n1cnt = P->n1_max - P->n1_min + 1;
-    auto kern = P->d_rec_gcut ? k_j_walk<0, true> : k_j_walk<0, false>;
-    kern<<<g, kTile, j_smem_bytes(P), s>>>(P->d_tiles, make_layout(P), P->d_walk, P->d_lines, P->d_chunks, nch,
+    j_kernel<0>(P)<<<g, kTile, j_smem_bytes(P, P->xtab64), s>>>(P->d_tiles, make_layout(P), P->d_walk, P->d_lines, P->d_chunks, nch,
                                                reinterpret_cast<const double2*>(W), P->ng_half, P->n1_min, n1cnt,
-                                               P->max_chunk_pts, P->d_Jp, P->cc);
+                                               P->max_chunk_pts, P->d_Jp, P->cc, P->xtab64);
     FTCJ_CUDA(cudaGetLastError());
     return FTCJ_OK;
 }
@@ -704,10 +834,9 @@ int launch_j_walk_grad(ftcj_plan* P, int ndens, const double* W, cudaStream_t s)
     }
     dim3 g((unsigned)P->tiles.size(), nch, ndens);
     int n1cnt = P->n1_max - P->n1_min + 1;
-    auto kern = P->d_rec_gcut ? k_j_walk<1, true> : k_j_walk<1, false>;
-    kern<<<g, kTile, j_smem_bytes(P), s>>>(P->d_tiles, make_grad_layout(P), P->d_walk, P->d_lines,
+    j_kernel<1>(P)<<<g, kTile, j_smem_bytes(P, P->xtab64), s>>>(P->d_tiles, make_grad_layout(P), P->d_walk, P->d_lines,
                                                   P->d_chunks, nch, reinterpret_cast<const double2*>(W), P->ng_half,
-                                                  P->n1_min, n1cnt, P->max_chunk_pts, P->d_Jg, P->cc);
+                                                  P->n1_min, n1cnt, P->max_chunk_pts, P->d_Jg, P->cc, P->xtab64);
     FTCJ_CUDA(cudaGetLastError());
     return FTCJ_OK;
 }
