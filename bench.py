@@ -596,9 +596,10 @@ def gpw_leg(ctx, forms=("split_tc", "fp64")):
     """The molecular crystal with the compact/diffuse classification (Sec. 2.6):
     the default alpha_cut = w^2/2 = 0.125 makes the 0.1 s exponent of every
     centre diffuse, and the s-s pairs of those primitives (with their lattice
-    images) take the GPW route (App. E): collocation on the real-space grid,
-    the separable transform onto the sphere, the full-range potential and the
-    adjoint integration, all FP64.  The classified build is a different
+    images) take the route of the DD records: their transform onto the sphere,
+    the full-range potential and the adjoint.  In this orthorhombic cell the
+    transforms run as the sliced separable product; the grid of App. E serves
+    other cells and callers that set one.  The classified build is a different
     Coulomb operator from the long-range headline (every integral touching a
     DD density takes the full-range kernel), so its time is context for the
     route, not a comparison."""
@@ -626,28 +627,23 @@ def gpw_leg(ctx, forms=("split_tc", "fp64")):
         phase_ms, batches, launches = p.profile_read()
         p.profile_enable(0)
         ph = {k: v / max(batches, 1) for k, v in phase_ms.items()}
-        npts = float(np.prod(info["gpw_grid"]))
-        # collocation and integration: 2 (L + 1) flops per DD record, grid point and density each
-        flops = sum(2.0 * (c + 1) * n for c, n in enumerate(info["dd_pairs_by_class"])) * npts * w.ndens * 2
+        # the method's flops of the DD records' two passes, as for the other records
+        flops = sum(method_flops_per_unit(c) * n for c, n in enumerate(info["dd_pairs_by_class"])) * (
+            info["ng_half"] * w.ndens * 2)
         gpw_ms = ph["gpw_rho"] + ph["gpw_j"]
-        # the split form runs the two grid contractions in double-float on the FP32 pipe
-        dfp = info["gpw_separable"] == 2
-        peak = ctx["peaks"]["split" if dfp else "fp64"]
         r = {"ms_per_step": ms, "value": units / (ms * 1e-3), "unit": UNIT,
              "dd_records": info["dd_pairs"], "dd_ordered_pairs": info["dd_pairs_ordered"],
              "dd_records_by_class": info["dd_pairs_by_class"], "compact_records": info["npairs"],
              "alpha_cut": info["alpha_cut"], "gpw_grid": info["gpw_grid"], "gpw_separable": info["gpw_separable"],
              "gpw_launches": info["gpw_launches"], "phase_ms_per_step": ph, "gpw_ms_per_step": gpw_ms,
              "gpw_share": gpw_ms / ms,
-             "gpw_roofline": {"bound": "alu", "pipe": "fp32 (double-float)" if dfp else "fp64",
-                              "achieved": flops / (gpw_ms * 1e-3) * 1e-12,
-                              "peak": peak * 1e-12, "unit": "TFLOP/s",
-                              "frac": flops / (gpw_ms * 1e-3) / peak,
+             "gpw_roofline": {"bound": "alu", "pipe": "fp32", "achieved": flops / (gpw_ms * 1e-3) * 1e-12,
+                              "peak": ctx["peaks"]["split"] * 1e-12, "unit": "TFLOP/s",
+                              "frac": flops / (gpw_ms * 1e-3) / ctx["peaks"]["split"],
                               "flops_per_step": flops,
-                              "note": "algorithmic flops of the collocation and integration contractions over "
-                                      "the time of both GPW phases (their reduction, six transform passes and "
-                                      "row sums included); peak: the FMA probe of this run for the pipe the "
-                                      "contractions run on (FP64, or FP32 for double-float), measured"}}
+                              "note": "4L + 14 flops per DD record and half-sphere point in each of the two passes "
+                                      "over the time of both phases; peak: the FP32 FMA probe of this run (the "
+                                      "slices are formed on that pipe), measured"}}
         if con == ftcj.FTCJ_CONTRACT_TC:
             r["status"] = p.status()
         out[form] = r

@@ -143,7 +143,9 @@ typedef struct {
     int gpw_grid[3];    /* classify = 1: grid points along a_1, a_2, a_3; each <= 0: the smallest count
                            N_i with N_i |b_i| >= Gcut + sqrt(184 p_max) (every alias of a DD transform,
                            exponent p <= p_max, below e^{-46} on the sphere) and N_i > 2 max|n_i|;
-                           an explicit count below 2 max|n_i| + 1 is refused (EINVAL) */
+                           an explicit count below 2 max|n_i| + 1 is refused (EINVAL).  Orthorhombic cells
+                           whose caller leaves all three open transform the DD records by the sliced
+                           separable product instead, which gives what the grid gives to rounding */
 } ftcj_params;
 
 #define FTCJ_CONTRACT_WALK 0
@@ -198,7 +200,8 @@ typedef struct {
                                  the pair*G counts above cover the compact records only */
     int64_t dd_pairs_ordered; /* the DD records' ordered primitive-shell pairs */
     double alpha_cut;         /* classified plan: the exponent boundary in use, else 0 */
-    int gpw_grid[3];          /* the GPW grid (0 without DD records) */
+    int gpw_grid[3];          /* the GPW grid (0 without DD records); where the separable product takes its place,
+                                 the grid that would serve */
     int gpw_separable;        /* 1: orthorhombic cell, per-axis factor tables (FP64); 2: the same with the grid
                                  contractions in double-float (split form); 0: per-point lattice images (FP64) */
     int gpw_launches;         /* kernel launches of the GPW route in one build over max_dens densities */

@@ -224,12 +224,15 @@ int ftcj_grad(ftcj_plan* P, int ndens, const double* Dk, double* EJ, double* gra
 int ftcj_plan_status(ftcj_plan* P, int* flags, void* stream) {
     if (!P || !flags) return fail(FTCJ_EINVAL, "null argument");
     cudaStream_t s = as_stream(stream);
-    *flags = 0;
-    if (P->d_tc_err) {
-        FTCJ_CUDA(cudaMemcpyAsync(flags, P->d_tc_err, sizeof(int), cudaMemcpyDeviceToHost, s));
-        FTCJ_CUDA(cudaMemsetAsync(P->d_tc_err, 0, sizeof(int), s));
-    }
+    int word[2] = {0, 0};  // the plan's kernels, and those of its DD records
+    int* const err[2] = {P->d_tc_err, P->dd ? P->dd->d_tc_err : nullptr};
+    for (int i = 0; i < 2; ++i)
+        if (err[i]) {
+            FTCJ_CUDA(cudaMemcpyAsync(&word[i], err[i], sizeof(int), cudaMemcpyDeviceToHost, s));
+            FTCJ_CUDA(cudaMemsetAsync(err[i], 0, sizeof(int), s));
+        }
     FTCJ_CUDA(cudaStreamSynchronize(s));
+    *flags = word[0] | word[1];
     return FTCJ_OK;
 }
 
