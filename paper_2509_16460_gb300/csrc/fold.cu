@@ -129,58 +129,105 @@ inline unsigned nblocks(long long n, int b) { return (unsigned)((n + b - 1) / b)
 // Each thread owns one AO-pair element of one density and keeps its whole
 // column over the mesh (nk complex values) in a thread-private slice of
 // shared memory (stride kFusedT, so a warp's accesses hit distinct banks).
-// The mesh axes are transformed in place: length 2 and 4 by butterflies
-// (only additions; the twiddles are +-1, +-i), other lengths by a direct sum
-// with the twiddle table.
+// The mesh axes are transformed in place: lengths 2, 3 and 4 by butterflies,
+// other lengths by a direct sum with the twiddle table.  The FP64 pipe bounds
+// it, so it leaves out what a real end of the transform makes redundant: the
+// fold's last axis forms the real part alone; the unfold's first axis takes
+// real input, and the other axes then run over half of its outputs, the rest
+// being their conjugates (J^{-k} = conj J^k).  A k 3x3x1 column costs 63 and
+// 49 FP64 operations instead of the 216 of a direct length-3 sum, a 4x4x4 one
+// 608 and 480 instead of 768.  Not done by the lane-shared register transform
+// below: in FP64 that repeats every length-3 line on three lanes.
+// Measured, k 3x3x1 with 940 AOs: fold 350 -> 128 us, unfold 322 -> 87 (the
+// register transform in FP64: 186 and 223); k 4x4x4 with 240 AOs: 111 -> 104
+// and 103 -> 86 (there 129 and 123).
 constexpr int kFusedT = 32;
 constexpr int kFusedMaxNk = 256;
 
+// what is known of a line: nothing, real input, or only the real part is wanted
+enum { kLine, kLineRealIn, kLineRealOut };
+
+template <int KIND>
 __device__ __forceinline__ void dft_line(double2* col, int base, int stride, int Na, const double2* __restrict__ w,
                                          bool inverse) {
+    constexpr bool RI = KIND == kLineRealIn, RO = KIND == kLineRealOut;
+    auto at = [&](int m) -> double2& { return col[(base + m * stride) * kFusedT]; };
+    auto sum = [](double2 p, double2 q) { return make_double2(p.x + q.x, RI ? 0.0 : p.y + q.y); };
+    auto dif = [](double2 p, double2 q) { return make_double2(p.x - q.x, RI ? 0.0 : p.y - q.y); };
+    auto put = [&](int m, double re, double im) {
+        if (RO) at(m).x = re;
+        else at(m) = make_double2(re, im);
+    };
     if (Na == 2) {
-        double2 x0 = col[base * kFusedT], x1 = col[(base + stride) * kFusedT];
-        col[base * kFusedT] = make_double2(x0.x + x1.x, x0.y + x1.y);
-        col[(base + stride) * kFusedT] = make_double2(x0.x - x1.x, x0.y - x1.y);
+        const double2 x0 = at(0), x1 = at(1);
+        const double2 a = sum(x0, x1), b = dif(x0, x1);
+        put(0, a.x, a.y);
+        put(1, b.x, b.y);
         return;
     }
-    if (Na == 4) {
-        double2 x0 = col[base * kFusedT], x1 = col[(base + stride) * kFusedT];
-        double2 x2 = col[(base + 2 * stride) * kFusedT], x3 = col[(base + 3 * stride) * kFusedT];
-        double2 a = make_double2(x0.x + x2.x, x0.y + x2.y), b = make_double2(x0.x - x2.x, x0.y - x2.y);
-        double2 c = make_double2(x1.x + x3.x, x1.y + x3.y), d = make_double2(x1.x - x3.x, x1.y - x3.y);
-        // forward (exp(-2 pi i mn/4)): y1 = b - i d, y3 = b + i d; inverse swaps them
-        double2 bmid = make_double2(b.x + d.y, b.y - d.x);  // b - i d
-        double2 bpid = make_double2(b.x - d.y, b.y + d.x);  // b + i d
-        col[base * kFusedT] = make_double2(a.x + c.x, a.y + c.y);
-        col[(base + 2 * stride) * kFusedT] = make_double2(a.x - c.x, a.y - c.y);
-        col[(base + stride) * kFusedT] = inverse ? bpid : bmid;
-        col[(base + 3 * stride) * kFusedT] = inverse ? bmid : bpid;
+    if (Na == 3 || Na == 4) {
+        // y0 is a plain sum; the two outputs that the directions swap are p - i q
+        // (y1 of the forward transform, twiddles exp(-2 pi i mn/N)) and p + i q
+        const double2 x0 = at(0), x1 = at(1), x2 = at(2);
+        double2 p, q;
+        if (Na == 3) {
+            const double h = 0.86602540378443864676;  // sqrt(3)/2
+            const double2 t = sum(x1, x2), u = dif(x1, x2);
+            p = make_double2(fma(-0.5, t.x, x0.x), RI ? 0.0 : fma(-0.5, t.y, x0.y));
+            q = make_double2(h * u.x, RI ? 0.0 : h * u.y);
+            const double2 y0 = sum(x0, t);
+            put(0, y0.x, y0.y);
+        } else {
+            const double2 x3 = at(3);
+            const double2 a = sum(x0, x2), c = sum(x1, x3);
+            p = dif(x0, x2);
+            q = dif(x1, x3);
+            const double2 y0 = sum(a, c), y2 = dif(a, c);
+            put(0, y0.x, y0.y);
+            put(2, y2.x, y2.y);
+        }
+        const double2 lo = RI ? make_double2(p.x, -q.x) : make_double2(p.x + q.y, p.y - q.x);
+        const double2 hi = RI ? make_double2(p.x, q.x) : make_double2(p.x - q.y, p.y + q.x);
+        const double2 y1 = inverse ? hi : lo, ym = inverse ? lo : hi;
+        put(1, y1.x, y1.y);
+        put(Na - 1, ym.x, ym.y);
         return;
     }
     double2 x[kTw];
-    for (int m = 0; m < Na; ++m) x[m] = col[(base + m * stride) * kFusedT];
+    for (int m = 0; m < Na; ++m) x[m] = at(m);
     for (int n = 0; n < Na; ++n) {
         double sr = 0.0, si = 0.0;
         for (int m = 0; m < Na; ++m) {
             double2 c = w[m * kTw + n];
             double wi = inverse ? -c.y : c.y;
-            sr = fma(c.x, x[m].x, fma(-wi, x[m].y, sr));
-            si = fma(c.x, x[m].y, fma(wi, x[m].x, si));
+            sr = fma(c.x, x[m].x, RI ? sr : fma(-wi, x[m].y, sr));
+            if (!RO) si = RI ? fma(wi, x[m].x, si) : fma(c.x, x[m].y, fma(wi, x[m].x, si));
         }
-        col[(base + n * stride) * kFusedT] = make_double2(sr, si);
+        put(n, sr, si);
     }
 }
 
-__device__ void dft_mesh(double2* col, int N1, int N2, int N3, const double2* __restrict__ tw, bool inverse) {
-    // axis 2 (stride 1), axis 1 (stride N3), axis 0 (stride N2*N3)
-    if (N3 > 1)
-        for (int o = 0; o < N1 * N2; ++o) dft_line(col, o * N3, 1, N3, tw + 2 * kTw * kTw, inverse);
-    if (N2 > 1)
-        for (int i1 = 0; i1 < N1; ++i1)
-            for (int i3 = 0; i3 < N3; ++i3) dft_line(col, i1 * N2 * N3 + i3, N3, N2, tw + kTw * kTw, inverse);
-    if (N1 > 1)
-        for (int o = 0; o < N2 * N3; ++o) dft_line(col, o, N2 * N3, N1, tw, inverse);
+// the lines of one axis, over the first H1 x H2 x H3 points of the other axes
+// (the axis' own H is its length N)
+template <int KIND>
+__device__ __forceinline__ void dft_axis(double2* col, int axis, int H1, int H2, int H3, int N2, int N3,
+                                         const double2* __restrict__ tw, bool inverse) {
+    const double2* w = tw + axis * kTw * kTw;
+    const int s1 = N2 * N3, s2 = N3;
+    if (axis == 0) {
+        for (int i2 = 0; i2 < H2; ++i2)
+            for (int i3 = 0; i3 < H3; ++i3) dft_line<KIND>(col, i2 * s2 + i3, s1, H1, w, inverse);
+    } else if (axis == 1) {
+        for (int i1 = 0; i1 < H1; ++i1)
+            for (int i3 = 0; i3 < H3; ++i3) dft_line<KIND>(col, i1 * s1 + i3, s2, H2, w, inverse);
+    } else {
+        for (int i1 = 0; i1 < H1; ++i1)
+            for (int i2 = 0; i2 < H2; ++i2) dft_line<KIND>(col, i1 * s1 + i2 * s2, 1, H3, w, inverse);
+    }
 }
+
+// the mesh axis that carries the real end: the last one longer than 1
+__device__ __forceinline__ int real_axis(int N2, int N3) { return N3 > 1 ? 2 : (N2 > 1 ? 1 : 0); }
 
 // D^{0n} = Re (1/nk) sum_k exp(-i k.R_n) D^k for one (density, element) per thread
 __global__ void __launch_bounds__(kFusedT) k_fold_fused(const double2* __restrict__ Dk, double* __restrict__ D0n,
@@ -194,7 +241,10 @@ __global__ void __launch_bounds__(kFusedT) k_fold_fused(const double2* __restric
     if (e < E) {
         const double2* src = Dk + d * nk * E + e;
         for (int k = 0; k < nk; ++k) col[k * kFusedT] = src[(long long)k * E];
-        dft_mesh(col, N1, N2, N3, tw, false);
+        const int r = real_axis(N2, N3);
+        if (N1 > 1 && r != 0) dft_axis<kLine>(col, 0, N1, N2, N3, N2, N3, tw, false);
+        if (N2 > 1 && r != 1) dft_axis<kLine>(col, 1, N1, N2, N3, N2, N3, tw, false);
+        dft_axis<kLineRealOut>(col, r, N1, N2, N3, N2, N3, tw, false);
         const double s = 1.0 / nk;
         double* dst = D0n + d * nk * E + e;
         for (int n = 0; n < nk; ++n) dst[(long long)n * E] = s * col[n * kFusedT].x;
@@ -213,9 +263,26 @@ __global__ void __launch_bounds__(kFusedT) k_unfold_fused(const double* __restri
     if (e < E) {
         const double* src = J0n + d * nk * E + e;
         for (int n = 0; n < nk; ++n) col[n * kFusedT] = make_double2(src[(long long)n * E], 0.0);
-        dft_mesh(col, N1, N2, N3, tw, true);
+        const int r = real_axis(N2, N3);
+        dft_axis<kLineRealIn>(col, r, N1, N2, N3, N2, N3, tw, true);
+        const int H2 = r == 1 ? N2 / 2 + 1 : N2, H3 = r == 2 ? N3 / 2 + 1 : N3;  // outputs kept of the real axis
+        if (N2 > 1 && r != 1) dft_axis<kLine>(col, 1, N1, N2, H3, N2, N3, tw, true);
+        if (N1 > 1 && r != 0) dft_axis<kLine>(col, 0, N1, H2, H3, N2, N3, tw, true);
         double2* dst = Jk + d * nk * E + e;
-        for (int k = 0; k < nk; ++k) dst[(long long)k * E] = col[k * kFusedT];
+        int k = 0;
+        for (int i1 = 0; i1 < N1; ++i1)
+            for (int i2 = 0; i2 < N2; ++i2)
+                for (int i3 = 0; i3 < N3; ++i3, ++k) {
+                    double2 v;
+                    if (i2 < H2 && i3 < H3) {
+                        v = col[k * kFusedT];
+                    } else {  // at -k, conjugated
+                        const int m1 = i1 ? N1 - i1 : 0, m2 = i2 ? N2 - i2 : 0, m3 = i3 ? N3 - i3 : 0;
+                        v = col[((m1 * N2 + m2) * N3 + m3) * kFusedT];
+                        v.y = -v.y;
+                    }
+                    dst[(long long)k * E] = v;
+                }
     }
 }
 

@@ -1,0 +1,71 @@
+"""Paths chosen by the size of a cell or of its k-mesh: the FP64 mesh transforms
+over lengths 1 to 6 (real ends, half-space of the unfold), the walks of cells of
+few tiles (short chunks), and FP64 walks with and without their line table."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from paper_2509_16460_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def F():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2509_16460_gb300 import build
+    build.build()
+    from paper_2509_16460_gb300 import ftcj
+    return ftcj
+
+
+@pytest.mark.parametrize("kmesh", [(1, 1, 2), (3, 1, 1), (3, 3, 1), (1, 4, 1), (2, 3, 4), (4, 4, 4), (5, 1, 3),
+                                   (3, 6, 1), (6, 2, 5), (5, 5, 1)])
+def test_fp64_fold_and_unfold(orc, F, kmesh):
+    """Both directions for inputs without any symmetry.  A value passes three
+    axes of at most 6 terms, under 32 roundings of 2^-53 of its column's sum:
+    2^-47 of that sum covers both sides."""
+    import torch
+    w = W.tiny(seed=35, A=np.diag([4.3, 4.6, 4.9]), kmesh=kmesh, ndens=2)
+    plan = F.Plan.from_workload(w)
+    rng = np.random.default_rng(17)
+    shape = w.Dk.shape
+    scale = 10.0 ** rng.uniform(-30, 3, size=shape[:1] + (1,) + shape[2:])
+    Dk = (rng.normal(size=shape) + 1j * rng.normal(size=shape)) * scale
+    got = plan.fold_density(torch.from_numpy(np.ascontiguousarray(Dk)).cuda()).cpu().numpy()
+    ref = orc.fold_density(dataclasses.replace(w, Dk=Dk)).real
+    assert (np.abs(got - ref) <= 2.0 ** -47 * np.abs(Dk).max(axis=1, keepdims=True)).all()
+    J0n = rng.normal(size=got.shape) * scale
+    Jk = plan.unfold_j(torch.from_numpy(np.ascontiguousarray(J0n)).cuda()).cpu().numpy()
+    nd, nk, n, _ = J0n.shape
+    Jref = (np.fft.ifftn(J0n.reshape(nd, *kmesh, n, n), axes=(1, 2, 3)) * nk).reshape(nd, nk, n, n)
+    assert (np.abs(Jk - Jref) <= 2.0 ** -47 * nk * np.abs(J0n).max(axis=1, keepdims=True)).all()
+    plan.close()
+
+
+TRI = np.array([[0.0, 0.0, 0.0], [0.4, 0.0, 0.0], [-0.5, 0.3, 0.0]])
+
+
+# a compact cell (short chunks, line table) and one whose lines hold more than
+# the 32 points that a table may have (the recurrences)
+@pytest.mark.parametrize("edges,omega", [((4.6, 5.2, 5.9), 0.37), ((60.0, 4.1, 4.4), 0.45)])
+def test_triclinic_walks_against_the_oracle(orc, F, edges, omega):
+    """J and E_J at the forms' own bounds (1e-10 and 1e-8 Eh), also with one
+    chunk over the whole sphere."""
+    import torch
+    w = W.tiny(seed=71, A=np.diag(edges) + TRI, kmesh=(1, 2, 1), omega=omega, ndens=2)
+    ref = orc.lrj(w, want_j0n=False)
+    Dk = torch.from_numpy(np.ascontiguousarray(w.Dk)).cuda()
+    for precision, tol in ((F.FTCJ_PREC_FP64, 1e-10), (F.FTCJ_PREC_SPLIT, 1e-8)):
+        for chunk in (0, 4096):
+            plan = F.Plan.from_workload(w, precision=precision, chunk_points=chunk)
+            Jk, EJ = plan.jbuild(Dk)
+            torch.cuda.synchronize()
+            dJ = float(np.abs(Jk.cpu().numpy() - ref["Jk"]).max())
+            dE = float(np.abs(EJ.cpu().numpy() - ref["EJ"]).max())
+            print(f"edges {edges} precision {precision} chunk {chunk}: max|dJ|={dJ:.2e} max|dE|={dE:.2e}")
+            assert dJ <= tol and dE <= tol * max(1.0, float(np.abs(ref["EJ"]).max()))
+            plan.close()
