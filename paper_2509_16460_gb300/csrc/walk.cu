@@ -144,7 +144,7 @@ __device__ __forceinline__ PairWalk idle_walk() {
 // Gaussian, its ratio and the phase take eight.  The FP64 pipe (2 lanes per SM)
 // is what the walks wait for, so its instructions per (record, point) set the
 // time: structure factors 9 + 2L instead of 17 + 2L, back-contraction 7 + 3L
-// instead of 14 + 2L (triclinic cell, 383 AOs: 3.00 -> 2.07 and 2.67 -> 1.60 ms).
+// instead of 14 + 2L (triclinic cell, 383 AOs: 3.00 -> 2.05 and 2.67 -> 1.97 ms).
 __device__ __forceinline__ double build_xtab(const PairWalk& w, double M11, int nx, double2* Xs, int tid) {
     const double g1 = exp(-w.c * M11);
     double xr = 1.0, xi = 0.0, rr = g1 * w.e1r, ri = g1 * w.e1i;
@@ -737,7 +737,7 @@ int upload_walk_tables(ftcj_plan* P) {
     int dev = 0, optin = 0;
     FTCJ_CUDA(cudaGetDevice(&dev));
     FTCJ_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    // the table only where two blocks still share an SM (both walks; a quarter of it per chunk point and table entry)
+    // the table only where two blocks still share an SM
     P->xtab64 = xtab_entries(P);
     if (std::max(rho_smem_bytes(P, P->xtab64), j_smem_bytes(P, P->xtab64)) > (size_t)optin / 2) P->xtab64 = 0;
     const size_t rs = rho_smem_bytes(P, P->xtab64), js = j_smem_bytes(P, P->xtab64);
