@@ -222,7 +222,8 @@ def make_workload(W, name):
 
 
 # form -> (pipe, per-pair cutoff eps, contraction): "split_tc" is the split form with the
-# tensor-core separable contraction of the structure-factor pass (orthorhombic cells)
+# tensor-core separable contraction of both passes (orthorhombic cells); "split" has its J walk
+# and, in larger orthorhombic cells, the structure factors of the eight-slice contraction
 FORMS = {"split_tc": ("split", 0.0, 1), "split": ("split", 0.0, 0), "fp64": ("fp64", 0.0, 0),
          "split_pair_gcut": ("split", PAIR_GCUT_EPS, 0), "fp64_pair_gcut": ("fp64", PAIR_GCUT_EPS, 0)}
 
@@ -353,7 +354,7 @@ def measure_form(ctx, w, wname, form):
         tc = {}
         for key, kern, mma, t_ms, note in (
                 ("tc_rho", "k_tc_rho", float(info["tc_mma_flops"]) * reps, rho_pass_ms,
-                 ("36 bf16 slice products per product (8 slices a side)" if pipe == "fp64" else
+                 ("36 bf16 slice products per product (8 slices a side)" if form != "split_tc" else
                   "21 bf16 slice products per product exact to 2^-41 (6 slices a side)") +
                  ", real products of the sign-symmetric rows (2 real per complex multiply-add)"),
                 ("tc_j", "k_tc_j", float(info["tc_j_mma_flops"]) * reps, j_pass_ms,

@@ -120,7 +120,10 @@ typedef struct {
                            (EUNSUPPORTED otherwise), whole sphere (pair_gcut_eps = 0).  The FP64 form
                            keeps 0 and takes the same product, cut finely enough for errors below FP64
                            accumulation's, by itself in orthorhombic cells (whole sphere, |n_i| <= 63,
-                           no chunk_points or rho_blocks of the caller's); the
+                           no chunk_points or rho_blocks of the caller's).  So do the structure
+                           factors of a split plan with 0, in place of its walk, where the sphere has
+                           at least 512 half-sphere points and 3e6 (record, point) units
+                           (ftcj_info.contraction says so).  With 1 the
                            back-contraction (Alg. S1) takes the same form where its columns fit the
                            MMA width and its factor tables shared memory, else the split walk
                            (ftcj_info.j_contraction says which) */
@@ -183,7 +186,8 @@ typedef struct {
                                  split form runs it as two class parts, else 1 (0: nothing to walk) */
     int j_walk_launches;      /* the same for the back-contraction walk */
     int contraction;          /* FTCJ_CONTRACT_WALK or FTCJ_CONTRACT_TC (the plan's structure-factor pass; the
-                                 FP64 form runs TC in orthorhombic cells without a walk shape of the caller's) */
+                                 FP64 form, and larger split plans, run TC in orthorhombic cells without a
+                                 walk shape of the caller's) */
     int64_t tc_mma_flops;     /* tensor-core contraction: bf16 MMA flops (2 per multiply-add, every slice
                                  product and padding column included) of one structure-factor pass over
                                  max_dens densities; 0 for the walks */

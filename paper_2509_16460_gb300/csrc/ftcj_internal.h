@@ -234,6 +234,7 @@ struct ftcj_plan {
     void* d_split_const = nullptr;   // split form: recurrence multipliers, [npairs]
     // tensor-core separable contraction of the structure-factor pass (tc.cu)
     bool tc = false;
+    bool tc_rho_only = false;  // split plan whose walks take the structure factors from the eight-slice product
     int tc_axis[3] = {0, 1, 2};  // row axes a, b and the column axis c
     int tc_ncols = 0, tc_nd = 0, tc_npad = 0;  // n_c = 0..ncols-1; densities per launch; MMA N
     int tc_colw = 0, tc_G = 0;                 // real columns per (i, j) block; blocks per window

@@ -125,8 +125,8 @@ struct TcArgs {
     const void* tabz;    // Z(0..), [ncols] per record in the same order
     const float* clk;    // c log2(e) in the same order
     long long kbase[kNclass];  // first record of each class in that order
-    const void* Dp;      // Hermite densities: split form double-float in the K order, [dens][class][term][position];
-                         // FP64 form doubles in record order, [dens][class][term][record]
+    const void* Dp;      // Hermite densities: split plans double-float in the K order, [dens][class][term][position];
+                         // FP64 plans doubles in record order, [dens][class][term][record]
     const int* korder;   // FP64 form: class-local record of each position of the K order of all classes
     long long dp_total;
     long long dp_base[kNclass];
@@ -637,9 +637,12 @@ constexpr int kTcBThreads = 512;
 // records of one (block, n_c, density), both columns (Re, Im), as halves of
 // 16-byte core-matrix rows; neighbouring lanes take the other half, neighbouring
 // columns and record octets, so a warp's stores of one slice fill 512-byte runs.
-template <class P>
+// DF: D' as the split form's Hermite map writes it, double-float in the K
+// order; otherwise (FP64 form) doubles in record order.
+template <class P, bool DF>
 __global__ void __launch_bounds__(kTcBThreads, P::S == 8 ? 1 : 2) k_tc_rho_b(TcArgs g) {
     constexpr bool kF64 = P::S == 8;
+    static_assert(kF64 || DF, "the six-slice operands are cut from double-float terms");
     constexpr int kS = P::S;
     __shared__ int mx[kTcNmax / 2];  // bits of the column bounds (non-negative floats order as integers)
     __shared__ int pairs[kTcGmax], tidx[kTcGmax][5];
@@ -656,7 +659,7 @@ __global__ void __launch_bounds__(kTcBThreads, P::S == 8 ? 1 : 2) k_tc_rho_b(TcA
     if (tid == 0) clmin_bits = __float_as_int(INFINITY);
     __syncthreads();
     const long long stride = g.dp_stride[L];
-    // split form: this window's positions; FP64 form: the class's records
+    // double-float terms: this window's positions; doubles: the class's records
     const float2* dpw = reinterpret_cast<const float2*>(g.Dp) + g.dp_base[L] + (long long)g.d0 * g.dp_total + wi.w;
     const double* dp64 = reinterpret_cast<const double*>(g.Dp) + g.dp_base[L] + (long long)g.d0 * g.dp_total;
     const long long kb = g.kbase[L] + wi.w;  // the window's first record in the K order
@@ -668,7 +671,7 @@ __global__ void __launch_bounds__(kTcBThreads, P::S == 8 ? 1 : 2) k_tc_rho_b(TcA
         const int k = tid + q * kTcBThreads;
         cr[q] = k < cnt ? __ldg(g.clk + kb + k) : 0.f;
         if (k < cnt) cmin = fminf(cmin, cr[q]);
-        ko[q] = kF64 && k < cnt ? __ldg(g.korder + kb + k) : 0;
+        ko[q] = !DF && k < cnt ? __ldg(g.korder + kb + k) : 0;
     }
     for (int gb = 0; gb < npair; ++gb)
         for (int d = 0; d < g.nd; ++d) {
@@ -682,7 +685,7 @@ __global__ void __launch_bounds__(kTcBThreads, P::S == 8 ? 1 : 2) k_tc_rho_b(TcA
                     cm[q][kk] = 0.f;
                     if (t < 0 || k >= cnt) continue;
                     const long long off = (long long)d * g.dp_total + (long long)t * stride;
-                    cm[q][kk] = 1.0001f * (kF64 ? fabsf((float)__ldg(dp64 + off + ko[q])) : fabsf(__ldg(dpw + off + k).x));
+                    cm[q][kk] = 1.0001f * (DF ? fabsf(__ldg(dpw + off + k).x) : fabsf((float)__ldg(dp64 + off + ko[q])));
                 }
             }
             for (int nc = 0; nc < g.ncols; ++nc) {
@@ -726,21 +729,30 @@ __global__ void __launch_bounds__(kTcBThreads, P::S == 8 ? 1 : 2) k_tc_rho_b(TcA
                     const int k = k0 + 2 * u + e;
                     double br = 0.0, bi = 0.0;
                     if (k < cnt) {
-                        const double* dp = dp64 + (long long)d * g.dp_total + __ldg(g.korder + kb + k);
+                        const long long at = (long long)d * g.dp_total + (DF ? (long long)k : (long long)__ldg(g.korder + kb + k));
+                        auto term = [&](int kk) {
+                            const long long o = at + (long long)tidx[gb][kk] * stride;
+                            if constexpr (DF) {
+                                const float2 v = __ldg(dpw + o);
+                                return join_df(df{v.x, v.y});
+                            } else {
+                                return __ldg(dp64 + o);
+                            }
+                        };
                         const double2 z = __ldg(reinterpret_cast<const double2*>(g.tabz) + (kb + k) * g.ncols + nc);
                         // sum_k D'_k (-i n_c)^k: terms of even k real, of odd k imaginary (few FP64 instructions:
                         // the pipe has 2 lanes per SM)
-                        double re = __ldg(dp + (long long)tidx[gb][0] * stride);
+                        double re = term(0);
                         if (nk == 0) {
                             br = z.x * re;
                             bi = z.y * re;
                         } else {
                             const double x = widen((float)nc);
-                            double im = -x * __ldg(dp + (long long)tidx[gb][1] * stride);
-                            if (nk > 1) re = fma(-widen((float)(nc * nc)), __ldg(dp + (long long)tidx[gb][2] * stride), re);
-                            if (nk > 2) im = fma(widen((float)(nc * nc * nc)), __ldg(dp + (long long)tidx[gb][3] * stride), im);
+                            double im = -x * term(1);
+                            if (nk > 1) re = fma(-widen((float)(nc * nc)), term(2), re);
+                            if (nk > 2) im = fma(widen((float)(nc * nc * nc)), term(3), im);
                             if (nk > 3)
-                                re = fma(widen((float)(nc * nc * nc * nc)), __ldg(dp + (long long)tidx[gb][4] * stride), re);
+                                re = fma(widen((float)(nc * nc * nc * nc)), term(4), re);
                             br = z.x * re - z.y * im;
                             bi = z.x * im + z.y * re;
                         }
@@ -1148,11 +1160,11 @@ __global__ void k_tc_tables(const PairWalk* __restrict__ walk, long long npairs,
     }
     const long long k = kpos[r];
     if (e < nna + nnb) {
-        tab[r * tws + e] = v;
+        if (tab) tab[r * tws + e] = v;  // tab, tabz3: the back-contraction's
         tabk[k * tws + e] = v;
     } else {
         tabz[k * nnc + n] = v;
-        if (F64) {
+        if (F64 && tabz3) {
             const double z[2] = {gval * c, -gval * s};
             for (int q = 0; q < 2; ++q) {
                 const float h = (float)z[q], m = (float)(z[q] - (double)h);
@@ -1842,9 +1854,12 @@ int setup_tc_j(ftcj_plan* P);
 // Plan-time set-up of the tensor-core form: the column axis, the slots and the
 // half-sphere map, the factor tables, the windows (class, block group, records
 // sorted by width), their deal to CTA groups and the B tiles.
+// FP64 plans and the structure factors of split walks: the finer of the two precisions
+inline bool tc_eight_slices(const ftcj_plan* P) { return P->precision == FTCJ_PREC_FP64 || P->tc_rho_only; }
+
 int setup_tc(ftcj_plan* P) {
     if (!P->ortho) return fail(FTCJ_EUNSUPPORTED, "the tensor-core contraction needs an orthorhombic cell");
-    const bool f64 = P->precision == FTCJ_PREC_FP64;
+    const bool f64 = tc_eight_slices(P);
     const int nmax = f64 ? Prec64::kNmax : PrecRho::kNmax, slices = f64 ? Prec64::S : PrecRho::S;
     const int nprod = slices * (slices + 1) / 2;
     if (P->d_rec_gcut) return fail(FTCJ_EUNSUPPORTED, "the tensor-core contraction walks the whole sphere");
@@ -2077,14 +2092,14 @@ int setup_tc(ftcj_plan* P) {
     if ((rc = tc_upload(P, &P->d_tc_wpairs, wpairs))) return rc;
     if ((rc = tc_upload(P, &P->d_tc_pos, pos))) return rc;
     if ((rc = tc_upload(P, &P->d_tc_kpos, kpos))) return rc;
-    if (f64 && (rc = tc_upload(P, &P->d_tc_korder, korder))) return rc;
+    if (P->precision == FTCJ_PREC_FP64 && (rc = tc_upload(P, &P->d_tc_korder, korder))) return rc;
     FTCJ_CUDA(cudaMemcpy(P->d_tc_cl, clk.data(), sizeof(float) * nrec, cudaMemcpyHostToDevice));
-    if ((rc = tc_alloc(P, &P->d_tc_tab, sizeof(float4) * nrec * tws))) return rc;
+    if (!P->tc_rho_only && (rc = tc_alloc(P, &P->d_tc_tab, sizeof(float4) * nrec * tws))) return rc;
     if ((rc = tc_alloc(P, &P->d_tc_tabk, sizeof(float4) * nrec * tws))) return rc;
     if ((rc = tc_alloc(P, &P->d_tc_tabz, sizeof(float4) * nrec * P->tc_ncols))) return rc;
-    if (f64 && (rc = tc_alloc(P, &P->d_tc_tabz3, 2 * sizeof(float4) * nrec * P->tc_ncols))) return rc;
+    if (f64 && !P->tc_rho_only && (rc = tc_alloc(P, &P->d_tc_tabz3, 2 * sizeof(float4) * nrec * P->tc_ncols))) return rc;
     // the odd stride's spare entry is copied along but never read
-    FTCJ_CUDA(cudaMemset(P->d_tc_tab, 0, sizeof(float4) * nrec * tws));
+    if (P->d_tc_tab) FTCJ_CUDA(cudaMemset(P->d_tc_tab, 0, sizeof(float4) * nrec * tws));
     FTCJ_CUDA(cudaMemset(P->d_tc_tabk, 0, sizeof(float4) * nrec * tws));
     if (P->npairs > 0) {
         const long long n = P->npairs * (long long)(P->tc_nna + P->tc_nnb + P->tc_ncols);
@@ -2125,17 +2140,18 @@ int launch_tc_rho(ftcj_plan* P, int ndens, cudaStream_t s) {
     g.wcnt = P->d_tc_wcnt;
     g.boff = P->d_tc_boff;
     g.wpairs = P->d_tc_wpairs;
-    const bool f64 = P->precision == FTCJ_PREC_FP64;
+    const bool f64 = tc_eight_slices(P);
     g.tabk = P->d_tc_tabk;
     g.tabz = P->d_tc_tabz;
     g.korder = P->d_tc_korder;
     g.clk = P->d_tc_cl;
     for (int cc = 0; cc < kNclass; ++cc) g.kbase[cc] = P->class_start[cc];
     g.Dp = P->d_Dp;
-    g.dp_total = f64 ? P->total_terms : P->tc_dp_total;
+    const bool df_terms = P->precision == FTCJ_PREC_SPLIT;
+    g.dp_total = df_terms ? P->tc_dp_total : P->total_terms;
     for (int cc = 0; cc < kNclass; ++cc) {
-        g.dp_base[cc] = f64 ? P->term_base[cc] : P->tc_dp_base[cc];
-        g.dp_stride[cc] = f64 ? P->class_start[cc + 1] - P->class_start[cc] : P->tc_dp_stride[cc];
+        g.dp_base[cc] = df_terms ? P->tc_dp_base[cc] : P->term_base[cc];
+        g.dp_stride[cc] = df_terms ? P->tc_dp_stride[cc] : P->class_start[cc + 1] - P->class_start[cc];
     }
     g.bs = reinterpret_cast<uint4*>(P->d_tc_b);
     g.clw = P->d_tc_clw;
@@ -2167,8 +2183,9 @@ int launch_tc_rho(ftcj_plan* P, int ndens, cudaStream_t s) {
             g.w0 = ps.w0;
             g.out_row0 = ps.out_row0;
             g.sched = P->d_tc_sched + ps.sched;
-            if (f64) k_tc_rho_b<Prec64><<<(unsigned)ps.nwin, kTcBThreads, 0, s>>>(g);
-            else k_tc_rho_b<PrecRho><<<(unsigned)ps.nwin, kTcBThreads, 0, s>>>(g);
+            if (!f64) k_tc_rho_b<PrecRho, true><<<(unsigned)ps.nwin, kTcBThreads, 0, s>>>(g);
+            else if (df_terms) k_tc_rho_b<Prec64, true><<<(unsigned)ps.nwin, kTcBThreads, 0, s>>>(g);
+            else k_tc_rho_b<Prec64, false><<<(unsigned)ps.nwin, kTcBThreads, 0, s>>>(g);
             FTCJ_CUDA(cudaGetLastError());
             const dim3 grid((unsigned)ps.ngroups, (unsigned)P->tc_mtiles);
             int nbuf = P->tc_nbuf, nts = P->tc_tslots;
@@ -2190,7 +2207,8 @@ int tc_rho_launches(const ftcj_plan* P, int nd) {
 // factor tables exceed shared memory.
 int setup_tc_j(ftcj_plan* P) {
     P->tc_j = false;
-    const bool f64 = P->precision == FTCJ_PREC_FP64;
+    if (P->tc_rho_only) return FTCJ_OK;
+    const bool f64 = tc_eight_slices(P);
     const int nmax = f64 ? Prec64::kNmax : PrecJ::kNmax, slices = f64 ? Prec64::S : PrecJ::S;
     const int nprod = slices * (slices + 1) / 2, part_stages = (f64 ? Prec64::kWin : PrecJ::kWin) / kTcJStageM;
     const int gw = round_up(2 * P->tc_ncols, 8);
@@ -2314,7 +2332,7 @@ int launch_tc_j(ftcj_plan* P, int ndens, const double* W, cudaStream_t s) {
         FTCJ_CUDA(cudaMemsetAsync(P->d_Jp, 0, sizeof(double) * (size_t)ndens * P->tc_jparts * P->total_terms, s));
         return FTCJ_OK;
     }
-    const bool f64 = P->precision == FTCJ_PREC_FP64;
+    const bool f64 = tc_eight_slices(P);
     TcJArgs g;
     g.slots = P->d_tc_slots;
     g.quads = P->d_tc_quads;

@@ -88,3 +88,54 @@ def test_fp64_walks_agree_with_contraction(F):
     assert float(((Ea - Eb).abs() / Eb.abs().clamp_min(1.0)).max()) <= 1e-12
     a.close()
     b.close()
+
+
+#       edges               kmesh      omega  ndens  taken
+SPLIT_CELLS = [
+    ([11.0, 12.3, 11.6], (1, 1, 1), 0.42, 1, True),
+    ([9.1, 9.7, 18.0], (2, 1, 1), 0.45, 3, True),   # three densities, a long axis
+    ([26.0, 10.0, 8.0], (1, 1, 1), 0.40, 2, True),  # odd counts of records and points
+    ([6.3, 6.0, 5.7], (1, 2, 1), 0.40, 2, False),   # below 512 points: the walk
+]
+EVEN = [(c, l, [0.12 * 2.1 ** q for q in range(n)]) for c in range(4) for l, n in ((0, 9), (1, 5), (2, 2))]
+
+
+@pytest.mark.parametrize("index", range(len(SPLIT_CELLS)))
+def test_split_walk_plans_take_structure_factors_from_the_product(orc, F, index):
+    """Above the size rule a split plan's rho comes from the eight-slice product and its J' from the walk; both
+    against the oracle and a caller's own walk shape.  Bar: double-float steps of 2^-45, at most 40 along a chain
+    (the walk), 1e-10 of max|J| (at least 1); the gradient likewise."""
+    import torch
+    edges, kmesh, omega, ndens, taken = SPLIT_CELLS[index]
+    w = W.tiny(seed=90 + index, A=np.diag(edges), shell_spec=EVEN, kmesh=kmesh, omega=omega, ndens=ndens,
+               centres=[[0.1, 0.2, 0.3], [1.9, 0.9, -0.4], [0.7, 3.1, 1.0], [-1.2, 1.0, 2.6]])
+    ref = orc.lrj(w, want_j0n=False)
+    scale = max(1.0, float(np.abs(ref["Jk"]).max()))
+    Dk = torch.from_numpy(np.ascontiguousarray(w.Dk)).cuda()
+    got = []
+    for chunk in (0, 4096):
+        plan = F.Plan.from_workload(w, precision=F.FTCJ_PREC_SPLIT, chunk_points=chunk)
+        info = plan.info
+        want = F.FTCJ_CONTRACT_TC if taken and not chunk else F.FTCJ_CONTRACT_WALK
+        assert (info["contraction"], info["j_contraction"]) == (want, F.FTCJ_CONTRACT_WALK), info
+        Jk, EJ = plan.jbuild(Dk)
+        E2, grad = plan.grad(Dk)
+        J1, _ = plan.jbuild(Dk[-1:].contiguous())  # fewer densities than the plan holds
+        torch.cuda.synchronize()
+        assert plan.status() == 0
+        dJ = float(np.abs(Jk.cpu().numpy() - ref["Jk"]).max())
+        d1 = float(np.abs(J1.cpu().numpy() - ref["Jk"][-1:]).max())
+        dE = float((np.abs(EJ.cpu().numpy() - ref["EJ"]) / np.maximum(1.0, np.abs(ref["EJ"]))).max())
+        print(f"cell {index} chunk {chunk}: records {info['npairs']} points {info['ng_half']} max|dJ|={dJ:.2e} "
+              f"rel dE={dE:.2e}")
+        assert dJ <= 1e-10 * scale and d1 <= 1e-10 * scale and dE <= 1e-10
+        assert bool(torch.equal(E2, EJ))
+        got.append((rho_of(plan, Dk), grad))
+        plan.close()
+    (ra, ga), (rb, gb) = got
+    assert float((ra - rb).abs().max()) <= 1e-10 * max(1.0, float(rb.abs().max()))
+    assert float((ga - gb).abs().max()) <= 1e-10 * max(1.0, float(gb.abs().max()))
+
+
+def rho_of(plan, Dk):
+    return plan.rho(plan.fold_density(Dk))
