@@ -29,7 +29,7 @@ int rho_walk(ftcj_plan* P, int nd, cudaStream_t s) {
 }
 
 int j_walk(ftcj_plan* P, int nd, const double* W, cudaStream_t s) {
-    if (P->tc_j) return launch_tc_j(P, nd, W, s);
+    if (P->tcj.on) return launch_tc_j(P, nd, W, s);
     return P->precision == FTCJ_PREC_SPLIT ? launch_j_walk_split(P, nd, W, s) : launch_j_walk(P, nd, W, s);
 }
 
@@ -214,8 +214,9 @@ int ftcj_grad(ftcj_plan* P, int ndens, const double* Dk, double* EJ, double* gra
         if ((rc = launch_rho_reduce(P, nd, P->d_rho, P->d_W, EJ + b0, nullptr, s))) return rc;
         // the degree-(L+1) sums in the plan's form where FP32 holds their powers of n exactly
         const bool split = P->precision == FTCJ_PREC_SPLIT && split_grad_walk_exact(P);
-        if ((rc = split ? launch_j_walk_grad_split(P, nd, P->d_W, s) : launch_j_walk_grad(P, nd, P->d_W, s)))
-            return rc;
+        if (P->tcg.on) rc = launch_tc_j_grad(P, nd, P->d_W, s);
+        else rc = split ? launch_j_walk_grad_split(P, nd, P->d_W, s) : launch_j_walk_grad(P, nd, P->d_W, s);
+        if (rc) return rc;
         if ((rc = launch_grad_assemble(P, nd, P->d_D0n, grad + (size_t)b0 * P->ncentre * 3, s))) return rc;
     }
     return FTCJ_OK;

@@ -154,6 +154,25 @@ struct TcPass {
 
 }  // namespace ftcj
 
+// One back-contraction in the tensor-core form: shape, work units and the V_ij buffer.
+struct TcBack {
+    bool on = false;                             // false: the walks run it
+    int extra = 0;                               // degree of the sums beyond the record's class (gradient: 1)
+    int nd = 0, gw = 0, G = 0, npad = 0;         // densities per launch, columns per density, blocks per group, MMA N
+    int nstage = 0, grid = 0, nbuf = 0;          // 16-slot stages, CTAs, stage buffers
+    int parts = 0, spp = 0;                      // partial arrays of J' (slot parts x column splits), stages per part
+    int sub = 1;                                 // column splits of the epilogue
+    int64_t mma_flops = 0;                       // bf16 MMA flops of one pass over max_dens densities
+    void* items = nullptr;                       // int4 [units]: class | part << 8, first block group, block groups, first record
+    void* groups = nullptr;                      // int2 [groups]: first block, blocks
+    int* pairs = nullptr;                        // (i | j << 3) of the groups' blocks
+    int* sched = nullptr;                        // CTA offsets, then unit ids
+    void* vs = nullptr;                          // bf16 sliced V_ij stage tiles by block group
+    long long* voff = nullptr;                   // start of each block group's tiles
+    int* vplace = nullptr;                       // block groups that hold each (i, j)
+    int* ev = nullptr;                           // their column bounds
+};
+
 struct ftcj_plan {
     // geometry and parameters
     double A[9], B[9], M[9];
@@ -265,21 +284,8 @@ struct ftcj_plan {
     int* d_tc_pos = nullptr;     // [npairs]: position of each record in its class's K order
     float* d_tc_clw = nullptr;   // [nwin]: the windows' smallest widths
     long long tc_dp_base[ftcj::kNclass] = {}, tc_dp_stride[ftcj::kNclass] = {}, tc_dp_total = 0;
-    // tensor-core form of the back-contraction (tc.cu); false: the split walk runs it
-    bool tc_j = false;
-    int tc_jnd = 0, tc_jgw = 0, tc_jG = 0, tc_jnpad = 0;  // densities per launch, columns per density, blocks per group, MMA N
-    int tc_jnstage = 0, tc_jgrid = 0, tc_jnbuf = 0;         // 16-slot stages, CTAs, stage buffers
-    int tc_jparts = 0, tc_jspp = 0;                         // partial arrays of J' (slot parts x column splits), stages per part
-    int tc_jsub = 1;                                        // column splits of the epilogue
-    int64_t tc_j_mma_flops = 0;                             // bf16 MMA flops of one pass over max_dens densities
-    void* d_tc_jitems = nullptr;   // int4 [units]: class | part << 8, first block group, block groups, first record
-    void* d_tc_jgroups = nullptr;  // int2 [groups]: first block, blocks
-    int* d_tc_jpairs = nullptr;    // (i | j << 3) of the groups' blocks
-    int* d_tc_jsched = nullptr;    // CTA offsets, then unit ids
-    void* d_tc_vs = nullptr;       // bf16 sliced V_ij stage tiles by block group
-    long long* d_tc_voff = nullptr;  // start of each block group's tiles
-    int* d_tc_vplace = nullptr;    // block groups that hold each (i, j)
-    int* d_tc_ev = nullptr;        // their column bounds
+    // the back-contraction as a tensor-core product (tc.cu), of a build and of the nuclear gradient
+    TcBack tcj, tcg;
     int rho_rows = 0;            // partial rows the rho reduction sums (walk blocks or tensor-core groups)
     // density classification (Sec. 2.6): the records a plan keeps (0 all, 1 compact, 2 DD)
     int rec_filter = 0;
@@ -366,6 +372,7 @@ void release_tc(ftcj_plan* P);  // back to a plan without the tensor-core form
 int launch_tc_rho(ftcj_plan* P, int ndens, cudaStream_t s);
 int tc_rho_launches(const ftcj_plan* P, int nd);
 int launch_tc_j(ftcj_plan* P, int ndens, const double* W, cudaStream_t s);
+int launch_tc_j_grad(ftcj_plan* P, int ndens, const double* W, cudaStream_t s);
 // one persistent launch of the walks of a batch of cells (walk_split.cu)
 struct BatchWalks;
 int batch_walks_create(const std::vector<ftcj_plan*>& plans, BatchWalks** out);
@@ -376,7 +383,7 @@ void batch_walks_destroy(BatchWalks* bw);
 int tc_j_launches(const ftcj_plan* P, int nd);
 // partial back-contraction sums the J -> AO map adds: one per walk chunk, or per row part of the tensor-core form
 inline int jp_chunks(const ftcj_plan* P) {
-    return P->jp_fixed > 0 ? P->jp_fixed : (P->tc_j ? P->tc_jparts : (int)P->chunks.size());
+    return P->jp_fixed > 0 ? P->jp_fixed : (P->tcj.on ? P->tcj.parts : (int)P->chunks.size());
 }
 
 // --- GPW route of the DD pair densities (gpw.cu) ---

@@ -975,9 +975,9 @@ int setup_product(ftcj_plan* P, ftcj_plan* D) {
     D->n_abs_max = P->n_abs_max;
     int rc = setup_tc(D);
     if (rc) return rc;
-    if (!D->tc_j) return FTCJ_EUNSUPPORTED;
+    if (!D->tcj.on) return FTCJ_EUNSUPPORTED;
     double* jp = nullptr;
-    const size_t terms = (size_t)D->max_dens * (size_t)D->total_terms * (size_t)D->tc_jparts;
+    const size_t terms = (size_t)D->max_dens * (size_t)D->total_terms * (size_t)D->tcj.parts;
     const size_t rows = 2 * (size_t)D->max_dens * (size_t)D->tc_out_rows * (size_t)D->ng_half;
     if (cudaMalloc(&jp, sizeof(double) * terms) != cudaSuccess ||
         cudaMalloc(&D->d_rho_part, sizeof(double) * rows) != cudaSuccess) {
@@ -987,7 +987,7 @@ int setup_product(ftcj_plan* P, ftcj_plan* D) {
     }
     cudaFree(D->d_Jp);
     D->d_Jp = jp;
-    D->jp_fixed = D->tc_jparts;
+    D->jp_fixed = D->tcj.parts;
     D->tc = true;
     D->rho_rows = D->tc_out_rows;
     D->nEblocks = (int)std::max<int64_t>(1, (D->ng_half + kRedPoints - 1) / kRedPoints);

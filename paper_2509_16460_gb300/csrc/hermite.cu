@@ -318,7 +318,8 @@ int launch_grad_assemble(ftcj_plan* P, int ndens, const double* D0n, double* gra
     for (int c = 0; c < kNclass; ++c) lg.base[c] = P->term_base_g[c];
     lg.total = P->total_terms_g;
     dim3 g((unsigned)((P->npairs + 127) / 128), ndens);
-    k_grad_assemble<<<g, 128, 0, s>>>(P->d_pairs, P->d_groups, P->d_members, D0n, P->d_Jg, (int)P->chunks.size(),
+    k_grad_assemble<<<g, 128, 0, s>>>(P->d_pairs, P->d_groups, P->d_members, D0n, P->d_Jg,
+                                      P->tcg.on ? P->tcg.parts : (int)P->chunks.size(),
                                       P->nao, P->nk, lg, grad, P->ncentre, P->d_Tmat, P->cc);
     FTCJ_CUDA(cudaGetLastError());
     return FTCJ_OK;

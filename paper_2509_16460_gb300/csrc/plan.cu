@@ -590,7 +590,7 @@ int create(const ftcj_cell* cell, const ftcj_basis* basis, const int kmesh[3], c
         size_t room = 0, all = 0;
         FTCJ_CUDA(cudaMemGetInfo(&room, &all));
         // what the plan has yet to allocate, roughly
-        const size_t rest = 8 * md * (10 * (size_t)P->nk * nn + (size_t)(nch + 1) * (size_t)(P->total_terms + P->total_terms_g) +
+        const size_t rest = 8 * md * (10 * (size_t)P->nk * nn + (size_t)std::max(nch + 1, P->tcg.parts) * (size_t)(P->total_terms + P->total_terms_g) +
                                       2 * (size_t)std::max(P->npb, P->tc_out_rows) * (size_t)P->ng_half);
         if (rc == FTCJ_EUNSUPPORTED || rc == FTCJ_ENOMEM || (rc == FTCJ_OK && room < rest)) {
             release_tc(P);
@@ -609,7 +609,7 @@ int create(const ftcj_cell* cell, const ftcj_basis* basis, const int kmesh[3], c
     // the tensor-core layout pads each class to 16 positions (and the last bulk copy may read 16 past a class)
     if ((rc = dalloc(P, &P->d_Dp, md * (size_t)std::max<long long>(P->total_terms, P->tc_dp_total) + 64))) return rc;
     if ((rc = dalloc(P, &P->d_Jp, md * (size_t)std::max(nch, jp_chunks(P)) * (size_t)P->total_terms))) return rc;
-    if ((rc = dalloc(P, &P->d_Jg, md * (size_t)nch * (size_t)P->total_terms_g))) return rc;
+    if ((rc = dalloc(P, &P->d_Jg, md * (size_t)std::max(nch, P->tcg.parts) * (size_t)P->total_terms_g))) return rc;
     if ((rc = dalloc(P, &P->d_rho_part, 2 * md * (size_t)std::max(P->npb, P->rho_rows) * (size_t)P->ng_half)))
         return rc;
     if ((rc = dalloc(P, &P->d_rho, 2 * md * (size_t)P->ng_half))) return rc;
@@ -707,12 +707,12 @@ int ftcj_plan_info(const ftcj_plan* P, ftcj_info* o) {
     const bool walks = P->ng_half > 0 && !P->tiles.empty();
     o->rho_walk_launches = walks ? (P->tc ? tc_rho_launches(P, P->max_dens) : (P->rho_hi_tiles > 0 ? 2 : 1)) : 0;
     o->j_walk_launches =
-        walks ? (P->tc_j ? tc_j_launches(P, P->max_dens) : (P->precision == FTCJ_PREC_SPLIT ? split_j_launches(P) : 1))
+        walks ? (P->tcj.on ? tc_j_launches(P, P->max_dens) : (P->precision == FTCJ_PREC_SPLIT ? split_j_launches(P) : 1))
               : 0;
     o->contraction = P->tc ? FTCJ_CONTRACT_TC : FTCJ_CONTRACT_WALK;
     o->tc_mma_flops = P->tc ? P->tc_mma_flops : 0;
-    o->j_contraction = P->tc_j ? FTCJ_CONTRACT_TC : FTCJ_CONTRACT_WALK;
-    o->tc_j_mma_flops = P->tc_j ? P->tc_j_mma_flops : 0;
+    o->j_contraction = P->tcj.on ? FTCJ_CONTRACT_TC : FTCJ_CONTRACT_WALK;
+    o->tc_j_mma_flops = P->tcj.on ? P->tcj.mma_flops : 0;
     if (P->tc) {
         o->tc_column_axis = P->tc_axis[2];
         o->tc_rows = P->tc_rows;

@@ -1160,11 +1160,11 @@ __global__ void k_tc_tables(const PairWalk* __restrict__ walk, long long npairs,
     }
     const long long k = kpos[r];
     if (e < nna + nnb) {
-        if (tab) tab[r * tws + e] = v;  // tab, tabz3: the back-contraction's
+        tab[r * tws + e] = v;
         tabk[k * tws + e] = v;
     } else {
         tabz[k * nnc + n] = v;
-        if (F64 && tabz3) {
+        if (F64) {
             const double z[2] = {gval * c, -gval * s};
             for (int q = 0; q < 2; ++q) {
                 const float h = (float)z[q], m = (float)(z[q] - (double)h);
@@ -1319,14 +1319,16 @@ void tc_slots(const std::set<std::pair<int, int>>& pts, std::vector<int>& slots,
 
 constexpr int kTcJStageM = 16;       // slots per stage: one MMA k-step
 constexpr int kTcJAsliceBytes = kTcM * kTcJStageM * 2;        // 128 records x 16 K x bf16
-constexpr int kTcPairsAll = 15;      // (i, j) with i + j <= 4
 
-__host__ __device__ constexpr int pair_index(int i, int j) { return i * 5 - i * (i - 1) / 2 + j; }
+// the (i, j) with i + j <= deg (4, for the gradient 5) in a row
+__host__ __device__ constexpr int pairs_all(int deg) { return (deg + 1) * (deg + 2) / 2; }
 
-__device__ __forceinline__ void pair_of_index(int pr, int& i, int& j) {
+__host__ __device__ constexpr int pair_index(int deg, int i, int j) { return i * (deg + 1) - i * (i - 1) / 2 + j; }
+
+__device__ __forceinline__ void pair_of_index(int deg, int pr, int& i, int& j) {
     i = 0;
-    while (pr > 4 - i) {
-        pr -= 5 - i;
+    while (pr > deg - i) {
+        pr -= deg + 1 - i;
         ++i;
     }
     j = pr;
@@ -1342,13 +1344,13 @@ struct TcJArgs {
     const int2* groups;     // block groups: first index into ipairs, blocks
     const int* ipairs;      // (i | j << 3) of each block
     const long long* voff;  // start of each block group's V tiles in vs (elements)
-    const int* vplace;      // [15 (i, j)][kNclass]: block group << 8 | place of the block in it, -1 none
+    const int* vplace;      // [(i, j)][kNclass]: block group << 8 | place of the block in it, -1 none
     const void* tab;        // X(0..), Y(0..) as complex double-float or double, [tws] per record
     const void* tabz;       // Z(0..), [ncols] per record in the K order: complex double-float, or triple-float as two
                             // float4 (FP64 form)
     const int* kpos;        // position of each record in the K order of all classes
     __nv_bfloat16* vs;      // sliced V_ij: [block group][stage][slice][columns of its MMA x 16 K] stage tiles
-    int* ev;                // column bounds of V_ij: [15][nd][ncols]
+    int* ev;                // column bounds of V_ij: [(i, j)][nd][ncols]
     double* Jp;             // partial back-contraction sums [dens][part][term] in the split form's class layout
     long long ng_half;
     long long jp_total;     // doubles per density of Jp
@@ -1356,6 +1358,7 @@ struct TcJArgs {
     long long term_base[kNclass];
     int* err;               // device error word (bit 0: a bounded wait gave up)
     int ax, bx, cx;
+    int deg;                // largest i + j + k: 4, for the gradient's sums 5
     int nam, nbm;
     int tws, offY;          // table entries per record (odd: conflict-free across records), start of Y
     int ncols, nd, d0;
@@ -1410,7 +1413,7 @@ __global__ void __launch_bounds__(256) k_tc_vbound(TcJArgs g) {
     const int col = blockIdx.x;  // ((i, j) nd + d) ncols + n_c
     const int nc = col % g.ncols, d = (col / g.ncols) % g.nd, pr = col / (g.ncols * g.nd);
     int i, j;
-    pair_of_index(pr, i, j);
+    pair_of_index(g.deg, pr, i, j);
     float mx = 0.f;
     for (int m = threadIdx.x; m < g.nslots; m += blockDim.x) {
         mx = fmaxf(mx, v_abs(v_entry<P>(g, m, i, j, d, nc)));
@@ -1434,7 +1437,7 @@ __global__ void __launch_bounds__(256) k_tc_vslice(TcJArgs g) {
     constexpr int kS = P::S;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long per_pair = (long long)g.nstage * (kTcJStageM / 2) * g.nd * g.ncols;
-    if (t >= kTcPairsAll * per_pair) return;
+    if (t >= pairs_all(g.deg) * per_pair) return;
     const int pr = (int)(t / per_pair);
     long long rem = t - pr * per_pair;
     const int nc = (int)(rem % g.ncols);
@@ -1443,7 +1446,7 @@ __global__ void __launch_bounds__(256) k_tc_vslice(TcJArgs g) {
     rem /= g.nd;
     const int m2 = (int)(rem % (kTcJStageM / 2)), q = (int)(rem / (kTcJStageM / 2));
     int i, j;
-    pair_of_index(pr, i, j);
+    pair_of_index(g.deg, pr, i, j);
     const int ev = g.ev[(pr * g.nd + d) * g.ncols + nc];
     uint32_t sr[kS], si[kS];
     if constexpr (P::S == 8) {
@@ -1512,7 +1515,8 @@ struct TcJSmem {
 // tables and warp 18 the V_ij stage tiles in with bulk copies; warps 0-15 then
 // form J' from tensor memory (lane quadrant w & 3; (block, density) pairs,
 // their columns split further where a group has fewer than four, w / 4 mod 4).  Waits are bounded as in the structure-factor kernel.
-template <class P>
+// E = 1: the gradient's sums, one degree above the record's class.
+template <class P, int E>
 __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) {
     extern __shared__ __align__(1024) unsigned char tsm[];
     const int bbytes = P::S * g.npad * 32;
@@ -1718,10 +1722,10 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) 
                     (size_t)__ldg(g.kpos + (rvalid ? r : un.w)) * g.ncols * (P::S == 8 ? 2 : 1);
                 for (int ps = es; ps < gr.y * g.nd * g.nsub; ps += kTcProdWarps / 4) {
                     const int pd = ps / g.nsub, sub = ps - pd * g.nsub, gb = pd / g.nd, d = pd - gb * g.nd;
-                    const int pr = __ldg(g.ipairs + gr.x + gb), i = pr & 7, j = pr >> 3, nk = L - i - j;
-                    typename P::Sum J[5];
+                    const int pr = __ldg(g.ipairs + gr.x + gb), i = pr & 7, j = pr >> 3, nk = L + E - i - j;
+                    typename P::Sum J[5 + E];
 #pragma unroll
-                    for (int kk = 0; kk < 5; ++kk) J[kk] = sum_zero(typename P::Sum());
+                    for (int kk = 0; kk < 5 + E; ++kk) J[kk] = sum_zero(typename P::Sum());
                     for (int c4 = sub; c4 < g.gw / 4; c4 += g.nsub) {
                         float T[P::ACC][4];
                         typename P::Sum zr[2], zi[2];  // Z: double-float in one float4, triple-float in two
@@ -1755,12 +1759,13 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) 
                                     if (nk > 1) J[2] = tf_add(J[2], tf_mulf(re, x * x));
                                     if (nk > 2) J[3] = tf_add(J[3], tf_mulf(im, x * x * x));
                                     if (nk > 3) J[4] = tf_add(J[4], tf_mulf(re, x * x * x * x));
+                                    if (E && nk > 4) J[4 + E] = tf_add(J[4 + E], tf_mulf(im, x * x * x * x * x));
                                 }
                             } else {
                                 const cdf zu = cdf_mul_u(cdf{zr[u], zi[u]}, cdf{vr, vi});
                                 float pw = 1.f;
 #pragma unroll
-                                for (int kk = 0; kk < 5; ++kk) {
+                                for (int kk = 0; kk < 5 + E; ++kk) {
                                     if (kk <= nk) J[kk] = df_add(J[kk], df_mulf_u(kk & 1 ? zu.im : zu.re, pw));
                                     pw *= (float)nc;
                                 }
@@ -1771,7 +1776,7 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) 
                         double* jp = g.Jp + ((long long)(g.d0 + d) * g.nparts + part * g.nsub + sub) * g.jp_total + g.term_base[L] +
                                      (r - g.cls_start[L]);
 #pragma unroll
-                        for (int kk = 0; kk < 5; ++kk)
+                        for (int kk = 0; kk < 5 + E; ++kk)
                             if (kk <= nk) {
                                 const double v = sum_double(sum_mulf(J[kk], P::row_scale(1)));  // exact power of two
                                 jp[(long long)term_of(g.ax, g.bx, i, j, kk) * cnt] = kk == 2 || kk == 3 ? -v : v;
@@ -1801,6 +1806,12 @@ size_t tc_j_smem_bytes(int slices, int npad, int tws, int nbuf) {
 
 // work dealt to nbin bins, largest first, each to the least loaded bin (ties
 // to the lower one): nbin + 1 offsets, then the item ids of each bin
+// the gradient's sums keep to the eight-slice form (double-float or FP64 precision)
+const void* tc_j_kernel(bool f64, int extra) {
+    if (extra) return (const void*)k_tc_j<Prec64, 1>;
+    return f64 ? (const void*)k_tc_j<Prec64, 0> : (const void*)k_tc_j<PrecJ, 0>;
+}
+
 std::vector<int> deal(const std::vector<double>& cost, int nbin) {
     std::vector<int> order(cost.size());
     for (size_t k = 0; k < order.size(); ++k) order[k] = (int)k;
@@ -1833,13 +1844,15 @@ void release_tc(ftcj_plan* P) {
                      &P->d_tc_winfo, (void**)&P->d_tc_wcnt, (void**)&P->d_tc_boff, (void**)&P->d_tc_sched, &P->d_tc_b,
                      &P->d_tc_tab, &P->d_tc_tabk, &P->d_tc_tabz, &P->d_tc_tabz3, (void**)&P->d_tc_cl, (void**)&P->d_tc_kpos,
                      (void**)&P->d_tc_korder, (void**)&P->d_tc_err, (void**)&P->d_tc_pos, (void**)&P->d_tc_clw,
-                     &P->d_tc_jitems, &P->d_tc_jgroups, (void**)&P->d_tc_jpairs, (void**)&P->d_tc_jsched, &P->d_tc_vs,
-                     (void**)&P->d_tc_voff, (void**)&P->d_tc_vplace, (void**)&P->d_tc_ev};
+                     &P->tcj.items, &P->tcj.groups, (void**)&P->tcj.pairs, (void**)&P->tcj.sched, &P->tcj.vs,
+                     (void**)&P->tcj.voff, (void**)&P->tcj.vplace, (void**)&P->tcj.ev,
+                     &P->tcg.items, &P->tcg.groups, (void**)&P->tcg.pairs, (void**)&P->tcg.sched, &P->tcg.vs,
+                     (void**)&P->tcg.voff, (void**)&P->tcg.vplace, (void**)&P->tcg.ev};
     for (void** p : ptrs) {
         if (*p) cudaFree(*p);
         *p = nullptr;
     }
-    P->tc = P->tc_j = false;
+    P->tc = P->tcj.on = P->tcg.on = false;
     P->tc_dp_total = 0;
     P->tc_passes.clear();
 }
@@ -1849,7 +1862,7 @@ long long tc_spin(const ftcj_plan* P) {
     return P->params.tc_wait_log2 > 0 ? (1LL << P->params.tc_wait_log2) : kTcSpinCycles;
 }
 
-int setup_tc_j(ftcj_plan* P);
+int setup_tc_j(ftcj_plan* P, int extra);
 
 // Plan-time set-up of the tensor-core form: the column axis, the slots and the
 // half-sphere map, the factor tables, the windows (class, block group, records
@@ -2094,12 +2107,12 @@ int setup_tc(ftcj_plan* P) {
     if ((rc = tc_upload(P, &P->d_tc_kpos, kpos))) return rc;
     if (P->precision == FTCJ_PREC_FP64 && (rc = tc_upload(P, &P->d_tc_korder, korder))) return rc;
     FTCJ_CUDA(cudaMemcpy(P->d_tc_cl, clk.data(), sizeof(float) * nrec, cudaMemcpyHostToDevice));
-    if (!P->tc_rho_only && (rc = tc_alloc(P, &P->d_tc_tab, sizeof(float4) * nrec * tws))) return rc;
+    if ((rc = tc_alloc(P, &P->d_tc_tab, sizeof(float4) * nrec * tws))) return rc;
     if ((rc = tc_alloc(P, &P->d_tc_tabk, sizeof(float4) * nrec * tws))) return rc;
     if ((rc = tc_alloc(P, &P->d_tc_tabz, sizeof(float4) * nrec * P->tc_ncols))) return rc;
-    if (f64 && !P->tc_rho_only && (rc = tc_alloc(P, &P->d_tc_tabz3, 2 * sizeof(float4) * nrec * P->tc_ncols))) return rc;
+    if (f64 && (rc = tc_alloc(P, &P->d_tc_tabz3, 2 * sizeof(float4) * nrec * P->tc_ncols))) return rc;
     // the odd stride's spare entry is copied along but never read
-    if (P->d_tc_tab) FTCJ_CUDA(cudaMemset(P->d_tc_tab, 0, sizeof(float4) * nrec * tws));
+    FTCJ_CUDA(cudaMemset(P->d_tc_tab, 0, sizeof(float4) * nrec * tws));
     FTCJ_CUDA(cudaMemset(P->d_tc_tabk, 0, sizeof(float4) * nrec * tws));
     if (P->npairs > 0) {
         const long long n = P->npairs * (long long)(P->tc_nna + P->tc_nnb + P->tc_ncols);
@@ -2125,7 +2138,10 @@ int setup_tc(ftcj_plan* P) {
         if ((rc = allow_dynamic_smem(tc_rho_kernel(f64, round_up(2 * nd * P->tc_ncols, 8)),
                                      tc_smem_bytes(slices, P->tc_npad, tws, P->tc_nbuf, P->tc_tslots))))
             return rc;
-    return setup_tc_j(P);
+    if (!P->tc_rho_only && (rc = setup_tc_j(P, 0))) return rc;
+    // the gradient's sums, where ftcj_grad takes the plan and n^5 is exact in FP32
+    if (f64 && P->shard_count <= 1 && !P->rec_filter && split_grad_walk_exact(P)) return setup_tc_j(P, 1);
+    return FTCJ_OK;
 }
 
 int launch_tc_rho(ftcj_plan* P, int ndens, cudaStream_t s) {
@@ -2205,9 +2221,11 @@ int tc_rho_launches(const ftcj_plan* P, int nd) {
 // the V_ij tile buffer.  tc_j stays false, and the split walk runs the
 // back-contraction, where one density's columns exceed the MMA width or the
 // factor tables exceed shared memory.
-int setup_tc_j(ftcj_plan* P) {
-    P->tc_j = false;
-    if (P->tc_rho_only) return FTCJ_OK;
+int setup_tc_j(ftcj_plan* P, int extra) {
+    TcBack& B = extra ? P->tcg : P->tcj;
+    B.on = false;
+    B.extra = extra;
+    const int deg = kNclass - 1 + extra, npairs_all = pairs_all(deg);
     const bool f64 = tc_eight_slices(P);
     const int nmax = f64 ? Prec64::kNmax : PrecJ::kNmax, slices = f64 ? Prec64::S : PrecJ::S;
     const int nprod = slices * (slices + 1) / 2, part_stages = (f64 ? Prec64::kWin : PrecJ::kWin) / kTcJStageM;
@@ -2223,7 +2241,7 @@ int setup_tc_j(ftcj_plan* P) {
         const int G = std::min(kTcGmax, nmax / colw);
         double items = 0.0;
         for (int L = 0; L < kNclass; ++L) {
-            const int nb = (L + 1) * (L + 2) / 2;
+            const int nb = pairs_all(L + extra);
             items += (double)tiles[L] * ((nb + G - 1) / G);
         }
         const double cost = (double)((P->max_dens + nd - 1) / nd) * items;
@@ -2243,7 +2261,7 @@ int setup_tc_j(ftcj_plan* P) {
     int nbuf = kTcNbufMax;
     while (nbuf > 2 && tc_j_smem_bytes(slices, npad, tws, nbuf) > (size_t)optin) --nbuf;
     if (tc_j_smem_bytes(slices, npad, tws, nbuf) > (size_t)optin) return FTCJ_OK;
-    P->tc_jnbuf = nbuf;
+    B.nbuf = nbuf;
     // slot parts of one exact accumulation each (1024 slots, 512 in the FP64 form), as even as the stage count allows
     const int nstage = (P->tc_nslots + kTcJStageM - 1) / kTcJStageM;
     const int nsplit = std::max(1, (nstage + part_stages - 1) / part_stages);
@@ -2253,10 +2271,10 @@ int setup_tc_j(ftcj_plan* P) {
     std::vector<int> ipairs;
     std::vector<int4> units;
     std::vector<double> cost;
-    std::vector<int> vplace((size_t)kTcPairsAll * kNclass, -1);
+    std::vector<int> vplace((size_t)npairs_all * kNclass, -1);
     std::vector<long long> voff;
     long long nvs = 0;
-    P->tc_j_mma_flops = 0;
+    B.mma_flops = 0;
     // a unit holds all block groups of its class, or one group each where there are too few units to fill the GPU
     int64_t whole = 0;
     for (int L = 0; L < kNclass; ++L) whole += tiles[L] * nparts;
@@ -2264,13 +2282,13 @@ int setup_tc_j(ftcj_plan* P) {
     for (int L = kNclass - 1; L >= 0; --L) {
         if (!tiles[L]) continue;
         std::vector<int> blocks;
-        for (int i = 0; i <= L; ++i)
-            for (int j = 0; i + j <= L; ++j) blocks.push_back(i | (j << 3));
+        for (int i = 0; i <= L + extra; ++i)
+            for (int j = 0; i + j <= L + extra; ++j) blocks.push_back(i | (j << 3));
         const int first = (int)groups.size();
         for (size_t g0 = 0; g0 < blocks.size(); g0 += G_best) {
             const int nb = (int)std::min<size_t>(G_best, blocks.size() - g0);
             for (int k = 0; k < nb; ++k)
-                vplace[(size_t)pair_index(blocks[g0 + k] & 7, blocks[g0 + k] >> 3) * kNclass + L] =
+                vplace[(size_t)pair_index(deg, blocks[g0 + k] & 7, blocks[g0 + k] >> 3) * kNclass + L] =
                     (int)groups.size() << 8 | k;
             voff.push_back(nvs);
             nvs += (long long)nstage * slices * mma_cols(nb, nd_best * gw) * 16;
@@ -2288,7 +2306,7 @@ int setup_tc_j(ftcj_plan* P) {
                         const int nb = groups[first + g0 + k].y;
                         cc += nst * (nprod * (25.0 + 0.25 * mma_cols(nb, nd_best * gw)) + 500.0) + 110.0 * nb * nd_best * gw;
                         for (int d0 = 0; d0 < P->max_dens; d0 += nd_best)
-                            P->tc_j_mma_flops += (long long)nst * nprod * 2LL * kTcM *
+                            B.mma_flops += (long long)nst * nprod * 2LL * kTcM *
                                                  mma_cols(nb, std::min(nd_best, P->max_dens - d0) * gw) * 16;
                     }
                     units.push_back(make_int4(L | (h << 8), first + g0, n, (int)(P->class_start[L] + t * kTcM)));
@@ -2296,40 +2314,43 @@ int setup_tc_j(ftcj_plan* P) {
                 }
             }
     }
-    P->tc_jnd = nd_best;
-    P->tc_jgw = gw;
-    P->tc_jG = G_best;
-    P->tc_jnpad = npad;
-    P->tc_jnstage = nstage;
-    P->tc_jsub = std::max(1, 4 / (G_best * nd_best) == 3 ? 2 : 4 / (G_best * nd_best));
-    P->tc_jparts = nparts * P->tc_jsub;
-    P->tc_jspp = spp;
-    P->tc_jgrid = std::max(1, std::min(P->num_sms, (int)units.size()));
-    const std::vector<int> sched = deal(cost, P->tc_jgrid);
+    B.nd = nd_best;
+    B.gw = gw;
+    B.G = G_best;
+    B.npad = npad;
+    B.nstage = nstage;
+    B.sub = std::max(1, 4 / (G_best * nd_best) == 3 ? 2 : 4 / (G_best * nd_best));
+    B.parts = nparts * B.sub;
+    B.spp = spp;
+    B.grid = std::max(1, std::min(P->num_sms, (int)units.size()));
+    const std::vector<int> sched = deal(cost, B.grid);
     int rc;
     int4* units_dev = nullptr;
     if ((rc = tc_upload(P, &units_dev, units))) return rc;
-    P->d_tc_jitems = units_dev;
+    B.items = units_dev;
     int2* groups_dev = nullptr;
     if ((rc = tc_upload(P, &groups_dev, groups))) return rc;
-    P->d_tc_jgroups = groups_dev;
-    if ((rc = tc_upload(P, &P->d_tc_jpairs, ipairs))) return rc;
-    if ((rc = tc_upload(P, &P->d_tc_jsched, sched))) return rc;
-    if ((rc = tc_upload(P, &P->d_tc_voff, voff))) return rc;
-    if ((rc = tc_upload(P, &P->d_tc_vplace, vplace))) return rc;
+    B.groups = groups_dev;
+    if ((rc = tc_upload(P, &B.pairs, ipairs))) return rc;
+    if ((rc = tc_upload(P, &B.sched, sched))) return rc;
+    if ((rc = tc_upload(P, &B.voff, voff))) return rc;
+    if ((rc = tc_upload(P, &B.vplace, vplace))) return rc;
     nvs = std::max(nvs, 1LL);
-    if ((rc = tc_alloc(P, &P->d_tc_vs, sizeof(__nv_bfloat16) * (size_t)nvs))) return rc;
-    FTCJ_CUDA(cudaMemset(P->d_tc_vs, 0, sizeof(__nv_bfloat16) * (size_t)nvs));
-    const size_t nev = (size_t)kTcPairsAll * nd_best * P->tc_ncols;
-    if ((rc = tc_alloc(P, (void**)&P->d_tc_ev, sizeof(int) * nev))) return rc;
-    if ((rc = allow_dynamic_smem(f64 ? (const void*)k_tc_j<Prec64> : (const void*)k_tc_j<PrecJ>, tc_j_smem_bytes(slices, npad, tws, nbuf)))) return rc;
-    P->tc_j = true;
+    if ((rc = tc_alloc(P, &B.vs, sizeof(__nv_bfloat16) * (size_t)nvs))) return rc;
+    FTCJ_CUDA(cudaMemset(B.vs, 0, sizeof(__nv_bfloat16) * (size_t)nvs));
+    const size_t nev = (size_t)npairs_all * nd_best * P->tc_ncols;
+    if ((rc = tc_alloc(P, (void**)&B.ev, sizeof(int) * nev))) return rc;
+    if ((rc = allow_dynamic_smem(tc_j_kernel(f64, extra), tc_j_smem_bytes(slices, npad, tws, nbuf)))) return rc;
+    B.on = true;
     return FTCJ_OK;
 }
 
-int launch_tc_j(ftcj_plan* P, int ndens, const double* W, cudaStream_t s) {
+namespace {
+
+int launch_back(ftcj_plan* P, const TcBack& B, int ndens, const double* W, double* Jp, long long jp_total,
+                const int64_t* term_base, cudaStream_t s) {
     if (P->ng_half == 0 || P->npairs == 0) {
-        FTCJ_CUDA(cudaMemsetAsync(P->d_Jp, 0, sizeof(double) * (size_t)ndens * P->tc_jparts * P->total_terms, s));
+        FTCJ_CUDA(cudaMemsetAsync(Jp, 0, sizeof(double) * (size_t)ndens * B.parts * jp_total, s));
         return FTCJ_OK;
     }
     const bool f64 = tc_eight_slices(P);
@@ -2338,22 +2359,23 @@ int launch_tc_j(ftcj_plan* P, int ndens, const double* W, cudaStream_t s) {
     g.quads = P->d_tc_quads;
     g.map = P->d_tc_map;
     g.W = reinterpret_cast<const double2*>(W);
-    g.sched = P->d_tc_jsched;
-    g.units = reinterpret_cast<const int4*>(P->d_tc_jitems);
-    g.groups = reinterpret_cast<const int2*>(P->d_tc_jgroups);
-    g.ipairs = P->d_tc_jpairs;
-    g.voff = P->d_tc_voff;
-    g.vplace = P->d_tc_vplace;
+    g.sched = B.sched;
+    g.units = reinterpret_cast<const int4*>(B.items);
+    g.groups = reinterpret_cast<const int2*>(B.groups);
+    g.ipairs = B.pairs;
+    g.voff = B.voff;
+    g.vplace = B.vplace;
     g.tab = P->d_tc_tab;
     g.tabz = f64 ? P->d_tc_tabz3 : P->d_tc_tabz;
     g.kpos = P->d_tc_kpos;
-    g.vs = reinterpret_cast<__nv_bfloat16*>(P->d_tc_vs);
-    g.ev = P->d_tc_ev;
-    g.Jp = P->d_Jp;
+    g.vs = reinterpret_cast<__nv_bfloat16*>(B.vs);
+    g.ev = B.ev;
+    g.Jp = Jp;
+    g.deg = kNclass - 1 + B.extra;
     g.ng_half = P->ng_half;
-    g.jp_total = P->total_terms;
+    g.jp_total = jp_total;
     for (int c = 0; c <= kNclass; ++c) g.cls_start[c] = P->class_start[c];
-    for (int c = 0; c < kNclass; ++c) g.term_base[c] = P->term_base[c];
+    for (int c = 0; c < kNclass; ++c) g.term_base[c] = term_base[c];
     g.err = P->d_tc_err;
     g.ax = P->tc_axis[0];
     g.bx = P->tc_axis[1];
@@ -2363,36 +2385,47 @@ int launch_tc_j(ftcj_plan* P, int ndens, const double* W, cudaStream_t s) {
     g.tws = P->tc_tws;
     g.offY = P->tc_nna;
     g.ncols = P->tc_ncols;
-    g.gw = P->tc_jgw;
+    g.gw = B.gw;
     g.nslots = P->tc_nslots;
-    g.nstage = P->tc_jnstage;
-    g.nparts = P->tc_jparts;
-    g.nsub = P->tc_jsub;
+    g.nstage = B.nstage;
+    g.nparts = B.parts;
+    g.nsub = B.sub;
     g.spin = tc_spin(P);
-    g.spp = P->tc_jspp;
-    const size_t smem = tc_j_smem_bytes(f64 ? Prec64::S : PrecJ::S, P->tc_jnpad, P->tc_tws, P->tc_jnbuf);
-    for (int d0 = 0; d0 < ndens; d0 += P->tc_jnd) {
+    g.spp = B.spp;
+    const size_t smem = tc_j_smem_bytes(f64 ? Prec64::S : PrecJ::S, B.npad, P->tc_tws, B.nbuf);
+    for (int d0 = 0; d0 < ndens; d0 += B.nd) {
         g.d0 = d0;
-        g.nd = std::min(P->tc_jnd, ndens - d0);
+        g.nd = std::min(B.nd, ndens - d0);
         // the plan's block count is kept; a smaller last density group only narrows each block
         g.colw = g.nd * g.gw;
-        g.npad = mma_cols(P->tc_jG, g.colw);
-        const unsigned nbound = (unsigned)(kTcPairsAll * g.nd * g.ncols);
+        g.npad = mma_cols(B.G, g.colw);
+        const unsigned nbound = (unsigned)(pairs_all(g.deg) * g.nd * g.ncols);
         if (f64) k_tc_vbound<Prec64><<<nbound, 256, 0, s>>>(g);
         else k_tc_vbound<PrecJ><<<nbound, 256, 0, s>>>(g);
         FTCJ_CUDA(cudaGetLastError());
-        const long long nv = (long long)kTcPairsAll * g.nstage * (kTcJStageM / 2) * g.nd * g.ncols;
+        const long long nv = (long long)pairs_all(g.deg) * g.nstage * (kTcJStageM / 2) * g.nd * g.ncols;
         const unsigned nslice = (unsigned)((nv + 255) / 256);
         if (f64) k_tc_vslice<Prec64><<<nslice, 256, 0, s>>>(g);
         else k_tc_vslice<PrecJ><<<nslice, 256, 0, s>>>(g);
         FTCJ_CUDA(cudaGetLastError());
-        if (f64) k_tc_j<Prec64><<<(unsigned)P->tc_jgrid, kTcThreadsAll, smem, s>>>(g, P->tc_jnbuf);
-        else k_tc_j<PrecJ><<<(unsigned)P->tc_jgrid, kTcThreadsAll, smem, s>>>(g, P->tc_jnbuf);
-        FTCJ_CUDA(cudaGetLastError());
+        int nbuf = B.nbuf;
+        void* args[] = {&g, &nbuf};
+        FTCJ_CUDA(cudaLaunchKernel(tc_j_kernel(f64, B.extra), dim3((unsigned)B.grid), dim3(kTcThreadsAll), args, smem, s));
     }
     return FTCJ_OK;
 }
 
-int tc_j_launches(const ftcj_plan* P, int nd) { return 3 * ((nd + P->tc_jnd - 1) / P->tc_jnd); }
+}  // namespace
+
+int launch_tc_j(ftcj_plan* P, int ndens, const double* W, cudaStream_t s) {
+    return launch_back(P, P->tcj, ndens, W, P->d_Jp, P->total_terms, P->term_base, s);
+}
+
+// the degree-(L+1) sums of the nuclear gradient, into d_Jg
+int launch_tc_j_grad(ftcj_plan* P, int ndens, const double* W, cudaStream_t s) {
+    return launch_back(P, P->tcg, ndens, W, P->d_Jg, P->total_terms_g, P->term_base_g, s);
+}
+
+int tc_j_launches(const ftcj_plan* P, int nd) { return 3 * ((nd + P->tcj.nd - 1) / P->tcj.nd); }
 
 }  // namespace ftcj

@@ -139,3 +139,29 @@ def test_split_walk_plans_take_structure_factors_from_the_product(orc, F, index)
 
 def rho_of(plan, Dk):
     return plan.rho(plan.fold_density(Dk))
+
+
+@pytest.mark.parametrize("index", range(len(CELLS)))
+def test_gradient_sums_of_the_product(orc, F, index):
+    """The degree-(L+1) sums of the FP64 form's gradient from the product, against the oracle and the walks.  Bar: the
+    derivative's terms are at most 2 alpha n^5 times the build's, held to 2^-42 of their bounds as above; 1e-10 of
+    max|dE/dR| (at least 1) leaves room for the cancellation between the two centres."""
+    import torch
+    w = cell(index)
+    Dk = torch.from_numpy(np.ascontiguousarray(w.Dk)).cuda()
+    ref = orc.grad(w)
+    scale = max(1.0, float(np.abs(ref).max()))
+    got = []
+    for chunk in (0, 4096):
+        plan = F.Plan.from_workload(w, chunk_points=chunk)
+        _, grad = plan.grad(Dk)
+        _, last = plan.grad(Dk[-1:].contiguous())  # fewer densities than the plan holds
+        torch.cuda.synchronize()
+        assert plan.status() == 0
+        got.append(grad.cpu().numpy())
+        err = float(np.abs(got[-1] - ref).max())
+        print(f"cell {index} chunk {chunk}: max|dgrad|={err:.2e} of {scale:.2e}")
+        assert err <= 1e-10 * scale
+        assert float(np.abs(last.cpu().numpy() - ref[-1:]).max()) <= 1e-10 * scale
+        plan.close()
+    assert float(np.abs(got[0] - got[1]).max()) <= 1e-10 * scale
