@@ -69,3 +69,23 @@ def test_triclinic_walks_against_the_oracle(orc, F, edges, omega):
             print(f"edges {edges} precision {precision} chunk {chunk}: max|dJ|={dJ:.2e} max|dE|={dE:.2e}")
             assert dJ <= tol and dE <= tol * max(1.0, float(np.abs(ref["EJ"]).max()))
             plan.close()
+
+
+@pytest.mark.parametrize("centres,exps", [(1, [0.4]), (2, [0.5, 1.4]), (7, [0.6])])
+def test_gradient_assembly_over_few_and_many_centres(orc, F, centres, exps):
+    """Blocks of 32 records: fewer than 32, more than four centres within a warp, a ragged last block.  Bar: FP64
+    sums of up to 1e4 terms, 1e-10 of max|dE/dR| (at least 1)."""
+    import torch
+    rng = np.random.default_rng(centres)
+    spec = [(c, l, exps) for c in range(centres) for l in ((0, 2) if c % 2 else (0, 1))]
+    w = W.tiny(seed=70 + centres, A=np.array([[5.0, 0.0, 0.0], [0.6, 5.4, 0.0], [-0.3, 0.8, 5.2]]), shell_spec=spec,
+               centres=(rng.random((centres, 3)) * 4.0).tolist(), kmesh=(1, 2, 1), omega=0.4, ndens=2)
+    ref = orc.grad(w)
+    for precision in (F.FTCJ_PREC_FP64, F.FTCJ_PREC_SPLIT):
+        plan = F.Plan.from_workload(w, precision=precision)
+        _, grad = plan.grad(torch.from_numpy(np.ascontiguousarray(w.Dk)).cuda())
+        torch.cuda.synchronize()
+        err = float(np.abs(grad.cpu().numpy() - ref).max())
+        print(f"{centres} centres precision {precision}: records {plan.info['npairs']} max|dgrad|={err:.2e}")
+        assert err <= 1e-10 * max(1.0, float(np.abs(ref).max()))
+        plan.close()
