@@ -180,8 +180,9 @@ typedef struct {
                                       work actually done in the units of pair_g_units */
     int n_abs_max;            /* largest |n_i| of the sphere's G = sum_i n_i b_i (the split form
                                  needs <= 63) */
-    int grad_split;           /* 1: ftcj_grad's back-contraction runs in double-float (split
-                                 form with n_abs_max <= 27), 0: in FP64 */
+    int grad_split;           /* 1: the plan's gradient walk is the double-float one (split form
+                                 with n_abs_max <= 27), 0: the FP64 one; plans whose contraction
+                                 is TC by themselves and n_abs_max <= 27 run the sliced product */
     int rho_walk_launches;    /* kernel launches of one structure-factor walk pass: 2 where the
                                  split form runs it as two class parts, else 1 (0: nothing to walk) */
     int j_walk_launches;      /* the same for the back-contraction walk */
@@ -326,7 +327,9 @@ int ftcj_unfold_j(ftcj_plan* plan, int ndens, const double* J0n, double* Jk, voi
  * The derivative of E_J with respect to D^k is J^k/Nk (ftcj_jbuild).
  * Runs a2..a5 and a back-contraction one degree higher than the build's,
  * in the plan's form (split: double-float on the FP32 pipe where every
- * |n_i| <= 27, so that FP32 holds the fifth powers exactly; else FP64),
+ * |n_i| <= 27, so that FP32 holds the fifth powers exactly; else FP64; with
+ * that bound, plans that take the eight-slice product by themselves (see
+ * ftcj_params.contraction) run these sums as one too),
  * followed by an FP64 assembly per centre.  With pair_gcut_eps > 0 the
  * double-float back-contraction walks the same points as the build's, so the
  * result is the derivative of the screened energy that ftcj_jbuild returns

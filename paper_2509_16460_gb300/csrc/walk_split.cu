@@ -31,7 +31,6 @@ constexpr int kSBatch = 8;  // points per reduction batch of the split rho walk 
 // crystal with per-pair cutoffs: 4.93 -> 4.22 ms and 3.16 -> 2.82).
 enum : int { kRec = 0, kOrtho = 1 };
 
-
 struct Layout {
     long long start[kNclass + 1];
     long long base[kNclass];
@@ -412,7 +411,7 @@ __device__ void rho_tile_split(const Tile& tl, const Layout& lay, const float2* 
                     }
         }
         if (ORTHO) {
-            // the line value gp(0) goes into the coefficients; X(n1) (and u^n1) carry the rest
+            // the line value gp(0) goes into the coefficients; X(n1) carries the rest
 #pragma unroll
             for (int i = 0; i <= L; ++i) c[i] = cdf_mul_u(s.gpL, c[i]);
         }
