@@ -229,11 +229,19 @@ int default_split_chunk(ftcj_plan* P) {
 // triclinic cell of 108 AOs, split form: a build 470 -> 242 us.
 int balance_chunks(ftcj_plan* P) {
     const int64_t tiles = (int64_t)P->tiles.size(), want = 4 * (int64_t)P->num_sms;
-    if (tiles == 0 || tiles * (int64_t)P->chunks.size() >= want) return FTCJ_OK;
-    const int64_t nch = (want + tiles - 1) / tiles;
     int longest = 1;
     for (const WLine& l : P->lines) longest = std::max(longest, l.hi - l.lo + 1);
-    const int chunk = (int)std::max<int64_t>({(P->ng_half + nch - 1) / nch, 48, longest});
+    int chunk;
+    if (tiles == 0 || tiles * (int64_t)P->chunks.size() >= want) {
+        // persistent blocks, a fixed number for every chunk: even chunks, or those of a short last one leave their
+        // SMs idle (24 centres, 1,354 points as 1024 + 330: structure factors 2631 -> 2035 us as 2 x 677)
+        const int64_t nch = (int64_t)P->chunks.size();
+        if (tiles < want || nch < 2) return FTCJ_OK;
+        chunk = (int)((P->ng_half + nch - 1) / nch + longest);  // no more chunks than there are
+    } else {
+        const int64_t nch = (want + tiles - 1) / tiles;
+        chunk = (int)std::max<int64_t>({(P->ng_half + nch - 1) / nch, 48, longest});
+    }
     if (chunk >= P->max_chunk_pts) return FTCJ_OK;
     P->chunk_max = chunk;
     return build_walk(P);
@@ -548,7 +556,10 @@ int create(const ftcj_cell* cell, const ftcj_basis* basis, const int kmesh[3], c
         if ((rc = rho_walk_blocks_per_sm(P, &bps))) return rc;
     }
     int nch = std::max<int>(1, (int)P->chunks.size());
-    P->npb = std::max(1, std::min<int>((int)std::max<size_t>(1, P->tiles.size()), P->num_sms * bps / nch));
+    // with per-pair cutoffs the outer chunks hold little of most tiles: more blocks than fit at once even that out
+    // (molecular crystal, a build: 7.57 ms with one wave of blocks, 7.47 with two, 7.45 with four, 7.37 with six)
+    const int waves = P->precision == FTCJ_PREC_SPLIT && P->d_rec_gcut && nch > 1 ? 6 : 1;
+    P->npb = std::max(1, std::min<int>((int)std::max<size_t>(1, P->tiles.size()), waves * P->num_sms * bps / nch));
     // several short chunks of few tiles: one block per (tile, chunk), dealt by the hardware, comes out more even than
     // one wave of blocks of which some hold two tiles
     if (nch > 1 && P->tiles.size() < 4 * (size_t)P->num_sms && prm->chunk_points <= 0)
@@ -563,8 +574,8 @@ int create(const ftcj_cell* cell, const ftcj_basis* basis, const int kmesh[3], c
         if ((rc = rho_walk_split_blocks_per_sm(P, 2, &bps_hi))) return rc;
         if ((rc = rho_walk_split_blocks_per_sm(P, 1, &bps_lo))) return rc;
         const int nlo = (int)P->tiles.size() - P->rho_hi_tiles;
-        P->npb_hi = std::max(1, std::min(P->rho_hi_tiles, P->num_sms * bps_hi / nch));
-        P->npb = P->npb_hi + std::max(1, std::min(nlo, P->num_sms * bps_lo / nch));
+        P->npb_hi = std::max(1, std::min(P->rho_hi_tiles, waves * P->num_sms * bps_hi / nch));
+        P->npb = P->npb_hi + std::max(1, std::min(nlo, waves * P->num_sms * bps_lo / nch));
     }
     if ((rc = build_rho_schedule(P))) return rc;
     if (P->tc && !P->ortho) return fail(FTCJ_EUNSUPPORTED, "the tensor-core contraction needs an orthorhombic cell");
