@@ -126,6 +126,15 @@ __device__ __forceinline__ bool locate(const MapThreads& mt, long long gid, int&
     return false;
 }
 
+// where D'_t of record i (class c) of density d goes: the walks' layout, or the
+// tensor-core form's K order where that form reads the split form's terms
+__device__ __forceinline__ long long term_offset(const MapLayout& lay, const TermDest& dst, int d, int c, int t,
+                                                 long long i) {
+    return dst.pos ? (long long)d * dst.total + dst.base[c] + (long long)t * dst.stride[c] + dst.pos[i]
+                   : (long long)d * lay.total + lay.base[c] + (i - lay.start[c]) +
+                         (long long)t * (lay.start[c + 1] - lay.start[c]);
+}
+
 // a3: one thread per (record, term): D'_term = sum over member pairs, f, q of
 // M[f][q][term] times the combined density element
 template <bool OUT_DF>
@@ -134,7 +143,7 @@ __global__ void __launch_bounds__(256) k_hermite_map(const PairDev* __restrict__
                                                      const MemberDev* __restrict__ mem,
                                                      const long long* __restrict__ moff,
                                                      const double* __restrict__ maps, const double* __restrict__ D0n,
-                                                     int nao, int nk, MapLayout lay, MapThreads mt,
+                                                     int nao, int nk, MapLayout lay, MapThreads mt, TermDest dst,
                                                      double* __restrict__ Dp) {
     const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int d = blockIdx.y;
@@ -167,13 +176,13 @@ __global__ void __launch_bounds__(256) k_hermite_map(const PairDev* __restrict__
             M += (long long)NT * nfa * nfb;
         }
     }
-    const long long off = (long long)d * lay.total + lay.base[L] + (i - lay.start[L]) +
-                          (long long)t * (lay.start[L + 1] - lay.start[L]);
     if (OUT_DF) {
+        const long long off = term_offset(lay, dst, d, L, t, i);
         const float hi = (float)acc;
         reinterpret_cast<float2*>(Dp)[off] = make_float2(hi, (float)(acc - (double)hi));
     } else {
-        Dp[off] = acc;
+        // FP64 plans keep the record order in both forms
+        Dp[term_offset(lay, TermDest{}, d, L, t, i)] = acc;
     }
 }
 
@@ -317,10 +326,7 @@ __global__ void __launch_bounds__(256) k_hermite_map_df(const PairDev* __restric
         const float2 x = v[e];
         acc = df_add(acc, df_mul_u(df{m.x, m.y}, df{x.x, x.y}));
     }
-    const long long off = dst.pos ? (long long)d * dst.total + dst.base[c] + (long long)t * dst.stride[c] + dst.pos[i]
-                                  : (long long)d * lay.total + lay.base[c] + (i - lay.start[c]) +
-                                        (long long)t * (lay.start[c + 1] - lay.start[c]);
-    Dp[off] = make_float2(acc.hi, acc.lo);
+    Dp[term_offset(lay, dst, d, c, t, i)] = make_float2(acc.hi, acc.lo);
 }
 
 __global__ void __launch_bounds__(256) k_jtransform_map_df(const PairDev* __restrict__ pairs,
@@ -608,10 +614,10 @@ int launch_hermite_map(ftcj_plan* P, int ndens, const double* D0n, cudaStream_t 
     dim3 g((unsigned)((n + 255) / 256), ndens);
     if (P->precision == FTCJ_PREC_SPLIT)
         k_hermite_map<true><<<g, 256, 0, s>>>(P->d_pairs, P->d_groups, P->d_members, P->d_map_off, P->d_maps, D0n,
-                                              P->nao, P->nk, make_map_layout(P), P->mt_terms, P->d_Dp);
+                                              P->nao, P->nk, make_map_layout(P), P->mt_terms, term_dest(P), P->d_Dp);
     else
         k_hermite_map<false><<<g, 256, 0, s>>>(P->d_pairs, P->d_groups, P->d_members, P->d_map_off, P->d_maps, D0n,
-                                               P->nao, P->nk, make_map_layout(P), P->mt_terms, P->d_Dp);
+                                               P->nao, P->nk, make_map_layout(P), P->mt_terms, TermDest{}, P->d_Dp);
     FTCJ_CUDA(cudaGetLastError());
     return FTCJ_OK;
 }
