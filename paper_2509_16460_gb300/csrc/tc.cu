@@ -103,6 +103,10 @@ constexpr int kTcTabSlotsMax = 6;              // stage tables in flight at most
 constexpr int kTcAsliceBytes = kTcM * kTcStageK * 2;      // 128 rows x 16 K x bf16
 constexpr long long kTcBWorkMax = 8LL << 30;              // bytes of B tiles per pass
 constexpr long long kTcSpinCycles = 1LL << 32;            // ~2 s of SM clock per wait
+// Exponent bound of a column with a NaN or an infinity.  Slices hold neither
+// (their digits come from integer operations or cancelling sums), so the sums
+// of such a column become NaN where they leave the product.
+constexpr int kNonFinite = 1 << 20;
 
 // a slot: bits 0-7 |n_a|, 8-15 |n_b|, 16 ta, 17 tb, 18 / 19: the lane's bit 0
 // (1) is the sign of n_a (n_b), 20: valid
@@ -133,6 +137,7 @@ struct TcArgs {
     long long dp_stride[kNclass];
     uint4* bs;           // sliced B stage tiles of this pass
     float* clw;          // [nwin]: smallest c log2(e) of each window's records
+    int* ew;             // [nwin][nd]: kNonFinite where a term of the window's records is not finite, else 0
     double2* out;        // partial rows [dens][out_rows][ng_half], this pass's from out_row0
     long long ng_half;
     int out_rows, out_row0;
@@ -343,6 +348,8 @@ __device__ __forceinline__ double tf_double(tf a) { return widen(a.h) + (widen(a
 // Operations that the kernels need on their sums, double-float or triple-float
 __device__ __forceinline__ df sum_zero(df) { return df{0.f, 0.f}; }
 __device__ __forceinline__ tf sum_zero(tf) { return tf{0.f, 0.f, 0.f}; }
+__device__ __forceinline__ df sum_nan(df) { return df{NAN, 0.f}; }
+__device__ __forceinline__ tf sum_nan(tf) { return tf{NAN, 0.f, 0.f}; }
 __device__ __forceinline__ df sum_neg(df a) { return df_neg(a); }
 __device__ __forceinline__ tf sum_neg(tf a) { return tf{-a.h, -a.m, -a.l}; }
 __device__ __forceinline__ df sum_add(df a, df b) { return df_add(a, b); }
@@ -644,13 +651,15 @@ __global__ void __launch_bounds__(kTcBThreads, P::S == 8 ? 1 : 2) k_tc_rho_b(TcA
     constexpr bool kF64 = P::S == 8;
     static_assert(kF64 || DF, "the six-slice operands are cut from double-float terms");
     constexpr int kS = P::S;
-    __shared__ int mx[kTcNmax / 2];  // bits of the column bounds (non-negative floats order as integers)
+    __shared__ int mx[kTcNmax / 2];  // bits of the column bounds (non-negative floats order as integers, NaN on top)
+    __shared__ int bad[kTcNmax / 2];
     __shared__ int pairs[kTcGmax], tidx[kTcGmax][5];
     __shared__ int clmin_bits;
     const int w = g.w0 + blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     const int4 wi = __ldg(g.winfo + w);
     const int L = wi.x, npair = wi.y, npo = g.nd * g.ncols, cnt = __ldg(g.wcnt + w);
     for (int i = tid; i < npair * npo; i += blockDim.x) mx[i] = 0;
+    if (tid < g.nd) bad[tid] = 0;
     if (tid < npair) {
         const int pr = __ldg(g.wpairs + wi.z + tid), i = pr & 7, j = pr >> 3;
         pairs[tid] = pr;
@@ -690,20 +699,22 @@ __global__ void __launch_bounds__(kTcBThreads, P::S == 8 ? 1 : 2) k_tc_rho_b(TcA
             }
             for (int nc = 0; nc < g.ncols; ++nc) {
                 const float x = (float)nc, mq = -g.Mcc * x * x;
-                float m = 0.f;
+                unsigned m = 0u;
 #pragma unroll
                 for (int q = 0; q < kIt; ++q) {
                     const float sv = cm[q][0] + x * (cm[q][1] + x * (cm[q][2] + x * (cm[q][3] + x * cm[q][4])));
-                    m = fmaxf(m, sv * exp2f(cr[q] * mq));
+                    m = max(m, __float_as_uint(sv * exp2f(cr[q] * mq)) & 0x7fffffffu);
                 }
-                const unsigned mb = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+                const unsigned mb = __reduce_max_sync(0xffffffffu, m);
                 if (lane == 0 && mb) atomicMax(&mx[gb * npo + nc * g.nd + d], (int)mb);
+                if (lane == 0 && mb >= 0x7f800000u) bad[d] = 1;
             }
         }
     for (int o = 16; o > 0; o >>= 1) cmin = fminf(cmin, __shfl_xor_sync(0xffffffffu, cmin, o));
     if (lane == 0 && cmin < INFINITY) atomicMin(&clmin_bits, __float_as_int(cmin));
     __syncthreads();
     if (tid == 0) g.clw[w] = __int_as_float(clmin_bits);
+    if (tid < g.nd) g.ew[w * g.nd + tid] = bad[tid] ? kNonFinite : 0;
     const int nst = (cnt + kTcStageK - 1) / kTcStageK, npc = (npo + 3) / 4, nw = mma_cols(npair, g.colw);
     uint4* base = g.bs + __ldg(g.boff + w);
     const int ntask = nst * npair * npc * 16;
@@ -717,7 +728,7 @@ __global__ void __launch_bounds__(kTcBThreads, P::S == 8 ? 1 : 2) k_tc_rho_b(TcA
         const int pr = pairs[gb], nk = L - (pr & 7) - (pr >> 3);  // k = 0 .. L - i - j
         const int k0 = q * kTcStageK + oc * 8 + half * 4;
         const float mb = __int_as_float(mx[gb * npo + p]);
-        const int eb = mb > 0.f ? bound_exp<P>(log2f(mb)) : -60;
+        const int eb = bad[d] ? kNonFinite : mb > 0.f ? bound_exp<P>(log2f(mb)) : -60;
         uint32_t s0[kS][2], s1[kS][2];
         if constexpr (kF64) {
             const float sc = pow2f(eb - 6);  // B's digits carry their column's bound
@@ -1028,6 +1039,13 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf,
             const int4 wi = __ldg(g.winfo + w);
             const uint32_t nw = (uint32_t)mma_cols(wi.y, g.colw);
             const float rsc = P::row_scale(bound_exp<P>(-cl * eQ));
+#pragma unroll
+            for (int x = 0; x < NU; ++x)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int p = 2 * (es + 4 * x) + h, d = g.nd == 1 ? 0 : p % g.nd;
+                    if (__ldg(g.ew + w * g.nd + d) == kNonFinite) S[x][2 * h] = S[x][2 * h + 1] = sum_nan(typename P::Sum());
+                }
             for (int gb = 0; gb < wi.y; ++gb) {
                 const int pr = __ldg(g.wpairs + wi.z + gb), i = pr & 7, j = pr >> 3;
                 // type (ta, tb) of lane ^ mask adds to this lane's character; i^{ta - i} = i^{ca} times a real sign
@@ -1351,6 +1369,7 @@ struct TcJArgs {
     const int* kpos;        // position of each record in the K order of all classes
     __nv_bfloat16* vs;      // sliced V_ij: [block group][stage][slice][columns of its MMA x 16 K] stage tiles
     int* ev;                // column bounds of V_ij: [(i, j)][nd][ncols]
+    int* er;                // [(i, j)][nd]: kNonFinite where one of their columns is, else 0
     double* Jp;             // partial back-contraction sums [dens][part][term] in the split form's class layout
     long long ng_half;
     long long jp_total;     // doubles per density of Jp
@@ -1404,8 +1423,12 @@ __device__ __forceinline__ auto v_entry(const TcJArgs& g, int slot, int i, int j
     else return cdf{df_mulf(v.re, p), df_mulf(v.im, p)};
 }
 
-__device__ __forceinline__ float v_abs(cdf v) { return fmaxf(fabsf(v.re.hi), fabsf(v.im.hi)); }
-__device__ __forceinline__ float v_abs(double2 v) { return fmaxf(fabsf((float)v.x), fabsf((float)v.y)); }
+// the larger of |Re|, |Im| as the bits of an FP32 number, NaN on top
+__device__ __forceinline__ unsigned abs_bits(float x, float y) {
+    return max(__float_as_uint(x) & 0x7fffffffu, __float_as_uint(y) & 0x7fffffffu);
+}
+__device__ __forceinline__ unsigned v_abs(cdf v) { return abs_bits(v.re.hi, v.im.hi); }
+__device__ __forceinline__ unsigned v_abs(double2 v) { return abs_bits((float)v.x, (float)v.y); }
 
 // column bounds: the exponent bound of max over the slots of |Re V_ij|, |Im V_ij|
 template <class P>
@@ -1414,19 +1437,22 @@ __global__ void __launch_bounds__(256) k_tc_vbound(TcJArgs g) {
     const int nc = col % g.ncols, d = (col / g.ncols) % g.nd, pr = col / (g.ncols * g.nd);
     int i, j;
     pair_of_index(g.deg, pr, i, j);
-    float mx = 0.f;
+    unsigned mx = 0u;
     for (int m = threadIdx.x; m < g.nslots; m += blockDim.x) {
-        mx = fmaxf(mx, v_abs(v_entry<P>(g, m, i, j, d, nc)));
+        mx = max(mx, v_abs(v_entry<P>(g, m, i, j, d, nc)));
     }
-    __shared__ float red[256];
+    __shared__ unsigned red[256];
     red[threadIdx.x] = mx;
     __syncthreads();
     for (int st = 128; st > 0; st >>= 1) {
-        if ((int)threadIdx.x < st) red[threadIdx.x] = fmaxf(red[threadIdx.x], red[threadIdx.x + st]);
+        if ((int)threadIdx.x < st) red[threadIdx.x] = max(red[threadIdx.x], red[threadIdx.x + st]);
         __syncthreads();
     }
     // |Re V|, |Im V| <= mx up to the FP32 rounding of the bound
-    if (threadIdx.x == 0) g.ev[col] = red[0] > 0.f ? bound_exp<P>(log2f(red[0] * 1.0001f)) : -60;
+    if (threadIdx.x == 0)
+        g.ev[col] = red[0] >= 0x7f800000u ? kNonFinite
+                    : red[0] > 0u         ? bound_exp<P>(log2f(__uint_as_float(red[0]) * 1.0001f))
+                                          : -60;
 }
 
 // V_ij sliced into stage tiles: block group, stage q, slice s holds the columns
@@ -1447,7 +1473,13 @@ __global__ void __launch_bounds__(256) k_tc_vslice(TcJArgs g) {
     const int m2 = (int)(rem % (kTcJStageM / 2)), q = (int)(rem / (kTcJStageM / 2));
     int i, j;
     pair_of_index(g.deg, pr, i, j);
-    const int ev = g.ev[(pr * g.nd + d) * g.ncols + nc];
+    const int* evr = g.ev + (pr * g.nd + d) * g.ncols;
+    const int ev = evr[nc];
+    if (nc == 0 && q == 0 && m2 == 0) {
+        int top = 0;
+        for (int k = 0; k < g.ncols; ++k) top = max(top, evr[k]);
+        g.er[pr * g.nd + d] = top == kNonFinite ? kNonFinite : 0;
+    }
     uint32_t sr[kS], si[kS];
     if constexpr (P::S == 8) {
         unsigned long long fr[2], fi[2];
@@ -1773,12 +1805,13 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) 
                         }
                     }
                     if (rvalid) {
+                        const bool finite = __ldg(g.er + pair_index(g.deg, i, j) * g.nd + d) != kNonFinite;
                         double* jp = g.Jp + ((long long)(g.d0 + d) * g.nparts + part * g.nsub + sub) * g.jp_total + g.term_base[L] +
                                      (r - g.cls_start[L]);
 #pragma unroll
                         for (int kk = 0; kk < 5 + E; ++kk)
                             if (kk <= nk) {
-                                const double v = sum_double(sum_mulf(J[kk], P::row_scale(1)));  // exact power of two
+                                const double v = finite ? sum_double(sum_mulf(J[kk], P::row_scale(1))) : NAN;  // exact power of two
                                 jp[(long long)term_of(g.ax, g.bx, i, j, kk) * cnt] = kk == 2 || kk == 3 ? -v : v;
                             }
                     }
@@ -1843,11 +1876,11 @@ void release_tc(ftcj_plan* P) {
     void** ptrs[] = {(void**)&P->d_tc_slots, (void**)&P->d_tc_quads, (void**)&P->d_tc_map, (void**)&P->d_tc_wpairs,
                      &P->d_tc_winfo, (void**)&P->d_tc_wcnt, (void**)&P->d_tc_boff, (void**)&P->d_tc_sched, &P->d_tc_b,
                      &P->d_tc_tab, &P->d_tc_tabk, &P->d_tc_tabz, &P->d_tc_tabz3, (void**)&P->d_tc_cl, (void**)&P->d_tc_kpos,
-                     (void**)&P->d_tc_korder, (void**)&P->d_tc_err, (void**)&P->d_tc_pos, (void**)&P->d_tc_clw,
+                     (void**)&P->d_tc_korder, (void**)&P->d_tc_err, (void**)&P->d_tc_pos, (void**)&P->d_tc_clw, (void**)&P->d_tc_ew,
                      &P->tcj.items, &P->tcj.groups, (void**)&P->tcj.pairs, (void**)&P->tcj.sched, &P->tcj.vs,
-                     (void**)&P->tcj.voff, (void**)&P->tcj.vplace, (void**)&P->tcj.ev,
+                     (void**)&P->tcj.voff, (void**)&P->tcj.vplace, (void**)&P->tcj.ev, (void**)&P->tcj.er,
                      &P->tcg.items, &P->tcg.groups, (void**)&P->tcg.pairs, (void**)&P->tcg.sched, &P->tcg.vs,
-                     (void**)&P->tcg.voff, (void**)&P->tcg.vplace, (void**)&P->tcg.ev};
+                     (void**)&P->tcg.voff, (void**)&P->tcg.vplace, (void**)&P->tcg.ev, (void**)&P->tcg.er};
     for (void** p : ptrs) {
         if (*p) cudaFree(*p);
         *p = nullptr;
@@ -2130,6 +2163,7 @@ int setup_tc(ftcj_plan* P) {
     if ((rc = tc_upload(P, &winfo_dev, winfo))) return rc;
     P->d_tc_winfo = winfo_dev;
     if ((rc = tc_upload(P, &P->d_tc_clw, std::vector<float>((size_t)std::max(1, nwin), 0.f)))) return rc;
+    if ((rc = tc_alloc(P, (void**)&P->d_tc_ew, sizeof(int) * (size_t)std::max(1, nwin) * P->tc_nd))) return rc;
     if ((rc = tc_alloc(P, &P->d_tc_b, (size_t)bmax * 16))) return rc;
     // columns between a window's blocks and the MMA's multiple of 16 are never written nor read back: finite once
     FTCJ_CUDA(cudaMemset(P->d_tc_b, 0, (size_t)bmax * 16));
@@ -2171,6 +2205,7 @@ int launch_tc_rho(ftcj_plan* P, int ndens, cudaStream_t s) {
     }
     g.bs = reinterpret_cast<uint4*>(P->d_tc_b);
     g.clw = P->d_tc_clw;
+    g.ew = P->d_tc_ew;
     g.out = reinterpret_cast<double2*>(P->d_rho_part);
     g.ng_half = P->ng_half;
     g.out_rows = P->tc_out_rows;
@@ -2340,6 +2375,7 @@ int setup_tc_j(ftcj_plan* P, int extra) {
     FTCJ_CUDA(cudaMemset(B.vs, 0, sizeof(__nv_bfloat16) * (size_t)nvs));
     const size_t nev = (size_t)npairs_all * nd_best * P->tc_ncols;
     if ((rc = tc_alloc(P, (void**)&B.ev, sizeof(int) * nev))) return rc;
+    if ((rc = tc_alloc(P, (void**)&B.er, sizeof(int) * (size_t)npairs_all * nd_best))) return rc;
     if ((rc = allow_dynamic_smem(tc_j_kernel(f64, extra), tc_j_smem_bytes(slices, npad, tws, nbuf)))) return rc;
     B.on = true;
     return FTCJ_OK;
@@ -2370,6 +2406,7 @@ int launch_back(ftcj_plan* P, const TcBack& B, int ndens, const double* W, doubl
     g.kpos = P->d_tc_kpos;
     g.vs = reinterpret_cast<__nv_bfloat16*>(B.vs);
     g.ev = B.ev;
+    g.er = B.er;
     g.Jp = Jp;
     g.deg = kNclass - 1 + B.extra;
     g.ng_half = P->ng_half;

@@ -1,5 +1,5 @@
 """What the sliced product has to take as the walks do: general contractions
-with many functions per primitive."""
+with many functions per primitive, and densities that are not finite."""
 import numpy as np
 import pytest
 
@@ -50,4 +50,58 @@ def test_wide_contractions_in_split_plans(orc, F, contraction):
     dE = float(np.abs(EJ.cpu().numpy() - ref["EJ"]).max()) / max(1.0, float(np.abs(ref["EJ"]).max()))
     print(f"contraction {contraction}: records {plan.info['npairs']} max|dJ|={dJ:.2e} of {scale:.2e} rel dE={dE:.2e}")
     assert dJ <= 1e-10 * scale and dE <= 1e-10
+    plan.close()
+
+
+EVEN = [(c, l, [0.12 * 2.1 ** q for q in range(n)]) for c in range(4) for l, n in ((0, 9), (1, 5), (2, 2))]
+DIFFUSE = [(c, l, [0.07, 0.4, 1.3]) for c in range(4) for l in (0, 1)]
+
+
+def pair_of_densities(kind):
+    """A cell whose passes run as sliced products in the named form, two densities, and the plan's arguments."""
+    spec = DIFFUSE if kind == "classified" else EVEN
+    w = W.tiny(seed=91, A=np.diag([11.0, 12.3, 11.6]), shell_spec=spec, kmesh=(1, 1, 1), omega=0.42, ndens=2,
+               centres=CENTRES)
+    args = {"fp64": dict(precision=0), "split": dict(precision=1), "tensor": dict(precision=1, contraction=1),
+            "classified": dict(precision=0, classify=True)}[kind]
+    return w, args
+
+
+def touched(J):
+    """The elements that some pair record contributes to."""
+    return J != 0
+
+
+KINDS = ["fp64", "split", "tensor", "classified"]
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), float("-inf")])
+def test_a_non_finite_density_stays_non_finite(F, kind, bad):
+    """One element of the first density is not finite: its E_J, J^k, rho and gradient show it, as the walks' do; the
+    second density's results are those without it."""
+    import torch
+    w, args = pair_of_densities(kind)
+    D = device(w)
+    plan = F.Plan.from_workload(w, **args)
+    assert plan.info["contraction"] == F.FTCJ_CONTRACT_TC
+    J0, E0 = plan.jbuild(D)
+    g0 = plan.grad(D)[1] if kind != "classified" else None
+    D[0, 0, 3, 3] = bad
+    J, E = plan.jbuild(D)
+    torch.cuda.synchronize()
+    assert plan.status() == 0
+    assert not bool(torch.isfinite(E[0])) and not bool(torch.isfinite(J[0].real)[touched(J0[0])].any())
+    scale = max(1.0, float(J0.abs().max()))
+    assert float((J[1] - J0[1]).abs().max()) <= 1e-12 * scale and float((E[1] - E0[1]).abs()) <= 1e-12 * float(E0[1].abs())
+    if g0 is not None:
+        rho = plan.rho(plan.fold_density(D))
+        assert not bool(torch.isfinite(rho[0].real).any()) and bool(torch.isfinite(rho[1].real).all())
+        E2, g = plan.grad(D)
+        assert not bool(torch.isfinite(E2[0])) and not bool(torch.isfinite(g[0]).any())
+        assert float((g[1] - g0[1]).abs().max()) <= 1e-12 * max(1.0, float(g0.abs().max()))
+        Wp = torch.ones((2, plan.ng_half), dtype=torch.complex128, device="cuda")
+        Wp[0, 5] = bad
+        J0n = plan.jback(Wp)
+        assert not bool(torch.isfinite(J0n[0])[touched(J0n[1])].any()) and bool(torch.isfinite(J0n[1]).all())
     plan.close()
