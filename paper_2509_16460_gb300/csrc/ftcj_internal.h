@@ -171,7 +171,7 @@ struct TcBack {
     long long* voff = nullptr;                   // start of each block group's tiles
     int* vplace = nullptr;                       // block groups that hold each (i, j)
     int* ev = nullptr;                           // their column bounds
-    int* er = nullptr;                           // per (i, j) and density: one of the columns is not finite
+    int* er = nullptr;                           // the exponent they are relative to, per (i, j) and density
 };
 
 struct ftcj_plan {
@@ -284,7 +284,7 @@ struct ftcj_plan {
     int* d_tc_err = nullptr;     // device error word of the bounded waits
     int* d_tc_pos = nullptr;     // [npairs]: position of each record in its class's K order
     float* d_tc_clw = nullptr;   // [nwin]: the windows' smallest widths
-    int* d_tc_ew = nullptr;      // [nwin][tc_nd]: windows with terms that are not finite
+    int* d_tc_ew = nullptr;      // [nwin][tc_nd]: exponents that the windows' B slices are relative to
     long long tc_dp_base[ftcj::kNclass] = {}, tc_dp_stride[ftcj::kNclass] = {}, tc_dp_total = 0;
     // the back-contraction as a tensor-core product (tc.cu), of a build and of the nuclear gradient
     TcBack tcj, tcg;

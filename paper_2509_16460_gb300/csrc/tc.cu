@@ -37,8 +37,10 @@
 // routines of matrix multiplication", Numer. Algorithms 59, 2012): every row
 // of A and every column of B, over a window of at most 1024 records, gets a
 // power-of-two bound 2^e of its entries, and each entry is cut into six slices
-// m_s 2^{e-6-7s} with integers |m_s| <= 64 (kept at their own magnitude: bf16
-// has FP32's exponent range, so no scaling is undone later).  Slice s of A
+// m_s 2^{e-6-7s} with integers |m_s| <= 64.  The columns' exponents are taken
+// relative to the largest of their window and density, which multiplies the
+// sums when they are drained: a build scales with its density over FP64's range
+// (the split form's terms over FP32's).  Slice s of A
 // times slice t of B is a tcgen05.mma of kind::f16 (bf16 operands, FP32
 // accumulator in tensor memory); products with s + t <= 5 are formed (21 per
 // k-step), the others fall below 2^-40 of the window's scale.  Products of the
@@ -97,6 +99,7 @@ constexpr int kTcWinMax = 1024;                // records per exact-accumulation
 constexpr int kTcNmax = 96;                    // MMA N at most in the split form: five accumulators in 512 columns
 constexpr int kTcNmax64 = 64;                  // in the FP64 form: eight
 constexpr int kTcTmemCols = 512;
+constexpr int kTcDensMax = 32;                 // densities per launch at most: one per lane of a drain warp
 constexpr int kTcGmax = 15;                    // (i, j) blocks per window at most (class 4 has 15)
 constexpr int kTcNbufMax = 4;                  // stage buffers at most
 constexpr int kTcTabSlotsMax = 6;              // stage tables in flight at most
@@ -137,7 +140,8 @@ struct TcArgs {
     long long dp_stride[kNclass];
     uint4* bs;           // sliced B stage tiles of this pass
     float* clw;          // [nwin]: smallest c log2(e) of each window's records
-    int* ew;             // [nwin][nd]: kNonFinite where a term of the window's records is not finite, else 0
+    int* ew;             // [nwin][nd]: exponent that the B slices of a window and density are relative to, kNonFinite
+                         // where a term of its records is not finite
     double2* out;        // partial rows [dens][out_rows][ng_half], this pass's from out_row0
     long long ng_half;
     int out_rows, out_row0;
@@ -528,6 +532,34 @@ __device__ __forceinline__ cdf rot_mi(cdf z, int p) {
     }
 }
 
+// exponent of |x|, x < 2^(exponent + 1): one above FP32's (FP64's) largest for infinities and NaN, one below the
+// smallest for zero and subnormals
+__device__ __forceinline__ int exponent(float x) { return (int)((__float_as_uint(x) >> 23) & 0xffu) - 127; }
+__device__ __forceinline__ int exponent(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) - 1023; }
+
+// |x| 2^-es for es >= its exponent, rounded up; FP64 (off its pipe): 0 where it is below 2^-100
+__device__ __forceinline__ float relative(float x, int es) { return fabsf(x) * (1.0001f * pow2f(-es)); }
+__device__ __forceinline__ float relative(double x, int es) {
+    const int k = exponent(x) - es;
+    const unsigned hi = (unsigned)__double2hiint(x), mantissa = ((hi & 0xfffffu) << 3) | ((unsigned)__double2loint(x) >> 29);
+    return k < -100 ? 0.f : __uint_as_float(((unsigned)(k + 127) << 23) + mantissa + 2u);
+}
+
+// log2 of a number that is zero (-infinity) or normal
+__device__ __forceinline__ float log2_normal(float x) {
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// x 2^k for a sum of FP32 numbers and |k| <= 860, so that the result is a normal number: by its exponent field, off the
+// FP64 pipe
+__device__ __forceinline__ double scale_pow2(double x, int k) {
+    const int hi = __double2hiint(x);
+    const bool normal = (unsigned)((hi & 0x7ff00000) - 0x100000) < 0x7fe00000u;  // neither zero nor infinite nor NaN
+    return __hiloint2double(normal ? hi + (k << 20) : hi, __double2loint(x));
+}
+
 __device__ __forceinline__ int exp_bound(float log2_bound) {
     // smallest e with 2^e > the bound, from a log2 estimate good to ~1e-4
     if (!(log2_bound > -100.f)) return -100;
@@ -593,6 +625,7 @@ struct SplitPrec {
     __device__ static __forceinline__ Entry entry(float2 x) { return df{x.x, x.y}; }
     __device__ static __forceinline__ float row_scale(int) { return 1.f; }
     static constexpr int kWin = kTcWinMax, kNmax = kTcNmax;
+    static constexpr int kRefMin = -120, kRefMax = 126, kColMin = -100;  // as for Prec64, in FP32
 };
 using PrecRho = SplitPrec<6, Slicer6>;
 using PrecJ = SplitPrec<7, Slicer7>;
@@ -617,9 +650,24 @@ struct Prec64 {
     __device__ static __forceinline__ Entry entry(double x) { return x; }
     __device__ static __forceinline__ float row_scale(int e) { return pow2f(e - 6); }
     static constexpr int kWin = kTcWinMax / 2, kNmax = kTcNmax64;
+    // B's (V's) digits carry their column's exponent relative to the largest of their window (their (i, j)) and density:
+    // at most 60 below it, where the last digit is 2^-115 of the largest bound and every product is still a normal FP32
+    // number.  The reference itself covers FP64's range but for its ends (scale_pow2).
+    static constexpr int kRefMin = -850, kRefMax = 850, kColMin = -60;
 };
 
-// the exponent of a bound (log2), not below -60 in the FP64 form, where the last slice sits 2^-55 under it
+// the reference exponent of columns whose largest exponent is top, and a column's own relative to it
+template <class P>
+__device__ __forceinline__ int ref_exp(int top) {
+    return max(P::kRefMin, min(P::kRefMax, top));
+}
+template <class P>
+__device__ __forceinline__ int col_exp(int e, int ref) {
+    return max(e - ref, P::kColMin);
+}
+
+// the exponent of a row bound of A (log2; at most 1), not below -60 in the FP64 form, where the last slice sits 2^-55
+// under it
 template <class P>
 __device__ __forceinline__ int bound_exp(float log2_bound) {
     return P::S == 8 ? max(exp_bound(log2_bound), -60) : exp_bound(log2_bound);
@@ -651,15 +699,18 @@ __global__ void __launch_bounds__(kTcBThreads, P::S == 8 ? 1 : 2) k_tc_rho_b(TcA
     constexpr bool kF64 = P::S == 8;
     static_assert(kF64 || DF, "the six-slice operands are cut from double-float terms");
     constexpr int kS = P::S;
-    __shared__ int mx[kTcNmax / 2];  // bits of the column bounds (non-negative floats order as integers, NaN on top)
+    __shared__ int mx[kTcNmax / 2], top[kTcNmax / 2];  // exponents of the column bounds; the largest per density
     __shared__ int bad[kTcNmax / 2];
     __shared__ int pairs[kTcGmax], tidx[kTcGmax][5];
     __shared__ int clmin_bits;
     const int w = g.w0 + blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     const int4 wi = __ldg(g.winfo + w);
     const int L = wi.x, npair = wi.y, npo = g.nd * g.ncols, cnt = __ldg(g.wcnt + w);
-    for (int i = tid; i < npair * npo; i += blockDim.x) mx[i] = 0;
-    if (tid < g.nd) bad[tid] = 0;
+    for (int i = tid; i < npair * npo; i += blockDim.x) mx[i] = INT_MIN / 2;
+    if (tid < g.nd) {
+        bad[tid] = 0;
+        top[tid] = INT_MIN / 2;
+    }
     if (tid < npair) {
         const int pr = __ldg(g.wpairs + wi.z + tid), i = pr & 7, j = pr >> 3;
         pairs[tid] = pr;
@@ -684,37 +735,50 @@ __global__ void __launch_bounds__(kTcBThreads, P::S == 8 ? 1 : 2) k_tc_rho_b(TcA
     }
     for (int gb = 0; gb < npair; ++gb)
         for (int d = 0; d < g.nd; ++d) {
-            float cm[kIt][5];
+            using Term = std::conditional_t<DF, float, double>;
+            float cm[kIt][5], es[kIt];
 #pragma unroll
             for (int q = 0; q < kIt; ++q) {
                 const int k = tid + q * kTcBThreads;
+                Term v[5];
 #pragma unroll
                 for (int kk = 0; kk < 5; ++kk) {
                     const int t = tidx[gb][kk];
-                    cm[q][kk] = 0.f;
+                    v[kk] = 0;
                     if (t < 0 || k >= cnt) continue;
                     const long long off = (long long)d * g.dp_total + (long long)t * stride;
-                    cm[q][kk] = 1.0001f * (DF ? fabsf(__ldg(dpw + off + k).x) : fabsf((float)__ldg(dp64 + off + ko[q])));
+                    if constexpr (DF) v[kk] = __ldg(dpw + off + k).x;
+                    else v[kk] = __ldg(dp64 + off + ko[q]);
                 }
+                // relative to the record's largest term, so that a bound neither overflows nor underflows
+                int e = exponent(v[0]);
+#pragma unroll
+                for (int kk = 1; kk < 5; ++kk) e = max(e, exponent(v[kk]));
+                if (e == (DF ? 128 : 1024)) bad[d] = 1;
+#pragma unroll
+                for (int kk = 0; kk < 5; ++kk) cm[q][kk] = k < cnt ? relative(v[kk], e) : 0.f;
+                es[q] = (float)e;
             }
+            int etop = INT_MIN / 2;
             for (int nc = 0; nc < g.ncols; ++nc) {
                 const float x = (float)nc, mq = -g.Mcc * x * x;
-                unsigned m = 0u;
+                float m = -1e9f;
 #pragma unroll
                 for (int q = 0; q < kIt; ++q) {
                     const float sv = cm[q][0] + x * (cm[q][1] + x * (cm[q][2] + x * (cm[q][3] + x * cm[q][4])));
-                    m = max(m, __float_as_uint(sv * exp2f(cr[q] * mq)) & 0x7fffffffu);
+                    m = fmaxf(m, log2_normal(sv) + (es[q] + cr[q] * mq));
                 }
-                const unsigned mb = __reduce_max_sync(0xffffffffu, m);
-                if (lane == 0 && mb) atomicMax(&mx[gb * npo + nc * g.nd + d], (int)mb);
-                if (lane == 0 && mb >= 0x7f800000u) bad[d] = 1;
+                const int me = __reduce_max_sync(0xffffffffu, __float2int_rd(m + 1e-3f) + 1);
+                etop = max(etop, me);
+                if (lane == 0) atomicMax(&mx[gb * npo + nc * g.nd + d], me);
             }
+            if (lane == 0) atomicMax(&top[d], etop);
         }
     for (int o = 16; o > 0; o >>= 1) cmin = fminf(cmin, __shfl_xor_sync(0xffffffffu, cmin, o));
     if (lane == 0 && cmin < INFINITY) atomicMin(&clmin_bits, __float_as_int(cmin));
     __syncthreads();
     if (tid == 0) g.clw[w] = __int_as_float(clmin_bits);
-    if (tid < g.nd) g.ew[w * g.nd + tid] = bad[tid] ? kNonFinite : 0;
+    if (tid < g.nd) g.ew[w * g.nd + tid] = bad[tid] ? kNonFinite : ref_exp<P>(top[tid]);
     const int nst = (cnt + kTcStageK - 1) / kTcStageK, npc = (npo + 3) / 4, nw = mma_cols(npair, g.colw);
     uint4* base = g.bs + __ldg(g.boff + w);
     const int ntask = nst * npair * npc * 16;
@@ -727,11 +791,11 @@ __global__ void __launch_bounds__(kTcBThreads, P::S == 8 ? 1 : 2) k_tc_rho_b(TcA
         const int nc = p / g.nd, d = p - nc * g.nd;
         const int pr = pairs[gb], nk = L - (pr & 7) - (pr >> 3);  // k = 0 .. L - i - j
         const int k0 = q * kTcStageK + oc * 8 + half * 4;
-        const float mb = __int_as_float(mx[gb * npo + p]);
-        const int eb = bad[d] ? kNonFinite : mb > 0.f ? bound_exp<P>(log2f(mb)) : -60;
+        const int er = ref_exp<P>(top[d]), ec = col_exp<P>(mx[gb * npo + p], er);
         uint32_t s0[kS][2], s1[kS][2];
         if constexpr (kF64) {
-            const float sc = pow2f(eb - 6);  // B's digits carry their column's bound
+            const float sc = pow2f(ec - 6);  // B's digits carry their column's relative bound
+            const int eb = bad[d] ? kNonFinite : er + ec;
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 unsigned long long fr[2], fi[2];
@@ -783,7 +847,8 @@ __global__ void __launch_bounds__(kTcBThreads, P::S == 8 ? 1 : 2) k_tc_rho_b(TcA
                 }
             }
         } else {
-            const typename P::Cut cut(eb);
+            const typename P::Cut cut(ec);
+            const float unref = pow2f(-er);
             const float2* dpd = dpw + (long long)d * g.dp_total + k0;
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
@@ -809,7 +874,8 @@ __global__ void __launch_bounds__(kTcBThreads, P::S == 8 ? 1 : 2) k_tc_rho_b(TcA
                     bv[e] = cdf{{0.f, 0.f}, {0.f, 0.f}};
                     if (k < cnt) {
                         const float4 zv = __ldg(reinterpret_cast<const float4*>(g.tabz) + (kb + k) * g.ncols + nc);
-                        bv[e] = cdf_mul(cdf{{zv.x, zv.y}, {zv.z, zv.w}}, cdf{re[e], im[e]});
+                        const cdf t = cdf_mul(cdf{{zv.x, zv.y}, {zv.z, zv.w}}, cdf{re[e], im[e]});
+                        bv[e] = cdf{{t.re.hi * unref, t.re.lo * unref}, {t.im.hi * unref, t.im.lo * unref}};
                     }
                 }
                 uint32_t o[kS];
@@ -993,12 +1059,18 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf,
 #pragma unroll
             for (int v = 0; v < 4; ++v) S[x][v] = sum_zero(typename P::Sum());
         const float eQ = g.Maa * ea * ea + g.Mbb * eb * eb;
+        // the sums of a density are relative to the largest exponent of the CTA's windows, lane d density d's
+        int eref = 0;
+        auto of_density = [](auto v, int d) { return __shfl_sync(0xffffffffu, v, d); };
+        // densities of a unit's two outputs: p = 2 un + h belongs to p mod nd, the next unit's is 8 on
+        const int d00 = (2 * es) % g.nd, d01 = (2 * es + 1) % g.nd, dstep = 8 % g.nd;
         Ring b(nbuf), t(ntslots);
         int gs = 0;  // stages so far (mod 2 the group that forms it)
         bool full = false;  // every buffer used once
         for (int jw = j0; jw < j1 && ok; ++jw) {
             const int w = __ldg(wlist + jw), nst = (__ldg(g.wcnt + w) + kTcStageK - 1) / kTcStageK;
             const float cl = __ldg(g.clw + w);
+            const int ew = lane < g.nd ? __ldg(g.ew + w * g.nd + lane) : P::kRefMin;
             const typename P::Cut cut(bound_exp<P>(-cl * Q));
             for (int q = 0; q < nst; ++q, ++gs, b.next(), t.next()) {
                 full = full || gs >= nbuf;
@@ -1032,6 +1104,42 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf,
                 }
             }
             if (!ok) break;
+            // (read before the wait below, which hides it)
+            if (jw == j0)
+                for (int d = 0; d < g.nd; ++d) {
+                    int e = INT_MIN / 2;
+                    for (int k = j0 + lane; k < j1; k += 32) {
+                        const int ek = __ldg(g.ew + __ldg(wlist + k) * g.nd + d);
+                        if (ek != kNonFinite) e = max(e, ek);
+                    }
+                    e = __reduce_max_sync(0xffffffffu, e);
+                    if (lane == d) eref = e;
+                }
+            // powers of two of this window's densities (lane d density d's), relative to the sums', 0 where they are
+            // below 2^-126; then of the two outputs of each unit, as the upper halves of two floats
+            const unsigned half = (unsigned)max(min(ew - eref, 0) + 127, 0) << 7;
+            unsigned rel[NU];
+            int d0 = d00, d1 = d01;
+#pragma unroll
+            for (int x = 0; x < NU; ++x) {
+                if (x > 0 && dstep == 0) {  // 1, 2, 4 or 8 densities: every unit holds the same two
+                    rel[x] = rel[0];
+                    continue;
+                }
+                rel[x] = of_density(half, d0) | (of_density(half, d1) << 16);
+                d0 += dstep;
+                d1 += dstep;
+                if (d0 >= g.nd) d0 -= g.nd;
+                if (d1 >= g.nd) d1 -= g.nd;
+            }
+            if (__any_sync(0xffffffffu, ew == kNonFinite)) {
+#pragma unroll
+                for (int x = 0; x < NU; ++x)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v)
+                        if (of_density(ew, (2 * (es + 4 * x) + (v >> 1)) % g.nd) == kNonFinite)
+                            S[x][v] = sum_nan(typename P::Sum());
+            }
             // ---- drain: each block's level sums, times (-i)^{i+j} n_a^i n_b^j, into the sums by character ----
             ok = __all_sync(0xffffffffu, mbar_wait(&sm.accf, (uint32_t)((jw - j0) & 1), abort_flag, g.spin));
             if (!ok) break;
@@ -1039,13 +1147,6 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf,
             const int4 wi = __ldg(g.winfo + w);
             const uint32_t nw = (uint32_t)mma_cols(wi.y, g.colw);
             const float rsc = P::row_scale(bound_exp<P>(-cl * eQ));
-#pragma unroll
-            for (int x = 0; x < NU; ++x)
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int p = 2 * (es + 4 * x) + h, d = g.nd == 1 ? 0 : p % g.nd;
-                    if (__ldg(g.ew + w * g.nd + d) == kNonFinite) S[x][2 * h] = S[x][2 * h + 1] = sum_nan(typename P::Sum());
-                }
             for (int gb = 0; gb < wi.y; ++gb) {
                 const int pr = __ldg(g.wpairs + wi.z + gb), i = pr & 7, j = pr >> 3;
                 // type (ta, tb) of lane ^ mask adds to this lane's character; i^{ta - i} = i^{ca} times a real sign
@@ -1058,11 +1159,12 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf,
                     if (un < nunit) {
                         float T[P::ACC][4];
                         tc_ld_levels4(tmem + tlane + (uint32_t)(gb * g.colw + 4 * un), nw, T);
+                        const float fu[2] = {f * __uint_as_float(rel[x] << 16), f * __uint_as_float(rel[x] & 0xffff0000u)};
 #pragma unroll
                         for (int v = 0; v < 4; ++v) {
                             typename P::Sum l = level_sum(T, v);
                             if (mask) l = sum_xor(l, mask);
-                            S[x][v] = sum_add(S[x][v], sum_mulf(l, f));
+                            S[x][v] = sum_add(S[x][v], sum_mulf(l, fu[v >> 1]));
                         }
                     }
                 }
@@ -1100,14 +1202,13 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf,
                             o = sum_xor(c[r], 2);
                             if (db) c[r] = (lane & 2) ? sum_add(o, sum_neg(c[r])) : sum_add(c[r], o);
                         }
-                        const int p = 2 * un + h;
+                        const int p = 2 * un + h, nc = p / g.nd, d = p - nc * g.nd, er = of_density(eref, d);
                         if (valid && p < npo) {
-                            const int nc = p / g.nd, d = p - nc * g.nd;
                             int idx = __ldg(mrow + nc);
                             if (idx != INT_MIN) {
                                 const bool cj = idx < 0;
                                 if (cj) idx = ~idx;
-                                const double re = sum_double(c[0]), im = sum_double(c[1]);
+                                const double re = scale_pow2(sum_double(c[0]), er), im = scale_pow2(sum_double(c[1]), er);
                                 g.out[((long long)(g.d0 + d) * g.out_rows + g.out_row0 + kg) * g.ng_half + idx] =
                                     make_double2(re, cj ? -im : im);
                             }
@@ -1322,18 +1423,16 @@ void tc_slots(const std::set<std::pair<int, int>>& pts, std::vector<int>& slots,
 // factor tables.  Every entry of A^T has modulus <= 1 (bound 2^1 for all of
 // them); each column of V_ij gets its own bound over all slots, so that entries
 // far out in the sphere (where W has decayed) sit many bits below their
-// column's bound.  Seven slices (products with s + t <= 6, 28 per k-step) keep
-// the truncation below 2^-45 of the bounds.  The slots are cut into parts of at
-// most 1024, each a work unit of its own: within a part, levels 0-3 are exact
-// (the level-3 sums stay below 1024 x 14848 < 2^24 in units of 2^-21: |A| <= 1
-// bounds the leading slice of A by 32) and only levels 4-6 share the rounded
-// fifth accumulator.  The tensor core's FP32 accumulation does not round to
-// nearest, so the rounded accumulator's error grows with the number of MMAs
-// that add into it and with its size; keeping level 3 out of it keeps that
-// error ~2^-7 of a four-accumulator scheme's.  The level sums go straight
-// to the epilogue, which forms the part's J' for k <= L - i - j in
-// double-float and writes it as one of the partial FP64 sums the J -> AO map
-// adds.
+// column's bound (again relative to the largest of their (i, j) and density,
+// which multiplies J').  Seven slices (products with s + t <= 6, 28 per k-step) keep the truncation
+// below 2^-45 of the bounds.  The slots are cut into parts of at most 1024, each a work unit of its
+// own: within a part, levels 0-3 are exact (the level-3 sums stay below 1024 x 14848 < 2^24 in units
+// of 2^-21: |A| <= 1 bounds the leading slice of A by 32) and only levels 4-6 share the rounded fifth
+// accumulator.  The tensor core's FP32 accumulation does not round to nearest, so the rounded
+// accumulator's error grows with the number of MMAs that add into it and with its size; keeping level
+// 3 out of it keeps that error ~2^-7 of a four-accumulator scheme's.  The level sums go straight to
+// the epilogue, which forms the part's J' for k <= L - i - j in double-float and writes it as one of
+// the partial FP64 sums the J -> AO map adds.
 
 constexpr int kTcJStageM = 16;       // slots per stage: one MMA k-step
 constexpr int kTcJAsliceBytes = kTcM * kTcJStageM * 2;        // 128 records x 16 K x bf16
@@ -1369,7 +1468,8 @@ struct TcJArgs {
     const int* kpos;        // position of each record in the K order of all classes
     __nv_bfloat16* vs;      // sliced V_ij: [block group][stage][slice][columns of its MMA x 16 K] stage tiles
     int* ev;                // column bounds of V_ij: [(i, j)][nd][ncols]
-    int* er;                // [(i, j)][nd]: kNonFinite where one of their columns is, else 0
+    int* er;                // [(i, j)][nd]: exponent that their slices are relative to, kNonFinite where a column is not
+                            // finite
     double* Jp;             // partial back-contraction sums [dens][part][term] in the split form's class layout
     long long ng_half;
     long long jp_total;     // doubles per density of Jp
@@ -1423,14 +1523,21 @@ __device__ __forceinline__ auto v_entry(const TcJArgs& g, int slot, int i, int j
     else return cdf{df_mulf(v.re, p), df_mulf(v.im, p)};
 }
 
-// the larger of |Re|, |Im| as the bits of an FP32 number, NaN on top
-__device__ __forceinline__ unsigned abs_bits(float x, float y) {
-    return max(__float_as_uint(x) & 0x7fffffffu, __float_as_uint(y) & 0x7fffffffu);
+// the larger of |Re|, |Im| by their leading bits (an FP32 number's, the high word of an FP64 one; non-negative numbers
+// order as integers, infinities and NaN on top), and the exponent e, |x| < 2^e, that they give
+__device__ __forceinline__ unsigned v_top(cdf v) {
+    return max(__float_as_uint(v.re.hi) & 0x7fffffffu, __float_as_uint(v.im.hi) & 0x7fffffffu);
 }
-__device__ __forceinline__ unsigned v_abs(cdf v) { return abs_bits(v.re.hi, v.im.hi); }
-__device__ __forceinline__ unsigned v_abs(double2 v) { return abs_bits((float)v.x, (float)v.y); }
+__device__ __forceinline__ unsigned v_top(double2 v) {
+    return max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
+}
+template <class P>
+__device__ __forceinline__ int top_exp(unsigned top) {
+    if (P::S == 8) return top >= 0x7ff00000u ? kNonFinite : (int)(top >> 20) - 1022;
+    return top >= 0x7f800000u ? kNonFinite : (int)(top >> 23) - 126;
+}
 
-// column bounds: the exponent bound of max over the slots of |Re V_ij|, |Im V_ij|
+// column bounds: the exponent of the maximum over the slots of |Re V_ij|, |Im V_ij|
 template <class P>
 __global__ void __launch_bounds__(256) k_tc_vbound(TcJArgs g) {
     const int col = blockIdx.x;  // ((i, j) nd + d) ncols + n_c
@@ -1439,7 +1546,7 @@ __global__ void __launch_bounds__(256) k_tc_vbound(TcJArgs g) {
     pair_of_index(g.deg, pr, i, j);
     unsigned mx = 0u;
     for (int m = threadIdx.x; m < g.nslots; m += blockDim.x) {
-        mx = max(mx, v_abs(v_entry<P>(g, m, i, j, d, nc)));
+        mx = max(mx, v_top(v_entry<P>(g, m, i, j, d, nc)));
     }
     __shared__ unsigned red[256];
     red[threadIdx.x] = mx;
@@ -1448,11 +1555,7 @@ __global__ void __launch_bounds__(256) k_tc_vbound(TcJArgs g) {
         if ((int)threadIdx.x < st) red[threadIdx.x] = max(red[threadIdx.x], red[threadIdx.x + st]);
         __syncthreads();
     }
-    // |Re V|, |Im V| <= mx up to the FP32 rounding of the bound
-    if (threadIdx.x == 0)
-        g.ev[col] = red[0] >= 0x7f800000u ? kNonFinite
-                    : red[0] > 0u         ? bound_exp<P>(log2f(__uint_as_float(red[0]) * 1.0001f))
-                                          : -60;
+    if (threadIdx.x == 0) g.ev[col] = top_exp<P>(red[0]);
 }
 
 // V_ij sliced into stage tiles: block group, stage q, slice s holds the columns
@@ -1474,12 +1577,11 @@ __global__ void __launch_bounds__(256) k_tc_vslice(TcJArgs g) {
     int i, j;
     pair_of_index(g.deg, pr, i, j);
     const int* evr = g.ev + (pr * g.nd + d) * g.ncols;
-    const int ev = evr[nc];
-    if (nc == 0 && q == 0 && m2 == 0) {
-        int top = 0;
-        for (int k = 0; k < g.ncols; ++k) top = max(top, evr[k]);
-        g.er[pr * g.nd + d] = top == kNonFinite ? kNonFinite : 0;
-    }
+    int top = evr[0];
+    for (int k = 1; k < g.ncols; ++k) top = max(top, evr[k]);
+    const bool finite = top != kNonFinite;
+    const int er = ref_exp<P>(top), ec = col_exp<P>(evr[nc], er);
+    if (nc == 0 && q == 0 && m2 == 0) g.er[pr * g.nd + d] = finite ? er : kNonFinite;
     uint32_t sr[kS], si[kS];
     if constexpr (P::S == 8) {
         unsigned long long fr[2], fi[2];
@@ -1490,10 +1592,10 @@ __global__ void __launch_bounds__(256) k_tc_vslice(TcJArgs g) {
             const double2 v = v_entry<P>(g, slot, i, j, d, nc);
             const int rot = (i + j + 8 - ((sl >> 16) & 1) - ((sl >> 17) & 1)) & 3;  // times (-i)^rot
             const double re = rot & 1 ? v.y : v.x, im = rot & 1 ? -v.x : v.y;
-            fr[e] = fixed8(rot & 2 ? -re : re, ev);
-            fi[e] = fixed8(rot & 2 ? -im : im, ev);
+            fr[e] = fixed8(rot & 2 ? -re : re, finite ? er + ec : kNonFinite);
+            fi[e] = fixed8(rot & 2 ? -im : im, finite ? er + ec : kNonFinite);
         }
-        float w = pow2f(ev - 6);
+        float w = pow2f(ec - 6);
 #pragma unroll
         for (int s = 0; s < kS; ++s, w *= 0x1p-7f) {
             const int sh = 7 * (7 - s);
@@ -1504,13 +1606,15 @@ __global__ void __launch_bounds__(256) k_tc_vslice(TcJArgs g) {
             si[s] = pack_bf2(digit(fi[0]), digit(fi[1]));
         }
     } else {
-        const typename P::Cut cut(ev);
+        const typename P::Cut cut(ec);
+        const float unref = pow2f(-er);
         cdf v[2];
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const int slot = q * kTcJStageM + 2 * m2 + e;
             const int sl = slot < g.nslots ? __ldg(g.slots + slot) : 0;
-            v[e] = rot_mi(v_entry<P>(g, slot, i, j, d, nc), i + j + 8 - ((sl >> 16) & 1) - ((sl >> 17) & 1));
+            const cdf t = rot_mi(v_entry<P>(g, slot, i, j, d, nc), i + j + 8 - ((sl >> 16) & 1) - ((sl >> 17) & 1));
+            v[e] = cdf{{t.re.hi * unref, t.re.lo * unref}, {t.im.hi * unref, t.im.lo * unref}};
         }
         cut.pair(v[0].re, v[1].re, sr);
         cut.pair(v[0].im, v[1].im, si);
@@ -1744,17 +1848,24 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) 
                     if (lane == 0) mbar_arrive(&sm.tempty);
                 }
                 // ---- J'_{r,ijk} = Re (-i)^k sum_{n_c} n_c^k Z_r(n_c) U_ij[r, n_c] ----
+                // lane l holds the l-th (block, density) of the group: (i, j) and the exponent of its sums
+                const int2 gr = __ldg(g.groups + un.y + gi);
+                int lpr = 0, ler = 0;
+                if (lane < gr.y * g.nd) {
+                    lpr = __ldg(g.ipairs + gr.x + lane / g.nd);
+                    ler = __ldg(g.er + pair_index(g.deg, lpr & 7, lpr >> 3) * g.nd + lane % g.nd);
+                }
                 ok = __all_sync(0xffffffffu, mbar_wait(&sm.accf, (uint32_t)(ng & 1), abort_flag, g.spin));
                 if (!ok) break;
                 tc_fence_after();
-                const int2 gr = __ldg(g.groups + un.y + gi);
                 const uint32_t nw = (uint32_t)mma_cols(gr.y, g.colw);
                 const float4* zrec =
                     reinterpret_cast<const float4*>(g.tabz) +
                     (size_t)__ldg(g.kpos + (rvalid ? r : un.w)) * g.ncols * (P::S == 8 ? 2 : 1);
                 for (int ps = es; ps < gr.y * g.nd * g.nsub; ps += kTcProdWarps / 4) {
                     const int pd = ps / g.nsub, sub = ps - pd * g.nsub, gb = pd / g.nd, d = pd - gb * g.nd;
-                    const int pr = __ldg(g.ipairs + gr.x + gb), i = pr & 7, j = pr >> 3, nk = L + E - i - j;
+                    const int pr = __shfl_sync(0xffffffffu, lpr, pd), i = pr & 7, j = pr >> 3, nk = L + E - i - j;
+                    const int er = __shfl_sync(0xffffffffu, ler, pd);
                     typename P::Sum J[5 + E];
 #pragma unroll
                     for (int kk = 0; kk < 5 + E; ++kk) J[kk] = sum_zero(typename P::Sum());
@@ -1805,13 +1916,13 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) 
                         }
                     }
                     if (rvalid) {
-                        const bool finite = __ldg(g.er + pair_index(g.deg, i, j) * g.nd + d) != kNonFinite;
+                        const int eo = P::S == 8 ? er + 1 - 6 : er;  // with A's bound 2^1 (row_scale)
                         double* jp = g.Jp + ((long long)(g.d0 + d) * g.nparts + part * g.nsub + sub) * g.jp_total + g.term_base[L] +
                                      (r - g.cls_start[L]);
 #pragma unroll
                         for (int kk = 0; kk < 5 + E; ++kk)
                             if (kk <= nk) {
-                                const double v = finite ? sum_double(sum_mulf(J[kk], P::row_scale(1))) : NAN;  // exact power of two
+                                const double v = er == kNonFinite ? NAN : scale_pow2(sum_double(J[kk]), eo);
                                 jp[(long long)term_of(g.ax, g.bx, i, j, kk) * cnt] = kk == 2 || kk == 3 ? -v : v;
                             }
                     }
@@ -1943,7 +2054,7 @@ int setup_tc(ftcj_plan* P) {
         }
         ap.rows = rs.size();
         ap.ncols = ncmax + 1;
-        for (ap.nd = P->max_dens; ap.nd >= 1; --ap.nd) {
+        for (ap.nd = std::min(P->max_dens, kTcDensMax); ap.nd >= 1; --ap.nd) {
             tc_columns(nmax, ap.nd, ap.ncols, &ap.colw, &ap.G, &ap.npad);
             if (ap.G > 0) break;
         }

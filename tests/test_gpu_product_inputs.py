@@ -1,5 +1,6 @@
 """What the sliced product has to take as the walks do: general contractions
-with many functions per primitive, and densities that are not finite."""
+with many functions per primitive, densities that are not finite, and very small
+and very large ones."""
 import numpy as np
 import pytest
 
@@ -104,4 +105,39 @@ def test_a_non_finite_density_stays_non_finite(F, kind, bad):
         Wp[0, 5] = bad
         J0n = plan.jback(Wp)
         assert not bool(torch.isfinite(J0n[0])[touched(J0n[1])].any()) and bool(torch.isfinite(J0n[1]).all())
+    plan.close()
+
+
+# FP64: any power of two that keeps E_J (quadratic) in FP64's range; split: double-float drops what lies below 2^-126,
+# so one whose operands' last bits (2^-48, and W another 2^-14) lie above that
+SCALES = {"fp64": (-300, -120, -90, 60, 300), "classified": (-300, -90, 300), "split": (-60, 40), "tensor": (-60, 40)}
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_builds_scale_with_the_density(F, kind):
+    """J(sD) = s J(D), E(sD) = s^2 E(D) and so on for powers of two s, in the first of two densities of a call, the
+    second unscaled.  A power of two changes no significand, so the FP64 forms differ by the order of the atomic sums
+    alone (1e-12 of max|J|); the split form's by what it drops below 2^-126 too (1e-10 of max|J|)."""
+    import torch
+    w, args = pair_of_densities(kind)
+    D = device(w)
+    plan = F.Plan.from_workload(w, **args)
+    J0, E0 = plan.jbuild(D)
+    g0 = plan.grad(D)[1] if kind != "classified" else None
+    tol = 1e-12 if args["precision"] == 0 else 1e-10
+    for e in SCALES[kind]:
+        s = 2.0 ** e
+        Ds = D.clone()
+        Ds[0] *= s
+        J, E = plan.jbuild(Ds)
+        torch.cuda.synchronize()
+        dJ = float((J[0] / s - J0[0]).abs().max()) / float(J0[0].abs().max())
+        dE = float((E[0] / s / s - E0[0]).abs()) / float(E0[0].abs())
+        d1 = float((J[1] - J0[1]).abs().max()) / float(J0[1].abs().max())
+        print(f"{kind} 2^{e}: rel dJ={dJ:.2e} dE={dE:.2e} unscaled {d1:.2e}")
+        assert dJ <= tol and dE <= tol and d1 <= 1e-12, (e, dJ, dE, d1)
+        if g0 is not None:
+            _, g = plan.grad(Ds)
+            dg = float((g[0] / s / s - g0[0]).abs().max()) / float(g0[0].abs().max())
+            assert dg <= tol * 10, (e, dg)
     plan.close()
