@@ -129,8 +129,8 @@ typedef struct {
                            (ftcj_info.j_contraction says which) */
     int tc_wait_log2;   /* tensor-core kernels: each wait between their roles gives up after
                            2^tc_wait_log2 clock cycles (0: 2^32, about 2 s), raises the plan's device
-                           error word (ftcj_plan_status) and lets the kernel drain and return; 1..40,
-                           small values are for tests of that path */
+                           error word (ftcj_plan_status), writes NaN in place of its results and lets
+                           the kernel drain and return; 1..40, small values are for tests of that path */
     int classify;       /* 1: compact/diffuse classification of the pair densities (Sec. 2.6).  A pair
                            record whose two primitives both have exponents below alpha_cut is DD; the
                            DD records leave the planewave walks and take the GPW route (App. E): their
@@ -254,7 +254,9 @@ int ftcj_jbuild(ftcj_plan* plan, int ndens, const double* Dk, double* Jk, double
  * managed D^k or J^k is read or written by the k-mesh transform kernels
  * directly over the host link, so its transfer overlaps that kernel; a
  * pageable buffer is copied through plan-owned staging sized at plan creation
- * for max_dens densities.  ndens may exceed max_dens (batched). */
+ * for max_dens densities.  ndens may exceed max_dens (batched).  Returns
+ * ETIMEOUT where ftcj_plan_status would report a wait that gave up (and clears
+ * that word). */
 int ftcj_jbuild_host(ftcj_plan* plan, int ndens, const double* Dk_host, double* Jk_host, double* EJ_host,
                      void* stream);
 
@@ -338,9 +340,11 @@ int ftcj_unfold_j(ftcj_plan* plan, int ndens, const double* J0n, double* Jk, voi
 int ftcj_grad(ftcj_plan* plan, int ndens, const double* Dk, double* EJ, double* grad, void* stream);
 
 /* Device error word of the plan's kernels that wait on one another inside a
- * block (the tensor-core contraction): bit 0 set when a bounded wait gave up
- * (the results of that build are invalid).  Synchronises `stream`, returns
- * the word in *flags and clears it.  A plan without such kernels reports 0. */
+ * block (the tensor-core contraction, which FP64 plans and larger split plans
+ * of orthorhombic cells run by themselves, see ftcj_params.contraction): bit 0
+ * set when a bounded wait gave up.  J^k (and E_J, where the structure factors
+ * gave up) of that build are then NaN.  Synchronises `stream`, returns the word
+ * in *flags and clears it.  A plan without such kernels reports 0. */
 int ftcj_plan_status(ftcj_plan* plan, int* flags, void* stream);
 
 /* Largest |Im D^{0n}| and largest |D^{0n}_{mu nu} - D^{0,-n}_{nu mu}| of
@@ -405,9 +409,10 @@ int ftcj_batch_replay(ftcj_batch* batch, void* stream);
  * raises the batch's error word and skips its work.  0..40, else EINVAL. */
 int ftcj_batch_set_wait(ftcj_batch* batch, int wait_log2);
 
-/* The error word of the last persistent launch (bit 0: a wait gave up),
- * read on `stream` (synchronises it).  Returns FTCJ_ETIMEOUT when bit 0 is
- * set, FTCJ_OK otherwise (and for batches that are not persistent). */
+/* The error words of the batch, read on `stream` (synchronises it): of the last
+ * persistent launch, and of the cells' plans since they were last read (as
+ * ftcj_plan_status, cleared); bit 0: a wait gave up.  Returns FTCJ_ETIMEOUT
+ * when bit 0 is set, FTCJ_OK otherwise. */
 int ftcj_batch_status(ftcj_batch* batch, int* flags, void* stream);
 
 void ftcj_batch_destroy(ftcj_batch* batch);

@@ -1,5 +1,6 @@
 // Public build entry points: argument checks and the order of the steps.
 #include <algorithm>
+#include <array>
 
 #include "ftcj_internal.h"
 
@@ -47,6 +48,11 @@ int single_potential(const ftcj_plan* P) {
     if (P->rec_filter)
         return fail(FTCJ_EUNSUPPORTED, "a classified plan (compact/diffuse) runs ftcj_jbuild or ftcj_jbuild_host only");
     return FTCJ_OK;
+}
+
+// device error words of a plan: its own, its DD records'
+std::array<int*, 2> error_words(const ftcj_plan* P) {
+    return {P->d_tc_err, P->dd ? P->dd->d_tc_err : nullptr};
 }
 
 int check(const ftcj_plan* P, int ndens, bool batch_limit) {
@@ -101,6 +107,23 @@ int build_batch(ftcj_plan* P, int nd, const double* Dk, double* Jk, double* EJ, 
 }
 
 }  // namespace
+
+namespace ftcj {
+
+int take_error_word(ftcj_plan* P, int* flags, cudaStream_t s) {
+    int word[2] = {0, 0};
+    const auto err = error_words(P);
+    for (int i = 0; i < 2; ++i)
+        if (err[i]) {
+            FTCJ_CUDA(cudaMemcpyAsync(&word[i], err[i], sizeof(int), cudaMemcpyDeviceToHost, s));
+            FTCJ_CUDA(cudaMemsetAsync(err[i], 0, sizeof(int), s));
+        }
+    FTCJ_CUDA(cudaStreamSynchronize(s));
+    *flags = word[0] | word[1];
+    return FTCJ_OK;
+}
+
+}  // namespace ftcj
 
 extern "C" {
 
@@ -194,8 +217,14 @@ int ftcj_jbuild_host(ftcj_plan* P, int ndens, const double* Dk_host, double* Jk_
                                       cudaMemcpyDeviceToHost, s));
         FTCJ_CUDA(cudaMemcpyAsync(EJ_host + b0, P->d_EJ_stage, sizeof(double) * nd, cudaMemcpyDeviceToHost, s));
     }
+    int word[2] = {0, 0};
+    const auto err = error_words(P);
+    for (int i = 0; i < 2; ++i)
+        if (err[i]) FTCJ_CUDA(cudaMemcpyAsync(&word[i], err[i], sizeof(int), cudaMemcpyDeviceToHost, s));
     FTCJ_CUDA(cudaStreamSynchronize(s));
-    return FTCJ_OK;
+    if ((word[0] | word[1]) == 0) return FTCJ_OK;
+    if ((rc = take_error_word(P, word, s))) return rc;  // cleared
+    return fail(FTCJ_ETIMEOUT, "a bounded wait of the tensor-core contraction gave up: J^k and E_J are invalid");
 }
 
 int ftcj_grad(ftcj_plan* P, int ndens, const double* Dk, double* EJ, double* grad, void* stream) {
@@ -224,17 +253,7 @@ int ftcj_grad(ftcj_plan* P, int ndens, const double* Dk, double* EJ, double* gra
 
 int ftcj_plan_status(ftcj_plan* P, int* flags, void* stream) {
     if (!P || !flags) return fail(FTCJ_EINVAL, "null argument");
-    cudaStream_t s = as_stream(stream);
-    int word[2] = {0, 0};  // the plan's kernels, and those of its DD records
-    int* const err[2] = {P->d_tc_err, P->dd ? P->dd->d_tc_err : nullptr};
-    for (int i = 0; i < 2; ++i)
-        if (err[i]) {
-            FTCJ_CUDA(cudaMemcpyAsync(&word[i], err[i], sizeof(int), cudaMemcpyDeviceToHost, s));
-            FTCJ_CUDA(cudaMemsetAsync(err[i], 0, sizeof(int), s));
-        }
-    FTCJ_CUDA(cudaStreamSynchronize(s));
-    *flags = word[0] | word[1];
-    return FTCJ_OK;
+    return take_error_word(P, flags, as_stream(stream));
 }
 
 int ftcj_check_density(ftcj_plan* P, int ndens, const double* Dk, double* max_imag, double* max_asym,

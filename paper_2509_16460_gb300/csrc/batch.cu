@@ -343,12 +343,23 @@ int ftcj_batch_set_wait(ftcj_batch* B, int wait_log2) {
 int ftcj_batch_status(ftcj_batch* B, int* flags, void* stream) {
     if (!B || !flags) return fail(FTCJ_EINVAL, "null argument");
     *flags = 0;
-    if (!B->walks) return FTCJ_OK;
-    int rc = batch_walks_error(B->walks, flags, reinterpret_cast<cudaStream_t>(stream));
-    if (rc) return rc;
-    if (*flags & 1)
-        return fail(FTCJ_ETIMEOUT, "a back-contraction item of the persistent batch gave up waiting for its "
-                                   "cell's potential");
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    if (B->walks) {
+        int rc = batch_walks_error(B->walks, flags, s);
+        if (rc) return rc;
+        if (*flags & 1)
+            return fail(FTCJ_ETIMEOUT, "a back-contraction item of the persistent batch gave up waiting for its "
+                                       "cell's potential");
+    }
+    // cells whose passes run as tensor-core products
+    for (ftcj_plan* P : B->plans) {
+        int word = 0;
+        if (!P->d_tc_err) continue;
+        int rc = take_error_word(P, &word, s);
+        if (rc) return rc;
+        *flags |= word;
+    }
+    if (*flags & 1) return fail(FTCJ_ETIMEOUT, "a bounded wait of a cell's tensor-core contraction gave up");
     return FTCJ_OK;
 }
 

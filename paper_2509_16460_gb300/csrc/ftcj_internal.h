@@ -373,6 +373,8 @@ int setup_tc(ftcj_plan* P);
 void release_tc(ftcj_plan* P);  // back to a plan without the tensor-core form
 int launch_tc_rho(ftcj_plan* P, int ndens, cudaStream_t s);
 int tc_rho_launches(const ftcj_plan* P, int nd);
+// the error word of a plan's bounded waits (its DD records' included), read on s (synchronised) and cleared
+int take_error_word(ftcj_plan* P, int* flags, cudaStream_t s);
 int launch_tc_j(ftcj_plan* P, int ndens, const double* W, cudaStream_t s);
 int launch_tc_j_grad(ftcj_plan* P, int ndens, const double* W, cudaStream_t s);
 // one persistent launch of the walks of a batch of cells (walk_split.cu)

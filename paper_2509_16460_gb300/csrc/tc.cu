@@ -66,7 +66,8 @@
 // the MMA side).  Every wait is bounded: past ~2 s of clock a waiting thread
 // raises the CTA's abort flag and the plan's device error word, every thread
 // leaves its loops, the copies and MMAs in flight are waited for (again
-// bounded) and tensor memory is freed before the CTA exits.
+// bounded), the CTA's outputs become NaN and tensor memory is freed before it
+// exits.
 //
 // What bounds it (molecular crystal, 1056 AOs, 2 densities, GB300): the product
 // takes 1.07 ms, of which the MMAs alone (operands left unformed) need 0.89 ms:
@@ -1220,7 +1221,14 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf,
     }
     tc_fence_before();
     __syncthreads();
-    if (*abort_flag && tid == 0) atomicOr(g.err, 1);
+    if (*abort_flag) {
+        if (tid == 0) atomicOr(g.err, 1);
+        // NaN over the group's rows: of this CTA's points at least nobody writes them again
+        for (long long i = tid; i < g.nd * g.ng_half; i += kTcThreadsAll) {
+            const long long d = i / g.ng_half;
+            g.out[((g.d0 + d) * g.out_rows + g.out_row0 + kg) * g.ng_half + (i - d * g.ng_half)] = make_double2(NAN, NAN);
+        }
+    }
     if (warp == kTcMmaWarp) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols) : "memory");
@@ -1935,7 +1943,20 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) 
     }
     tc_fence_before();
     __syncthreads();
-    if (*abort_flag && tid == 0) atomicOr(g.err, 1);
+    if (*abort_flag) {
+        if (tid == 0) atomicOr(g.err, 1);
+        // NaN over the terms of the CTA's units: what its own block groups hold nobody writes again
+        for (int ju = j0; ju < j1; ++ju) {
+            const int4 un = __ldg(g.units + __ldg(ulist + ju));
+            const int L = un.x & 255, part = un.x >> 8;
+            const long long cnt = g.cls_start[L + 1] - g.cls_start[L], loc = un.w - g.cls_start[L];
+            const int nv = (int)min((long long)kTcM, cnt - loc), nt = nterms(L + E);
+            for (int i = tid; i < g.nd * g.nsub * nt * nv; i += kTcThreadsAll) {
+                const int r = i % nv, t = (i / nv) % nt, sub = (i / nv / nt) % g.nsub, d = i / nv / nt / g.nsub;
+                g.Jp[((long long)(g.d0 + d) * g.nparts + part * g.nsub + sub) * g.jp_total + g.term_base[L] + t * cnt + loc + r] = NAN;
+            }
+        }
+    }
     if (warp == kTcMmaWarp) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols) : "memory");

@@ -309,7 +309,8 @@ class Batch:
         _check(lib().ftcj_batch_set_wait(self._h, int(wait_log2)), "ftcj_batch_set_wait")
 
     def status(self, stream=None) -> int:
-        """Error word of the last persistent launch; raises FtcjError (FTCJ_ETIMEOUT) when a wait gave up."""
+        """Error word of the last persistent launch and of the cells' plans; raises FtcjError (FTCJ_ETIMEOUT) when a
+        wait gave up."""
         w = _c_int(0)
         _check(lib().ftcj_batch_status(self._h, ctypes.byref(w), _stream_ptr(stream)), "ftcj_batch_status")
         return int(w.value)

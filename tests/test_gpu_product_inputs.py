@@ -1,6 +1,6 @@
 """What the sliced product has to take as the walks do: general contractions
 with many functions per primitive, densities that are not finite, and very small
-and very large ones."""
+and very large ones; and what a caller sees of a bounded wait that gave up."""
 import numpy as np
 import pytest
 
@@ -141,3 +141,46 @@ def test_builds_scale_with_the_density(F, kind):
             dg = float((g[0] / s / s - g0[0]).abs().max()) / float(g0[0].abs().max())
             assert dg <= tol * 10, (e, dg)
     plan.close()
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_a_wait_that_gives_up_is_seen(F, kind, monkeypatch):
+    """With a wait budget of 2 clock cycles the products give up and return: J^k and E_J are NaN, not what an earlier
+    build left, the host call raises, and a batch reports it.  The next plan on the same GPU builds as before."""
+    import torch
+    w, args = pair_of_densities(kind)
+    D = device(w)
+    good = F.Plan.from_workload(w, **args)
+    J0, E0 = good.jbuild(D)
+    plan = F.Plan.from_workload(w, tc_wait_log2=1, **args)
+    J, E = plan.jbuild(D)
+    torch.cuda.synchronize()
+    assert not bool(torch.isfinite(E).any()) and not bool(torch.isfinite(J.real)[touched(J0)].any())
+    assert plan.status() & 1 and plan.status() == 0
+    if kind != "classified":
+        _, g = plan.grad(D)
+        assert not bool(torch.isfinite(g).any()) and plan.status() & 1
+    with pytest.raises(F.FtcjError, match="timed out"):
+        plan.jbuild_host(w.Dk)
+    assert plan.status() == 0
+    plan.close()
+    if kind == "fp64":
+        params = F._params_of
+
+        def impatient(*a, **k):
+            p = params(*a, **k)
+            p.tc_wait_log2 = 1
+            return p
+
+        monkeypatch.setattr(F, "_params_of", impatient)
+        batch = F.Batch([w, w])
+        assert batch.infos[0]["contraction"] == F.FTCJ_CONTRACT_TC
+        batch.jbuild([D, D])
+        with pytest.raises(F.FtcjError, match="timed out"):
+            batch.status()
+        assert batch.status() == 0
+        batch.close()
+    J, E = good.jbuild(D)
+    torch.cuda.synchronize()
+    assert good.status() == 0 and float((J - J0).abs().max()) <= 1e-12 * max(1.0, float(J0.abs().max()))
+    good.close()
