@@ -560,10 +560,14 @@ int create(const ftcj_cell* cell, const ftcj_basis* basis, const int kmesh[3], c
     // (molecular crystal, a build: 7.57 ms with one wave of blocks, 7.47 with two, 7.45 with four, 7.37 with six)
     const int waves = P->precision == FTCJ_PREC_SPLIT && P->d_rec_gcut && nch > 1 ? 6 : 1;
     P->npb = std::max(1, std::min<int>((int)std::max<size_t>(1, P->tiles.size()), waves * P->num_sms * bps / nch));
-    // several short chunks of few tiles: one block per (tile, chunk), dealt by the hardware, comes out more even than
-    // one wave of blocks of which some hold two tiles
-    if (nch > 1 && P->tiles.size() < 4 * (size_t)P->num_sms && prm->chunk_points <= 0)
-        P->npb = (int)std::max<size_t>(1, P->tiles.size());
+    // several chunks of few tiles: one block per (tile, chunk), dealt by the hardware, comes out more even than one wave
+    // of blocks of which some hold two tiles (1,481 records, 158,239 points in 160 chunks: structure factors 2162 us with
+    // 11 blocks a chunk, 2042 with 14).  Each block has a row of partial sums as long as the sphere: up to 128 MB of
+    // them a density, so that sphere and tiles do not multiply without limit
+    if (nch > 1 && P->tiles.size() < 4 * (size_t)P->num_sms && prm->chunk_points <= 0) {
+        const int64_t rows = std::max<int64_t>(1, (int64_t)(128u << 20) / (int64_t)(sizeof(double2) * P->ng_half));
+        P->npb = std::max(P->npb, (int)std::min<int64_t>((int64_t)P->tiles.size(), rows));
+    }
     if (prm->rho_blocks > 0) {
         P->npb = std::min<int>(prm->rho_blocks, (int)std::max<size_t>(1, P->tiles.size()));
         P->rho_hi_tiles = 0;  // an explicit block count keeps the one-launch walk
@@ -602,7 +606,7 @@ int create(const ftcj_cell* cell, const ftcj_basis* basis, const int kmesh[3], c
         FTCJ_CUDA(cudaMemGetInfo(&room, &all));
         // what the plan has yet to allocate, roughly
         const size_t rest = 8 * md * (10 * (size_t)P->nk * nn + (size_t)std::max(nch + 1, P->tcg.parts) * (size_t)(P->total_terms + P->total_terms_g) +
-                                      2 * (size_t)std::max(P->npb, P->tc_out_rows) * (size_t)P->ng_half);
+                                      2 * (size_t)P->tc_out_rows * (size_t)P->ng_half);
         if (rc == FTCJ_EUNSUPPORTED || rc == FTCJ_ENOMEM || (rc == FTCJ_OK && room < rest)) {
             release_tc(P);
             P->device_bytes = bytes;
@@ -621,7 +625,7 @@ int create(const ftcj_cell* cell, const ftcj_basis* basis, const int kmesh[3], c
     if ((rc = dalloc(P, &P->d_Dp, md * (size_t)std::max<long long>(P->total_terms, P->tc_dp_total) + 64))) return rc;
     if ((rc = dalloc(P, &P->d_Jp, md * (size_t)std::max(nch, jp_chunks(P)) * (size_t)P->total_terms))) return rc;
     if ((rc = dalloc(P, &P->d_Jg, md * (size_t)std::max(nch, P->tcg.parts) * (size_t)P->total_terms_g))) return rc;
-    if ((rc = dalloc(P, &P->d_rho_part, 2 * md * (size_t)std::max(P->npb, P->rho_rows) * (size_t)P->ng_half)))
+    if ((rc = dalloc(P, &P->d_rho_part, 2 * md * (size_t)P->rho_rows * (size_t)P->ng_half)))
         return rc;
     if ((rc = dalloc(P, &P->d_rho, 2 * md * (size_t)P->ng_half))) return rc;
     if ((rc = dalloc(P, &P->d_W, 2 * md * (size_t)P->ng_half))) return rc;

@@ -89,3 +89,26 @@ def test_gradient_assembly_over_few_and_many_centres(orc, F, centres, exps):
         print(f"{centres} centres precision {precision}: records {plan.info['npairs']} max|dgrad|={err:.2e}")
         assert err <= 1e-10 * max(1.0, float(np.abs(ref).max()))
         plan.close()
+
+
+def test_rows_of_partial_sums_of_a_long_sphere(F):
+    """Few tiles over many chunks: a walk block per tile as long as the partial rows, each as long as the sphere, stay
+    within 128 MB; the same J as from two blocks (the form's 1e-8 of max|J|)."""
+    import torch
+    spec = [(c, l, [0.2 * 1.15 ** q for q in range(n)]) for c in range(12) for l, n in ((0, 14), (1, 8), (2, 4))]
+    w = W.tiny(seed=77, A=np.diag([30.0, 32.0, 34.0]) + 4.0 * TRI, shell_spec=spec, omega=0.5, eps_g=1e-30,
+               centres=[[1.7 * i, 1.9 * j, 0.3 * (i + j)] for i in range(4) for j in range(3)])
+    Dk = torch.from_numpy(np.ascontiguousarray(w.Dk)).cuda()
+    got = []
+    for blocks in (0, 2):
+        plan = F.Plan.from_workload(w, precision=F.FTCJ_PREC_SPLIT, rho_blocks=blocks)
+        info = plan.info
+        if not blocks:
+            tiles = sum(-(-n // 128) for n in info["pairs_by_class"])
+            print(f"points {info['ng_half']} chunks {info['nchunks']} tiles {tiles} blocks {info['rho_blocks']}")
+            assert info["nchunks"] > 100 and info["rho_blocks"] * info["ng_half"] * 16 <= 128 << 20
+            assert info["rho_blocks"] < tiles
+        got.append(plan.jbuild(Dk)[0])
+        torch.cuda.synchronize()
+        plan.close()
+    assert float((got[0] - got[1]).abs().max()) <= 1e-8 * max(1.0, float(got[1].abs().max()))
