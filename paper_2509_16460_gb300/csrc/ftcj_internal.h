@@ -252,6 +252,7 @@ struct ftcj_plan {
     double* d_check = nullptr;       // [2]
     void* d_split_init = nullptr;    // split form: walk state at each chunk start, [nchunks][npairs]
     void* d_split_const = nullptr;   // split form: recurrence multipliers, [npairs]
+    bool products = true;  // the plan may take sliced products of its own choice (false: short of device memory)
     // tensor-core separable contraction of the structure-factor pass (tc.cu)
     bool tc = false;
     bool tc_rho_only = false;  // split plan whose walks take the structure factors from the eight-slice product

@@ -898,6 +898,7 @@ int galloc(ftcj_plan* P, Gpw* g, T** ptr, size_t count) {
     const size_t bytes = sizeof(T) * count;
     cudaError_t e = cudaMalloc((void**)ptr, bytes);
     if (e != cudaSuccess) {
+        cudaGetLastError();  // clear the non-sticky error
         *ptr = nullptr;
         return fail(FTCJ_ENOMEM, std::string("cudaMalloc of ") + std::to_string(bytes) +
                                      " bytes for the GPW grid failed: " + cudaGetErrorString(e));
@@ -1055,7 +1056,7 @@ int setup_gpw(ftcj_plan* P) {
         k_gpw_vfr<<<(unsigned)((P->ng_half + 255) / 256), 256>>>(P->d_gvec, P->ng_half, P->cc, g->d_vfr);
         FTCJ_CUDA(cudaGetLastError());
     }
-    if (g->sep && own_grid && P->ng_half > 0 && P->n_abs_max <= kSplitNmax) {
+    if (P->products && g->sep && own_grid && P->ng_half > 0 && P->n_abs_max <= kSplitNmax) {
         rc = setup_product(P, D);
         if (rc == FTCJ_OK) {
             g->product = true;

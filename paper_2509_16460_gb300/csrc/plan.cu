@@ -253,6 +253,7 @@ int dalloc(ftcj_plan* P, T** ptr, size_t count) {
     size_t bytes = sizeof(T) * count;
     cudaError_t e = cudaMalloc((void**)ptr, bytes);
     if (e != cudaSuccess) {
+        cudaGetLastError();  // clear the non-sticky error
         *ptr = nullptr;
         return fail(FTCJ_ENOMEM, std::string("cudaMalloc of ") + std::to_string(bytes) + " bytes failed: " +
                                      cudaGetErrorString(e));
@@ -589,11 +590,11 @@ int create(const ftcj_cell* cell, const ftcj_basis* basis, const int kmesh[3], c
     // throughput for each FP64 lane that the walks would use (both passes: slab of 940 AOs, walks 36.7 ms, contraction
     // 1.55 ms; diamond cell 2.02 and 0.30 ms; 18 AOs 0.33 and 0.08 ms).
     // A caller's own walk shape, |n_i| above 63 (powers of n exact in FP32 no longer), spheres wider than the MMA
-    // and plans short of memory keep the walks.  The split form's walks take the structure factors from it too where
+    // and plans short of memory (see ftcj_plan_create) keep the walks.  The split form's walks take the structure factors from it too where
     // the sphere fills the product's tiles of 128 rows and the work its launches (slab 3.03 -> 0.82 ms; 706 half-sphere
     // points, 34,131 records: 174 -> 119 us; 582, 6,695: 55 -> 48; but 230, 111,640: 162 -> 193 and 1,026, 814:
     // 31 -> 44).
-    const bool whole = P->ortho && !P->tc && !P->d_rec_gcut && prm->chunk_points <= 0 && prm->rho_blocks <= 0 &&
+    const bool whole = P->products && P->ortho && !P->tc && !P->d_rec_gcut && prm->chunk_points <= 0 && prm->rho_blocks <= 0 &&
                        P->n_abs_max <= kSplitNmax && P->npairs > 0 && P->ng_half > 0;
     const bool split_rho = P->precision == FTCJ_PREC_SPLIT && P->ng_half >= 512 && P->npairs * P->ng_half >= 3000000;
     const size_t nn = (size_t)P->nao * P->nao, md = (size_t)P->max_dens;
@@ -602,12 +603,7 @@ int create(const ftcj_cell* cell, const ftcj_basis* basis, const int kmesh[3], c
         P->tc = true;
         P->tc_rho_only = split_rho;
         rc = setup_tc(P);
-        size_t room = 0, all = 0;
-        FTCJ_CUDA(cudaMemGetInfo(&room, &all));
-        // what the plan has yet to allocate, roughly
-        const size_t rest = 8 * md * (10 * (size_t)P->nk * nn + (size_t)std::max(nch + 1, P->tcg.parts) * (size_t)(P->total_terms + P->total_terms_g) +
-                                      2 * (size_t)P->tc_out_rows * (size_t)P->ng_half);
-        if (rc == FTCJ_EUNSUPPORTED || rc == FTCJ_ENOMEM || (rc == FTCJ_OK && room < rest)) {
+        if (rc == FTCJ_EUNSUPPORTED) {
             release_tc(P);
             P->device_bytes = bytes;
             P->tc_rho_only = false;
@@ -676,23 +672,32 @@ int ftcj_plan_create(const ftcj_cell* cell, const ftcj_basis* basis, const int k
                      ftcj_plan** out) {
     if (!out) return fail(FTCJ_EINVAL, "null output pointer");
     *out = nullptr;
-    ftcj_plan* P = new (std::nothrow) ftcj_plan();
-    if (!P) return fail(FTCJ_ENOMEM, "host allocation failed");
-    int rc;
-    try {
-        rc = create(cell, basis, kmesh, params, P);
-    } catch (const std::bad_alloc&) {
-        rc = fail(FTCJ_ENOMEM, "host allocation failed");
-    } catch (...) {
-        rc = fail(FTCJ_EINVAL, "unexpected host exception");
-    }
-    if (rc != FTCJ_OK) {
+    // a plan that runs out of device memory with sliced products of its own choice is made again without them: the
+    // walks and the grid need less
+    for (const bool products : {true, false}) {
+        ftcj_plan* P = new (std::nothrow) ftcj_plan();
+        if (!P) return fail(FTCJ_ENOMEM, "host allocation failed");
+        P->products = products;
+        int rc;
+        try {
+            rc = create(cell, basis, kmesh, params, P);
+        } catch (const std::bad_alloc&) {
+            rc = fail(FTCJ_ENOMEM, "host allocation failed");
+        } catch (...) {
+            rc = fail(FTCJ_EINVAL, "unexpected host exception");
+        }
+        if (rc == FTCJ_OK) {
+            *out = P;
+            return FTCJ_OK;
+        }
+        const bool chosen = (P->tc && P->params.contraction == FTCJ_CONTRACT_WALK) || (P->dd && P->dd->tc);
+        const bool memory = rc == FTCJ_ENOMEM || (rc == FTCJ_ECUDA && cudaPeekAtLastError() == cudaErrorMemoryAllocation);
         free_device(P);
         delete P;
-        return rc;
+        if (memory) cudaGetLastError();  // clear the non-sticky error
+        if (!(products && chosen && memory)) return rc;
     }
-    *out = P;
-    return FTCJ_OK;
+    return FTCJ_ENOMEM;
 }
 
 int ftcj_plan_info(const ftcj_plan* P, ftcj_info* o) {

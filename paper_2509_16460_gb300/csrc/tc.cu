@@ -105,7 +105,7 @@ constexpr int kTcGmax = 15;                    // (i, j) blocks per window at mo
 constexpr int kTcNbufMax = 4;                  // stage buffers at most
 constexpr int kTcTabSlotsMax = 6;              // stage tables in flight at most
 constexpr int kTcAsliceBytes = kTcM * kTcStageK * 2;      // 128 rows x 16 K x bf16
-constexpr long long kTcBWorkMax = 8LL << 30;              // bytes of B tiles per pass
+constexpr long long kTcBWorkMax = 8LL << 30;              // bytes of B tiles per pass at most
 constexpr long long kTcSpinCycles = 1LL << 32;            // ~2 s of SM clock per wait
 // Exponent bound of a column with a NaN or an infinity.  Slices hold neither
 // (their digits come from integer operations or cancelling sums), so the sums
@@ -2206,10 +2206,15 @@ int setup_tc(ftcj_plan* P) {
         }
     }
     // Passes: the B tiles of a pass's windows fill one workspace, bounded so that a large system reuses it
-    // instead of growing it; each pass deals its windows to CTA groups, one CTA per SM over all (group, row
+    // instead of growing it, by 8 GB and by 1/32 of the memory that is free now, so that further plans and the caller
+    // find theirs (each further pass costs 70 to 130 us: crystal of 1056 AOs, FP64, 2461 us in one pass, 2529 in two,
+    // 2660 in four); each pass deals its windows to CTA groups, one CTA per SM over all (group, row
     // tile) pairs, so that the grid is a single wave (a partial second wave would double the pass)
     const int nwin = (int)wins.size();
     P->tc_nwin = nwin;
+    size_t room = 0, all = 0;
+    FTCJ_CUDA(cudaMemGetInfo(&room, &all));
+    const long long work_max = std::min(kTcBWorkMax, (long long)(room / 32));
     std::vector<int4> winfo((size_t)std::max(1, nwin), make_int4(0, 0, 0, 0));
     std::vector<int> wcnt((size_t)std::max(1, nwin), 0);
     std::vector<long long> boff((size_t)std::max(1, nwin), 0);
@@ -2223,7 +2228,7 @@ int setup_tc(ftcj_plan* P) {
         while (w1 < nwin) {
             const Win& w = wins[w1];
             const long long n = (long long)((w.cnt + kTcStageK - 1) / kTcStageK) * slices * mma_cols(w.info.y, P->tc_colw) * 2;
-            if (w1 > w0 && (off + n) * 16 > kTcBWorkMax) break;
+            if (w1 > w0 && (off + n) * 16 > work_max) break;
             winfo[w1] = w.info;
             wcnt[w1] = w.cnt;
             boff[w1] = off;
