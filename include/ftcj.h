@@ -181,8 +181,8 @@ typedef struct {
     int n_abs_max;            /* largest |n_i| of the sphere's G = sum_i n_i b_i (the split form
                                  needs <= 63) */
     int grad_split;           /* 1: the plan's gradient walk is the double-float one (split form
-                                 with n_abs_max <= 27), 0: the FP64 one; plans whose contraction
-                                 is TC by themselves and n_abs_max <= 27 run the sliced product */
+                                 with n_abs_max <= 27), 0: the FP64 one (grad_contraction says
+                                 whether it runs) */
     int rho_walk_launches;    /* kernel launches of one structure-factor walk pass: 2 where the
                                  split form runs it as two class parts, else 1 (0: nothing to walk) */
     int j_walk_launches;      /* the same for the back-contraction walk */
@@ -212,6 +212,8 @@ typedef struct {
     int gpw_launches;         /* kernel launches of the GPW route in one build over max_dens densities */
     int64_t dd_pairs_by_class[5]; /* DD records of class L = l_a + l_b (the GPW route's cost per grid point
                                      and density is 2 (L + 1) flops in each of collocation and integration) */
+    int grad_contraction;     /* the form of ftcj_grad's degree-(L+1) sums: FTCJ_CONTRACT_TC (the eight-slice
+                                 product) or FTCJ_CONTRACT_WALK (grad_split says in which precision) */
 } ftcj_info;
 
 typedef struct ftcj_plan ftcj_plan;

@@ -733,6 +733,7 @@ int ftcj_plan_info(const ftcj_plan* P, ftcj_info* o) {
     o->tc_mma_flops = P->tc ? P->tc_mma_flops : 0;
     o->j_contraction = P->tcj.on ? FTCJ_CONTRACT_TC : FTCJ_CONTRACT_WALK;
     o->tc_j_mma_flops = P->tcj.on ? P->tcj.mma_flops : 0;
+    o->grad_contraction = P->tcg.on ? FTCJ_CONTRACT_TC : FTCJ_CONTRACT_WALK;
     if (P->tc) {
         o->tc_column_axis = P->tc_axis[2];
         o->tc_rows = P->tc_rows;

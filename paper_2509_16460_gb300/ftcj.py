@@ -60,7 +60,7 @@ class Info(ctypes.Structure):
                 ("tc_blocks_per_window", _c_int), ("tc_dens_per_launch", _c_int),
                 ("dd_pairs", ctypes.c_int64), ("dd_pairs_ordered", ctypes.c_int64), ("alpha_cut", _c_double),
                 ("gpw_grid", _c_int * 3), ("gpw_separable", _c_int), ("gpw_launches", _c_int),
-                ("dd_pairs_by_class", ctypes.c_int64 * 5)]
+                ("dd_pairs_by_class", ctypes.c_int64 * 5), ("grad_contraction", _c_int)]
 
     def as_dict(self):
         d = {k: getattr(self, k) for k, _ in self._fields_}

@@ -165,3 +165,27 @@ def test_gradient_sums_of_the_product(orc, F, index):
         assert float(np.abs(last.cpu().numpy() - ref[-1:]).max()) <= 1e-10 * scale
         plan.close()
     assert float(np.abs(got[0] - got[1]).max()) <= 1e-10 * scale
+
+
+#       edges               omega  the sums' form
+GRADIENT_CELLS = [([5.0, 6.1, 7.3], 0.45, "product"),
+                  ([4.1, 4.4, 34.0], 0.50, "walk")]  # |n| up to 30: n^5 is not exact in FP32
+
+
+@pytest.mark.parametrize("edges,omega,form", GRADIENT_CELLS)
+def test_form_of_the_gradient_sums(orc, F, edges, omega, form):
+    """Which form runs the degree-(L+1) sums, and that the structure factors' product with the walk's sums gives the
+    oracle's gradient too (the bar of the product's, above)."""
+    import torch
+    w = W.tiny(seed=66, A=np.diag(edges), centres=[[0.1, 0.2, 0.3], [1.3, 0.9, -0.4]], shell_spec=SP, omega=omega)
+    ref = orc.grad(w)
+    plan, walk = F.Plan.from_workload(w), F.Plan.from_workload(w, chunk_points=4096)
+    assert plan.info["contraction"] == F.FTCJ_CONTRACT_TC and walk.info["contraction"] == F.FTCJ_CONTRACT_WALK
+    assert plan.info["grad_contraction"] == (F.FTCJ_CONTRACT_TC if form == "product" else F.FTCJ_CONTRACT_WALK)
+    assert walk.info["grad_contraction"] == F.FTCJ_CONTRACT_WALK
+    _, grad = plan.grad(torch.from_numpy(np.ascontiguousarray(w.Dk)).cuda())
+    torch.cuda.synchronize()
+    assert plan.status() == 0
+    assert float(np.abs(grad.cpu().numpy() - ref).max()) <= 1e-10 * max(1.0, float(np.abs(ref).max()))
+    plan.close()
+    walk.close()
