@@ -1969,14 +1969,14 @@ size_t tc_j_smem_bytes(int slices, int npad, int tws, int nbuf) {
     return std::max<size_t>(need, 120 * 1024);
 }
 
-// work dealt to nbin bins, largest first, each to the least loaded bin (ties
-// to the lower one): nbin + 1 offsets, then the item ids of each bin
 // the gradient's sums keep to the eight-slice form (double-float or FP64 precision)
 const void* tc_j_kernel(bool f64, int extra) {
     if (extra) return (const void*)k_tc_j<Prec64, 1>;
     return f64 ? (const void*)k_tc_j<Prec64, 0> : (const void*)k_tc_j<PrecJ, 0>;
 }
 
+// work dealt to nbin bins, largest first, each to the least loaded bin (ties
+// to the lower one): nbin + 1 offsets, then the item ids of each bin
 std::vector<int> deal(const std::vector<double>& cost, int nbin) {
     std::vector<int> order(cost.size());
     for (size_t k = 0; k < order.size(); ++k) order[k] = (int)k;
@@ -2029,12 +2029,12 @@ long long tc_spin(const ftcj_plan* P) {
 
 int setup_tc_j(ftcj_plan* P, int extra);
 
-// Plan-time set-up of the tensor-core form: the column axis, the slots and the
-// half-sphere map, the factor tables, the windows (class, block group, records
-// sorted by width), their deal to CTA groups and the B tiles.
 // FP64 plans and the structure factors of split walks: the finer of the two precisions
 inline bool tc_eight_slices(const ftcj_plan* P) { return P->precision == FTCJ_PREC_FP64 || P->tc_rho_only; }
 
+// Plan-time set-up of the tensor-core form: the column axis, the slots and the
+// half-sphere map, the factor tables, the windows (class, block group, records
+// sorted by width), their deal to CTA groups and the B tiles.
 int setup_tc(ftcj_plan* P) {
     if (!P->ortho) return fail(FTCJ_EUNSUPPORTED, "the tensor-core contraction needs an orthorhombic cell");
     const bool f64 = tc_eight_slices(P);
@@ -2390,9 +2390,9 @@ int tc_rho_launches(const ftcj_plan* P, int nd) {
 
 // Plan-time set-up of the tensor-core back-contraction: densities per
 // launch, (i, j) blocks per group, the work units, their deal to the CTAs and
-// the V_ij tile buffer.  tc_j stays false, and the split walk runs the
-// back-contraction, where one density's columns exceed the MMA width or the
-// factor tables exceed shared memory.
+// the V_ij tile buffer.  TcBack::on stays false, and the walks run the
+// back-contraction (the gradient's sums), where one density's columns exceed
+// the MMA width or the factor tables exceed shared memory.
 int setup_tc_j(ftcj_plan* P, int extra) {
     TcBack& B = extra ? P->tcg : P->tcj;
     B.on = false;
@@ -2491,7 +2491,7 @@ int setup_tc_j(ftcj_plan* P, int extra) {
     B.G = G_best;
     B.npad = npad;
     B.nstage = nstage;
-    B.sub = std::max(1, 4 / (G_best * nd_best) == 3 ? 2 : 4 / (G_best * nd_best));
+    B.sub = std::max(1, 4 / (G_best * nd_best));
     B.parts = nparts * B.sub;
     B.spp = spp;
     B.grid = std::max(1, std::min(P->num_sms, (int)units.size()));

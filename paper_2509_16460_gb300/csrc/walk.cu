@@ -562,7 +562,7 @@ __device__ void j_tile(const double* M6, const Tile& tl, const Layout& lay, cons
                         Ar[0] += tr;
                         Ai[0] += ti;
                         const double* pwm = pw + (m - n1min) * kPw;
-    #pragma unroll
+#pragma unroll
                         for (int i = 1; i <= L; ++i) {
                             Ar[i] = fma(tr, pwm[i], Ar[i]);
                             Ai[i] = fma(ti, pwm[i], Ai[i]);
@@ -585,7 +585,7 @@ __device__ void j_tile(const double* M6, const Tile& tl, const Layout& lay, cons
                         Ar[0] += tr;
                         Ai[0] += ti;
                         const double* pwm = pw + (m - n1min) * kPw;
-    #pragma unroll
+#pragma unroll
                         for (int i = 1; i <= L; ++i) {
                             Ar[i] = fma(tr, pwm[i], Ar[i]);
                             Ai[i] = fma(ti, pwm[i], Ai[i]);

@@ -692,7 +692,7 @@ __device__ void j_tile_split(const Tile& tl, const Layout& lay, const SConst* __
             for (int dir = 0; dir < 2; ++dir) {
                 int m0, m1, step;
                 cdf gp, R;
-                    if (dir == 0) {
+                if (dir == 0) {
                     if (hi < 0) continue;
                     m0 = 0;
                     m1 = hi;
