@@ -266,6 +266,7 @@ struct ftcj_plan {
     int tc_out_rows = 0;                       // partial rows over all passes
     int tc_nbuf = 0, tc_tslots = 0;            // stage buffers and stage-table slots in shared memory
     int64_t tc_mma_flops = 0;                  // bf16 MMA flops of one pass over max_dens densities
+    void* d_tc_arena = nullptr;  // holds the tables below but for the factor tables, widths and operand tiles
     int* d_tc_slots = nullptr;   // [mtiles * 128]
     int* d_tc_quads = nullptr;   // [nslots / 4]
     int* d_tc_map = nullptr;     // [2 nna - 1][2 nnb - 1][ncols]

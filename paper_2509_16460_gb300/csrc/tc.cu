@@ -83,8 +83,8 @@
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <cstring>
 #include <queue>
-#include <set>
 #include <type_traits>
 #include <vector>
 
@@ -1322,12 +1322,62 @@ int tc_alloc(ftcj_plan* P, void** ptr, size_t bytes) {
     return FTCJ_OK;
 }
 
-template <class T>
-int tc_upload(ftcj_plan* P, T** ptr, const std::vector<T>& v) {
-    const int rc = tc_alloc(P, (void**)ptr, sizeof(T) * std::max<size_t>(v.size(), 1));
-    if (rc) return rc;
-    if (!v.empty()) FTCJ_CUDA(cudaMemcpy(*ptr, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice));
-    return FTCJ_OK;
+// The plan's host-made tables, gathered into one allocation and one copy
+// (some thirty of each took a third of a small plan's set-up)
+struct TcArena {
+    std::vector<unsigned char> host;
+    std::vector<std::pair<void**, size_t>> at;
+    // n elements, of which v gives the first (the rest start at zero)
+    template <class T>
+    void add(T** ptr, const std::vector<T>& v, size_t n = 0) {
+        const size_t off = (host.size() + 255) / 256 * 256;
+        at.push_back({(void**)ptr, off});
+        host.resize(off + sizeof(T) * std::max<size_t>({v.size(), n, 1}), 0);
+        if (!v.empty()) std::memcpy(host.data() + off, v.data(), sizeof(T) * v.size());
+    }
+    int commit(ftcj_plan* P) {
+        const int rc = tc_alloc(P, &P->d_tc_arena, host.size());
+        if (rc) return rc;
+        for (const auto& q : at) *q.first = (unsigned char*)P->d_tc_arena + q.second;
+        FTCJ_CUDA(cudaMemcpy(P->d_tc_arena, host.data(), host.size(), cudaMemcpyHostToDevice));
+        return FTCJ_OK;
+    }
+};
+
+// Records [first, last) in the order of their widths, stable.  Positive floats
+// order as their bits: one counting pass by the upper 17, then the buckets that
+// hold several widths are sorted.
+std::vector<int> sort_by_width(int64_t first, int64_t last, const std::vector<float>& width) {
+    using Item = std::pair<uint32_t, int>;
+    const auto less = [](const Item& x, const Item& y) { return x.first < y.first; };
+    std::vector<Item> a((size_t)(last - first));
+    const auto item = [&](int64_t r) {
+        Item q{0u, (int)r};
+        std::memcpy(&q.first, &width[r], 4);
+        return q;
+    };
+    if (last - first < 4096) {  // fewer than the buckets are worth
+        for (int64_t r = first; r < last; ++r) a[r - first] = item(r);
+        std::stable_sort(a.begin(), a.end(), less);
+    } else {
+        constexpr int kShift = 15;
+        std::vector<int> start((1u << (32 - kShift)) + 1, 0);
+        for (int64_t r = first; r < last; ++r) ++start[(item(r).first >> kShift) + 1];
+        for (size_t d = 1; d < start.size(); ++d) start[d] += start[d - 1];
+        for (int64_t r = first; r < last; ++r) {
+            const Item q = item(r);
+            a[start[q.first >> kShift]++] = q;
+        }
+        for (size_t i = 0, j; i < a.size(); i = j) {
+            bool sorted = true;
+            for (j = i + 1; j < a.size() && (a[j].first >> kShift) == (a[i].first >> kShift); ++j)
+                sorted = sorted && a[j - 1].first <= a[j].first;
+            if (!sorted) std::stable_sort(a.begin() + i, a.begin() + j, less);
+        }
+    }
+    std::vector<int> out(a.size());
+    for (size_t k = 0; k < a.size(); ++k) out[k] = a[k].second;
+    return out;
 }
 
 int round_up(int x, int m) { return (x + m - 1) / m * m; }
@@ -1377,7 +1427,7 @@ void tc_columns(int nmax, int nd, int ncols, int* colw, int* G, int* npad) {
 // points share a group (the free bit says which); the origin takes one more.
 // quads: the same groups for the back-contraction's operand former (bit 0:
 // both indices positive, bit 1: n_b = 0, then two indices of 8 bits).
-void tc_slots(const std::set<std::pair<int, int>>& pts, std::vector<int>& slots, std::vector<int>& quads) {
+void tc_slots(const std::vector<std::pair<int, int>>& pts, std::vector<int>& slots, std::vector<int>& quads) {
     std::vector<int> axa, axb;  // n_a > 0, n_b = 0 and n_a = 0, n_b > 0
     bool origin = false;
     slots.clear();
@@ -2005,18 +2055,15 @@ std::vector<int> deal(const std::vector<double>& cost, int nbin) {
 }  // namespace
 
 void release_tc(ftcj_plan* P) {
-    void** ptrs[] = {(void**)&P->d_tc_slots, (void**)&P->d_tc_quads, (void**)&P->d_tc_map, (void**)&P->d_tc_wpairs,
-                     &P->d_tc_winfo, (void**)&P->d_tc_wcnt, (void**)&P->d_tc_boff, (void**)&P->d_tc_sched, &P->d_tc_b,
-                     &P->d_tc_tab, &P->d_tc_tabk, &P->d_tc_tabz, &P->d_tc_tabz3, (void**)&P->d_tc_cl, (void**)&P->d_tc_kpos,
-                     (void**)&P->d_tc_korder, (void**)&P->d_tc_err, (void**)&P->d_tc_pos, (void**)&P->d_tc_clw, (void**)&P->d_tc_ew,
-                     &P->tcj.items, &P->tcj.groups, (void**)&P->tcj.pairs, (void**)&P->tcj.sched, &P->tcj.vs,
-                     (void**)&P->tcj.voff, (void**)&P->tcj.vplace, (void**)&P->tcj.ev, (void**)&P->tcj.er,
-                     &P->tcg.items, &P->tcg.groups, (void**)&P->tcg.pairs, (void**)&P->tcg.sched, &P->tcg.vs,
-                     (void**)&P->tcg.voff, (void**)&P->tcg.vplace, (void**)&P->tcg.ev, (void**)&P->tcg.er};
-    for (void** p : ptrs) {
+    void** owned[] = {&P->d_tc_arena, (void**)&P->d_tc_cl, &P->d_tc_tab, &P->d_tc_tabk, &P->d_tc_tabz, &P->d_tc_tabz3,
+                      &P->d_tc_b, &P->tcj.vs, &P->tcg.vs};
+    for (void** p : owned) {
         if (*p) cudaFree(*p);
         *p = nullptr;
     }
+    // tables inside the arena; of these, callers ask for the error word and the K order
+    P->d_tc_err = nullptr;
+    P->d_tc_pos = nullptr;
     P->tc = P->tcj.on = P->tcg.on = false;
     P->tc_dp_total = 0;
     P->tc_passes.clear();
@@ -2027,7 +2074,7 @@ long long tc_spin(const ftcj_plan* P) {
     return P->params.tc_wait_log2 > 0 ? (1LL << P->params.tc_wait_log2) : kTcSpinCycles;
 }
 
-int setup_tc_j(ftcj_plan* P, int extra);
+int setup_tc_j(ftcj_plan* P, int extra, TcArena& arena);
 
 // FP64 plans and the structure factors of split walks: the finer of the two precisions
 inline bool tc_eight_slices(const ftcj_plan* P) { return P->precision == FTCJ_PREC_FP64 || P->tc_rho_only; }
@@ -2051,7 +2098,6 @@ int setup_tc(ftcj_plan* P) {
     // block, n_c) the epilogue.  The per-entry costs are measured ones.
     const double kB = f64 ? 5.0 : 3.7, kE = f64 ? 5.0 : 2.9;
     struct AxisPlan {
-        std::set<std::pair<int, int>> pts;
         std::vector<int> slots, quads;
         size_t rows = 0;
         int ncols = 0, nd = 0, colw = 0, G = 0, npad = 0, nam = 0, nbm = 0;
@@ -2061,26 +2107,32 @@ int setup_tc(ftcj_plan* P) {
     for (int c = 0; c < 3; ++c) {
         const int a = (c + 1) % 3, b = (c + 2) % 3;
         AxisPlan ap;
-        std::set<std::pair<int, int>> rs;
         int ncmax = 0;
         for (int64_t q = 0; q < ngh; ++q) {
-            int n[3] = {P->gvec[3 * q], P->gvec[3 * q + 1], P->gvec[3 * q + 2]};
-            if (n[c] < 0)
-                for (int x = 0; x < 3; ++x) n[x] = -n[x];
-            rs.insert({n[a], n[b]});
-            ap.pts.insert({std::abs(n[a]), std::abs(n[b])});
-            ap.nam = std::max(ap.nam, std::abs(n[a]));
-            ap.nbm = std::max(ap.nbm, std::abs(n[b]));
-            ncmax = std::max(ncmax, n[c]);
+            ap.nam = std::max(ap.nam, std::abs(P->gvec[3 * q + a]));
+            ap.nbm = std::max(ap.nbm, std::abs(P->gvec[3 * q + b]));
+            ncmax = std::max(ncmax, std::abs(P->gvec[3 * q + c]));
         }
-        ap.rows = rs.size();
+        // (n_a, n_b) at n_c >= 0, and their absolute values
+        std::vector<char> signed_seen((size_t)(2 * ap.nam + 1) * (2 * ap.nbm + 1), 0);
+        std::vector<char> seen((size_t)(ap.nam + 1) * (ap.nbm + 1), 0);
+        for (int64_t q = 0; q < ngh; ++q) {
+            const int sg = P->gvec[3 * q + c] < 0 ? -1 : 1, na = sg * P->gvec[3 * q + a], nb = sg * P->gvec[3 * q + b];
+            signed_seen[(size_t)(na + ap.nam) * (2 * ap.nbm + 1) + nb + ap.nbm] = 1;
+            seen[(size_t)std::abs(na) * (ap.nbm + 1) + std::abs(nb)] = 1;
+        }
+        std::vector<std::pair<int, int>> pts;
+        for (int na = 0; na <= ap.nam; ++na)
+            for (int nb = 0; nb <= ap.nbm; ++nb)
+                if (seen[(size_t)na * (ap.nbm + 1) + nb]) pts.push_back({na, nb});
+        ap.rows = (size_t)std::count(signed_seen.begin(), signed_seen.end(), 1);
         ap.ncols = ncmax + 1;
         for (ap.nd = std::min(P->max_dens, kTcDensMax); ap.nd >= 1; --ap.nd) {
             tc_columns(nmax, ap.nd, ap.ncols, &ap.colw, &ap.G, &ap.npad);
             if (ap.G > 0) break;
         }
         if (ap.nd < 1 || ap.G < 1) continue;
-        tc_slots(ap.pts, ap.slots, ap.quads);
+        tc_slots(pts, ap.slots, ap.quads);
         const double mt = (double)((ap.slots.size() + kTcM - 1) / kTcM);
         const double launches = (double)((P->max_dens + ap.nd - 1) / ap.nd);
         double cost = 0.0;
@@ -2134,8 +2186,9 @@ int setup_tc(ftcj_plan* P) {
     P->tc_tws = tws;
     const size_t nrec = (size_t)std::max<int64_t>(P->npairs, 1);
     int rc;
-    if ((rc = tc_alloc(P, (void**)&P->d_tc_err, sizeof(int)))) return rc;
-    FTCJ_CUDA(cudaMemset(P->d_tc_err, 0, sizeof(int)));
+    TcArena arena;
+    arena.host.reserve(16 * nrec + 8 * map.size() + (1 << 18));
+    arena.add(&P->d_tc_err, std::vector<int>(1, 0));
     if ((rc = tc_alloc(P, (void**)&P->d_tc_cl, sizeof(float) * nrec))) return rc;
     std::vector<float> clh(nrec, 0.f);
     if (P->npairs > 0) {
@@ -2155,9 +2208,8 @@ int setup_tc(ftcj_plan* P) {
     std::vector<int> pos(nrec, 0), kpos(nrec, 0), korder(nrec, 0);
     std::vector<float> clk(nrec, 0.f);
     for (int L = 0; L < kNclass; ++L) {
-        std::vector<int>& recs = order[L];
-        for (int64_t r = P->class_start[L]; r < P->class_start[L + 1]; ++r) recs.push_back((int)r);
-        std::stable_sort(recs.begin(), recs.end(), [&](int x, int y) { return clh[x] < clh[y]; });
+        order[L] = sort_by_width(P->class_start[L], P->class_start[L + 1], clh);
+        const std::vector<int>& recs = order[L];
         for (size_t k = 0; k < recs.size(); ++k) {
             pos[recs[k]] = (int)k;
             kpos[recs[k]] = (int)(P->class_start[L] + (int64_t)k);
@@ -2269,13 +2321,24 @@ int setup_tc(ftcj_plan* P) {
             }
     if (!P->tc_tslots)
         return fail(FTCJ_EUNSUPPORTED, "the G sphere is too long for the tensor-core kernel's shared-memory tables");
-    if ((rc = tc_upload(P, &P->d_tc_slots, slots))) return rc;
-    if ((rc = tc_upload(P, &P->d_tc_quads, best.quads))) return rc;
-    if ((rc = tc_upload(P, &P->d_tc_map, map))) return rc;
-    if ((rc = tc_upload(P, &P->d_tc_wpairs, wpairs))) return rc;
-    if ((rc = tc_upload(P, &P->d_tc_pos, pos))) return rc;
-    if ((rc = tc_upload(P, &P->d_tc_kpos, kpos))) return rc;
-    if (P->precision == FTCJ_PREC_FP64 && (rc = tc_upload(P, &P->d_tc_korder, korder))) return rc;
+    arena.add(&P->d_tc_slots, slots);
+    arena.add(&P->d_tc_quads, best.quads);
+    arena.add(&P->d_tc_map, map);
+    arena.add(&P->d_tc_wpairs, wpairs);
+    arena.add(&P->d_tc_pos, pos);
+    arena.add(&P->d_tc_kpos, kpos);
+    if (P->precision == FTCJ_PREC_FP64) arena.add(&P->d_tc_korder, korder);
+    arena.add(&P->d_tc_wcnt, wcnt);
+    arena.add(&P->d_tc_boff, boff);
+    arena.add(&P->d_tc_sched, sched);
+    arena.add((int4**)&P->d_tc_winfo, winfo);
+    arena.add(&P->d_tc_clw, std::vector<float>(), (size_t)std::max(1, nwin));
+    arena.add(&P->d_tc_ew, std::vector<int>(), (size_t)std::max(1, nwin) * P->tc_nd);
+    // the back-contraction's, and those of the gradient's sums where ftcj_grad takes the plan and n^5 is exact in FP32
+    if (!P->tc_rho_only && (rc = setup_tc_j(P, 0, arena))) return rc;
+    if (f64 && P->shard_count <= 1 && !P->rec_filter && split_grad_walk_exact(P) && (rc = setup_tc_j(P, 1, arena)))
+        return rc;
+    if ((rc = arena.commit(P))) return rc;
     FTCJ_CUDA(cudaMemcpy(P->d_tc_cl, clk.data(), sizeof(float) * nrec, cudaMemcpyHostToDevice));
     if ((rc = tc_alloc(P, &P->d_tc_tab, sizeof(float4) * nrec * tws))) return rc;
     if ((rc = tc_alloc(P, &P->d_tc_tabk, sizeof(float4) * nrec * tws))) return rc;
@@ -2293,14 +2356,6 @@ int setup_tc(ftcj_plan* P) {
             reinterpret_cast<float4*>(P->d_tc_tabz), reinterpret_cast<float4*>(P->d_tc_tabz3));
         FTCJ_CUDA(cudaGetLastError());
     }
-    if ((rc = tc_upload(P, &P->d_tc_wcnt, wcnt))) return rc;
-    if ((rc = tc_upload(P, &P->d_tc_boff, boff))) return rc;
-    if ((rc = tc_upload(P, &P->d_tc_sched, sched))) return rc;
-    int4* winfo_dev = nullptr;
-    if ((rc = tc_upload(P, &winfo_dev, winfo))) return rc;
-    P->d_tc_winfo = winfo_dev;
-    if ((rc = tc_upload(P, &P->d_tc_clw, std::vector<float>((size_t)std::max(1, nwin), 0.f)))) return rc;
-    if ((rc = tc_alloc(P, (void**)&P->d_tc_ew, sizeof(int) * (size_t)std::max(1, nwin) * P->tc_nd))) return rc;
     if ((rc = tc_alloc(P, &P->d_tc_b, (size_t)bmax * 16))) return rc;
     // columns between a window's blocks and the MMA's multiple of 16 are never written nor read back: finite once
     FTCJ_CUDA(cudaMemset(P->d_tc_b, 0, (size_t)bmax * 16));
@@ -2309,9 +2364,6 @@ int setup_tc(ftcj_plan* P) {
         if ((rc = allow_dynamic_smem(tc_rho_kernel(f64, round_up(2 * nd * P->tc_ncols, 8)),
                                      tc_smem_bytes(slices, P->tc_npad, tws, P->tc_nbuf, P->tc_tslots))))
             return rc;
-    if (!P->tc_rho_only && (rc = setup_tc_j(P, 0))) return rc;
-    // the gradient's sums, where ftcj_grad takes the plan and n^5 is exact in FP32
-    if (f64 && P->shard_count <= 1 && !P->rec_filter && split_grad_walk_exact(P)) return setup_tc_j(P, 1);
     return FTCJ_OK;
 }
 
@@ -2393,7 +2445,7 @@ int tc_rho_launches(const ftcj_plan* P, int nd) {
 // the V_ij tile buffer.  TcBack::on stays false, and the walks run the
 // back-contraction (the gradient's sums), where one density's columns exceed
 // the MMA width or the factor tables exceed shared memory.
-int setup_tc_j(ftcj_plan* P, int extra) {
+int setup_tc_j(ftcj_plan* P, int extra, TcArena& arena) {
     TcBack& B = extra ? P->tcg : P->tcj;
     B.on = false;
     B.extra = extra;
@@ -2496,23 +2548,18 @@ int setup_tc_j(ftcj_plan* P, int extra) {
     B.spp = spp;
     B.grid = std::max(1, std::min(P->num_sms, (int)units.size()));
     const std::vector<int> sched = deal(cost, B.grid);
+    arena.add((int4**)&B.items, units);
+    arena.add((int2**)&B.groups, groups);
+    arena.add(&B.pairs, ipairs);
+    arena.add(&B.sched, sched);
+    arena.add(&B.voff, voff);
+    arena.add(&B.vplace, vplace);
+    arena.add(&B.ev, std::vector<int>(), (size_t)npairs_all * nd_best * P->tc_ncols);
+    arena.add(&B.er, std::vector<int>(), (size_t)npairs_all * nd_best);
     int rc;
-    int4* units_dev = nullptr;
-    if ((rc = tc_upload(P, &units_dev, units))) return rc;
-    B.items = units_dev;
-    int2* groups_dev = nullptr;
-    if ((rc = tc_upload(P, &groups_dev, groups))) return rc;
-    B.groups = groups_dev;
-    if ((rc = tc_upload(P, &B.pairs, ipairs))) return rc;
-    if ((rc = tc_upload(P, &B.sched, sched))) return rc;
-    if ((rc = tc_upload(P, &B.voff, voff))) return rc;
-    if ((rc = tc_upload(P, &B.vplace, vplace))) return rc;
     nvs = std::max(nvs, 1LL);
     if ((rc = tc_alloc(P, &B.vs, sizeof(__nv_bfloat16) * (size_t)nvs))) return rc;
     FTCJ_CUDA(cudaMemset(B.vs, 0, sizeof(__nv_bfloat16) * (size_t)nvs));
-    const size_t nev = (size_t)npairs_all * nd_best * P->tc_ncols;
-    if ((rc = tc_alloc(P, (void**)&B.ev, sizeof(int) * nev))) return rc;
-    if ((rc = tc_alloc(P, (void**)&B.er, sizeof(int) * (size_t)npairs_all * nd_best))) return rc;
     if ((rc = allow_dynamic_smem(tc_j_kernel(f64, extra), tc_j_smem_bytes(slices, npad, tws, nbuf)))) return rc;
     B.on = true;
     return FTCJ_OK;
