@@ -10,6 +10,8 @@ is timed beside it; the diamond-like 240-AO cell (k 4x4x4) is a secondary
 line, checked whole against the CPU oracle.
 
 One step = one whole build from D^k (resident in HBM) to J^k and E_J.
+stdout gets one JSON line with the headline figures; a second one with every
+figure measured (rooflines, phases, the extra workloads' rates) goes to stderr.
 Metric value = pair*G evaluations per second, the unit being one ordered
 screened primitive-shell pair times one G != 0 of the full sphere, times the
 densities of the call.
@@ -578,8 +580,9 @@ def slab_leg(ftcj, W, torch, flush, steps):
             torch.cuda.synchronize()
             out["gradient"] = {"ms_per_step": ms, "value": units / (ms * 1e-3), "unit": UNIT,
                                "note": "one call: fold, Hermite map and rho pass of the plan's form, the adjoint "
-                                       "walk of degree L+1 (double-float where grad_split is 1), then the FP64 "
-                                       "per-centre assembly",
+                                       "sums of degree L+1 (the eight-slice product where grad_contraction is 1, else "
+                                       "a walk, double-float where grad_split is 1), then the FP64 per-centre assembly",
+                               "grad_contraction": int(p.info["grad_contraction"]),
                                "grad_split": int(p.info["grad_split"]),
                                "abs_dEJ_vs_build": float((EJ - E).abs().max()),
                                "max_abs_force": float(G.abs().max()),
@@ -692,6 +695,47 @@ def run_reference(args, world, rank):
     }
     print(json.dumps(line), flush=True)
     return 0
+
+
+def headline(line):
+    """The line for stdout, short enough to be read whole from the end of a log (under 3,000 bytes): the headline
+    figures, and per extra workload and form the time alone.  Everything measured is in the details on stderr."""
+    short = {k: v for k, v in line.items() if not isinstance(v, dict)}
+    short["dtype"] = "bf16 slices (exact level sums), f32x2 sums, f64 setup and E_J" if "bf16" in line["dtype"] else line["dtype"]
+    cfg = line["config"]
+    short["config"] = {k: cfg[k] for k in ("workload", "form", "ndens", "pair_g_units_per_step", "parallelism")}
+    short["config"]["l2"] = f"{L2_FLUSH_BYTES >> 20} MB written between timed steps"
+    for k in ("e2e", "clocks"):
+        short[k] = line[k]
+    roof = line["roofline"]
+    short["roofline"] = {k: roof.get(k) for k in ("bound", "kernel", "achieved", "peak", "unit", "frac", "peak_source")}
+    short["forms"] = {f: {k: r[k] for k in ("ms_per_step", "value", "max_abs_dJ_vs_fp64") if k in r}
+                      for f, r in line["forms"].items()}
+
+    def times(leg):
+        out = {}
+        for k, v in leg.items():
+            if k == "ms_per_step":
+                out[k] = v
+            elif isinstance(v, dict) and times(v):
+                t = times(v)
+                out[k] = t["ms_per_step"] if list(t) == ["ms_per_step"] else t
+        return out
+
+    short["extra_ms"] = {k: times(line[k]) for k in ("diamond", "batch", "gpw", "workloads") if k in line}
+    if "cpu_baseline" in line:
+        b = line["cpu_baseline"]
+        short["cpu_baseline"] = {k: b[k] for k in ("value", "unit", "cores", "kind", "seconds")}
+        short["cpu_baseline"]["sample"] = f"every {CPU_BASELINE_STRIDE}th ordered screened pair, whole sphere"
+
+    def rounded(v):
+        if isinstance(v, float):
+            return float(f"{v:.6g}")
+        if isinstance(v, dict):
+            return {k: rounded(x) for k, x in v.items()}
+        return v
+
+    return {k: v if k in ("value", "ms_per_step", "e2e", "config") else rounded(v) for k, v in short.items()}
 
 
 def main():
@@ -812,7 +856,8 @@ def main():
                        "whole k-mesh transforms of the build (not scaled down), one run"),
             "seconds": r["seconds"], "pair_g_units_in_sample": cu}
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print(json.dumps({"details": line}), file=sys.stderr, flush=True)
+        print(json.dumps(headline(line)), flush=True)
     if dist is not None:
         dist.destroy_process_group()
     return 0

@@ -118,9 +118,12 @@ typedef struct {
                            orthorhombic fully separable case): rho(n) as a sliced bf16 tcgen05 matrix
                            product over (pair record, i, j), split form and orthorhombic cells only
                            (EUNSUPPORTED otherwise), whole sphere (pair_gcut_eps = 0).  The FP64 form
-                           keeps 0 and takes the same product, cut finely enough for errors below FP64
-                           accumulation's, by itself in orthorhombic cells (whole sphere, |n_i| <= 63,
-                           no chunk_points or rho_blocks of the caller's).  So do the structure
+                           keeps 0 and takes the same product by itself in orthorhombic cells (whole
+                           sphere, |n_i| <= 63, no chunk_points or rho_blocks of the caller's, device
+                           memory for it): operands in fixed point to 2^-55 of the largest of their row
+                           or column over up to 512 records, summed exactly, which leaves J^k and E_J a
+                           smaller error than FP64 accumulation does; a rho(G) far below the largest has
+                           fewer bits of its own than the walks give it.  So do the structure
                            factors of a split plan with 0, in place of its walk, where the sphere has
                            at least 512 half-sphere points and 3e6 (record, point) units
                            (ftcj_info.contraction says so).  With 1 the
