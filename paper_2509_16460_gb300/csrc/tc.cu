@@ -1224,9 +1224,9 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf,
     if (*abort_flag) {
         if (tid == 0) atomicOr(g.err, 1);
         // NaN over the group's rows: of this CTA's points at least nobody writes them again
-        for (long long i = tid; i < g.nd * g.ng_half; i += kTcThreadsAll) {
-            const long long d = i / g.ng_half;
-            g.out[((g.d0 + d) * g.out_rows + g.out_row0 + kg) * g.ng_half + (i - d * g.ng_half)] = make_double2(NAN, NAN);
+        for (int d = 0; d < g.nd; ++d) {
+            double2* row = g.out + ((long long)(g.d0 + d) * g.out_rows + g.out_row0 + blockIdx.x) * g.ng_half;
+            for (long long i = tid; i < g.ng_half; i += kTcThreadsAll) row[i] = make_double2(NAN, NAN);
         }
     }
     if (warp == kTcMmaWarp) {
@@ -1995,9 +1995,12 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) 
     __syncthreads();
     if (*abort_flag) {
         if (tid == 0) atomicOr(g.err, 1);
-        // NaN over the terms of the CTA's units: what its own block groups hold nobody writes again
-        for (int ju = j0; ju < j1; ++ju) {
-            const int4 un = __ldg(g.units + __ldg(ulist + ju));
+        // NaN over the terms of the CTA's units: what its own block groups hold nobody writes again (the bounds are read
+        // anew, so that they hold no registers until here)
+        const volatile int* sched = g.sched;
+        const int first = sched[blockIdx.x], last = sched[blockIdx.x + 1];
+        for (int ju = first; ju < last; ++ju) {
+            const int4 un = __ldg(g.units + sched[gridDim.x + 1 + ju]);
             const int L = un.x & 255, part = un.x >> 8;
             const long long cnt = g.cls_start[L + 1] - g.cls_start[L], loc = un.w - g.cls_start[L];
             const int nv = (int)min((long long)kTcM, cnt - loc), nt = nterms(L + E);
