@@ -588,7 +588,7 @@ int create(const ftcj_cell* cell, const ftcj_basis* basis, const int kmesh[3], c
     // The FP64 form runs the same separable contraction where the cell is orthorhombic, with operands cut finely
     // enough for its errors to stay below FP64 accumulation's (tc.cu): GB300 has 64 FP32 lanes and far more tensor
     // throughput for each FP64 lane that the walks would use (both passes: slab of 940 AOs, walks 36.7 ms, contraction
-    // 1.55 ms; diamond cell 2.02 and 0.30 ms; 18 AOs 0.33 and 0.08 ms).
+    // 1.53 ms; diamond cell 2.02 and 0.32 ms; 18 AOs 0.33 and 0.08 ms).
     // A caller's own walk shape, |n_i| above 63 (powers of n exact in FP32 no longer), spheres wider than the MMA
     // and plans short of memory (see ftcj_plan_create) keep the walks.  The split form's walks take the structure factors from it too where
     // the sphere fills the product's tiles of 128 rows and the work its launches (slab 3.03 -> 0.82 ms; 706 half-sphere

@@ -70,7 +70,7 @@
 // exits.
 //
 // What bounds it (molecular crystal, 1056 AOs, 2 densities, GB300): the product
-// takes 1.07 ms, of which the MMAs alone (operands left unformed) need 0.89 ms:
+// takes 1.10 ms, of which the MMAs alone (operands left unformed) need 0.89 ms:
 // their operand reads from shared memory (15 MMAs of N = 96 or 192 per k-step,
 // 123 KB) beside the operand and table writes.  B tiles in global memory cost
 // 0.28 ms more (0.49 GB written).  What took the pass from 4.76 ms there: the
@@ -1117,7 +1117,8 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf,
                     if (lane == d) eref = e;
                 }
             // powers of two of this window's densities (lane d density d's), relative to the sums', 0 where they are
-            // below 2^-126; then of the two outputs of each unit, as the upper halves of two floats
+            // below 2^-126 (the crystal's pass 1350 -> 1378 us against unscaled sums; read after the wait, with an
+            // exponent and a division per output, 1397); then of the two outputs of each unit, as the upper halves of two floats
             const unsigned half = (unsigned)max(min(ew - eref, 0) + 127, 0) << 7;
             unsigned rel[NU];
             int d0 = d00, d1 = d01;
