@@ -590,12 +590,12 @@ int create(const ftcj_cell* cell, const ftcj_basis* basis, const int kmesh[3], c
     // throughput for each FP64 lane that the walks would use (both passes: slab of 940 AOs, walks 36.7 ms, contraction
     // 1.53 ms; diamond cell 2.02 and 0.32 ms; 18 AOs 0.33 and 0.08 ms).
     // A caller's own walk shape, |n_i| above 63 (powers of n exact in FP32 no longer), spheres wider than the MMA
-    // and plans short of memory (see ftcj_plan_create) keep the walks.  The split form's walks take the structure factors from it too where
-    // the sphere fills the product's tiles of 128 rows and the work its launches (slab 3.03 -> 0.82 ms; 706 half-sphere
-    // points, 34,131 records: 174 -> 119 us; 582, 6,695: 55 -> 48; but 230, 111,640: 162 -> 193 and 1,026, 814:
-    // 31 -> 44).
-    const bool whole = P->products && P->ortho && !P->tc && !P->d_rec_gcut && prm->chunk_points <= 0 && prm->rho_blocks <= 0 &&
-                       P->n_abs_max <= kSplitNmax && P->npairs > 0 && P->ng_half > 0;
+    // and plans short of memory (see ftcj_plan_create) keep the walks.  The split form's walks take the structure
+    // factors from it too where the sphere fills the product's tiles of 128 rows and the work its launches (slab 3.03 ->
+    // 0.82 ms; 706 half-sphere points, 34,131 records: 174 -> 119 us; 582, 6,695: 55 -> 48; but 230, 111,640: 162 ->
+    // 193 and 1,026, 814: 31 -> 44).
+    const bool whole = P->products && P->ortho && !P->tc && !P->d_rec_gcut && prm->chunk_points <= 0 &&
+                       prm->rho_blocks <= 0 && P->n_abs_max <= kSplitNmax && P->npairs > 0 && P->ng_half > 0;
     const bool split_rho = P->precision == FTCJ_PREC_SPLIT && P->ng_half >= 512 && P->npairs * P->ng_half >= 3000000;
     const size_t nn = (size_t)P->nao * P->nao, md = (size_t)P->max_dens;
     if (whole && (P->precision == FTCJ_PREC_FP64 || split_rho)) {
