@@ -1117,8 +1117,8 @@ __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_rho(TcArgs g, int nbuf,
                     if (lane == d) eref = e;
                 }
             // powers of two of this window's densities (lane d density d's), relative to the sums', 0 where they are
-            // below 2^-126 (the crystal's pass 1350 -> 1378 us against unscaled sums; read after the wait, with an
-            // exponent and a division per output, 1397); then of the two outputs of each unit, as the upper halves of two floats
+            // below 2^-126; then of the two outputs of each unit, as the upper halves of two floats (the crystal's pass
+            // against unscaled sums: 1348 -> 1375 us; 1383 with an exponent and a remainder per output and window)
             const unsigned half = (unsigned)max(min(ew - eref, 0) + 127, 0) << 7;
             unsigned rel[NU];
             int d0 = d00, d1 = d01;
@@ -1709,7 +1709,8 @@ struct TcJSmem {
 // per slice), lane 0 of warp 16 issues the MMAs, warp 17 brings the factor
 // tables and warp 18 the V_ij stage tiles in with bulk copies; warps 0-15 then
 // form J' from tensor memory (lane quadrant w & 3; (block, density) pairs,
-// their columns split further where a group has fewer than four, w / 4 mod 4).  Waits are bounded as in the structure-factor kernel.
+// their columns split further where a group has fewer than four, w / 4 mod 4).
+// Waits are bounded as in the structure-factor kernel.
 // E = 1: the gradient's sums, one degree above the record's class.
 template <class P, int E>
 __global__ void __launch_bounds__(kTcThreadsAll, 1) k_tc_j(TcJArgs g, int nbuf) {
